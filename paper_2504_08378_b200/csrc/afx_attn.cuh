@@ -4,7 +4,8 @@
 // grid = (S, kv_heads, T), cluster = (S,1,1): the S blocks of a cluster split the L = pos+1
 // cached positions of one (token, kv head) and meet their (max, sum, weighted V) partials
 // through distributed shared memory (softmax in base 2: exp(s) = 2^(s * log2 e)).  The block owning the last position first rotates and
-// stores the current token's k and v into the cache.  head_dim is fixed at 128.
+// stores the current token's k and v into the cache.  head_dim is fixed at 128.  This kernel takes one
+// query head per kv head, the one in afx_attn_mma.cuh several.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -20,7 +21,7 @@ constexpr int kAttnWarps = kAttnThreads / 32;
 constexpr int kAttnWorkers = 2 * kAttnWarps;  // half warps: each walks its own positions
 constexpr int kHeadDim = 128;
 constexpr int kAttnMaxRep = 8;  // query heads per kv head
-constexpr int kAttnUnroll = 4;  // cache rows (K and V each) in flight per half warp (8 with one query head)
+constexpr int kAttnUnroll = 8;  // cache rows (K and V each) in flight per half warp
 
 struct AttnArgs {
     const float* qkv;  // [T][n_qkv] fp32: q heads | k heads | v heads
@@ -33,14 +34,14 @@ struct AttnArgs {
     uint16_t* out;  // [T][q_heads*128] dtype bits
 };
 
+afx_status launch_attention(int dtype, const AttnArgs& a, cudaStream_t st);  // afx_attn.cu
+
 struct AttnSmem {
-    __align__(16) float q[kAttnMaxRep][kHeadDim];     // rotated queries times scale * log2(e)
-    __align__(16) float red[kAttnWorkers][kHeadDim];  // one query head's partial outputs
+    __align__(16) float q[kHeadDim];  // rotated query times scale * log2(e)
+    __align__(16) float red[kAttnWorkers][kHeadDim];
     float red_m[kAttnWorkers];
     float red_l[kAttnWorkers];
-    float part_m[kAttnMaxRep];  // this block's partials, read by the cluster
-    float part_l[kAttnMaxRep];
-    float part_acc[kAttnMaxRep][kHeadDim];
+    float part_m, part_l, part_acc[kHeadDim];  // this block's partials, read by the cluster
 };
 
 __device__ __forceinline__ void unpack8_f16(const uint4& raw, float (&w)[8]) {
@@ -59,12 +60,12 @@ __device__ __forceinline__ float fast_exp2(float x) {
     return y;
 }
 
-// One pass over the cache: every half warp keeps a running (max, sum, weighted V) per query
-// head for the positions it visits (16 lanes x 8 dims = one 128-wide row per load), K and V
+// One query head per kv head.  One pass over the cache: every half warp keeps a running (max, sum,
+// weighted V) for the positions it visits (16 lanes x 8 dims = one 128-wide row per load), K and V
 // rows of kAttnUnroll positions are requested together so that 2 * kAttnUnroll 16-byte loads
 // per lane are in flight; the half warps of a block meet in shared memory, the blocks of a
 // cluster through distributed shared memory, both in a fixed order.
-template <int DT, int REP>
+template <int DT>
 __device__ __forceinline__ void attention_block(const AttnArgs& a, AttnSmem* sm) {
     cg::cluster_group cluster = cg::this_cluster();
     const int S = static_cast<int>(cluster.num_blocks());
@@ -73,36 +74,35 @@ __device__ __forceinline__ void attention_block(const AttnArgs& a, AttnSmem* sm)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int half = lane >> 4, l16 = lane & 15;
     const int worker = 2 * warp + half;
-    const int rep = a.q_heads / a.kv_heads;
     const int L = a.pos + 1;
     const int l_lo = static_cast<int>(static_cast<int64_t>(rank) * L / S);
     const int l_hi = static_cast<int>(static_cast<int64_t>(rank + 1) * L / S);
     const float qscale = rsqrtf(static_cast<float>(kHeadDim)) * 1.4426950408889634f;
     const uint32_t half_mask = 0xFFFFu << (16 * half);  // the two halves of a warp work on different keys
+    constexpr int U = kAttnUnroll;
 
     AFX_TRACE_REGION(0);
     AFX_MARK(0);
+    const size_t row_stride = static_cast<size_t>(a.kv_heads) * kHeadDim;
+    const size_t head_off = static_cast<size_t>(hk) * kHeadDim + l16 * 8;
     uint16_t* kc = a.k_cache + static_cast<size_t>(t) * a.max_seq * a.kv_heads * kHeadDim;
     uint16_t* vc = a.v_cache + static_cast<size_t>(t) * a.max_seq * a.kv_heads * kHeadDim;
-    // With one query head per kv head the registers allow it: the past rows of this half
-    // warp's first batch were written by earlier tokens' attention kernels -- at least one
-    // layer step (five grids) back, so complete by the ordering rule stated in fused_op_block
-    // -- and are requested before the wait for q, k, v.
-    constexpr int U = REP == 1 ? 2 * kAttnUnroll : kAttnUnroll;
-    constexpr bool kEarly = REP == 1;
     uint4 kraw[U], vraw[U];
-    if (kEarly) {
-        const size_t rs = static_cast<size_t>(a.kv_heads) * kHeadDim;
-        const size_t ho = static_cast<size_t>(hk) * kHeadDim + l16 * 8;
+    // rows [from, to) of the batch of positions p0, p0 + kAttnWorkers, ..
+    auto fetch = [&](int p0, int from, int to) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int p = l_lo + worker + u * kAttnWorkers;
-            if (p < l_hi && p < a.pos) {
-                kraw[u] = *reinterpret_cast<const uint4*>(kc + static_cast<size_t>(p) * rs + ho);
-                vraw[u] = *reinterpret_cast<const uint4*>(vc + static_cast<size_t>(p) * rs + ho);
+            const int p = p0 + u * kAttnWorkers;
+            if (p >= from && p < to) {
+                kraw[u] = *reinterpret_cast<const uint4*>(kc + static_cast<size_t>(p) * row_stride + head_off);
+                vraw[u] = *reinterpret_cast<const uint4*>(vc + static_cast<size_t>(p) * row_stride + head_off);
             }
         }
-    }
+    };
+    // The past rows of this half warp's first batch were written by earlier tokens' attention kernels
+    // -- at least one layer step (five grids) back, so complete by the ordering rule stated in
+    // fused_op_block -- and are requested before the wait for q, k, v.
+    fetch(l_lo + worker, 0, min(l_hi, a.pos));
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // only after the wait (see fused_op_block)
     AFX_MARK(1);
@@ -110,16 +110,13 @@ __device__ __forceinline__ void attention_block(const AttnArgs& a, AttnSmem* sm)
     const float* row = a.qkv + static_cast<size_t>(t) * a.n_qkv;
     const float* cs = a.rope_cos + static_cast<size_t>(a.pos) * (kHeadDim / 2);
     const float* sn = a.rope_sin + static_cast<size_t>(a.pos) * (kHeadDim / 2);
-    const size_t row_stride = static_cast<size_t>(a.kv_heads) * kHeadDim;
-    const size_t head_off = static_cast<size_t>(hk) * kHeadDim + l16 * 8;
 
-    // rotated, pre-scaled queries of this kv head's group
-    for (int e = tid; e < rep * (kHeadDim / 2); e += kAttnThreads) {
-        const int r = e / (kHeadDim / 2), i = e - r * (kHeadDim / 2);
-        const float* qh = row + static_cast<size_t>(hk * rep + r) * kHeadDim;
-        const float x0 = qh[2 * i], x1 = qh[2 * i + 1];
-        sm->q[r][2 * i] = (x0 * cs[i] - x1 * sn[i]) * qscale;
-        sm->q[r][2 * i + 1] = (x0 * sn[i] + x1 * cs[i]) * qscale;
+    // rotated, pre-scaled query
+    if (tid < kHeadDim / 2) {
+        const float* qh = row + static_cast<size_t>(hk) * kHeadDim;
+        const float x0 = qh[2 * tid], x1 = qh[2 * tid + 1];
+        sm->q[2 * tid] = (x0 * cs[tid] - x1 * sn[tid]) * qscale;
+        sm->q[2 * tid + 1] = (x0 * sn[tid] + x1 * cs[tid]) * qscale;
     }
     // the block that owns the newest position appends the current k, v (fp16) first
     if (l_hi == L && l_lo < l_hi) {
@@ -138,125 +135,90 @@ __device__ __forceinline__ void attention_block(const AttnArgs& a, AttnSmem* sm)
     }
     __syncthreads();
 
-    float m_run[REP], l_run[REP], acc[REP][8];
+    float m_run = -INFINITY, l_run = 0.0f, acc[8];
 #pragma unroll
-    for (int r = 0; r < REP; ++r) {
-        m_run[r] = -INFINITY;
-        l_run[r] = 0.0f;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[r][j] = 0.0f;
-    }
-
-    // rows of a batch that are not in registers yet: all of them, or (first batch, requested
-    // before the wait) only the row this kernel has just appended
-    auto fetch = [&](int p0, bool only_new) {
+    for (int j = 0; j < 8; ++j) acc[j] = 0.0f;
+    AFX_MARK(2);
+    fetch(l_lo + worker, a.pos, l_hi);  // the first batch's row that this kernel has just appended
+    const float4 qa = *reinterpret_cast<const float4*>(&sm->q[l16 * 8]);
+    const float4 qb = *reinterpret_cast<const float4*>(&sm->q[l16 * 8 + 4]);
+    for (int p0 = l_lo + worker; p0 < l_hi; p0 += kAttnWorkers * U) {
+        float sc[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int p = p0 + u * kAttnWorkers;
-            if (p < l_hi && (!only_new || p >= a.pos)) {
-                kraw[u] = *reinterpret_cast<const uint4*>(kc + static_cast<size_t>(p) * row_stride + head_off);
-                vraw[u] = *reinterpret_cast<const uint4*>(vc + static_cast<size_t>(p) * row_stride + head_off);
+            float d = -INFINITY;
+            if (p0 + u * kAttnWorkers < l_hi) {  // uniform over the half warp
+                float kv[8];
+                unpack8_f16(kraw[u], kv);
+                d = qa.x * kv[0];
+                d = fmaf(qa.y, kv[1], d);
+                d = fmaf(qa.z, kv[2], d);
+                d = fmaf(qa.w, kv[3], d);
+                d = fmaf(qb.x, kv[4], d);
+                d = fmaf(qb.y, kv[5], d);
+                d = fmaf(qb.z, kv[6], d);
+                d = fmaf(qb.w, kv[7], d);
+                d += __shfl_xor_sync(half_mask, d, 8);
+                d += __shfl_xor_sync(half_mask, d, 4);
+                d += __shfl_xor_sync(half_mask, d, 2);
+                d += __shfl_xor_sync(half_mask, d, 1);
+            }
+            sc[u] = d;
+        }
+        float mn = m_run;
+#pragma unroll
+        for (int u = 0; u < U; ++u) mn = fmaxf(mn, sc[u]);
+        const float f = fast_exp2(m_run - mn);  // 0 on the first visit (m_run = -inf)
+        m_run = mn;
+        l_run *= f;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[j] *= f;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (p0 + u * kAttnWorkers < l_hi) {
+                const float pw = fast_exp2(sc[u] - mn);
+                l_run += pw;
+                float vv[8];
+                unpack8_f16(vraw[u], vv);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) acc[j] = fmaf(pw, vv[j], acc[j]);
             }
         }
-    };
-    AFX_MARK(2);
-    fetch(l_lo + worker, kEarly);
-    for (int p0 = l_lo + worker; p0 < l_hi; p0 += kAttnWorkers * U) {
-        float sc[REP][U];
-#pragma unroll
-        for (int r = 0; r < REP; ++r) {
-            if (r < rep) {
-                const float4 qa = *reinterpret_cast<const float4*>(&sm->q[r][l16 * 8]);
-                const float4 qb = *reinterpret_cast<const float4*>(&sm->q[r][l16 * 8 + 4]);
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    float d = -INFINITY;
-                    if (p0 + u * kAttnWorkers < l_hi) {  // uniform over the half warp
-                        float kv[8];
-                        unpack8_f16(kraw[u], kv);
-                        d = qa.x * kv[0];
-                        d = fmaf(qa.y, kv[1], d);
-                        d = fmaf(qa.z, kv[2], d);
-                        d = fmaf(qa.w, kv[3], d);
-                        d = fmaf(qb.x, kv[4], d);
-                        d = fmaf(qb.y, kv[5], d);
-                        d = fmaf(qb.z, kv[6], d);
-                        d = fmaf(qb.w, kv[7], d);
-                        d += __shfl_xor_sync(half_mask, d, 8);
-                        d += __shfl_xor_sync(half_mask, d, 4);
-                        d += __shfl_xor_sync(half_mask, d, 2);
-                        d += __shfl_xor_sync(half_mask, d, 1);
-                    }
-                    sc[r][u] = d;
-                }
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < REP; ++r) {
-            if (r < rep) {
-                float mn = m_run[r];
-#pragma unroll
-                for (int u = 0; u < U; ++u) mn = fmaxf(mn, sc[r][u]);
-                const float f = fast_exp2(m_run[r] - mn);  // 0 on the first visit (m_run = -inf)
-                m_run[r] = mn;
-                l_run[r] *= f;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) acc[r][j] *= f;
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    if (p0 + u * kAttnWorkers < l_hi) {
-                        const float pw = fast_exp2(sc[r][u] - mn);
-                        l_run[r] += pw;
-                        float vv[8];
-                        unpack8_f16(vraw[u], vv);
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) acc[r][j] = fmaf(pw, vv[j], acc[r][j]);
-                    }
-                }
-            }
-        }
-        if (p0 + kAttnWorkers * U < l_hi) fetch(p0 + kAttnWorkers * U, false);
+        if (p0 + kAttnWorkers * U < l_hi) fetch(p0 + kAttnWorkers * U, 0, l_hi);
     }
 
     AFX_MARK(3);
-    // meet the half warps of the block (fixed order), one query head at a time
+    // meet the half warps of the block (fixed order)
+    float4* dst = reinterpret_cast<float4*>(&sm->red[worker][l16 * 8]);
+    dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+    dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+    if (l16 == 0) {
+        sm->red_m[worker] = m_run;
+        sm->red_l[worker] = l_run;
+    }
+    __syncthreads();
+    if (tid <= kHeadDim) {
+        float M = -INFINITY;
 #pragma unroll
-    for (int r = 0; r < REP; ++r) {
-        if (r < rep) {
-            float4* dst = reinterpret_cast<float4*>(&sm->red[worker][l16 * 8]);
-            dst[0] = make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
-            dst[1] = make_float4(acc[r][4], acc[r][5], acc[r][6], acc[r][7]);
-            if (l16 == 0) {
-                sm->red_m[worker] = m_run[r];
-                sm->red_l[worker] = l_run[r];
-            }
-            __syncthreads();
-            if (tid <= kHeadDim) {
-                float M = -INFINITY;
+        for (int g = 0; g < kAttnWorkers; ++g) M = fmaxf(M, sm->red_m[g]);
+        float s = 0.0f;
 #pragma unroll
-                for (int g = 0; g < kAttnWorkers; ++g) M = fmaxf(M, sm->red_m[g]);
-                float s = 0.0f;
-#pragma unroll
-                for (int g = 0; g < kAttnWorkers; ++g) {
-                    // a half warp that saw no position has m = -inf, l = 0, acc = 0
-                    const float w = sm->red_m[g] == -INFINITY ? 0.0f : fast_exp2(sm->red_m[g] - M);
-                    s = fmaf(w, tid < kHeadDim ? sm->red[g][tid] : sm->red_l[g], s);
-                }
-                if (tid < kHeadDim) {
-                    sm->part_acc[r][tid] = s;
-                } else {
-                    sm->part_l[r] = s;
-                    sm->part_m[r] = M;
-                }
-            }
-            __syncthreads();
+        for (int g = 0; g < kAttnWorkers; ++g) {
+            // a half warp that saw no position has m = -inf, l = 0, acc = 0
+            const float w = sm->red_m[g] == -INFINITY ? 0.0f : fast_exp2(sm->red_m[g] - M);
+            s = fmaf(w, tid < kHeadDim ? sm->red[g][tid] : sm->red_l[g], s);
+        }
+        if (tid < kHeadDim) {
+            sm->part_acc[tid] = s;
+        } else {
+            sm->part_l = s;
+            sm->part_m = M;
         }
     }
     AFX_MARK(4);
     cluster.sync();
     AFX_MARK(5);
-    for (int e = rank + S * tid; e < rep * kHeadDim; e += S * kAttnThreads) {
-        const int r = e / kHeadDim, d = e - r * kHeadDim;
+    for (int d = rank + S * tid; d < kHeadDim; d += S * kAttnThreads) {
         // all remote reads first (they are independent), then the merge in block order
         float mq[8], aq[8], lq[8];
 #pragma unroll
@@ -265,9 +227,9 @@ __device__ __forceinline__ void attention_block(const AttnArgs& a, AttnSmem* sm)
             aq[q] = 0.0f;
             lq[q] = 0.0f;
             if (q < S) {
-                mq[q] = cluster.map_shared_rank(&sm->part_m[0], q)[r];
-                aq[q] = cluster.map_shared_rank(&sm->part_acc[0][0], q)[r * kHeadDim + d];
-                lq[q] = cluster.map_shared_rank(&sm->part_l[0], q)[r];
+                mq[q] = *cluster.map_shared_rank(&sm->part_m, q);
+                aq[q] = cluster.map_shared_rank(&sm->part_acc[0], q)[d];
+                lq[q] = *cluster.map_shared_rank(&sm->part_l, q);
             }
         }
         float M = -INFINITY;
@@ -280,7 +242,7 @@ __device__ __forceinline__ void attention_block(const AttnArgs& a, AttnSmem* sm)
             num = fmaf(w, aq[q], num);
             den = fmaf(w, lq[q], den);
         }
-        a.out[static_cast<size_t>(t) * a.q_heads * kHeadDim + static_cast<size_t>(hk * rep + r) * kHeadDim + d] =
+        a.out[static_cast<size_t>(t) * a.q_heads * kHeadDim + static_cast<size_t>(hk) * kHeadDim + d] =
             float_to_bits<DT>(num / den);
     }
     AFX_MARK(6);

@@ -102,6 +102,17 @@ __device__ __forceinline__ uint16_t float_to_bits(float v) {
     }
 }
 
+// Two values rounded to nearest even and packed (a in the low half); NaN becomes the canonical NaN.
+template <int DT>
+__device__ __forceinline__ uint32_t pack2_bits(float a, float b) {
+    uint32_t r;
+    if (DT == AFX_F16)
+        asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+    else
+        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+    return r;
+}
+
 // ---- memory access -------------------------------------------------------------------
 
 // 128-bit streaming read of weights: read-only path, no L1 allocation (each byte is used once).

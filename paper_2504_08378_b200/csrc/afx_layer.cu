@@ -61,20 +61,6 @@ __global__ void __launch_bounds__(kGemvThreads, 2) fused_q4_kernel(FusedArgs a) 
     fused_op_block<DT, 1, PW, CAP, IN, EP, true>(a, dyn, &sel, nullptr);
 }
 
-template <int DT, int REP>
-__global__ void __launch_bounds__(kAttnThreads, REP <= 2 ? 2 : 1) attention_kernel(AttnArgs a) {
-    __shared__ AttnSmem sm;
-    attention_block<DT, REP>(a, &sm);
-}
-
-template <int DT>
-static cudaError_t launch_attention_rep(const cudaLaunchConfig_t& cfg, int rep, const AttnArgs& a) {
-    if (rep <= 1) return cudaLaunchKernelEx(&cfg, attention_kernel<DT, 1>, a);
-    if (rep <= 2) return cudaLaunchKernelEx(&cfg, attention_kernel<DT, 2>, a);
-    if (rep <= 4) return cudaLaunchKernelEx(&cfg, attention_kernel<DT, 4>, a);
-    return cudaLaunchKernelEx(&cfg, attention_kernel<DT, 8>, a);
-}
-
 template <int DT, int TMAX, int IN, int EP>
 static afx_status launch_fused_t(const FusedArgs& a, cudaStream_t st) {
     // staged column offsets are 32-bit counts of 16-byte units
@@ -213,30 +199,6 @@ static afx_status launch_fused_dt(const FusedArgs& a, cudaStream_t st) {
 template <int IN, int EP>
 static afx_status launch_fused(int dtype, const FusedArgs& a, cudaStream_t st) {
     return dtype == AFX_F16 ? launch_fused_dt<AFX_F16, IN, EP>(a, st) : launch_fused_dt<AFX_BF16, IN, EP>(a, st);
-}
-
-static afx_status launch_attention(int dtype, const AttnArgs& a, cudaStream_t st) {
-    // split the cached positions so that kv_heads * T * S blocks fill the machine, S <= 8
-    const int groups = a.kv_heads * a.T;
-    int S = (2 * sm_count() + groups - 1) / groups;
-    S = S < 1 ? 1 : (S > 8 ? 8 : S);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(S, a.kv_heads, a.T);
-    cfg.blockDim = dim3(kAttnThreads, 1, 1);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = S;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
-    const int rep = a.q_heads / a.kv_heads;
-    const cudaError_t e = dtype == AFX_F16 ? launch_attention_rep<AFX_F16>(cfg, rep, a)
-                                           : launch_attention_rep<AFX_BF16>(cfg, rep, a);
-    return e == cudaSuccess ? AFX_OK : AFX_ERR_CUDA;
 }
 
 static size_t align256(size_t b) { return (b + 255) / 256 * 256; }
