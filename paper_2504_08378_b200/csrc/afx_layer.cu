@@ -39,17 +39,7 @@ template <int DT, int TMAX, int IN, int EP, int STAGES, int CAPM, int BPS>
 __global__ void __launch_bounds__(kGemvThreads, BPS) fused_mt_kernel(FusedArgs a) {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ SelectScratch sel;
-    fused_op_block<DT, TMAX, kMtTile, CAPM, IN, EP, false, false, STAGES>(a, dyn, &sel, nullptr);
-}
-
-// The one-token operator for a family of `groups` operators in one grid (mixture of experts).
-template <int DT, int PW, int IN, int EP>
-__global__ void __launch_bounds__(kGemvThreads, 2) fused_family_kernel(FusedArgs a) {
-    constexpr int CAP = FusedShape<1>::kStageCap;
-    extern __shared__ __align__(16) unsigned char dyn[];
-    __shared__ SelectScratch sel;
-    __shared__ GemvRecv<1> recv;
-    fused_op_block<DT, 1, PW, CAP, IN, EP, false, true>(a, dyn, &sel, &recv);
+    fused_op_block<DT, TMAX, kMtTile, CAPM, IN, EP, false, STAGES>(a, dyn, &sel, nullptr);
 }
 
 // The one-token operator over 4-bit rows: tiles of PW = 512, 256 or 128 outputs.
@@ -59,56 +49,6 @@ __global__ void __launch_bounds__(kGemvThreads, 2) fused_q4_kernel(FusedArgs a) 
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ SelectScratch sel;
     fused_op_block<DT, 1, PW, CAP, IN, EP, true>(a, dyn, &sel, nullptr);
-}
-
-template <int DT, int TMAX, int IN, int EP>
-static afx_status launch_fused_t(const FusedArgs& a, cudaStream_t st) {
-    // staged column offsets are 32-bit counts of 16-byte units
-    if (static_cast<uint64_t>(a.K) * static_cast<uint64_t>(a.ldw >> 3) > 0x100000000ull) return AFX_ERR_CAPACITY;
-    const size_t dyn = fused_dyn_smem(IN, a.K, a.T);
-    const void* kerns[3] = {reinterpret_cast<const void*>(fused_op_kernel<DT, TMAX, 256, IN, EP>),
-                            reinterpret_cast<const void*>(fused_op_kernel<DT, TMAX, 128, IN, EP>),
-                            reinterpret_cast<const void*>(fused_op_kernel<DT, TMAX, 64, IN, EP>)};
-    // side outputs, if any, come from one more cluster than there are column tiles
-    FusedArgs b = a;
-    b.side_cluster = (a.idx_out != nullptr || a.count_out != nullptr || a.bitmap_out != nullptr ||
-                      a.xnorm_out != nullptr || a.bitmap_pred != nullptr || a.kth_slot != nullptr ||
-                      (a.kth_multi != nullptr && a.T > 1))
-                         ? 1 : 0;
-    const GemvShapeChoice c = choose_gemv_shape(a.N, kerns, dyn, b.side_cluster);
-    if (c.tiles + b.side_cluster > 65535) return AFX_ERR_CAPACITY;
-    const int rows = c.tiles + b.side_cluster;
-    switch (c.pw) {
-        case 256: return launch_clustered(fused_op_kernel<DT, TMAX, 256, IN, EP>, c.S, rows, dyn, b, st);
-        case 128: return launch_clustered(fused_op_kernel<DT, TMAX, 128, IN, EP>, c.S, rows, dyn, b, st);
-        default: return launch_clustered(fused_op_kernel<DT, TMAX, 64, IN, EP>, c.S, rows, dyn, b, st);
-    }
-}
-
-// `groups` operators of one family (weights from a.wt_table through a.wt_sel[g]) in one grid;
-// one token, no side outputs.
-template <int DT, int IN, int EP>
-static afx_status launch_fused_family_dt(const FusedArgs& a, cudaStream_t st) {
-    if (static_cast<uint64_t>(a.K) * static_cast<uint64_t>(a.ldw >> 3) > 0x100000000ull) return AFX_ERR_CAPACITY;
-    if (a.T != 1 || a.groups < 1 || a.wt_table == nullptr || a.wt_sel == nullptr) return AFX_ERR_INVALID_ARG;
-    const size_t dyn = fused_dyn_smem(IN, a.K, 1);
-    const void* kerns[3] = {reinterpret_cast<const void*>(fused_family_kernel<DT, 256, IN, EP>),
-                            reinterpret_cast<const void*>(fused_family_kernel<DT, 128, IN, EP>),
-                            reinterpret_cast<const void*>(fused_family_kernel<DT, 64, IN, EP>)};
-    FusedArgs b = a;
-    b.side_cluster = 0;
-    const GemvShapeChoice c = choose_gemv_shape(a.N, kerns, dyn, 0, 256, a.groups);
-    if (c.tiles > 65535) return AFX_ERR_CAPACITY;
-    switch (c.pw) {
-        case 256: return launch_clustered(fused_family_kernel<DT, 256, IN, EP>, c.S, c.tiles, dyn, b, st);
-        case 128: return launch_clustered(fused_family_kernel<DT, 128, IN, EP>, c.S, c.tiles, dyn, b, st);
-        default: return launch_clustered(fused_family_kernel<DT, 64, IN, EP>, c.S, c.tiles, dyn, b, st);
-    }
-}
-
-template <int IN, int EP>
-static afx_status launch_fused_family(int dtype, const FusedArgs& a, cudaStream_t st) {
-    return dtype == AFX_F16 ? launch_fused_family_dt<AFX_F16, IN, EP>(a, st) : launch_fused_family_dt<AFX_BF16, IN, EP>(a, st);
 }
 
 // a.Wt = the 4-bit rows, a.ldw = their stride in units of 2 bytes, a.T == 1, a.N % 32 == 0.
@@ -191,7 +131,7 @@ static afx_status launch_fused_mt(const FusedArgs& a, cudaStream_t st) {
 
 template <int DT, int IN, int EP>
 static afx_status launch_fused_dt(const FusedArgs& a, cudaStream_t st) {
-    if (a.T <= 1) return launch_fused_t<DT, 1, IN, EP>(a, st);
+    if (a.T <= 1) return launch_one_token(DT, IN, EP, ONE_TOKEN_PLAIN, a, st);
     if (a.T <= 4) return launch_fused_mt<DT, 4, IN, EP>(a, st);
     return launch_fused_mt<DT, 8, IN, EP>(a, st);
 }
@@ -468,6 +408,7 @@ static afx_status launch_layer_kernel(afx_model* m, int layer, afx_state* s, int
             a.gain = L.g_attn;
             a.xnorm_out = reinterpret_cast<uint16_t*>(s->blob + s->off_xnorm[0]);
             a.ep = {qkv, nullptr, m->n_qkv};
+            a.beside_attention = 1;
             plan_selection(m, s, layer, AFX_OP_QKV, true, &a);
             return launch_fused<IN_NORM, EP_STORE>(d.dtype, a, st);
         case AFX_STEP_ATTN: {  // rotary, cache append, dense attention
@@ -494,6 +435,7 @@ static afx_status launch_layer_kernel(afx_model* m, int layer, afx_state* s, int
             a.N = d.hidden;
             a.x = attn;
             a.ep = {h, nullptr, d.hidden};
+            a.beside_attention = 1;
             plan_selection(m, s, layer, AFX_OP_O, true, &a);
             return launch_fused<IN_X, EP_ACCUM>(d.dtype, a, st);
         case AFX_STEP_GU:  // gate | up, silu(gate) * up
@@ -548,17 +490,16 @@ namespace afx {
 // launch's side-output block writes (normed input, active list, count, cross-layer bookkeeping).
 template <int IN>
 static afx_status launch_select_only(int dtype, const FusedArgs& a, cudaStream_t st) {
+    if (a.T <= 1) return launch_one_token(dtype, IN, EP_STORE, ONE_TOKEN_SELECT, a, st);
     FusedArgs b = a;
     b.side_cluster = 1;
     b.N = 8;  // no column tile is streamed: the grid holds the side-output cluster only
     const size_t dyn = fused_dyn_smem(IN, a.K, a.T);
     auto go = [&](auto kern) { return launch_clustered(kern, 1, 1, dyn, b, st); };
     if (dtype == AFX_F16) {
-        if (a.T <= 1) return go(fused_op_kernel<AFX_F16, 1, 64, IN, EP_STORE>);
         if (a.T <= 4) return go(fused_op_kernel<AFX_F16, 4, 64, IN, EP_STORE>);
         return go(fused_op_kernel<AFX_F16, 8, 64, IN, EP_STORE>);
     }
-    if (a.T <= 1) return go(fused_op_kernel<AFX_BF16, 1, 64, IN, EP_STORE>);
     if (a.T <= 4) return go(fused_op_kernel<AFX_BF16, 4, 64, IN, EP_STORE>);
     return go(fused_op_kernel<AFX_BF16, 8, 64, IN, EP_STORE>);
 }
@@ -808,30 +749,66 @@ template <int DT>
 __global__ void __launch_bounds__(kMoeThreads, 1)
 moe_router_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ Wr, int64_t ldr, int K, int E, int top,
                   MoeWork* __restrict__ w) {
-    __shared__ float part[kMoeThreads / 32][kMoeMaxExperts];
+    constexpr int NW = kMoeThreads / 32, U = 4;
+    __shared__ float part[NW][kMoeMaxExperts + 1];
+    __shared__ float logit[kMoeMaxExperts];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // the experts' operator selects its active channels meanwhile
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     float acc[kMoeMaxExperts];
 #pragma unroll
     for (int e = 0; e < kMoeMaxExperts; ++e) acc[e] = 0.0f;
-    for (int j = threadIdx.x; j < K; j += kMoeThreads) {
-        const float xv = bits_to_float<DT>(x[j]);
-        const uint16_t* row = Wr + static_cast<int64_t>(j) * ldr;
+    if (E == 8 && (ldr & 7) == 0 && (reinterpret_cast<uintptr_t>(Wr) & 15u) == 0) {
+        // a row in one 16-byte load, U rows in flight
+        for (int j0 = threadIdx.x; j0 < K; j0 += U * kMoeThreads) {
+            uint4 raw[U];
+            float xv[U];
 #pragma unroll
-        for (int e = 0; e < kMoeMaxExperts; ++e)
-            if (e < E) acc[e] = fmaf(xv, bits_to_float<DT>(row[e]), acc[e]);
+            for (int u = 0; u < U; ++u) {
+                const int j = j0 + u * kMoeThreads;
+                raw[u] = make_uint4(0u, 0u, 0u, 0u);
+                xv[u] = 0.0f;
+                if (j < K) {
+                    raw[u] = *reinterpret_cast<const uint4*>(Wr + static_cast<int64_t>(j) * ldr);
+                    xv[u] = bits_to_float<DT>(x[j]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint32_t r[4] = {raw[u].x, raw[u].y, raw[u].z, raw[u].w};
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    acc[e] = fmaf(xv[u], bits_to_float<DT>(static_cast<uint16_t>(r[e >> 1] >> (16 * (e & 1)))), acc[e]);
+            }
+        }
+    } else {
+        for (int j = threadIdx.x; j < K; j += kMoeThreads) {
+            const float xv = bits_to_float<DT>(x[j]);
+            const uint16_t* row = Wr + static_cast<int64_t>(j) * ldr;
+#pragma unroll
+            for (int e = 0; e < kMoeMaxExperts; ++e)
+                if (e < E) acc[e] = fmaf(xv, bits_to_float<DT>(row[e]), acc[e]);
+        }
     }
 #pragma unroll
     for (int e = 0; e < kMoeMaxExperts; ++e) {
-        const float v = warp_sum(acc[e]);
-        if (lane_id() == 0) part[warp_id()][e] = v;
+        if (e < E) {
+            const float v = warp_sum(acc[e]);
+            if (lane_id() == 0) part[warp_id()][e] = v;
+        }
+    }
+    __syncthreads();
+    for (int e = warp_id(); e < E; e += NW) {
+        static_assert(NW == 32, "one warp's sum per lane");
+        const float v = warp_sum(part[lane_id()][e]);
+        if (lane_id() == 0) logit[e] = v;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         float lg[kMoeMaxExperts];
         for (int e = 0; e < E; ++e) {
-            float s = 0.0f;
-            for (int g = 0; g < kMoeThreads / 32; ++g) s += part[g][e];
-            lg[e] = s;
-            w->logits[e] = s;
+            lg[e] = logit[e];
+            w->logits[e] = lg[e];
         }
         uint32_t taken = 0;
         float chosen[kMoeMaxTop];
@@ -856,6 +833,8 @@ moe_router_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ W
 __global__ void __launch_bounds__(256) moe_combine_kernel(const float* __restrict__ part, int64_t stride, int top, int n,
                                                           int accumulate, float* __restrict__ y) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (i >= n) return;
     float s = accumulate ? y[i] : 0.0f;
     for (int r = 0; r < top; ++r) s += part[r * stride + i];
@@ -898,11 +877,18 @@ extern "C" afx_status afx_moe_block(const afx_moe_desc* desc, const void* x, flo
     char* hm_base = static_cast<char*>(workspace) + align256(sizeof(MoeWork));
     const uint16_t* xb = static_cast<const uint16_t*>(x);
     const uint16_t* wr = static_cast<const uint16_t*>(d.w_router);
-    if (d.dtype == AFX_F16)
-        moe_router_kernel<AFX_F16><<<1, kMoeThreads, 0, st>>>(xb, wr, d.ld_router, d.hidden, d.n_experts, d.top, w);
-    else
-        moe_router_kernel<AFX_BF16><<<1, kMoeThreads, 0, st>>>(xb, wr, d.ld_router, d.hidden, d.n_experts, d.top, w);
-    if (cudaGetLastError() != cudaSuccess) return AFX_ERR_CUDA;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cfg.gridDim = dim3(1);
+    cfg.blockDim = dim3(kMoeThreads);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, d.dtype == AFX_F16 ? moe_router_kernel<AFX_F16> : moe_router_kernel<AFX_BF16>,
+                                             xb, wr, d.ld_router, d.hidden, d.n_experts, d.top, w);
+    if (e != cudaSuccess) return AFX_ERR_CUDA;
     // the chosen experts' gate | up operators in one grid (the same input, one silu(gate) * up vector each)
     float* part = reinterpret_cast<float*>(hm_base + static_cast<size_t>(d.top) * moe_hm_stride(d));
     afx_status rc;
@@ -917,13 +903,15 @@ extern "C" afx_status afx_moe_block(const afx_moe_desc* desc, const void* x, flo
     a.N = 2 * d.mlp;
     a.x = xb;
     a.x_stride = 0;
+    a.x_early = 1;
     a.k = d.k_gu;
     a.tau = d.tau_gu;
     a.ep = {nullptr, reinterpret_cast<uint16_t*>(hm_base), 2 * d.mlp, nullptr};
     a.out_stride = static_cast<int64_t>(moe_hm_stride(d) / 2);
-    if ((rc = launch_fused_family<IN_X, EP_SILU>(d.dtype, a, st)) != AFX_OK) return rc;
+    if ((rc = launch_one_token(d.dtype, IN_X, EP_SILU, ONE_TOKEN_FAMILY, a, st)) != AFX_OK) return rc;
     // their down projections in one grid, each on the active channels of its own input and
     // weighted by its routing weight, into one partial output per expert
+    a.x_early = 0;
     a.wt_table = reinterpret_cast<const uint16_t* const*>(d.w_down_table);
     a.ldw = d.hidden;
     a.K = d.mlp;
@@ -934,10 +922,13 @@ extern "C" afx_status afx_moe_block(const afx_moe_desc* desc, const void* x, flo
     a.tau = d.tau_down;
     a.ep = {part, nullptr, d.hidden, &w->weight[0]};
     a.out_stride = static_cast<int64_t>(moe_part_stride(d) / 4);
-    if ((rc = launch_fused_family<IN_X, EP_STORE>(d.dtype, a, st)) != AFX_OK) return rc;
+    if ((rc = launch_one_token(d.dtype, IN_X, EP_STORE, ONE_TOKEN_FAMILY, a, st)) != AFX_OK) return rc;
     // the experts' contributions meet in the order of the router's choice
-    moe_combine_kernel<<<(d.hidden + 255) / 256, 256, 0, st>>>(part, a.out_stride, d.top, d.hidden, accumulate ? 1 : 0, y);
-    if (cudaGetLastError() != cudaSuccess) return AFX_ERR_CUDA;
+    cfg.gridDim = dim3((d.hidden + 255) / 256);
+    cfg.blockDim = dim3(256);
+    if (cudaLaunchKernelEx(&cfg, moe_combine_kernel, static_cast<const float*>(part), a.out_stride, d.top, d.hidden, accumulate ? 1 : 0, y) !=
+        cudaSuccess)
+        return AFX_ERR_CUDA;
     return AFX_OK;
 }
 
@@ -1031,16 +1022,3 @@ extern "C" afx_status afx_mlp_block_noalloc(const void* w_gu, const void* w_down
     a.ep = {y, nullptr, hidden};
     return launch_fused<IN_X, EP_STORE>(dtype, a, st);
 }
-
-#ifdef AFX_EXPERIMENT
-// Experiment builds only (not part of the ABI): clusters of S blocks of the bf16 one-token operator (tile width pw,
-// plain input of K channels, h += epilogue) that the occupancy query reports as co-resident.
-extern "C" int afx_internal_max_clusters(int pw, int S, int K) {
-    using namespace afx;
-    const size_t dyn = fused_dyn_smem(IN_X, K, 1);
-    const void* kern = pw == 256 ? reinterpret_cast<const void*>(fused_op_kernel<AFX_BF16, 1, 256, IN_X, EP_ACCUM>)
-                     : pw == 128 ? reinterpret_cast<const void*>(fused_op_kernel<AFX_BF16, 1, 128, IN_X, EP_ACCUM>)
-                                 : reinterpret_cast<const void*>(fused_op_kernel<AFX_BF16, 1, 64, IN_X, EP_ACCUM>);
-    return max_active_clusters(kern, S, dyn);
-}
-#endif

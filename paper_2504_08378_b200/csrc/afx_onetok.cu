@@ -1,0 +1,95 @@
+// Launcher of the one-token sparse operator (afx_slice.cuh).
+#include "afx_launch.cuh"
+#include "afx_slice.cuh"
+
+namespace afx {
+
+template <int DT, int NT, int NW, int CH, int IN, int EP, bool GRP>
+__global__ void __launch_bounds__(NT, 1024 / NT) slice_op_kernel(FusedArgs a) {
+    extern __shared__ __align__(16) unsigned char dyn[];
+    __shared__ RegSelScratch s;
+    slice_op_block<DT, NT, NW, CH, IN, EP, GRP>(a, dyn, &s);
+}
+
+template <int DT, int NT, int NW, int CH, int IN, int EP, bool GRP>
+static afx_status launch_slice(const FusedArgs& a, bool select_only, cudaStream_t st) {
+    if (static_cast<uint64_t>(a.K) * static_cast<uint64_t>(a.ldw >> 3) > 0x100000000ull) return AFX_ERR_CAPACITY;
+    FusedArgs b = a;
+    b.side_cluster = select_only || a.idx_out != nullptr || a.count_out != nullptr || a.bitmap_out != nullptr ||
+                     a.xnorm_out != nullptr || a.bitmap_pred != nullptr || a.kth_slot != nullptr;
+    // one slice per SM, one SM left for the side outputs where there are any; more slices (in waves) only
+    // where one would exceed the widest a block can finish
+    const int groups = GRP ? a.groups : 1;
+    const int sms = sm_count() > 0 ? sm_count() : 148;
+    const int most = slice_max_pieces(NT) / kSlGranule;  // granules per slice
+    const int granules = (a.N / 8 + kSlGranule - 1) / kSlGranule;
+    int nb = (sms - b.side_cluster - (GRP && a.x_early ? 1 : 0)) / groups;  // (that kernel's block keeps one SM busy)
+    if (nb > granules) nb = granules;
+    if (nb < 1) nb = 1;
+    if ((granules + nb - 1) / nb > most) nb = ((granules + most - 1) / most + nb - 1) / nb * nb;
+    if (static_cast<int64_t>(nb) * granules >= 0x7FFFFFFF) return AFX_ERR_CAPACITY;
+    b.slices = nb;
+    size_t dyn = slice_dyn_smem(NT, a.K, a.idx_in != nullptr);
+    if (NT == 512 && dyn < kSlAlone) dyn = kSlAlone;
+    auto kern = slice_op_kernel<DT, NT, NW, CH, IN, EP, GRP>;
+    if (!ensure_dyn_smem(reinterpret_cast<const void*>(kern), dyn)) {
+        cudaGetLastError();
+        return AFX_ERR_CUDA;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((select_only ? 0 : nb * groups) + b.side_cluster, 1, 1);
+    cfg.blockDim = dim3(NT, 1, 1);
+    cfg.dynamicSmemBytes = dyn;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, b) == cudaSuccess ? AFX_OK : AFX_ERR_CUDA;
+}
+
+// Blocks of 512 threads beside the attention: its blocks become resident next to them, request their first
+// rows before the wait and start as soon as the operator's last block ends (4096 -> 12288, attention over
+// 2048 positions, 4096 -> 4096: 35.0 us, with 1024 threads 39.7).  Small operators too, which wait less
+// for fewer warps (1024 -> 5632: 6.2 us, with 1024 threads 8.0).  Elsewhere 1024 threads keep twice
+// the loads in flight (4096 -> 22016: 20.0 us, with 512 threads 24.1), and from K = 4096 on that is worth
+// more than the overlap (8 layers of 8192 channels, 8000 positions: 1573 us, with 512 threads 1613).
+constexpr int kSlNarrowMaxK = 4096;
+// Selecting warps and slots: as few warps as leave a lane enough registers.
+template <int DT, int IN, int EP, bool GRP>
+static afx_status launch_slice_k(const FusedArgs& a, bool select_only, cudaStream_t st) {
+    const bool narrow = (a.beside_attention && a.K <= kSlNarrowMaxK) || static_cast<int64_t>(a.K) * a.N <= (8 << 20);
+    if (narrow && a.K <= 4096) return launch_slice<DT, 512, 8, 4, IN, EP, GRP>(a, select_only, st);
+    if (narrow && a.K <= 12288) return launch_slice<DT, 512, 16, 6, IN, EP, GRP>(a, select_only, st);
+    if (a.K <= 4096) return launch_slice<DT, 1024, 8, 4, IN, EP, GRP>(a, select_only, st);
+    if (a.K <= 12288) return launch_slice<DT, 1024, 16, 6, IN, EP, GRP>(a, select_only, st);
+    if (a.K <= 16384) return launch_slice<DT, 1024, 16, 8, IN, EP, GRP>(a, select_only, st);
+    if (a.K <= 32768) return launch_slice<DT, 1024, 32, 8, IN, EP, GRP>(a, select_only, st);
+    return AFX_ERR_CAPACITY;
+}
+
+template <int DT>
+static afx_status launch_one_token_dt(int in, int ep, OneTokenForm form, const FusedArgs& a, cudaStream_t st) {
+    if (form == ONE_TOKEN_SELECT)
+        return in == IN_NORM ? launch_slice_k<DT, IN_NORM, EP_STORE, false>(a, true, st)
+                             : launch_slice_k<DT, IN_X, EP_STORE, false>(a, true, st);
+    if (form == ONE_TOKEN_FAMILY) {
+        if (a.T != 1 || a.groups < 1 || a.wt_table == nullptr || a.wt_sel == nullptr) return AFX_ERR_INVALID_ARG;
+        return ep == EP_SILU ? launch_slice_k<DT, IN_X, EP_SILU, true>(a, false, st)
+                             : launch_slice_k<DT, IN_X, EP_STORE, true>(a, false, st);
+    }
+    if (in == IN_NORM && ep == EP_STORE) return launch_slice_k<DT, IN_NORM, EP_STORE, false>(a, false, st);
+    if (in == IN_NORM && ep == EP_SILU) return launch_slice_k<DT, IN_NORM, EP_SILU, false>(a, false, st);
+    if (in == IN_X && ep == EP_ACCUM) return launch_slice_k<DT, IN_X, EP_ACCUM, false>(a, false, st);
+    if (in == IN_X && ep == EP_SILU) return launch_slice_k<DT, IN_X, EP_SILU, false>(a, false, st);
+    if (in == IN_X && ep == EP_STORE) return launch_slice_k<DT, IN_X, EP_STORE, false>(a, false, st);
+    return AFX_ERR_UNSUPPORTED;
+}
+
+afx_status launch_one_token(int dtype, int in, int ep, OneTokenForm form, const FusedArgs& a, cudaStream_t st) {
+    return dtype == AFX_F16 ? launch_one_token_dt<AFX_F16>(in, ep, form, a, st)
+                            : launch_one_token_dt<AFX_BF16>(in, ep, form, a, st);
+}
+
+}  // namespace afx
