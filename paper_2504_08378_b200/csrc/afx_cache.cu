@@ -3,9 +3,8 @@
 // The policy of one step runs in ONE thread block (it is integer bookkeeping over at most K
 // channels; what costs time in a step is the host -> device copy of the misses): usage
 // counts and an activity bitmap, ordered compactions (hits/misses in list order, free slots
-// ascending), a bitonic sort of the eviction candidates by (count, channel id), a short
-// sequential pass that pairs misses with candidates exactly as the step-by-step definition
-// does, and the table updates.  A second kernel copies the missed columns from the mapped
+// ascending), a bitonic sort of the eviction candidates by (count, channel id), a pass of one warp
+// that pairs misses with candidates exactly as the step-by-step definition does, and the table updates.  A second kernel copies the missed columns from the mapped
 // host memory with 128-bit loads.
 #include <new>
 #include <vector>
@@ -158,20 +157,42 @@ cache_policy_kernel(CacheTables tb, const int32_t* __restrict__ idx, const int32
             s_mfreq[tid] = static_cast<int>(tb.usage[j]);
         }
         __syncthreads();
-        if (tid == 0) {
-            int vp = s_vp, nt = s_nt;
+        if (warp_id() == 0) {
+            // 32 misses at a time, in runs: as long as misses take candidates, the r-th one left takes candidate
+            // vp + r; as long as they do not, all of them are compared with candidate vp.  One thread
+            // taking them one by one was most of the policy (172 us for 2400 misses; a cached step over 8192 x 8192,
+            // 800 us of it host link: 938 us, with runs 833).
+            const int lane = lane_id();
+            const uint32_t lt = (1u << lane) - 1u;
             const int m = min(static_cast<int>(blockDim.x), n_miss - base);
-            for (int q = 0; q < m; ++q) {
-                if (base + q < n_free) {
-                    s_assign[q] = 0;  // takes free_list[base + q]
-                } else if (vp < n_cand && static_cast<uint32_t>(s_mfreq[q]) >= static_cast<uint32_t>(keys[vp] >> 32)) {
-                    s_assign[q] = vp++;
-                } else {
-                    s_assign[q] = -1 - nt++;
+            int vp = s_vp, nt = s_nt;
+            auto takes = [&](int v, uint32_t f) { return v < n_cand && f >= static_cast<uint32_t>(keys[v] >> 32); };
+            for (int q0 = 0; q0 < m; q0 += 32) {
+                const int q = q0 + lane;
+                const uint32_t f = q < m ? static_cast<uint32_t>(s_mfreq[q]) : 0u;
+                int assign = 0;  // (a miss that takes free_list[base + q])
+                uint32_t left = __ballot_sync(0xFFFFFFFFu, q < m && base + q >= n_free);
+                while (left != 0u) {
+                    const bool mine = (left >> lane) & 1u;
+                    const int r = __popc(left & lt);
+                    const uint32_t no = __ballot_sync(0xFFFFFFFFu, mine && !takes(vp + r, f));
+                    const uint32_t run = left & (no == 0u ? 0xFFFFFFFFu : (no & (0u - no)) - 1u);
+                    if ((run >> lane) & 1u) assign = vp + r;
+                    vp += __popc(run);
+                    left &= ~run;
+                    if (left == 0u) break;
+                    const uint32_t yes = __ballot_sync(0xFFFFFFFFu, ((left >> lane) & 1u) && takes(vp, f));
+                    const uint32_t out = left & (yes == 0u ? 0xFFFFFFFFu : (yes & (0u - yes)) - 1u);
+                    if ((out >> lane) & 1u) assign = -1 - (nt + __popc(out & lt));
+                    nt += __popc(out);
+                    left &= ~out;
                 }
+                if (q < m) s_assign[q] = assign;
             }
-            s_vp = vp;
-            s_nt = nt;
+            if (lane == 0) {
+                s_vp = vp;
+                s_nt = nt;
+            }
         }
         __syncthreads();
         if (i < n_miss) {
