@@ -200,10 +200,19 @@ def _ptr(t):
     return t.data_ptr()
 
 
+_current_raw_stream = None
+
+
 def _stream(stream):
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        # torch.cuda.current_stream() builds a Stream object per call (7 us, half of a small operator's call)
+        global _current_raw_stream
+        if _current_raw_stream is None:
+            import torch
+            torch.cuda.init()
+            device, raw = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
+            _current_raw_stream = lambda: raw(device())
+        return _current_raw_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
