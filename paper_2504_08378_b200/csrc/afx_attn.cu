@@ -18,7 +18,7 @@ __global__ void __launch_bounds__(kAttnMmaThreads, 1) attention_mma_kernel(AttnA
 }
 
 // The largest cluster of at most `most` blocks that keeps all `groups` clusters resident at once.
-static int attn_cluster(const void* kern, size_t dyn, int groups, int most) {
+static int attn_mma_cluster(const void* kern, size_t dyn, int groups, int most) {
     if (most > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
         cudaGetLastError();
         most = 8;
@@ -48,7 +48,7 @@ static afx_status launch_attention_dt(const AttnArgs& a, cudaStream_t st) {
             cudaGetLastError();
             return AFX_ERR_CUDA;
         }
-        S = attn_cluster(kern, dyn, groups, useful < 1 ? 1 : useful > kAttnMaxCluster ? kAttnMaxCluster : useful);
+        S = attn_mma_cluster(kern, dyn, groups, useful < 1 ? 1 : useful > kAttnMaxCluster ? kAttnMaxCluster : useful);
     } else {
         // split the cached positions so that kv_heads * T * S blocks fill the machine, S <= 8
         S = (2 * sm_count() + groups - 1) / groups;

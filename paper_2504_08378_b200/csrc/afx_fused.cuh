@@ -71,10 +71,12 @@ struct FusedArgs {
     int64_t x_stride, out_stride;
 };
 
-// The one-token operator (afx_onetok.cu): a plain operator, `groups` operators of one family, or input stage
-// and selection with the side outputs only.
-enum OneTokenForm { ONE_TOKEN_PLAIN, ONE_TOKEN_FAMILY, ONE_TOKEN_SELECT };
+// The one-token operator (afx_onetok.cu): a plain operator or `groups` operators of one family.
+enum OneTokenForm { ONE_TOKEN_PLAIN, ONE_TOKEN_FAMILY };
 afx_status launch_one_token(int dtype, int in, int ep, OneTokenForm form, const FusedArgs& a, cudaStream_t st);
+
+// Input stage and selection of a.T tokens with the side outputs, as a kernel of its own (afx_seltok.cu).
+afx_status launch_select_tokens(int dtype, bool norm, const FusedArgs& a, cudaStream_t st);
 
 // Dynamic shared memory: [16-bit inputs: T tokens (IN_NORM) or one token (IN_X), each padded
 // to a multiple of 8 elements] [T bitmaps of ceil(K/32) flag words, each padded to 16 bytes: where

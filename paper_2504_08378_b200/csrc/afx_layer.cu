@@ -10,22 +10,6 @@
 
 namespace afx {
 
-template <int TMAX>
-struct FusedShape {
-    static constexpr int kBlocksPerSM = TMAX <= 1 ? 2 : 1;
-    static constexpr int kStageCap = TMAX <= 4 ? 2048 : 1024;
-};
-
-template <int DT, int TMAX, int PW, int IN, int EP>
-__global__ void __launch_bounds__(kGemvThreads, FusedShape<TMAX>::kBlocksPerSM)
-fused_op_kernel(FusedArgs a) {
-    constexpr int CAP = FusedShape<TMAX>::kStageCap;
-    extern __shared__ __align__(16) unsigned char dyn[];
-    __shared__ SelectScratch sel;
-    __shared__ GemvRecv<TMAX> recv;
-    fused_op_block<DT, TMAX, PW, CAP, IN, EP>(a, dyn, &sel, &recv);
-}
-
 // The operator for several tokens per step: the streaming stage runs on the tensor cores.  The
 // block is alone on its SM: staged entries per pass as many as the inputs of TMAX tokens leave room for.
 constexpr int kFusedMtStages = 3, kFusedMtStagesSmall = 2;  // pipeline stages of the several-token operator
@@ -45,7 +29,7 @@ __global__ void __launch_bounds__(kGemvThreads, BPS) fused_mt_kernel(FusedArgs a
 // The one-token operator over 4-bit rows: tiles of PW = 512, 256 or 128 outputs.
 template <int DT, int PW, int IN, int EP>
 __global__ void __launch_bounds__(kGemvThreads, 2) fused_q4_kernel(FusedArgs a) {
-    constexpr int CAP = FusedShape<1>::kStageCap;
+    constexpr int CAP = 2048;
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ SelectScratch sel;
     fused_op_block<DT, 1, PW, CAP, IN, EP, true>(a, dyn, &sel, nullptr);
@@ -129,9 +113,35 @@ static afx_status launch_fused_mt(const FusedArgs& a, cudaStream_t st) {
     return AFX_ERR_CAPACITY;
 }
 
+// Several tokens with room for the list in device memory: the selection of every token on an SM of its own,
+// then the list kernel, two blocks per SM.  In one kernel (launch_fused_mt) every cluster selects for itself
+// over all tokens before it streams, one block per SM.  Four tokens of 5120 channels, 60 %, split and in one:
+// 5120 -> 15360 34.1 and 39.2 us, 5120 -> 5120 22.6 and 24.2, 5120 -> 27648 53.6 and 63.1, 13824 -> 5120
+// 39.9 and 56.6.
+template <int DT, int IN, int EP>
+static afx_status launch_split(const FusedArgs& a, cudaStream_t st) {
+    const afx_status rc = launch_select_tokens(DT, IN == IN_NORM, a, st);
+    if (rc != AFX_OK) return rc;
+    GemvListArgs g = {};
+    g.Wt = a.Wt;
+    g.ldw = a.ldw;
+    g.K = a.K;
+    g.N = a.N;
+    g.T = a.T;
+    g.x = IN == IN_NORM ? a.xnorm_out : a.x;
+    g.idx = a.idx_in != nullptr ? a.idx_in : a.idx_out;
+    g.count = a.idx_in != nullptr ? a.count_in : a.count_out;
+    g.accumulate = EP == EP_ACCUM;
+    g.silu = EP == EP_SILU;
+    g.ep = a.ep;
+    return launch_list_gemv(DT, g, st);
+}
+
 template <int DT, int IN, int EP>
 static afx_status launch_fused_dt(const FusedArgs& a, cudaStream_t st) {
     if (a.T <= 1) return launch_one_token(DT, IN, EP, ONE_TOKEN_PLAIN, a, st);
+    const bool listed = a.idx_in != nullptr || (a.idx_out != nullptr && a.count_out != nullptr);
+    if (listed && (IN == IN_X || a.xnorm_out != nullptr) && a.K <= kSelectFastMaxK) return launch_split<DT, IN, EP>(a, st);
     if (a.T <= 4) return launch_fused_mt<DT, 4, IN, EP>(a, st);
     return launch_fused_mt<DT, 8, IN, EP>(a, st);
 }
@@ -486,24 +496,6 @@ extern "C" afx_status afx_layer_kernel(afx_model* m, int layer, afx_state* s, in
 
 namespace afx {
 
-// Input stage + selection of one operator WITHOUT its GEMV: one block that writes what a fused
-// launch's side-output block writes (normed input, active list, count, cross-layer bookkeeping).
-template <int IN>
-static afx_status launch_select_only(int dtype, const FusedArgs& a, cudaStream_t st) {
-    if (a.T <= 1) return launch_one_token(dtype, IN, EP_STORE, ONE_TOKEN_SELECT, a, st);
-    FusedArgs b = a;
-    b.side_cluster = 1;
-    b.N = 8;  // no column tile is streamed: the grid holds the side-output cluster only
-    const size_t dyn = fused_dyn_smem(IN, a.K, a.T);
-    auto go = [&](auto kern) { return launch_clustered(kern, 1, 1, dyn, b, st); };
-    if (dtype == AFX_F16) {
-        if (a.T <= 4) return go(fused_op_kernel<AFX_F16, 4, 64, IN, EP_STORE>);
-        return go(fused_op_kernel<AFX_F16, 8, 64, IN, EP_STORE>);
-    }
-    if (a.T <= 4) return go(fused_op_kernel<AFX_BF16, 4, 64, IN, EP_STORE>);
-    return go(fused_op_kernel<AFX_BF16, 8, 64, IN, EP_STORE>);
-}
-
 }  // namespace afx
 
 extern "C" afx_status afx_layer_step_hosted(afx_model* m, int layer, afx_state* s, int pos, const afx_hosted_ops* ops,
@@ -557,7 +549,7 @@ extern "C" afx_status afx_layer_step_hosted(afx_model* m, int layer, afx_state* 
             x16 = a.x;
         }
         plan_selection(m, s, layer, op, true, &a);
-        rc = norm ? launch_select_only<IN_NORM>(d.dtype, a, st) : launch_select_only<IN_X>(d.dtype, a, st);
+        rc = launch_select_tokens(d.dtype, norm, a, st);
         if (rc != AFX_OK) return rc;
         const int32_t* idx = a.idx_out;
         const int32_t* count = stats + (static_cast<size_t>(layer) * 4 + op) * 4;

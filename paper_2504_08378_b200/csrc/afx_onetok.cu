@@ -12,10 +12,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) slice_op_kernel(FusedArgs a) {
 }
 
 template <int DT, int NT, int NW, int CH, int IN, int EP, bool GRP>
-static afx_status launch_slice(const FusedArgs& a, bool select_only, cudaStream_t st) {
+static afx_status launch_slice(const FusedArgs& a, cudaStream_t st) {
     if (static_cast<uint64_t>(a.K) * static_cast<uint64_t>(a.ldw >> 3) > 0x100000000ull) return AFX_ERR_CAPACITY;
     FusedArgs b = a;
-    b.side_cluster = select_only || a.idx_out != nullptr || a.count_out != nullptr || a.bitmap_out != nullptr ||
+    b.side_cluster = a.idx_out != nullptr || a.count_out != nullptr || a.bitmap_out != nullptr ||
                      a.xnorm_out != nullptr || a.bitmap_pred != nullptr || a.kth_slot != nullptr;
     // one slice per SM, one SM left for the side outputs where there are any; more slices (in waves) only
     // where one would exceed the widest a block can finish
@@ -37,7 +37,7 @@ static afx_status launch_slice(const FusedArgs& a, bool select_only, cudaStream_
         return AFX_ERR_CUDA;
     }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((select_only ? 0 : nb * groups) + b.side_cluster, 1, 1);
+    cfg.gridDim = dim3(nb * groups + b.side_cluster, 1, 1);
     cfg.blockDim = dim3(NT, 1, 1);
     cfg.dynamicSmemBytes = dyn;
     cfg.stream = st;
@@ -58,32 +58,29 @@ static afx_status launch_slice(const FusedArgs& a, bool select_only, cudaStream_
 constexpr int kSlNarrowMaxK = 4096;
 // Selecting warps and slots: as few warps as leave a lane enough registers.
 template <int DT, int IN, int EP, bool GRP>
-static afx_status launch_slice_k(const FusedArgs& a, bool select_only, cudaStream_t st) {
+static afx_status launch_slice_k(const FusedArgs& a, cudaStream_t st) {
     const bool narrow = (a.beside_attention && a.K <= kSlNarrowMaxK) || static_cast<int64_t>(a.K) * a.N <= (8 << 20);
-    if (narrow && a.K <= 4096) return launch_slice<DT, 512, 8, 4, IN, EP, GRP>(a, select_only, st);
-    if (narrow && a.K <= 12288) return launch_slice<DT, 512, 16, 6, IN, EP, GRP>(a, select_only, st);
-    if (a.K <= 4096) return launch_slice<DT, 1024, 8, 4, IN, EP, GRP>(a, select_only, st);
-    if (a.K <= 12288) return launch_slice<DT, 1024, 16, 6, IN, EP, GRP>(a, select_only, st);
-    if (a.K <= 16384) return launch_slice<DT, 1024, 16, 8, IN, EP, GRP>(a, select_only, st);
-    if (a.K <= 32768) return launch_slice<DT, 1024, 32, 8, IN, EP, GRP>(a, select_only, st);
+    if (narrow && a.K <= 4096) return launch_slice<DT, 512, 8, 4, IN, EP, GRP>(a, st);
+    if (narrow && a.K <= 12288) return launch_slice<DT, 512, 16, 6, IN, EP, GRP>(a, st);
+    if (a.K <= 4096) return launch_slice<DT, 1024, 8, 4, IN, EP, GRP>(a, st);
+    if (a.K <= 12288) return launch_slice<DT, 1024, 16, 6, IN, EP, GRP>(a, st);
+    if (a.K <= 16384) return launch_slice<DT, 1024, 16, 8, IN, EP, GRP>(a, st);
+    if (a.K <= 32768) return launch_slice<DT, 1024, 32, 8, IN, EP, GRP>(a, st);
     return AFX_ERR_CAPACITY;
 }
 
 template <int DT>
 static afx_status launch_one_token_dt(int in, int ep, OneTokenForm form, const FusedArgs& a, cudaStream_t st) {
-    if (form == ONE_TOKEN_SELECT)
-        return in == IN_NORM ? launch_slice_k<DT, IN_NORM, EP_STORE, false>(a, true, st)
-                             : launch_slice_k<DT, IN_X, EP_STORE, false>(a, true, st);
     if (form == ONE_TOKEN_FAMILY) {
         if (a.T != 1 || a.groups < 1 || a.wt_table == nullptr || a.wt_sel == nullptr) return AFX_ERR_INVALID_ARG;
-        return ep == EP_SILU ? launch_slice_k<DT, IN_X, EP_SILU, true>(a, false, st)
-                             : launch_slice_k<DT, IN_X, EP_STORE, true>(a, false, st);
+        return ep == EP_SILU ? launch_slice_k<DT, IN_X, EP_SILU, true>(a, st)
+                             : launch_slice_k<DT, IN_X, EP_STORE, true>(a, st);
     }
-    if (in == IN_NORM && ep == EP_STORE) return launch_slice_k<DT, IN_NORM, EP_STORE, false>(a, false, st);
-    if (in == IN_NORM && ep == EP_SILU) return launch_slice_k<DT, IN_NORM, EP_SILU, false>(a, false, st);
-    if (in == IN_X && ep == EP_ACCUM) return launch_slice_k<DT, IN_X, EP_ACCUM, false>(a, false, st);
-    if (in == IN_X && ep == EP_SILU) return launch_slice_k<DT, IN_X, EP_SILU, false>(a, false, st);
-    if (in == IN_X && ep == EP_STORE) return launch_slice_k<DT, IN_X, EP_STORE, false>(a, false, st);
+    if (in == IN_NORM && ep == EP_STORE) return launch_slice_k<DT, IN_NORM, EP_STORE, false>(a, st);
+    if (in == IN_NORM && ep == EP_SILU) return launch_slice_k<DT, IN_NORM, EP_SILU, false>(a, st);
+    if (in == IN_X && ep == EP_ACCUM) return launch_slice_k<DT, IN_X, EP_ACCUM, false>(a, st);
+    if (in == IN_X && ep == EP_SILU) return launch_slice_k<DT, IN_X, EP_SILU, false>(a, st);
+    if (in == IN_X && ep == EP_STORE) return launch_slice_k<DT, IN_X, EP_STORE, false>(a, st);
     return AFX_ERR_UNSUPPORTED;
 }
 

@@ -1,18 +1,14 @@
 // afx_select_active / afx_diff_active: stand-alone selection and cross-layer set difference.
 #include "afx_launch.cuh"
+#include "afx_fused.cuh"
 #include "afx_select.cuh"
 
 namespace afx {
 
 constexpr int kSelectThreads = 1024;
 
-// Dynamic shared memory.  Fast path: [flag words, padded to 16 bytes] [one token's keys] [key
-// histogram].  Large-K path: flag words only.
-static size_t select_dyn_smem(int K) {
-    size_t b = (static_cast<size_t>((K + 31) >> 5) * 4 + 15) / 16 * 16;
-    if (K <= kSelectFastMaxK) b += (static_cast<size_t>(K) + 7) / 8 * 8 * 2 + kKeyHistBytes;
-    return b;
-}
+// Dynamic shared memory of the kernel for K > kSelectFastMaxK: flag words.
+static size_t select_dyn_smem(int K) { return (static_cast<size_t>((K + 31) >> 5) * 4 + 15) / 16 * 16; }
 
 template <int DT>
 __global__ void __launch_bounds__(kSelectThreads, 1)
@@ -21,32 +17,8 @@ select_kernel(const uint16_t* __restrict__ x, int K, int T, int mode, int k, flo
     extern __shared__ __align__(16) unsigned char s_dyn[];
     __shared__ SelectScratch scratch;
     const int nwords = (K + 31) >> 5;
-    const size_t flag_bytes = (static_cast<size_t>(nwords) * 4 + 15) / 16 * 16;
     uint32_t* s_flags = reinterpret_cast<uint32_t*>(s_dyn);
     const int lane = lane_id();
-    if (K <= kSelectFastMaxK) {
-        uint16_t* xs = reinterpret_cast<uint16_t*>(s_dyn + flag_bytes);
-        uint32_t* hist = reinterpret_cast<uint32_t*>(s_dyn + flag_bytes + (static_cast<size_t>(K) + 7) / 8 * 8 * 2);
-        const bool topk = mode == AFX_MODE_TOPK && k > 0 && k < K;
-        if (topk) block_clear_key_hist<kSelectThreads>(hist);
-        unsigned long long fl = 0ull;
-        int pos0 = 0, total = 0;
-        for (int t = 0; t < T; ++t) {
-            if (t > 0) __syncthreads();  // the previous token's keys are still being read
-            block_stage_token(x + static_cast<size_t>(t) * K, K, xs);
-            fl |= block_token_flags<DT, kSelectThreads>(xs, K, mode, k, tau, hist, t == 0, &scratch, T == 1,
-                                                        pos0, total);
-        }
-        if (T > 1) pos0 = block_prefix(__popcll(fl), scratch.wtot[2], total);
-        for_each_owned_active(fl, K, pos0, [&](int j, int pos) { idx[pos] = j; });
-        if (threadIdx.x == 0) *count = total;
-        if (bitmap != nullptr) {
-            store_flag_bytes(fl, K, s_flags);
-            __syncthreads();
-            for (int w = threadIdx.x; w < nwords; w += blockDim.x) bitmap[w] = s_flags[w];
-        }
-        return;
-    }
     int w0, w1;
     warp_word_range(nwords, w0, w1);
     int mine = 0;
@@ -134,6 +106,19 @@ extern "C" afx_status afx_select_active(const void* x, int dtype, int K, int T, 
     if ((reinterpret_cast<uintptr_t>(x) & 1u) || (reinterpret_cast<uintptr_t>(idx) & 3u) ||
         (reinterpret_cast<uintptr_t>(count) & 3u) || (reinterpret_cast<uintptr_t>(bitmap) & 3u))
         return AFX_ERR_ALIGNMENT;
+    if (K <= kSelectFastMaxK) {
+        FusedArgs a = {};
+        a.K = K;
+        a.T = T;
+        a.x = static_cast<const uint16_t*>(x);
+        a.mode = mode;
+        a.k = k;
+        a.tau = tau;
+        a.idx_out = idx;
+        a.count_out = count;
+        a.bitmap_out = bitmap;
+        return launch_select_tokens(dtype, false, a, static_cast<cudaStream_t>(stream));
+    }
     const size_t smem = select_dyn_smem(K);
     auto kern = dtype == AFX_F16 ? select_kernel<AFX_F16> : select_kernel<AFX_BF16>;
     if (!ensure_dyn_smem(reinterpret_cast<const void*>(kern), smem)) {

@@ -92,7 +92,7 @@ __device__ __forceinline__ void st_shared_if(uint32_t at, uint32_t v, bool on) {
 // warps select, with up to CH slots of 4 channels per lane (K <= 128 NW CH).
 template <int DT, int NT, int NW, int CH, int IN, int EP, bool GRP>
 __device__ __forceinline__ void slice_op_block(const FusedArgs& a, unsigned char* dyn, RegSelScratch* sc) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = tid >> 5;
     const int K = a.K, m = sel_slots<NW>(K);
     const bool selects = NW == NT / 32 || warp < NW;
     const int nb = a.slices, grp = GRP ? static_cast<int>(blockIdx.x) / nb : 0, b = static_cast<int>(blockIdx.x) - grp * nb;
@@ -116,10 +116,8 @@ __device__ __forceinline__ void slice_op_block(const FusedArgs& a, unsigned char
     // this operator (or by this launch's own scribe: only a better hint).
     constexpr bool kEarlyGain = IN == IN_NORM && CH < 8;
     float4 gv[kEarlyGain ? CH : 1];
-    if (kEarlyGain && selects) {
-#pragma unroll
-        for (int i = 0; i < CH; ++i)
-            if (i < m && sel_channel(m, i) < K) gv[i] = *reinterpret_cast<const float4*>(a.gain + sel_channel(m, i));
+    if constexpr (kEarlyGain) {
+        if (selects) sel_load_gain<CH>(a.gain, K, m, gv);
     }
     uint32_t hint = kNoHint;
     if (own && a.kth_slot != nullptr) {
@@ -146,52 +144,16 @@ __device__ __forceinline__ void slice_op_block(const FusedArgs& a, unsigned char
     }
     if (selects) {
         uint32_t kw[2 * CH];
-        if (IN == IN_NORM) {  // x = round(h / rms(h) * gain); K % 8 == 0
-            float4 hv[CH];
-            float ss = 0.0f;
-#pragma unroll
-            for (int i = 0; i < CH; ++i) {
-                hv[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                if (i < m && sel_channel(m, i) < K) hv[i] = *reinterpret_cast<const float4*>(a.h + sel_channel(m, i));
-            }
-#pragma unroll
-            for (int i = 0; i < CH; ++i) {
-                ss = fmaf(hv[i].x, hv[i].x, ss);
-                ss = fmaf(hv[i].y, hv[i].y, ss);
-                ss = fmaf(hv[i].z, hv[i].z, ss);
-                ss = fmaf(hv[i].w, hv[i].w, ss);
-            }
-            ss = warp_sum(ss);
-            if (lane == 0) sc->sum[warp] = ss;
-            sel_barrier<NW>();
-            float tot = 0.0f;
-#pragma unroll
-            for (int w = 0; w < NW; w += 4) {
-                const float4 v = *reinterpret_cast<const float4*>(sc->sum + w);
-                tot += (v.x + v.y) + (v.z + v.w);
-            }
-            const float inv = 1.0f / sqrtf(tot / static_cast<float>(K) + a.eps);
-#pragma unroll
-            for (int i = 0; i < CH; ++i) {
-                kw[2 * i] = 0u;
-                kw[2 * i + 1] = 0u;
-                const int j = sel_channel(m, i);
-                if (i < m && j < K) {
-                    const float4 gn = kEarlyGain ? gv[kEarlyGain ? i : 0] : *reinterpret_cast<const float4*>(a.gain + j);
-                    kw[2 * i] = pack2_bits<DT>(hv[i].x * inv * gn.x, hv[i].y * inv * gn.y);
-                    kw[2 * i + 1] = pack2_bits<DT>(hv[i].z * inv * gn.z, hv[i].w * inv * gn.w);
-                    if (scribe && a.xnorm_out != nullptr)
-                        *reinterpret_cast<uint2*>(a.xnorm_out + j) = make_uint2(kw[2 * i], kw[2 * i + 1]);
-                }
-            }
-        } else {
+        if (IN == IN_NORM)
+            sel_norm_keys<DT, NW, CH, kEarlyGain>(a.h, a.gain, gv, a.eps, K, m, sc, scribe ? a.xnorm_out : nullptr, kw);
+        else
             sel_load_keys<CH>(x, K, m, kw);
-        }
         AFX_MARK(2);
         if (own) {
-            int kth;
+            int kth, at, n;
             const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(list));
-            const int n = sel_select<DT, NW, CH>(kw, m, K, a.mode, a.k, a.tau, hint, sc, kth, [&](int i, int e, int pos, bool on) {
+            const uint32_t fl = sel_flags<DT, NW, CH>(kw, m, K, a.mode, a.k, a.tau, hint, sc, kth, at, n);
+            sel_emit<CH>(fl, m, at, [&](int i, int e, int pos, bool on) {
                 st_shared_if(base + 4 * pos, __byte_perm(kw[2 * i + (e >> 1)], static_cast<uint32_t>(sel_channel(m, i) + e), (e & 1) ? 0x3254 : 0x1054), on);
             });
             if (tid == 0) {

@@ -169,12 +169,12 @@ __device__ __forceinline__ int tau_key(float tau) {
     return static_cast<int>((__float_as_uint(tau) >> 16) & 0x7FFFu);
 }
 
-// Calls emit(slot, element, position, active) for the lane's channels -- the active ones' positions ascend
-// with the channel over the NW warps -- and returns the list's length.  Every thread of the NW warps calls
-// it.  `kth` receives the k-th key where one was searched (top-k with 0 < k < K), else 0.
-template <int DT, int NW, int CH, class Emit>
-__device__ __forceinline__ int sel_select(const uint32_t (&kw)[2 * CH], int m, int K, int mode, int k, float tau,
-                                          uint32_t hint, RegSelScratch* sc, int& kth, Emit emit) {
+// Flags (sel_bit) of the lane's active channels; `at` = the list position of the warp's first one,
+// `count` = the list's length.  Every thread of the NW warps calls it.  `kth` receives the k-th key where
+// one was searched (top-k with 0 < k < K), else 0.
+template <int DT, int NW, int CH>
+__device__ __forceinline__ uint32_t sel_flags(const uint32_t (&kw)[2 * CH], int m, int K, int mode, int k, float tau,
+                                              uint32_t hint, RegSelScratch* sc, int& kth, int& at, int& count) {
     static_assert(CH <= 8, "flags of one lane in a word");
     const int lane = lane_id(), warp = warp_id();
     const uint32_t lt = (1u << lane) - 1u;
@@ -238,13 +238,22 @@ __device__ __forceinline__ int sel_select(const uint32_t (&kw)[2 * CH], int m, i
         }
     }
     AFX_MARK(10);
+    at = static_cast<int>(pre >> 16) + min(pre_e, need_eq);
+    count = static_cast<int>(tot >> 16) + need_eq;
+    return fl;
+}
+
+// Calls emit(slot, element, position, active) for the lane's channels; the active ones' positions ascend with
+// the channel, from `at` for the warp's first.
+template <int CH, class Emit>
+__device__ __forceinline__ void sel_emit(uint32_t fl, int m, int at, Emit emit) {
+    const int lane = lane_id();
     // Active channels per slot, four slots to a word (bytes 0..3 = slots 0, 2, 1, 3, then 4, 6, 5, 7), and
     // their prefix over the lanes (a slot of a warp has at most 128).
     const uint32_t pairs = (fl & 0x55555555u) + ((fl >> 1) & 0x55555555u);
     uint32_t ev = pairs & 0x33333333u, od = (pairs >> 2) & 0x33333333u;  // slots 0, 2, 4, 6 and 1, 3, 5, 7
     ev += ev >> 16;
     od += od >> 16;
-    int at = static_cast<int>(pre >> 16) + min(pre_e, need_eq);
 #pragma unroll
     for (int h = 0; h < (CH + 3) / 4; ++h) {
         if (4 * h < m) {
@@ -273,7 +282,55 @@ __device__ __forceinline__ int sel_select(const uint32_t (&kw)[2 * CH], int m, i
             }
         }
     }
-    return static_cast<int>(tot >> 16) + need_eq;
+}
+
+// What a layer operator reads: x = round(h / rms(h) * gain), the lane's channels as sel_load_keys leaves them
+// (K % 8 == 0).  gv: the gains (sel_load_gain), or, with EARLY false, nothing: they are read here.
+template <int CH>
+__device__ __forceinline__ void sel_load_gain(const float* gain, int K, int m, float4 (&gv)[CH]) {
+#pragma unroll
+    for (int i = 0; i < CH; ++i)
+        if (i < m && sel_channel(m, i) < K) gv[i] = *reinterpret_cast<const float4*>(gain + sel_channel(m, i));
+}
+template <int DT, int NW, int CH, bool EARLY>
+__device__ __forceinline__ void sel_norm_keys(const float* h, const float* gain, const float4 (&gv)[EARLY ? CH : 1], float eps,
+                                              int K, int m, RegSelScratch* sc, uint16_t* xnorm_out, uint32_t (&kw)[2 * CH]) {
+    float4 hv[CH];
+    float ss = 0.0f;
+#pragma unroll
+    for (int i = 0; i < CH; ++i) {
+        hv[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (i < m && sel_channel(m, i) < K) hv[i] = *reinterpret_cast<const float4*>(h + sel_channel(m, i));
+    }
+#pragma unroll
+    for (int i = 0; i < CH; ++i) {
+        ss = fmaf(hv[i].x, hv[i].x, ss);
+        ss = fmaf(hv[i].y, hv[i].y, ss);
+        ss = fmaf(hv[i].z, hv[i].z, ss);
+        ss = fmaf(hv[i].w, hv[i].w, ss);
+    }
+    ss = warp_sum(ss);
+    if (lane_id() == 0) sc->sum[warp_id()] = ss;
+    sel_barrier<NW>();
+    float tot = 0.0f;
+#pragma unroll
+    for (int w = 0; w < NW; w += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(sc->sum + w);
+        tot += (v.x + v.y) + (v.z + v.w);
+    }
+    const float inv = 1.0f / sqrtf(tot / static_cast<float>(K) + eps);
+#pragma unroll
+    for (int i = 0; i < CH; ++i) {
+        kw[2 * i] = 0u;
+        kw[2 * i + 1] = 0u;
+        const int j = sel_channel(m, i);
+        if (i < m && j < K) {
+            const float4 gn = EARLY ? gv[EARLY ? i : 0] : *reinterpret_cast<const float4*>(gain + j);
+            kw[2 * i] = pack2_bits<DT>(hv[i].x * inv * gn.x, hv[i].y * inv * gn.y);
+            kw[2 * i + 1] = pack2_bits<DT>(hv[i].z * inv * gn.z, hv[i].w * inv * gn.w);
+            if (xnorm_out != nullptr) *reinterpret_cast<uint2*>(xnorm_out + j) = make_uint2(kw[2 * i], kw[2 * i + 1]);
+        }
+    }
 }
 
 }  // namespace afx
