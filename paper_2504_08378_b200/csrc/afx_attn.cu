@@ -4,11 +4,11 @@
 
 namespace afx {
 
-// One query head per kv head: dot products on the fp32 pipe.
-template <int DT>
-__global__ void __launch_bounds__(kAttnThreads, 2) attention_kernel(AttnArgs a) {
+// One query head per kv head: dot products on the fp32 pipe, U cache rows in flight per half warp.
+template <int DT, int U>
+__global__ void __launch_bounds__(kAttnThreads, U == 8 ? 2 : 3) attention_kernel(AttnArgs a) {
     __shared__ AttnSmem sm;
-    attention_block<DT>(a, &sm);
+    attention_block<DT, U>(a, &sm);
 }
 
 template <int DT>
@@ -36,10 +36,17 @@ static afx_status launch_attention_dt(const AttnArgs& a, cudaStream_t st) {
     // One query head uses an eighth of their rows, and the fp32 pipe keeps up (kv 32, 2048 positions: 11.3
     // and 12.3 us; kv 40, four tokens: 47.1 and 52.6).
     const bool mma = a.q_heads > a.kv_heads;
+    // one query head: split the cached positions so that kv_heads * T * S blocks fill the machine, S <= 8
+    int S = (2 * sm_count() + groups - 1) / groups;
+    S = S < 1 ? 1 : (S > 8 ? 8 : S);
+    // Two blocks per SM with 8 cache rows of K and V in flight per half warp, where all of them are resident that
+    // way; where some would stream alone in a second wave, three per SM with 4 rows (kv 40, four tokens, 2048
+    // positions, 320 blocks: 45.8 and 32.5 us).
+    const bool deep = groups * S <= 2 * sm_count();
     const void* kern = mma ? reinterpret_cast<const void*>(attention_mma_kernel<DT>)
-                           : reinterpret_cast<const void*>(attention_kernel<DT>);
+                           : deep ? reinterpret_cast<const void*>(attention_kernel<DT, 8>)
+                                  : reinterpret_cast<const void*>(attention_kernel<DT, 4>);
     size_t dyn = 0;
-    int S;
     if (mma) {
         // as many blocks as find a tile for every warp, at most what is resident in one wave
         const int useful = (a.pos + kAttnTile * kAttnMmaWarps - 1) / (kAttnTile * kAttnMmaWarps);
@@ -49,10 +56,6 @@ static afx_status launch_attention_dt(const AttnArgs& a, cudaStream_t st) {
             return AFX_ERR_CUDA;
         }
         S = attn_mma_cluster(kern, dyn, groups, useful < 1 ? 1 : useful > kAttnMaxCluster ? kAttnMaxCluster : useful);
-    } else {
-        // split the cached positions so that kv_heads * T * S blocks fill the machine, S <= 8
-        S = (2 * sm_count() + groups - 1) / groups;
-        S = S < 1 ? 1 : (S > 8 ? 8 : S);
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(S, a.kv_heads, a.T);
@@ -69,7 +72,8 @@ static afx_status launch_attention_dt(const AttnArgs& a, cudaStream_t st) {
     cfg.attrs = attr;
     cfg.numAttrs = 2;
     const cudaError_t e = mma ? cudaLaunchKernelEx(&cfg, attention_mma_kernel<DT>, a)
-                              : cudaLaunchKernelEx(&cfg, attention_kernel<DT>, a);
+                       : deep ? cudaLaunchKernelEx(&cfg, attention_kernel<DT, 8>, a)
+                              : cudaLaunchKernelEx(&cfg, attention_kernel<DT, 4>, a);
     return e == cudaSuccess ? AFX_OK : AFX_ERR_CUDA;
 }
 

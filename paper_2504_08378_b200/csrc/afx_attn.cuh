@@ -21,7 +21,6 @@ constexpr int kAttnWarps = kAttnThreads / 32;
 constexpr int kAttnWorkers = 2 * kAttnWarps;  // half warps: each walks its own positions
 constexpr int kHeadDim = 128;
 constexpr int kAttnMaxRep = 8;  // query heads per kv head
-constexpr int kAttnUnroll = 8;  // cache rows (K and V each) in flight per half warp
 
 struct AttnArgs {
     const float* qkv;  // [T][n_qkv] fp32: q heads | k heads | v heads
@@ -62,10 +61,10 @@ __device__ __forceinline__ float fast_exp2(float x) {
 
 // One query head per kv head.  One pass over the cache: every half warp keeps a running (max, sum,
 // weighted V) for the positions it visits (16 lanes x 8 dims = one 128-wide row per load), K and V
-// rows of kAttnUnroll positions are requested together so that 2 * kAttnUnroll 16-byte loads
+// rows of U positions are requested together so that 2 U 16-byte loads
 // per lane are in flight; the half warps of a block meet in shared memory, the blocks of a
 // cluster through distributed shared memory, both in a fixed order.
-template <int DT>
+template <int DT, int U>
 __device__ __forceinline__ void attention_block(const AttnArgs& a, AttnSmem* sm) {
     cg::cluster_group cluster = cg::this_cluster();
     const int S = static_cast<int>(cluster.num_blocks());
@@ -79,7 +78,6 @@ __device__ __forceinline__ void attention_block(const AttnArgs& a, AttnSmem* sm)
     const int l_hi = static_cast<int>(static_cast<int64_t>(rank + 1) * L / S);
     const float qscale = rsqrtf(static_cast<float>(kHeadDim)) * 1.4426950408889634f;
     const uint32_t half_mask = 0xFFFFu << (16 * half);  // the two halves of a warp work on different keys
-    constexpr int U = kAttnUnroll;
 
     AFX_TRACE_REGION(0);
     AFX_MARK(0);

@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("pos", [0, 1, 15, 16, 17, 127, 128, 129, 1100])
-@pytest.mark.parametrize("kvh,rep,T", [(3, 1, 2), (5, 2, 1), (2, 3, 3), (1, 8, 1)])
+@pytest.mark.parametrize("kvh,rep,T", [(3, 1, 2), (13, 1, 3), (5, 2, 1), (2, 3, 3), (1, 8, 1)])
 def test_attention_matches_oracle_at_tile_edges(pos, kvh, rep, T):
     dt, heads, scale = "f16", kvh * rep, [1.0, 30.0, 1e-3][pos % 3]
     hidden, mlp, max_seq = 128, 64, pos + 1
