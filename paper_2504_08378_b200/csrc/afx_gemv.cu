@@ -20,8 +20,10 @@ sparse_gemv_kernel(GemvListArgs a) {
 }
 
 // A few tokens at once: the tensor-core kernel (afx_mma.cuh).  2048 staged entries per pass
-// still leave room for two blocks per SM.
-using MtListSmem = MtSmem<2048, 4>;
+// leave room for two blocks per SM.  Six stages of 16 channels: a step of four tokens on a 13B-shaped stack
+// takes 200 us a layer, 208 with four stages of 32 (more shared memory: fewer attention blocks beside it),
+// 212 with four of 16, 217 with eight.
+using MtListSmem = MtSmem<2048, 6, 16>;
 template <int DT>
 __global__ void __launch_bounds__(kGemvThreads, 2) sparse_gemm_mt_kernel(GemvListArgs a) {
     extern __shared__ __align__(16) unsigned char mt_dyn[];
