@@ -4,21 +4,6 @@
 
 namespace afx {
 
-template <int TMAX>
-struct GemvShape {
-    static constexpr int kBlocksPerSM = TMAX <= 1 ? 2 : 1;
-    static constexpr int kStageCap = TMAX <= 4 ? 1024 : 512;
-};
-
-template <int DT, int TMAX, int PW>
-__global__ void __launch_bounds__(kGemvThreads, GemvShape<TMAX>::kBlocksPerSM)
-sparse_gemv_kernel(GemvListArgs a) {
-    constexpr int CAP = GemvShape<TMAX>::kStageCap;
-    __shared__ GemvSmem<TMAX, CAP> sm;
-    __shared__ GemvRecv<TMAX> recv;
-    gemv_list_block<DT, TMAX, PW, CAP>(a, &sm, &recv);
-}
-
 // A few tokens at once: the tensor-core kernel (afx_mma.cuh).  2048 staged entries per pass
 // leave room for two blocks per SM.  Six stages of 16 channels: a step of four tokens on a 13B-shaped stack
 // takes 200 us a layer, 208 with four stages of 32 (more shared memory: fewer attention blocks beside it),
@@ -71,27 +56,9 @@ int g_force_pw = 0, g_force_s = 0;  // experiment knobs, 0 = automatic
 int g_cluster_margin = -1;          // experiment knob, < 0 = automatic
 #endif
 
-template <int DT, int TMAX>
-static afx_status launch_gemv_t(const GemvListArgs& a, cudaStream_t st) {
-    const void* kerns[3] = {reinterpret_cast<const void*>(sparse_gemv_kernel<DT, TMAX, 256>),
-                            reinterpret_cast<const void*>(sparse_gemv_kernel<DT, TMAX, 128>),
-                            reinterpret_cast<const void*>(sparse_gemv_kernel<DT, TMAX, 64>)};
-    const GemvShapeChoice c = choose_gemv_shape(a.N, kerns, 0);
-    switch (c.pw) {
-        case 256: return launch_clustered(sparse_gemv_kernel<DT, TMAX, 256>, c.S, c.tiles, 0, a, st);
-        case 128: return launch_clustered(sparse_gemv_kernel<DT, TMAX, 128>, c.S, c.tiles, 0, a, st);
-        default: return launch_clustered(sparse_gemv_kernel<DT, TMAX, 64>, c.S, c.tiles, 0, a, st);
-    }
-}
-
-template <int DT>
-static afx_status launch_gemv(const GemvListArgs& a, cudaStream_t st) {
-    if (a.T <= 1) return launch_gemv_t<DT, 1>(a, st);
-    return launch_gemm_mt<DT>(a, st);
-}
-
 afx_status launch_list_gemv(int dtype, const GemvListArgs& a, cudaStream_t st) {
-    return dtype == AFX_F16 ? launch_gemv<AFX_F16>(a, st) : launch_gemv<AFX_BF16>(a, st);
+    if (a.T <= 1) return launch_list_one_token(dtype, a, st);
+    return dtype == AFX_F16 ? launch_gemm_mt<AFX_F16>(a, st) : launch_gemm_mt<AFX_BF16>(a, st);
 }
 
 }  // namespace afx

@@ -243,89 +243,6 @@ struct GemvListArgs {
 
 // afx_sparse_gemv's launcher (afx_gemv.cu), also used by the layer step over host-resident weights.
 afx_status launch_list_gemv(int dtype, const GemvListArgs& a, cudaStream_t st);
-
-// grid = (S, tiles), cluster = (S, 1, 1).
-template <int DT, int TMAX, int PW, int CAP>
-__device__ __forceinline__ void gemv_list_block(const GemvListArgs& a, GemvSmem<TMAX, CAP>* sm,
-                                                GemvRecv<TMAX>* recv) {
-    constexpr int LPC = PW / 8;
-    const int tid = threadIdx.x;
-    const int lane = tid & 31;
-    const int S = gridDim.x, s = blockIdx.x, tile = blockIdx.y;
-    const int T = a.T;
-    cluster_arrive();
-    // Programmatic dependent launch: global memory is touched only once the previous grid is
-    // complete, and the next grid in the stream may be scheduled (as SM resources free up)
-    // only after that -- so whatever a grid reads before its own wait was written at least
-    // two grids earlier and is complete.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    int cnt = *a.count;
-    if (cnt < 0 || cnt > a.K) {
-        if (tid == 0 && s == 0 && tile == 0) report_status(a.status, AFX_ERR_CAPACITY);
-        cnt = max(0, min(cnt, a.K));
-    }
-    const int c_lo = static_cast<int>(static_cast<int64_t>(s) * cnt / S);
-    const int c_hi = static_cast<int>(static_cast<int64_t>(s + 1) * cnt / S);
-    const int out0 = tile * PW + (lane % LPC) * 8;
-    const bool lane_ok = out0 < a.N;
-    const uint64_t ld16 = static_cast<uint64_t>(a.ldw >> 3);  // row stride in 16-byte units
-    const uint4* wbase16 = reinterpret_cast<const uint4*>(a.Wt + out0);
-
-    float acc[TMAX][8];
-#pragma unroll
-    for (int t = 0; t < TMAX; ++t)
-#pragma unroll
-        for (int q = 0; q < 8; ++q) acc[t][q] = 0.0f;
-
-    __shared__ int first_ok;
-    for (int c0 = c_lo; c0 < c_hi; c0 += CAP) {
-        int staged = min(CAP, c_hi - c0);
-        __syncthreads();
-        bool skipped = false;
-        for (int i = tid; i < staged; i += kGemvThreads) {
-            // An entry outside [0, K), or one whose cache slot is negative (a channel that found
-            // no row), takes no part: x = 0, and the status word says so.
-            const int j = a.idx[c0 + i];
-            const int col = a.slot != nullptr ? a.slot[c0 + i] : j;
-            const bool in_range = static_cast<unsigned>(j) < static_cast<unsigned>(a.K);
-            const uint64_t off = static_cast<uint64_t>(col < 0 ? 0 : col) * ld16;
-            const bool ok = in_range && col >= 0 && off + static_cast<uint64_t>(a.N >> 3) <= 0xFFFFFFFFull;
-            if (!ok && tile == 0) report_status(a.status, in_range ? AFX_ERR_CAPACITY : AFX_ERR_INVALID_ARG);
-            skipped |= !ok;
-            sm->col[i] = ok ? static_cast<uint32_t>(off) : kSkippedEntry;
-#pragma unroll
-            for (int t = 0; t < TMAX; ++t)
-                if (t < T) sm->xv[t][i] = ok ? bits_to_float<DT>(a.x[static_cast<size_t>(t) * a.K + j]) : 0.0f;
-        }
-        if (__syncthreads_or(skipped)) {
-            // Rare.  A skipped entry still costs a load in the streaming loop; whatever it reads
-            // is multiplied by 0, so it must read weights (finite), not a row nobody filled:
-            // send it to the column of the first entry that does take part.
-            if (tid == 0) first_ok = staged;
-            __syncthreads();
-            for (int i = tid; i < staged; i += kGemvThreads)
-                if (sm->col[i] != kSkippedEntry) atomicMin(&first_ok, i);
-            __syncthreads();
-            const int f = first_ok;
-            if (f < staged) {
-                const uint32_t safe = sm->col[f];
-                __syncthreads();
-                for (int i = tid; i < staged; i += kGemvThreads)
-                    if (sm->col[i] == kSkippedEntry) sm->col[i] = safe;
-            } else {
-                staged = 0;  // nothing in this part of the list takes part
-            }
-            __syncthreads();
-        }
-        if (lane_ok) gemv_stream<DT, TMAX, PW, CAP, true>(wbase16, T, sm, staged, acc);
-    }
-    if (a.silu)
-        gemv_finish_tile<DT, TMAX, PW, CAP, EP_SILU>(acc, T, tile, sm, recv, a.ep);
-    else if (a.accumulate)
-        gemv_finish_tile<DT, TMAX, PW, CAP, EP_ACCUM>(acc, T, tile, sm, recv, a.ep);
-    else
-        gemv_finish_tile<DT, TMAX, PW, CAP, EP_STORE>(acc, T, tile, sm, recv, a.ep);
-}
+afx_status launch_list_one_token(int dtype, const GemvListArgs& a, cudaStream_t st);  // afx_onetok.cu
 
 }  // namespace afx

@@ -46,6 +46,8 @@ diff_kernel(const int32_t* __restrict__ idxA, const int32_t* __restrict__ cntA,
             const uint32_t* __restrict__ bitmapP, int K, int32_t* __restrict__ miss,
             int32_t* __restrict__ miss_count, int32_t* __restrict__ hit_count, int32_t* __restrict__ status) {
     __shared__ int scan[2][33];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // only after the wait (ordering rule of the library)
     int n = *cntA;
     if (n < 0 || n > K) {
         if (threadIdx.x == 0) report_status(status, AFX_ERR_CAPACITY);
@@ -144,7 +146,16 @@ extern "C" afx_status afx_diff_active(const int32_t* idxA, const int32_t* cntA,
         (reinterpret_cast<uintptr_t>(miss_count) & 3u) || (reinterpret_cast<uintptr_t>(hit_count) & 3u) ||
         (reinterpret_cast<uintptr_t>(dev_status) & 3u))
         return AFX_ERR_ALIGNMENT;
-    diff_kernel<<<1, kSelectThreads, 0, static_cast<cudaStream_t>(stream)>>>(
-        idxA, cntA, bitmapP, K, miss, miss_count, hit_count, dev_status);
-    return launch_status();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1, 1, 1);
+    cfg.blockDim = dim3(kSelectThreads, 1, 1);
+    cfg.stream = static_cast<cudaStream_t>(stream);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, diff_kernel, idxA, cntA, bitmapP, K, miss, miss_count, hit_count, dev_status) == cudaSuccess
+               ? AFX_OK
+               : AFX_ERR_CUDA;
 }

@@ -88,6 +88,54 @@ __device__ __forceinline__ void st_shared_if(uint32_t at, uint32_t v, bool on) {
     asm volatile("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p st.shared.u32 [%0], %1; }" ::"r"(at), "r"(v), "r"(on ? 1u : 0u) : "memory");
 }
 
+// The row sets' sums (thread `tid` holds row set g = tid / P, piece tid - g P, of `rows` sets) meet and leave
+// as outputs 8 piece0 .. of the operator: `parts` threads per output add every parts-th set, then in order.
+template <int DT, int NT, int EP>
+__device__ __forceinline__ void slice_finish(const f32x2 (&acc)[4], int g, int rows, int P, int piece0, unsigned char* dyn, float* y,
+                                             uint16_t* out_bits, float scale, float y_old) {
+    const int tid = threadIdx.x, nout = P * 8;
+    const int parts = NT / nout, part = tid / nout, out = tid - part * nout;
+    __syncthreads();  // the list has been read
+    AFX_MARK(6);
+    float* red = reinterpret_cast<float*>(dyn);
+    if (g < rows) {
+        float4* d4 = reinterpret_cast<float4*>(red + tid * 8);
+#pragma unroll
+        for (int i = 0; i < 4; i += 2) {
+            float4 v;
+            unpack_f32x2(acc[i], v.x, v.y);
+            unpack_f32x2(acc[i + 1], v.z, v.w);
+            d4[i / 2] = v;
+        }
+    }
+    __syncthreads();
+    float* red2 = red + NT * 8;
+    if (part < parts) {
+        float sum = 0.0f;
+#pragma unroll 4
+        for (int r = part; r < rows; r += parts) sum += red[r * nout + out];
+        red2[tid] = sum;
+    }
+    __syncthreads();
+    auto total = [&](int o) {
+        float v = red2[o];
+#pragma unroll 4
+        for (int q = 1; q < parts; ++q) v += red2[q * nout + o];
+        return v;
+    };
+    if (EP == EP_SILU) {
+        // pair r of the slice: 8 gate then 8 up outputs per 16 columns
+        if (tid < nout / 2) {
+            const int o = (tid >> 3) * 16 + (tid & 7);
+            const float gate = total(o), up = total(o + 8);
+            out_bits[piece0 * 4 + tid] = float_to_bits<DT>(gate / (1.0f + expf(-gate)) * up);
+        }
+    } else if (tid < nout) {
+        const float v = total(tid) * scale;
+        y[piece0 * 8 + tid] = EP == EP_ACCUM ? y_old + v : v;
+    }
+}
+
 // GRP: the grid may hold several operators of one family (FusedArgs::groups).  The first NW of the NT / 32
 // warps select, with up to CH slots of 4 channels per lane (K <= 128 NW CH).
 template <int DT, int NT, int NW, int CH, int IN, int EP, bool GRP>
@@ -251,48 +299,104 @@ __device__ __forceinline__ void slice_op_block(const FusedArgs& a, unsigned char
     if (g < rows) slice_stream<DT>(Wt, a.ldw, piece0 + piece, list, cnt, g, rows, acc);
     AFX_MARK(5);
 
-    // ---- the row sets' sums meet: `parts` threads per output add every parts-th one, then in order ----
-    const int parts = NT / nout, part = tid / nout, out = tid - part * nout;
-    __syncthreads();  // the list has been read
-    AFX_MARK(6);
-    float* red = reinterpret_cast<float*>(dyn);
-    if (g < rows) {
-        float4* d4 = reinterpret_cast<float4*>(red + tid * 8);
-#pragma unroll
-        for (int i = 0; i < 4; i += 2) {
-            float4 v;
-            unpack_f32x2(acc[i], v.x, v.y);
-            unpack_f32x2(acc[i + 1], v.z, v.w);
-            d4[i / 2] = v;
-        }
-    }
-    __syncthreads();
-    float* red2 = red + NT * 8;
-    if (part < parts) {
-        float sum = 0.0f;
-#pragma unroll 4
-        for (int r = part; r < rows; r += parts) sum += red[r * nout + out];
-        red2[tid] = sum;
-    }
-    __syncthreads();
-    auto total = [&](int o) {
-        float v = red2[o];
-#pragma unroll 4
-        for (int q = 1; q < parts; ++q) v += red2[q * nout + o];
-        return v;
-    };
-    if (EP == EP_SILU) {
-        // pair r of the slice: 8 gate then 8 up outputs per 16 columns
-        if (tid < nout / 2) {
-            const int o = (tid >> 3) * 16 + (tid & 7);
-            const float gate = total(o), up = total(o + 8);
-            out_bits[piece0 * 4 + tid] = float_to_bits<DT>(gate / (1.0f + expf(-gate)) * up);
-        }
-    } else if (tid < nout) {
-        const float v = total(tid) * scale;
-        y[piece0 * 8 + tid] = EP == EP_ACCUM ? y_old + v : v;
-    }
+    slice_finish<DT, NT, EP>(acc, g, rows, P, piece0, dyn, y, out_bits, scale, y_old);
     AFX_MARK(7);
+}
+
+// ---- the operator on a list given by the caller (afx_sparse_gemv, one token) ----
+
+constexpr int kSlListCap = 8192;  // staged entries per pass: row offset in 16-byte units, 16-bit input
+
+__host__ __device__ inline size_t slice_given_smem(int threads) {
+    const size_t list = static_cast<size_t>(kSlListCap) * 6, sums = static_cast<size_t>(threads) * 9 * 4;
+    return list > sums ? list : sums;
+}
+
+template <int DT, int NT, int EP>
+__device__ __forceinline__ void slice_list_block(const GemvListArgs& a, unsigned char* dyn) {
+    const int tid = threadIdx.x;
+    // this block's slice, as in slice_op_block
+    const int nb = gridDim.x, b = blockIdx.x;
+    const int pieces = a.N / 8, granules = (pieces + kSlGranule - 1) / kSlGranule;
+    const int g_lo = b * granules / nb, g_hi = (b + 1) * granules / nb;
+    const int piece0 = g_lo * kSlGranule, P = max(1, min(g_hi * kSlGranule, pieces) - piece0), nout = P * 8;
+    const int rows = NT / P, g = tid / P, piece = tid - g * P;
+    uint32_t* const off = reinterpret_cast<uint32_t*>(dyn);
+    uint16_t* const xb = reinterpret_cast<uint16_t*>(dyn + static_cast<size_t>(kSlListCap) * 4);
+    const uint64_t ld16 = static_cast<uint64_t>(a.ldw >> 3);
+    const char* base = reinterpret_cast<const char*>(a.Wt + static_cast<size_t>(piece0 + piece) * 8);
+    __shared__ int first_ok;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // only after the wait (ordering rule)
+    int cnt = *a.count;
+    if (cnt < 0 || cnt > a.K) {
+        if (tid == 0 && b == 0) report_status(a.status, AFX_ERR_CAPACITY);
+        cnt = max(0, min(cnt, a.K));
+    }
+    float y_old = 0.0f;
+    if (EP == EP_ACCUM && tid < nout) y_old = a.ep.y[piece0 * 8 + tid];
+    f32x2 acc[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i] = pack_f32x2(0.0f, 0.0f);
+    for (int c0 = 0; c0 < cnt; c0 += kSlListCap) {
+        int staged = min(kSlListCap, cnt - c0);
+        if (c0 > 0) __syncthreads();  // the previous pass has been read
+        bool skipped = false;
+        for (int i = tid; i < staged; i += NT) {
+            // An entry outside [0, K), or one whose cache slot is negative (a channel that found
+            // no row), takes no part: x = 0, and the status word says so.
+            const int j = a.idx[c0 + i];
+            const int col = a.slot != nullptr ? a.slot[c0 + i] : j;
+            const bool in_range = static_cast<unsigned>(j) < static_cast<unsigned>(a.K);
+            const uint64_t o = static_cast<uint64_t>(col < 0 ? 0 : col) * ld16;
+            const bool ok = in_range && col >= 0 && o + static_cast<uint64_t>(a.N >> 3) <= 0xFFFFFFFFull;
+            if (!ok && b == 0) report_status(a.status, in_range ? AFX_ERR_CAPACITY : AFX_ERR_INVALID_ARG);
+            skipped |= !ok;
+            off[i] = ok ? static_cast<uint32_t>(o) : kSkippedEntry;
+            xb[i] = ok ? a.x[j] : uint16_t(0);
+        }
+        if (__syncthreads_or(skipped)) {
+            // Rare.  A skipped entry still costs a load in the streaming loop; whatever it reads is multiplied
+            // by 0, so it must read weights (finite): the row of the first entry that does take part.
+            if (tid == 0) first_ok = staged;
+            __syncthreads();
+            for (int i = tid; i < staged; i += NT)
+                if (off[i] != kSkippedEntry) atomicMin(&first_ok, i);
+            __syncthreads();
+            const int f = first_ok;
+            if (f < staged) {
+                const uint32_t safe = off[f];
+                __syncthreads();
+                for (int i = tid; i < staged; i += NT)
+                    if (off[i] == kSkippedEntry) off[i] = safe;
+            } else {
+                staged = 0;  // nothing in this part of the list takes part
+            }
+            __syncthreads();
+        }
+        if (g < rows) {
+            constexpr int U = 8;
+            for (int p = g; p < staged; p += U * rows) {
+                uint4 raw[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (p + u * rows < staged) raw[u] = ld_stream_16B(base + static_cast<uint64_t>(off[p + u * rows]) * 16);
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (p + u * rows < staged) {
+                        f32x2 w[4];
+                        unpack8_pairs<DT>(raw[u], w);
+                        const float xv = bits_to_float<DT>(xb[p + u * rows]);
+                        const f32x2 x2 = pack_f32x2(xv, xv);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) fma_f32x2(acc[i], w[i], x2);
+                    }
+                }
+            }
+        }
+    }
+    const float scale = EP != EP_SILU && a.ep.scale != nullptr ? *a.ep.scale : 1.0f;
+    slice_finish<DT, NT, EP>(acc, g, rows, P, piece0, dyn, a.ep.y, a.ep.out_bits, scale, y_old);
 }
 
 }  // namespace afx
