@@ -39,3 +39,42 @@ def test_one_token_operator_at_dispatch_edges(K, N, dt, mode):
         # sums of fp32 products in any order: at most K / 2 additions, each within 2^-24 of the running sum
         bound = (len(want) + 2) * 2.0 ** -24 * (w.abs() * xa.abs()[:, None]).sum(0)
         assert bool(((y.double() - (w * xa[:, None]).sum(0)).abs() <= bound).all())
+
+
+@pytest.mark.parametrize("K,N,keep,dt", [(20000, 64, 20000, "f16"), (8193, 1032, 8193, "bf16"), (64, 80000, 33, "bf16"),
+                                         (4096, 2056, 1, "f16"), (4096, 2048, 0, "bf16")])
+def test_given_list_at_pass_and_slice_edges(K, N, keep, dt):
+    """One token with a given list: more entries than a pass holds, both block sizes, waves of slices, none."""
+    rng = np.random.default_rng(K + N)
+    torch_dt = torch.float16 if dt == "f16" else torch.bfloat16
+    x = torch.from_numpy(rng.standard_normal(K).astype(np.float32)).to(torch_dt).cuda()
+    W = (0.02 * torch.from_numpy(rng.standard_normal((K, N), dtype=np.float32))).to(torch_dt).cuda()
+    want = np.sort(rng.permutation(K)[:keep]).astype(np.int32)
+    idx = torch.zeros(K, dtype=torch.int32, device="cuda")
+    idx[:keep] = torch.from_numpy(want).cuda()
+    count = torch.tensor([keep], dtype=torch.int32, device="cuda")
+    y = torch.full((N,), 0.5, device="cuda")
+    afx.afx_sparse_gemv(W.view(torch.int16), dt, K, N, N, x.view(torch.int16), 1, idx, count, None, y, 1)
+    a = torch.from_numpy(want.astype(np.int64)).cuda()
+    w, xa = W[a].double(), x[a].double()[:, None]
+    bound = (keep + 3) * 2.0 ** -24 * ((w.abs() * xa.abs()).sum(0) + 0.5)  # any order of fp32 additions
+    assert bool(((y.double() - 0.5 - (w * xa).sum(0)).abs() <= bound).all())
+
+
+@pytest.mark.parametrize("K", [33, 4096, 4097, 8193, 16385, 32768])
+@pytest.mark.parametrize("T", [1, 2, 8])
+@pytest.mark.parametrize("dt,mode", [("bf16", "topk"), ("f16", "topk"), ("f16", "threshold")])
+def test_selection_of_tokens_at_warp_limits(K, T, dt, mode):
+    """Union over tokens with few distinct magnitudes (ties at the boundary), one token all zero."""
+    rng = np.random.default_rng(K + T)
+    x = np.round(rng.laplace(size=(T, K)) * 4) / 4
+    x[-1] *= T == 1
+    bits = torch.from_numpy(x.astype(np.float32)).to(torch.float16 if dt == "f16" else torch.bfloat16).view(torch.int16).cuda()
+    k, tau = max(1, K // 3), 0.75
+    want = oracle.select_active(bits.cpu().numpy().view(np.uint16), dt, oracle.TOPK if mode == "topk" else oracle.THRESHOLD, k=k, tau=tau)
+    idx, count = torch.zeros(K, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    bitmap = torch.zeros((K + 31) // 32, dtype=torch.int32, device="cuda")
+    afx.afx_select_active(bits, dt, K, T, afx.MODE_TOPK if mode == "topk" else afx.MODE_THRESHOLD, k, tau, idx, count, bitmap)
+    assert np.array_equal(idx.cpu().numpy()[: int(count)], want)
+    flags = np.unpackbits(bitmap.cpu().numpy().view(np.uint8), bitorder="little")[:K]
+    assert np.array_equal(np.flatnonzero(flags), want)
