@@ -100,8 +100,8 @@ __host__ __device__ inline size_t fused_dyn_smem(int in_kind, int K, int T, size
 // ldw is the row stride in units of 2 bytes, the tile is PW = 512, 256 or 128 outputs wide and
 // the streaming loop and the reduction are the 4-bit kernel's.
 template <int DT, int TMAX, int PW, int CAP, int IN, int EP, bool WQ4 = false, int WMT = 0>
-__device__ __forceinline__ void fused_op_block(const FusedArgs& a, unsigned char* dyn, SelectScratch* sel,
-                                               GemvRecv<TMAX>* recv) {
+__device__ __forceinline__ void fused_op_block(const FusedArgs& a, unsigned char* dyn, SelectScratch* sel) {
+    static_assert(WQ4 || WMT > 0, "one token over 16-bit rows is afx_slice.cuh's");
     constexpr int LPC = WQ4 ? PW / kQ4Opl : PW / 8;
     static_assert(WMT > 0 || sizeof(GemvSmem<TMAX, CAP>) <= kKeyHistBytes, "work area too small");
     static_assert(!WQ4 || (TMAX == 1 && CAP * 8 + (kQ4Warps + 1) * PW * 4 <= kKeyHistBytes), "4-bit: one token, sums behind the staged list");
@@ -366,11 +366,6 @@ __device__ __forceinline__ void fused_op_block(const FusedArgs& a, unsigned char
     const int c_lo = s * cnt / S;  // S <= 8, cnt <= 2^20: no overflow
     const int c_hi = (s + 1) * cnt / S;
 
-    float acc[TMAX][8];
-#pragma unroll
-    for (int t = 0; t < TMAX; ++t)
-#pragma unroll
-        for (int q = 0; q < 8; ++q) acc[t][q] = 0.0f;
     f32x2 qacc[8];  // 4-bit weights: 16 outputs per lane
 #pragma unroll
     for (int i = 0; i < 8; ++i) qacc[i] = pack_f32x2(0.0f, 0.0f);
@@ -450,22 +445,15 @@ __device__ __forceinline__ void fused_op_block(const FusedArgs& a, unsigned char
         if (WQ4) {
             if (lane_ok)
                 q4_stream<LPC>(reinterpret_cast<const unsigned char*>(Wt), a.N, out0 / kQ4Opl, sm->col, sm->xv[0], staged, qacc);
-        } else if (lane_ok) {
-            gemv_stream<DT, TMAX, PW, CAP, false>(reinterpret_cast<const uint4*>(Wt + out0), T, sm, staged, acc);
         }
     }
     AFX_MARK(5);
 
     AFX_MARK(6);
 
-    EpilogueArgs ep = a.ep;
-    if (WQ4) {
-        cluster_wait();  // pairs with the cluster_arrive() at kernel start
-        q4_finish<DT, LPC>(qacc, reinterpret_cast<float*>(work) + 2 * CAP, tile, a.N,
-                           EP == EP_SILU ? Q4_SILU : (EP == EP_ACCUM ? Q4_ACCUM : Q4_STORE), ep.y, ep.out_bits);
-    } else {
-        gemv_finish_tile<DT, TMAX, PW, CAP, EP>(acc, T, tile, sm, recv, ep, !share);
-    }
+    cluster_wait();  // pairs with the cluster_arrive() at kernel start
+    q4_finish<DT, LPC>(qacc, reinterpret_cast<float*>(work) + 2 * CAP, tile, a.N,
+                       EP == EP_SILU ? Q4_SILU : (EP == EP_ACCUM ? Q4_ACCUM : Q4_STORE), a.ep.y, a.ep.out_bits);
     AFX_MARK(7);
 }
 

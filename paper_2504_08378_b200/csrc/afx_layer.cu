@@ -23,7 +23,7 @@ template <int DT, int TMAX, int IN, int EP, int STAGES, int CAPM, int BPS>
 __global__ void __launch_bounds__(kGemvThreads, BPS) fused_mt_kernel(FusedArgs a) {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ SelectScratch sel;
-    fused_op_block<DT, TMAX, kMtTile, CAPM, IN, EP, false, STAGES>(a, dyn, &sel, nullptr);
+    fused_op_block<DT, TMAX, kMtTile, CAPM, IN, EP, false, STAGES>(a, dyn, &sel);
 }
 
 // The one-token operator over 4-bit rows: tiles of PW = 512, 256 or 128 outputs.
@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(kGemvThreads, 2) fused_q4_kernel(FusedArgs a) 
     constexpr int CAP = 2048;
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ SelectScratch sel;
-    fused_op_block<DT, 1, PW, CAP, IN, EP, true>(a, dyn, &sel, nullptr);
+    fused_op_block<DT, 1, PW, CAP, IN, EP, true>(a, dyn, &sel);
 }
 
 // a.Wt = the 4-bit rows, a.ldw = their stride in units of 2 bytes, a.T == 1, a.N % 32 == 0.

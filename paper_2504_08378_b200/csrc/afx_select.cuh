@@ -509,17 +509,6 @@ __device__ __forceinline__ unsigned long long block_token_flags(const uint16_t* 
     return fl;
 }
 
-// Writes the calling thread's flag bytes into a ceil(K/32)-word bitmap in shared memory
-// (bit j % 32 of word j / 32) and clears the bytes past the last chunk.  No barrier.
-__device__ __forceinline__ void store_flag_bytes(unsigned long long fl, int K, uint32_t* flags) {
-    int c_lo, c_hi;
-    thread_chunk_range(K, c_lo, c_hi);
-    uint8_t* bytes = reinterpret_cast<uint8_t*>(flags);
-    for (int c = c_lo; c < c_hi; ++c) bytes[c] = static_cast<uint8_t>(fl >> (8 * (c - c_lo)));
-    const int nchunks = (K + 7) >> 3, nbytes = ((K + 31) >> 5) << 2;
-    for (int c = nchunks + threadIdx.x; c < nbytes; c += blockDim.x) bytes[c] = 0;
-}
-
 // Calls f(j, pos) for every active channel j of the calling thread, ascending, pos = its
 // position in the list.
 template <class F>
