@@ -34,10 +34,10 @@ sys.path.insert(0, ROOT)
 CFG = dict(name="llama7b_decode_32L_bf16_top50_xl3", dtype="bf16", n_layers=32, hidden=4096, n_heads=32,
            n_kv_heads=32, mlp=11008, past=2048, sparsity_percent=50, xl_depth=3, seed=3)
 ORACLE_SAMPLE_LAYERS = 16
-# dram__bytes_read.sum + dram__bytes_write.sum of one fused gate/up launch of this workload,
-# from the ncu capture summarised in profiles/fused_op_kernel_7b_ncu_full.md (None while the
+# DRAM bytes (dram__bytes.sum.per_second x duration) of one fused gate/up launch of this workload,
+# from the ncu capture summarised in profiles/slice_op_kernel_7b_ncu.md (None while the
 # kernel has changed since the counters were taken).
-NCU_TRAFFIC_BYTES_PER_LAUNCH = 93_864_960
+NCU_TRAFFIC_BYTES_PER_LAUNCH = 93_519_000
 
 
 def measured_peaks():
@@ -427,7 +427,7 @@ def run_afx(args):
     w_bytes, kv_bytes = active_bytes_per_token(cfg, k)
     step_s = ms / args.steps * 1e-3
     roofline = {"bound": "hbm",
-                "kernel": "fused_op_kernel<bf16,1,256,RMSNorm,silu*up> as the decode step launches it: gate|up 4096->22016, "
+                "kernel": "slice_op_kernel<bf16,1024 threads,8 selecting warps,RMSNorm,silu*up> as the decode step launches it: gate|up 4096->22016, "
                           "k=2048 (norm + hinted top-k + sparse GEMV + epilogue + cross-layer side outputs)",
                 "achieved": achieved, "peak": peak, "peak_kind": peak_kind, "unit": "GB/s",
                 "frac": round(achieved / peak, 4), "frac_of_8TBs": round(achieved / 8000.0, 4),
