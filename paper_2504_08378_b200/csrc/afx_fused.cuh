@@ -142,8 +142,8 @@ __device__ __forceinline__ void fused_op_block(const FusedArgs& a, unsigned char
     // only AFTER its own dependency wait.  When a grid runs its prologue, its predecessor has
     // therefore passed its wait, i.e. the grid before that one is complete: whatever is read
     // before the wait below must have been written at least two grids earlier (weights and
-    // gains: never; the search hint and the predicted set: by the same operator of an earlier
-    // token or layer, at least five grids back).
+    // gains: never; the predicted set: by the same operator of an earlier layer, at least five
+    // grids back).  The search hint is the exception: it may be rewritten while it is read.
     // the norm's gains are weights: they can be on their way before the wait for h
     constexpr int NH = 4;  // float4 pieces of h (and of the gain) a thread keeps in registers
     float4 gv[NH];
@@ -154,22 +154,14 @@ __device__ __forceinline__ void fused_op_block(const FusedArgs& a, unsigned char
             gv[i] = c < (K >> 2) ? reinterpret_cast<const float4*>(a.gain)[c] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
     }
-    // the hint was written by an earlier token's launch of this operator (a launch that reads
-    // the value its own scribe block has just rewritten only gets a better hint: the
-    // selection's result does not depend on it)
-    uint32_t hint = kNoKeyHint;
-    if (topk && T == 1 && a.kth_slot != nullptr) {
-        const uint32_t v = static_cast<uint32_t>(__ldcg(a.kth_slot));
-        if (v & 0x10000u) hint = v & 0x7FFFu;
-    }
-    uint32_t hint_t[TMAX];  // several tokens: one hint each
-#pragma unroll
-    for (int t = 0; t < TMAX; ++t) {
-        hint_t[t] = kNoKeyHint;
-        if (TMAX > 1 && topk && T > 1 && t < T && a.kth_multi != nullptr) {
-            const uint32_t v = static_cast<uint32_t>(__ldcg(a.kth_multi + t));
-            if (v & 0x10000u) hint_t[t] = v & 0x7FFFu;
-        }
+    // The hints, one per token, are written by an earlier launch of this operator, which may still be
+    // running, and by this launch's own scribe block.  The selection does not depend on them, but all
+    // threads of a block must search from the same one: a single thread reads it, the others
+    // take it from shared memory behind the barrier of the input stage.
+    if (tid < T) {
+        const int32_t* const slot = T == 1 ? a.kth_slot : a.kth_multi != nullptr ? a.kth_multi + tid : nullptr;
+        const uint32_t v = topk && slot != nullptr ? static_cast<uint32_t>(__ldcg(slot)) : 0u;
+        sel->hint[tid] = (v & 0x10000u) ? v & 0x7FFFu : kNoKeyHint;
     }
     // likewise the predicted set this selection is compared with: the same operator of the
     // predictor layer wrote it, at least one layer (five grids) ago (byte v = the flags of the
@@ -291,18 +283,14 @@ __device__ __forceinline__ void fused_op_block(const FusedArgs& a, unsigned char
                             sm->col[p] = static_cast<uint32_t>(j) * ld16;
                             sm->xv[0][p] = bits_to_float<DT>(bits);
                         }
-                    }, e_lo, e_lo + e_n, hint, xchg);
+                    }, e_lo, e_lo + e_n, sel->hint[0], xchg);
                 first_staged = true;
                 if (scribe && tid == 0 && a.kth_slot != nullptr) *a.kth_slot = 0x10000 | sel->res[0];
             } else {
                 uint32_t thr_t = 0;
-                uint32_t h_t = kNoKeyHint;
-#pragma unroll
-                for (int u = 0; u < TMAX; ++u)
-                    if (u == t) h_t = hint_t[u];
                 const unsigned long long ft =
                     block_token_flags<DT, kGemvThreads>(xt, K, a.mode, a.k, a.tau, hist, first, sel, T == 1, pos0, cnt,
-                                                        NoEmit(), 0, 0x7FFFFFFF, h_t, nullptr, &thr_t);
+                                                        NoEmit(), 0, 0x7FFFFFFF, sel->hint[t], nullptr, &thr_t);
                 if (scribe && tid == 0 && topk && T > 1 && a.kth_multi != nullptr) a.kth_multi[t] = 0x10000 | thr_t;
                 if (share) {
                     int q_lo, q_hi;

@@ -32,6 +32,7 @@ struct SelectScratch {
     int res[4];       // broadcast of the k-th key search
     __align__(16) int hist[256];  // large-K path; the fused operators borrow it for the norm's reduction
     int scan[33];
+    uint32_t hint[AFX_MAX_T];  // the fused operators: where each token's search starts
 };
 
 // Words [w0, w1) of a ceil(K/32)-word bitmap owned by the calling warp (contiguous, so that

@@ -47,19 +47,15 @@ __device__ __forceinline__ void select_tokens_block(const FusedArgs& a, SelTokSm
     const bool selects = NW == kStThreads / 32 || warp_id() < NW;
     const bool own = a.idx_in == nullptr;
     const bool topk = a.mode == AFX_MODE_TOPK && a.k > 0 && a.k < K;
-    // Read before the dependency wait: gains never change, the hint's only writer is this block's own
-    // predecessor for the same operator, several grids back (the ordering rule stated at fused_op_block).
+    // Read before the dependency wait: gains never change; the hint may be rewritten meanwhile by an earlier launch
+    // of the operator, and either value gives the same selection.
     constexpr bool kEarlyGain = IN == IN_NORM && CH < 8;
     float4 gv[kEarlyGain ? CH : 1];
     if constexpr (kEarlyGain) {
         if (selects) sel_load_gain<CH>(a.gain, K, m, gv);
     }
     int32_t* const slot = T == 1 ? a.kth_slot : a.kth_multi != nullptr ? a.kth_multi + t : nullptr;
-    uint32_t hint = kNoHint;
-    if (own && topk && slot != nullptr) {
-        const uint32_t v = static_cast<uint32_t>(__ldcg(slot));
-        if (v & 0x10000u) hint = v & 0x7FFFu;
-    }
+    if (own) sel_read_hint(slot, &sm->sel);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // only after the wait (ordering rule)
 
@@ -72,8 +68,9 @@ __device__ __forceinline__ void select_tokens_block(const FusedArgs& a, SelTokSm
         else if (own)
             sel_load_keys<CH>(a.x + static_cast<size_t>(t) * K, K, m, kw);
         if (own) {
+            if (IN == IN_X) sel_barrier<NW>();  // the hint is there (IN_NORM: since the norm's barrier)
             int kth, at;
-            const uint32_t fl = sel_flags<DT, NW, CH>(kw, m, K, a.mode, a.k, a.tau, hint, &sm->sel, kth, at, cnt);
+            const uint32_t fl = sel_flags<DT, NW, CH>(kw, m, K, a.mode, a.k, a.tau, sm->sel.hint, &sm->sel, kth, at, cnt);
             if (tid == 0 && topk && slot != nullptr) *slot = 0x10000 | kth;
 #pragma unroll
             for (int i = 0; i < CH; ++i) {

@@ -160,18 +160,14 @@ __device__ __forceinline__ void slice_op_block(const FusedArgs& a, unsigned char
     const int g = tid / P, piece = tid - g * P;
 
     // What the prologue reads before the dependency wait was written at least two grids earlier (the
-    // ordering rule stated at fused_op_block): gains never, the hint by an earlier token's launch of
-    // this operator (or by this launch's own scribe: only a better hint).
+    // ordering rule stated at fused_op_block): gains never.  The hint may be rewritten meanwhile (by the launch
+    // before, or by this launch's own scribe): either value gives the same selection.
     constexpr bool kEarlyGain = IN == IN_NORM && CH < 8;
     float4 gv[kEarlyGain ? CH : 1];
     if constexpr (kEarlyGain) {
         if (selects) sel_load_gain<CH>(a.gain, K, m, gv);
     }
-    uint32_t hint = kNoHint;
-    if (own && a.kth_slot != nullptr) {
-        const uint32_t v = static_cast<uint32_t>(__ldcg(a.kth_slot));
-        if (v & 0x10000u) hint = v & 0x7FFFu;
-    }
+    if (own) sel_read_hint(a.kth_slot, sc);
     const bool early = GRP && a.x_early != 0;  // the input is older than the kernel before this one: select first
     if (!early) {
         asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -198,9 +194,10 @@ __device__ __forceinline__ void slice_op_block(const FusedArgs& a, unsigned char
             sel_load_keys<CH>(x, K, m, kw);
         AFX_MARK(2);
         if (own) {
+            if (IN == IN_X) sel_barrier<NW>();  // sc->hint is there (IN_NORM: since the norm's barrier)
             int kth, at, n;
             const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(list));
-            const uint32_t fl = sel_flags<DT, NW, CH>(kw, m, K, a.mode, a.k, a.tau, hint, sc, kth, at, n);
+            const uint32_t fl = sel_flags<DT, NW, CH>(kw, m, K, a.mode, a.k, a.tau, sc->hint, sc, kth, at, n);
             sel_emit<CH>(fl, m, at, [&](int i, int e, int pos, bool on) {
                 st_shared_if(base + 4 * pos, __byte_perm(kw[2 * i + (e >> 1)], static_cast<uint32_t>(sel_channel(m, i) + e), (e & 1) ? 0x3254 : 0x1054), on);
             });

@@ -23,7 +23,8 @@ constexpr int kRegSelMaxWarps = 32;
 struct RegSelScratch {
     __align__(16) uint32_t part[2][kRegSelMaxWarps][4];  // per-warp counts of a search step (double-buffered)
     uint32_t scan[kRegSelMaxWarps];
-    int count;  // the list's length, for the warps that did not select
+    int count;      // the list's length, for the warps that did not select
+    uint32_t hint;  // where the search starts (sel_read_hint)
     __align__(16) float sum[kRegSelMaxWarps];
 };
 
@@ -31,6 +32,17 @@ struct RegSelScratch {
 template <int NW>
 __device__ __forceinline__ void sel_barrier() {
     asm volatile("bar.sync 1, %0;" ::"n"(NW * 32) : "memory");
+}
+
+// The search hint in `slot` (NULL: none) for the whole block: ONE thread of the first warp reads it and leaves it in
+// sc->hint, which the others read behind a barrier of the selecting warps.  Another launch of the operator, or
+// another block of this one, may be rewriting the word: threads that read it for themselves could start with
+// different hints, take different numbers of search steps, and wait at different barriers for each other.
+__device__ __forceinline__ void sel_read_hint(const int32_t* slot, RegSelScratch* sc) {
+    if (threadIdx.x == 0) {
+        const uint32_t v = slot != nullptr ? static_cast<uint32_t>(__ldcg(slot)) : 0u;
+        sc->hint = (v & 0x10000u) ? v & 0x7FFFu : kNoHint;
+    }
 }
 
 // Slots per lane for K channels on NW warps.

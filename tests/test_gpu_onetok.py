@@ -78,3 +78,27 @@ def test_selection_of_tokens_at_warp_limits(K, T, dt, mode):
     assert np.array_equal(idx.cpu().numpy()[: int(count)], want)
     flags = np.unpackbits(bitmap.cpu().numpy().view(np.uint8), bitorder="little")[:K]
     assert np.array_equal(np.flatnonzero(flags), want)
+
+
+@pytest.mark.parametrize("K,N,dt", [(512, 256, "f16"), (4096, 512, "bf16"), (11008, 1024, "bf16")])
+def test_calls_in_a_row_share_a_hint(K, N, dt):
+    """The next launch reads the hint while the one before rewrites it, and the hints are far apart: every block
+    must search from ONE of the two values, and the lists must not depend on which."""
+    rng = np.random.default_rng(K + N)
+    torch_dt = torch.float16 if dt == "f16" else torch.bfloat16
+    x = torch.from_numpy(rng.laplace(size=(2, K)) * np.array([[1.0], [1.0 / 64]])).to(torch_dt).cuda().view(torch.int16)
+    W = (0.02 * torch.from_numpy(rng.standard_normal((K, N), dtype=np.float32))).to(torch_dt).cuda().view(torch.int16)
+    k, calls = synth.keep_count(K, 50), 64
+    y = torch.zeros((calls, N), device="cuda")
+    idx = torch.zeros((calls, K), dtype=torch.int32, device="cuda")
+    count = torch.zeros(calls, dtype=torch.int32, device="cuda")
+    want = [oracle.select_active(v.cpu().numpy().view(np.uint16), dt, oracle.TOPK, k=k) for v in x]
+    hint = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for i in range(calls):
+        if i % 16 == 0:
+            hint.zero_()
+        afx.afx_select_gemv(W, dt, K, N, N, x[i % 2], 1, afx.MODE_TOPK, k, 0.0, y[i], 0, idx[i], count[i], kth_hint=hint)
+    assert count.tolist() == [k] * calls
+    for i in range(calls):
+        assert np.array_equal(idx[i, :k].cpu().numpy(), want[i % 2]), i
+        assert torch.equal(y[i], y[i % 2])
