@@ -1,8 +1,16 @@
 // afx_sparse_gemv: host-side shape selection and launch.
 #include "afx_launch.cuh"
+#include "afx_list.cuh"
 #include "afx_mma.cuh"
 
 namespace afx {
+
+template <int DT, int PW>
+__global__ void __launch_bounds__(kGemvThreads, 2) sparse_gemv_kernel(GemvListArgs a) {
+    __shared__ ListSmem<1, 1024> sm;
+    __shared__ GemvRecv<1> recv;
+    gemv_list_block<DT, 1, PW, 1024>(a, &sm, &recv);
+}
 
 // A few tokens at once: the tensor-core kernel (afx_mma.cuh).  2048 staged entries per pass
 // leave room for two blocks per SM.  Six stages of 16 channels: a step of four tokens on a 13B-shaped stack
@@ -56,9 +64,22 @@ int g_force_pw = 0, g_force_s = 0;  // experiment knobs, 0 = automatic
 int g_cluster_margin = -1;          // experiment knob, < 0 = automatic
 #endif
 
+template <int DT>
+static afx_status launch_gemv(const GemvListArgs& a, cudaStream_t st) {
+    if (a.T > 1) return launch_gemm_mt<DT>(a, st);
+    const void* kerns[3] = {reinterpret_cast<const void*>(sparse_gemv_kernel<DT, 256>),
+                            reinterpret_cast<const void*>(sparse_gemv_kernel<DT, 128>),
+                            reinterpret_cast<const void*>(sparse_gemv_kernel<DT, 64>)};
+    const GemvShapeChoice c = choose_gemv_shape(a.N, kerns, 0);
+    switch (c.pw) {
+        case 256: return launch_clustered(sparse_gemv_kernel<DT, 256>, c.S, c.tiles, 0, a, st);
+        case 128: return launch_clustered(sparse_gemv_kernel<DT, 128>, c.S, c.tiles, 0, a, st);
+        default: return launch_clustered(sparse_gemv_kernel<DT, 64>, c.S, c.tiles, 0, a, st);
+    }
+}
+
 afx_status launch_list_gemv(int dtype, const GemvListArgs& a, cudaStream_t st) {
-    if (a.T <= 1) return launch_list_one_token(dtype, a, st);
-    return dtype == AFX_F16 ? launch_gemm_mt<AFX_F16>(a, st) : launch_gemm_mt<AFX_BF16>(a, st);
+    return dtype == AFX_F16 ? launch_gemv<AFX_F16>(a, st) : launch_gemv<AFX_BF16>(a, st);
 }
 
 }  // namespace afx

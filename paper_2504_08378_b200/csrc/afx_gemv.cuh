@@ -61,6 +61,5 @@ struct GemvListArgs {
 
 // afx_sparse_gemv's launcher (afx_gemv.cu), also used by the layer step over host-resident weights.
 afx_status launch_list_gemv(int dtype, const GemvListArgs& a, cudaStream_t st);
-afx_status launch_list_one_token(int dtype, const GemvListArgs& a, cudaStream_t st);  // afx_onetok.cu
 
 }  // namespace afx

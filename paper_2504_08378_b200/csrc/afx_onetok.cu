@@ -89,48 +89,4 @@ afx_status launch_one_token(int dtype, int in, int ep, OneTokenForm form, const 
                             : launch_one_token_dt<AFX_BF16>(in, ep, form, a, st);
 }
 
-template <int DT, int NT, int EP>
-__global__ void __launch_bounds__(NT, 1024 / NT) slice_list_kernel(GemvListArgs a) {
-    extern __shared__ __align__(16) unsigned char dyn[];
-    slice_list_block<DT, NT, EP>(a, dyn);
-}
-
-template <int DT, int NT>
-static afx_status launch_slice_list(const GemvListArgs& a, cudaStream_t st) {
-    const int most = slice_max_pieces(NT) / kSlGranule;  // granules per slice
-    const int granules = (a.N / 8 + kSlGranule - 1) / kSlGranule;
-    int nb = sm_count() > 0 ? sm_count() : 148;
-    if (nb > granules) nb = granules;
-    if ((granules + nb - 1) / nb > most) nb = ((granules + most - 1) / most + nb - 1) / nb * nb;
-    if (static_cast<int64_t>(nb) * granules >= 0x7FFFFFFF) return AFX_ERR_CAPACITY;
-    size_t dyn = slice_given_smem(NT);
-    if (NT == 512 && dyn < kSlAlone) dyn = kSlAlone;
-    auto go = [&](auto kern) {
-        if (!ensure_dyn_smem(reinterpret_cast<const void*>(kern), dyn)) {
-            cudaGetLastError();
-            return AFX_ERR_CUDA;
-        }
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(nb, 1, 1);
-        cfg.blockDim = dim3(NT, 1, 1);
-        cfg.dynamicSmemBytes = dyn;
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        return cudaLaunchKernelEx(&cfg, kern, a) == cudaSuccess ? AFX_OK : AFX_ERR_CUDA;
-    };
-    if (a.silu) return go(slice_list_kernel<DT, NT, EP_SILU>);
-    return a.accumulate ? go(slice_list_kernel<DT, NT, EP_ACCUM>) : go(slice_list_kernel<DT, NT, EP_STORE>);
-}
-
-// 512 and 1024 threads: as in launch_slice_k.
-afx_status launch_list_one_token(int dtype, const GemvListArgs& a, cudaStream_t st) {
-    const bool narrow = static_cast<int64_t>(a.K) * a.N <= (8 << 20);
-    if (dtype == AFX_F16) return narrow ? launch_slice_list<AFX_F16, 512>(a, st) : launch_slice_list<AFX_F16, 1024>(a, st);
-    return narrow ? launch_slice_list<AFX_BF16, 512>(a, st) : launch_slice_list<AFX_BF16, 1024>(a, st);
-}
-
 }  // namespace afx

@@ -300,100 +300,4 @@ __device__ __forceinline__ void slice_op_block(const FusedArgs& a, unsigned char
     AFX_MARK(7);
 }
 
-// ---- the operator on a list given by the caller (afx_sparse_gemv, one token) ----
-
-constexpr int kSlListCap = 8192;  // staged entries per pass: row offset in 16-byte units, 16-bit input
-
-__host__ __device__ inline size_t slice_given_smem(int threads) {
-    const size_t list = static_cast<size_t>(kSlListCap) * 6, sums = static_cast<size_t>(threads) * 9 * 4;
-    return list > sums ? list : sums;
-}
-
-template <int DT, int NT, int EP>
-__device__ __forceinline__ void slice_list_block(const GemvListArgs& a, unsigned char* dyn) {
-    const int tid = threadIdx.x;
-    // this block's slice, as in slice_op_block
-    const int nb = gridDim.x, b = blockIdx.x;
-    const int pieces = a.N / 8, granules = (pieces + kSlGranule - 1) / kSlGranule;
-    const int g_lo = b * granules / nb, g_hi = (b + 1) * granules / nb;
-    const int piece0 = g_lo * kSlGranule, P = max(1, min(g_hi * kSlGranule, pieces) - piece0), nout = P * 8;
-    const int rows = NT / P, g = tid / P, piece = tid - g * P;
-    uint32_t* const off = reinterpret_cast<uint32_t*>(dyn);
-    uint16_t* const xb = reinterpret_cast<uint16_t*>(dyn + static_cast<size_t>(kSlListCap) * 4);
-    const uint64_t ld16 = static_cast<uint64_t>(a.ldw >> 3);
-    const char* base = reinterpret_cast<const char*>(a.Wt + static_cast<size_t>(piece0 + piece) * 8);
-    __shared__ int first_ok;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // only after the wait (ordering rule)
-    int cnt = *a.count;
-    if (cnt < 0 || cnt > a.K) {
-        if (tid == 0 && b == 0) report_status(a.status, AFX_ERR_CAPACITY);
-        cnt = max(0, min(cnt, a.K));
-    }
-    float y_old = 0.0f;
-    if (EP == EP_ACCUM && tid < nout) y_old = a.ep.y[piece0 * 8 + tid];
-    f32x2 acc[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) acc[i] = pack_f32x2(0.0f, 0.0f);
-    for (int c0 = 0; c0 < cnt; c0 += kSlListCap) {
-        int staged = min(kSlListCap, cnt - c0);
-        if (c0 > 0) __syncthreads();  // the previous pass has been read
-        bool skipped = false;
-        for (int i = tid; i < staged; i += NT) {
-            // An entry outside [0, K), or one whose cache slot is negative (a channel that found
-            // no row), takes no part: x = 0, and the status word says so.
-            const int j = a.idx[c0 + i];
-            const int col = a.slot != nullptr ? a.slot[c0 + i] : j;
-            const bool in_range = static_cast<unsigned>(j) < static_cast<unsigned>(a.K);
-            const uint64_t o = static_cast<uint64_t>(col < 0 ? 0 : col) * ld16;
-            const bool ok = in_range && col >= 0 && o + static_cast<uint64_t>(a.N >> 3) <= 0xFFFFFFFFull;
-            if (!ok && b == 0) report_status(a.status, in_range ? AFX_ERR_CAPACITY : AFX_ERR_INVALID_ARG);
-            skipped |= !ok;
-            off[i] = ok ? static_cast<uint32_t>(o) : kSkippedEntry;
-            xb[i] = ok ? a.x[j] : uint16_t(0);
-        }
-        if (__syncthreads_or(skipped)) {
-            // Rare.  A skipped entry still costs a load in the streaming loop; whatever it reads is multiplied
-            // by 0, so it must read weights (finite): the row of the first entry that does take part.
-            if (tid == 0) first_ok = staged;
-            __syncthreads();
-            for (int i = tid; i < staged; i += NT)
-                if (off[i] != kSkippedEntry) atomicMin(&first_ok, i);
-            __syncthreads();
-            const int f = first_ok;
-            if (f < staged) {
-                const uint32_t safe = off[f];
-                __syncthreads();
-                for (int i = tid; i < staged; i += NT)
-                    if (off[i] == kSkippedEntry) off[i] = safe;
-            } else {
-                staged = 0;  // nothing in this part of the list takes part
-            }
-            __syncthreads();
-        }
-        if (g < rows) {
-            constexpr int U = 8;
-            for (int p = g; p < staged; p += U * rows) {
-                uint4 raw[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u)
-                    if (p + u * rows < staged) raw[u] = ld_stream_16B(base + static_cast<uint64_t>(off[p + u * rows]) * 16);
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    if (p + u * rows < staged) {
-                        f32x2 w[4];
-                        unpack8_pairs<DT>(raw[u], w);
-                        const float xv = bits_to_float<DT>(xb[p + u * rows]);
-                        const f32x2 x2 = pack_f32x2(xv, xv);
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) fma_f32x2(acc[i], w[i], x2);
-                    }
-                }
-            }
-        }
-    }
-    const float scale = EP != EP_SILU && a.ep.scale != nullptr ? *a.ep.scale : 1.0f;
-    slice_finish<DT, NT, EP>(acc, g, rows, P, piece0, dyn, a.ep.y, a.ep.out_bits, scale, y_old);
-}
-
 }  // namespace afx
