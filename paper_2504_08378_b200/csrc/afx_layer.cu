@@ -120,6 +120,10 @@ static afx_status launch_fused_mt(const FusedArgs& a, cudaStream_t st) {
 // 39.9 and 56.6.
 template <int DT, int IN, int EP>
 static afx_status launch_split(const FusedArgs& a, cudaStream_t st) {
+    // The list kernel's 32-bit row offsets would drop the channels behind them, and nothing may fail behind the
+    // first of the two launches.
+    if (static_cast<uint64_t>(a.K) * static_cast<uint64_t>(a.ldw >> 3) > 0x100000000ull) return AFX_ERR_CAPACITY;
+    if ((a.N + kMtTile - 1) / kMtTile > 65535) return AFX_ERR_CAPACITY;
     const afx_status rc = launch_select_tokens(DT, IN == IN_NORM, a, st);
     if (rc != AFX_OK) return rc;
     GemvListArgs g = {};

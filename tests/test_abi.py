@@ -103,6 +103,17 @@ def test_gemv_rejects_bad_arguments_on_the_host():
     assert e.value.status == 2
 
 
+@pytest.mark.parametrize("T", [1, 2, 8])
+@pytest.mark.parametrize("lists", [True, False])
+def test_select_gemv_refuses_row_offsets_beyond_32_bits(T, lists):
+    """Rows are addressed in 16-byte units with 32 bits, with one token and several, with and without list outputs."""
+    K, N = 4096, 64
+    out = (FAKE, FAKE) if lists else (None, None)
+    with pytest.raises(afx.AfxError) as e:
+        afx.afx_select_gemv(FAKE, 1, K, N, (1 << 23) + 8, FAKE, T, 0, 8, 0.0, FAKE, 0, *out, stream=0)
+    assert e.value.status == 3
+
+
 def test_diff_rejects_bad_arguments_on_the_host():
     assert _status(afx.afx_diff_active, None, FAKE, FAKE, 8, FAKE, FAKE, FAKE) == 1
     assert _status(afx.afx_diff_active, FAKE, FAKE, FAKE, 0, FAKE, FAKE, FAKE) == 1
