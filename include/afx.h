@@ -282,7 +282,10 @@ afx_status afx_layer_step(afx_model* model, int layer, afx_state* state, int pos
  * ONE of the five kernels of afx_layer_step, on whatever the state holds (afx_layer_step is
  * exactly the five calls in order).  For per-operator timing and profiling of the launches a
  * decode step really makes -- the same kernel instantiation, launch shape and side outputs;
- * this library's own addition, the paper has no counterpart.
+ * this library's own addition, the paper has no counterpart.  One difference: inside
+ * afx_layer_step the attention requests its first cache rows before the q | k | v operator in
+ * front of it is done; AFX_STEP_ATTN by itself reads the cache only after everything before it
+ * on the stream, which may be the call that wrote those rows.
  */
 #define AFX_STEP_QKV 0
 #define AFX_STEP_ATTN 1

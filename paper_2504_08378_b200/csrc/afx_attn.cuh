@@ -31,6 +31,9 @@ struct AttnArgs {
     const float* rope_cos;  // [max_seq][64]
     const float* rope_sin;
     uint16_t* out;  // [T][q_heads*128] dtype bits
+    // The grid in front of this one waited for everything before it and writes no cache rows (a step's own q | k | v
+    // operator): the past rows are final when this grid starts and may be read before its dependency wait.
+    int past_final;
 };
 
 afx_status launch_attention(int dtype, const AttnArgs& a, cudaStream_t st);  // afx_attn.cu
@@ -97,10 +100,8 @@ __device__ __forceinline__ void attention_block(const AttnArgs& a, AttnSmem* sm)
             }
         }
     };
-    // The past rows of this half warp's first batch were written by earlier tokens' attention kernels
-    // -- at least one layer step (five grids) back, so complete by the ordering rule stated in
-    // fused_op_block -- and are requested before the wait for q, k, v.
-    fetch(l_lo + worker, 0, min(l_hi, a.pos));
+    // Inside a layer step the past rows of this half warp's first batch are requested before the wait for q, k, v.
+    if (a.past_final) fetch(l_lo + worker, 0, min(l_hi, a.pos));
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // only after the wait (see fused_op_block)
     AFX_MARK(1);
@@ -137,7 +138,7 @@ __device__ __forceinline__ void attention_block(const AttnArgs& a, AttnSmem* sm)
 #pragma unroll
     for (int j = 0; j < 8; ++j) acc[j] = 0.0f;
     AFX_MARK(2);
-    fetch(l_lo + worker, a.pos, l_hi);  // the first batch's row that this kernel has just appended
+    fetch(l_lo + worker, a.past_final ? a.pos : 0, l_hi);  // the row that this kernel has just appended, or all of the first batch
     const float4 qa = *reinterpret_cast<const float4*>(&sm->q[l16 * 8]);
     const float4 qb = *reinterpret_cast<const float4*>(&sm->q[l16 * 8 + 4]);
     for (int p0 = l_lo + worker; p0 < l_hi; p0 += kAttnWorkers * U) {

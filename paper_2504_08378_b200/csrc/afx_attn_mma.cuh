@@ -95,16 +95,19 @@ __device__ __forceinline__ void attention_mma_block(const AttnArgs& a, AttnMmaSm
                 for (int q = 0; q < 2; ++q) vr[h][e][q] = r[8 * q + gid];
             }
     };
-    // The past rows were written by earlier tokens' attention kernels -- at least one layer step (five
-    // grids) back, so complete by the ordering rule stated in fused_op_block -- and the first tile's are
-    // requested before the wait for q, k, v.
-    if (t_lo + warp < t_hi) {
+    // Inside a layer step the first tile's rows are requested before the wait for q, k, v.
+    const bool any = t_lo + warp < t_hi;
+    if (any && a.past_final) {
         fetch_k(t_lo + warp);
         fetch_v(t_lo + warp);
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // only after the wait (see fused_op_block)
     AFX_MARK(1);
+    if (any && !a.past_final) {
+        fetch_k(t_lo + warp);
+        fetch_v(t_lo + warp);
+    }
 
     const float* row = a.qkv + static_cast<size_t>(t) * a.n_qkv;
     const float2* cs = reinterpret_cast<const float2*>(a.rope_cos + static_cast<size_t>(a.pos) * (kHeadDim / 2));

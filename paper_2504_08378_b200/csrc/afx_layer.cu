@@ -398,8 +398,9 @@ static afx_status check_step(const afx_model* m, int layer, const afx_state* s) 
 
 namespace afx {
 
-// One of the five kernels of a layer step (which = AFX_STEP_*), on validated arguments.
-static afx_status launch_layer_kernel(afx_model* m, int layer, afx_state* s, int pos, int which, cudaStream_t st) {
+// One of the five kernels of a layer step (which = AFX_STEP_*), on validated arguments.  in_step: the launch in front
+// of an AFX_STEP_ATTN is the same step's q | k | v operator (by itself the kernel may follow anything).
+static afx_status launch_layer_kernel(afx_model* m, int layer, afx_state* s, int pos, int which, bool in_step, cudaStream_t st) {
     const afx_model_desc& d = m->d;
     const afx_layer_desc& L = m->layers[layer];
     float* h = reinterpret_cast<float*>(s->blob + s->off_h);
@@ -439,6 +440,7 @@ static afx_status launch_layer_kernel(afx_model* m, int layer, afx_state* s, int
             at.rope_cos = m->rope;
             at.rope_sin = m->rope + static_cast<size_t>(d.max_seq) * (kHeadDim / 2);
             at.out = attn;
+            at.past_final = in_step;
             return launch_attention(d.dtype, at, st);
         }
         case AFX_STEP_O:
@@ -486,7 +488,7 @@ extern "C" afx_status afx_layer_step(afx_model* m, int layer, afx_state* s, int 
     if (rc != AFX_OK) return rc;
     if (pos < 0 || pos >= m->d.max_seq) return AFX_ERR_INVALID_ARG;
     for (int which = AFX_STEP_QKV; which <= AFX_STEP_DOWN; ++which)
-        if ((rc = launch_layer_kernel(m, layer, s, pos, which, static_cast<cudaStream_t>(stream))) != AFX_OK) return rc;
+        if ((rc = launch_layer_kernel(m, layer, s, pos, which, true, static_cast<cudaStream_t>(stream))) != AFX_OK) return rc;
     return AFX_OK;
 }
 
@@ -495,7 +497,7 @@ extern "C" afx_status afx_layer_kernel(afx_model* m, int layer, afx_state* s, in
     afx_status rc = check_step(m, layer, s);
     if (rc != AFX_OK) return rc;
     if (pos < 0 || pos >= m->d.max_seq || which < AFX_STEP_QKV || which > AFX_STEP_DOWN) return AFX_ERR_INVALID_ARG;
-    return launch_layer_kernel(m, layer, s, pos, which, static_cast<cudaStream_t>(stream));
+    return launch_layer_kernel(m, layer, s, pos, which, false, static_cast<cudaStream_t>(stream));
 }
 
 namespace afx {
@@ -530,9 +532,9 @@ extern "C" afx_status afx_layer_step_hosted(afx_model* m, int layer, afx_state* 
     const afx_layer_desc& L = m->layers[layer];
     const int which_of[4] = {AFX_STEP_QKV, AFX_STEP_O, AFX_STEP_GU, AFX_STEP_DOWN};
     for (int op = 0; op < 4; ++op) {
-        if (op == AFX_OP_O && (rc = launch_layer_kernel(m, layer, s, pos, AFX_STEP_ATTN, st)) != AFX_OK) return rc;
+        if (op == AFX_OP_O && (rc = launch_layer_kernel(m, layer, s, pos, AFX_STEP_ATTN, true, st)) != AFX_OK) return rc;
         if (ops->cache[op] == nullptr && ops->swap[op] == nullptr) {  // resident weights: the fused kernel
-            if ((rc = launch_layer_kernel(m, layer, s, pos, which_of[op], st)) != AFX_OK) return rc;
+            if ((rc = launch_layer_kernel(m, layer, s, pos, which_of[op], true, st)) != AFX_OK) return rc;
             continue;
         }
         // 1. input stage + selection
@@ -615,9 +617,9 @@ extern "C" afx_status afx_layer_step_q4(afx_model* m, int layer, afx_state* s, i
     const afx_layer_desc& L = m->layers[layer];
     const int which_of[4] = {AFX_STEP_QKV, AFX_STEP_O, AFX_STEP_GU, AFX_STEP_DOWN};
     for (int op = 0; op < 4; ++op) {
-        if (op == AFX_OP_O && (rc = launch_layer_kernel(m, layer, s, pos, AFX_STEP_ATTN, st)) != AFX_OK) return rc;
+        if (op == AFX_OP_O && (rc = launch_layer_kernel(m, layer, s, pos, AFX_STEP_ATTN, true, st)) != AFX_OK) return rc;
         if (q4->wq[op] == nullptr) {  // 16-bit weights: the fused kernel
-            if ((rc = launch_layer_kernel(m, layer, s, pos, which_of[op], st)) != AFX_OK) return rc;
+            if ((rc = launch_layer_kernel(m, layer, s, pos, which_of[op], true, st)) != AFX_OK) return rc;
             continue;
         }
         // input stage + selection + the operator on the 4-bit rows of the active channels, one kernel

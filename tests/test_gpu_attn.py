@@ -38,3 +38,41 @@ def test_attention_matches_oracle_at_tile_edges(pos, kvh, rep, T):
         assert np.array_equal(have[:, :pos], before[:, :pos])
         assert np.abs(have[:, pos].astype(np.int32) - want[:, pos].astype(np.int32)).max() <= 1
     m.close()
+
+
+@pytest.mark.parametrize("kvh,rep,T", [(4, 1, 1), (8, 1, 4), (4, 4, 1), (2, 8, 2)])
+def test_attention_calls_in_a_row_see_each_others_rows(kvh, rep, T):
+    """The attention kernel of one layer at consecutive (and earlier) positions without any other kernel between: each
+    call must read the rows that the calls before it wrote, not what the cache held."""
+    dt, heads, start, n = "bf16", kvh * rep, 37, 24
+    hidden, mlp, max_seq = 128, 64, start + n
+    positions = list(range(start, max_seq)) + [5, max_seq - 1, 3, 6]
+    L = synth.layer_weights(43, 0, hidden, heads, kvh, mlp, dt)
+    kc0, vc0 = synth.kv_cache(43, 0, T, max_seq, kvh, max_seq)
+    L["k_cache"], L["v_cache"], L["k"] = kc0, vc0, [hidden, heads * 128, hidden, mlp]
+    m = DecoderModel(dt, hidden, heads, kvh, mlp, max_seq, [L], T=T)
+    qkv = torch.from_numpy(np.random.default_rng(7).standard_normal(m.qkv.shape).astype(np.float32)).cuda()
+    qkv[:, -kvh * 128:] *= 50  # values of new rows unlike the old ones
+    got = []
+    for sync in (True, False):
+        m.k_cache[0].copy_(torch.from_numpy(kc0.view(np.int16)))
+        m.v_cache[0].copy_(torch.from_numpy(vc0.view(np.int16)))
+        m.qkv.copy_(qkv)
+        torch.cuda.synchronize()
+        outs = torch.empty((len(positions), *m.bits(afx.BUF_ATTN).shape), dtype=torch.int16, device="cuda")
+        for i, pos in enumerate(positions):
+            m.layer_kernel(0, pos, afx.STEP_ATTN)
+            if sync:
+                torch.cuda.synchronize()
+                outs[i] = m.bits(afx.BUF_ATTN)
+        if not sync:
+            outs[-1] = m.bits(afx.BUF_ATTN)
+        got.append((outs[-1].clone(), m.k_cache[0].clone(), m.v_cache[0].clone()))
+    assert all(torch.equal(a, b) for a, b in zip(*got))
+    # the last call, at position 6, read the rows of the calls at 3 and 5
+    q = qkv.double().cpu().numpy()
+    kc, vc = (got[0][i].cpu().numpy().view(np.uint16).copy() for i in (1, 2))
+    ref = oracle.decode(ol.attention_stage(ol.Config(dt, hidden, heads, kvh, mlp), q, kc, vc, positions[-1]), dt)
+    out = oracle.decode(got[0][0].cpu().numpy().view(np.uint16), dt)
+    assert np.abs(out - ref).max() <= 2.0 ** -8 * np.abs(ref).max()  # one rounding to bf16
+    m.close()
