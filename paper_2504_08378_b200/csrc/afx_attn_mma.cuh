@@ -53,6 +53,10 @@ __device__ __forceinline__ void split_pair(float a, float b, uint32_t& hi, uint3
     lo = pack2_bits<AFX_F16>(a - f.x, b - f.y);
 }
 
+// A product's sums of the high and the low halves.  An infinity in the cache makes the high one what the product is
+// (infinite, or NaN); the low one may then be of the other sign, or 0 times infinity, and says nothing.
+__device__ __forceinline__ float whole(float hi, float lo) { return fabsf(hi) <= 3.402823466e38f ? hi + lo : hi; }
+
 template <int DT>
 __device__ __forceinline__ void attention_mma_block(const AttnArgs& a, AttnMmaSmem* sm) {
     constexpr int NW = kAttnMmaWarps, NT = kAttnMmaThreads;
@@ -74,7 +78,8 @@ __device__ __forceinline__ void attention_mma_block(const AttnArgs& a, AttnMmaSm
     uint16_t* kc = a.k_cache + (static_cast<size_t>(t) * a.max_seq * a.kv_heads + hk) * kHeadDim;
     uint16_t* vc = a.v_cache + (static_cast<size_t>(t) * a.max_seq * a.kv_heads + hk) * kHeadDim;
 
-    // Rows behind the last past position are read as the last one and masked below.
+    // Key rows behind the last past position are read as the last one, and their scores masked below; value rows are
+    // zero there (a probability of 0 times an infinity of the last row would be NaN).
     uint4 kr[2][4], vr[2][2][2];
     auto row_of = [&](int p) { return static_cast<size_t>(min(p, a.pos - 1)) * row_stride; };
     auto fetch_k = [&](int tile) {  // tile half h: the lane's position 8 h + gid, 16-byte pieces 4 j + tig
@@ -90,9 +95,10 @@ __device__ __forceinline__ void attention_mma_block(const AttnArgs& a, AttnMmaSm
         for (int h = 0; h < 2; ++h)
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                const uint4* r = reinterpret_cast<const uint4*>(vc + row_of(tile * 16 + 8 * h + 2 * tig + e));
+                const int p = tile * 16 + 8 * h + 2 * tig + e;
+                const uint4* r = reinterpret_cast<const uint4*>(vc + row_of(p));
 #pragma unroll
-                for (int q = 0; q < 2; ++q) vr[h][e][q] = r[8 * q + gid];
+                for (int q = 0; q < 2; ++q) vr[h][e][q] = p < a.pos ? r[8 * q + gid] : make_uint4(0u, 0u, 0u, 0u);
             }
     };
     // Inside a layer step the first tile's rows are requested before the wait for q, k, v.
@@ -221,14 +227,15 @@ __device__ __forceinline__ void attention_mma_block(const AttnArgs& a, AttnMmaSm
             for (int h = 0; h < 2; ++h)
 #pragma unroll
                 for (int e = 0; e < 2; ++e)
-                    s[h][e] = tile * 16 + 8 * h + 2 * tig + e < a.pos ? (c[h][e] + c[h][2 + e]) * unit : -INFINITY;
+                    s[h][e] = tile * 16 + 8 * h + 2 * tig + e < a.pos ? whole(c[h][e], c[h][2 + e]) * unit : -INFINITY;
         }
         float mn = fmaxf(fmaxf(s[0][0], s[0][1]), fmaxf(s[1][0], s[1][1]));
         mn = fmaxf(mn, __shfl_xor_sync(0xFFFFFFFFu, mn, 1));
         mn = fmaxf(mn, __shfl_xor_sync(0xFFFFFFFFu, mn, 2));
-        mn = fmaxf(mn, m_run);  // finite: a tile holds at least one past position
+        mn = fmaxf(mn, m_run);  // (-inf while every score has been)
+        const float ref = mn == -INFINITY ? 0.0f : mn;
         if (__any_sync(0xFFFFFFFFu, mn > m_run)) {
-            const float f = fast_exp2(m_run - mn);  // 0 on the first visit (m_run = -inf)
+            const float f = fast_exp2(m_run - ref);  // 0 on the first visit (m_run = -inf)
             m_run = mn;
             l_run *= f;
 #pragma unroll
@@ -241,7 +248,7 @@ __device__ __forceinline__ void attention_mma_block(const AttnArgs& a, AttnMmaSm
         uint32_t p[4];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const float p0 = fast_exp2(s[h][0] - mn) * kUp, p1 = fast_exp2(s[h][1] - mn) * kUp;
+            const float p0 = fast_exp2(s[h][0] - ref) * kUp, p1 = fast_exp2(s[h][1] - ref) * kUp;
             l_run += p0 + p1;
             split_pair(p0, p1, p[2 * h], p[2 * h + 1]);
         }
@@ -276,7 +283,7 @@ __device__ __forceinline__ void attention_mma_block(const AttnArgs& a, AttnMmaSm
                 float4* d = reinterpret_cast<float4*>(&sm->acc[warp][gid][64 * q + 16 * tig + 8 * c]);
                 float v[8];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) v[i] = (o[q][i][c] + o[q][i][2 + c]) * (1.0f / kUp);
+                for (int i = 0; i < 8; ++i) v[i] = whole(o[q][i][c], o[q][i][2 + c]) * (1.0f / kUp);
                 d[0] = make_float4(v[0], v[1], v[2], v[3]);
                 d[1] = make_float4(v[4], v[5], v[6], v[7]);
             }

@@ -97,3 +97,41 @@ def test_attention_keeps_32_bit_precision(kvh, rep, pos):
     ref = ol.attention_stage(cfg, qkv.astype(np.float64), kc, vc, pos)
     assert (m.bits(afx.BUF_ATTN).cpu().numpy().view(np.uint16) != ref).mean() <= 0.014
     m.close()
+
+
+@pytest.mark.parametrize("kvh,rep", [(3, 2), (2, 8)])
+@pytest.mark.parametrize("pos", [17, 200])
+def test_attention_with_infinities_in_the_cache(kvh, rep, pos):
+    """fp16 caches overflow to infinity.  A key that makes every head's score -inf leaves its position out (the only
+    past one of a tile among them); an infinite value makes its dimension infinite and nothing else."""
+    dt, heads, T = "f16", kvh * rep, 1
+    hidden, mlp, max_seq = 128, 64, pos + 1
+    cfg = ol.Config(dt, hidden, heads, kvh, mlp)
+    L = synth.layer_weights(53, 0, hidden, heads, kvh, mlp, dt)
+    kc, vc = synth.kv_cache(53, 0, T, max_seq, kvh, pos)
+    qkv = np.random.default_rng(pos).standard_normal((T, (heads + 2 * kvh) * 128)).astype(np.float32)
+    rot = np.stack([oracle.rope(qkv[0, h * 128:(h + 1) * 128].reshape(1, 1, 128), np.full(1, pos, np.int32))[0, 0] for h in range(heads)])
+    for g in range(kvh):
+        d = 127  # a dimension in which all queries of the group are made positive
+        for h in range(g * rep, (g + 1) * rep):
+            if rot[h, d] <= 0:
+                qkv[0, h * 128:(h + 1) * 128] *= -1
+        for p in (0, 5, 16):
+            kc[0, p, g, d] = 0xFC00  # -inf
+        vc[0, 3, g, 10] = 0x7C00
+        vc[0, pos - 1 if pos > 17 else 15, g, 77] = 0xFC00  # (200: the row that fills up the last tile)
+    L["k_cache"], L["v_cache"], L["k"] = kc.copy(), vc.copy(), [hidden, heads * 128, hidden, mlp]
+    m = DecoderModel(dt, hidden, heads, kvh, mlp, max_seq, [L], T=T)
+    m.qkv.copy_(torch.from_numpy(qkv).cuda())
+    m.layer_kernel(0, pos, afx.STEP_ATTN)
+    got = oracle.decode(m.bits(afx.BUF_ATTN).cpu().numpy().view(np.uint16), dt).reshape(heads, 128)
+    K, V = (oracle.decode(c.cpu().numpy().view(np.uint16), "f16")[0] for c in (m.k_cache[0], m.v_cache[0]))
+    for h in range(heads):
+        q = oracle.rope(qkv[0, h * 128:(h + 1) * 128].reshape(1, 1, 128).astype(np.float64), np.full(1, pos, np.int32))[0, 0]
+        sc = K[:, h // rep] @ q / np.sqrt(128.0)
+        w = np.exp(sc - sc.max())
+        want = (w[:, None] * V[:, h // rep]).sum(0) / w.sum()
+        fin = np.isfinite(want)
+        assert (~fin).sum() >= 1 and np.array_equal(got[h][~fin], want[~fin])
+        assert np.abs(got[h][fin] - want[fin]).max() <= 2 * 2.0 ** -11 * np.abs(want[fin]).max()
+    m.close()
