@@ -86,3 +86,20 @@ def test_router_breaks_ties_toward_the_lower_expert():
         assert abs(wsel.sum() - 1.0) < 1e-6 and np.isfinite(y).all()
         ids, w, _ = ol.moe_router(xb, synth.f32_to_bits(Wr, dt), dt, top)
         assert ids.tolist() == want and np.allclose(wsel, w, rtol=1e-5)
+
+
+@pytest.mark.parametrize("E,ld", [(3, 3), (4, 8), (5, 16), (8, 8), (8, 12), (9, 16), (12, 12), (12, 24), (16, 16)])
+@pytest.mark.parametrize("hidden", [264, 4104])
+def test_router_rows_in_pieces(E, ld, hidden):
+    """Expert counts and row strides with and without whole 16-byte pieces; what lies behind the experts is NaN."""
+    dt, mlp = "bf16", 64
+    experts_np = [synth.layer_weights(503, 0, hidden, 1, 1, mlp, dt)] * E
+    Wr = np.full((hidden, ld), 0x7FC0, np.uint16)
+    Wr[:, :E] = synth.weight(503, 9, hidden, E, dt, sigma=0.05)
+    x = synth.laplace_bits(503, 7, (1, hidden), dt)
+    ids, w, logits = ol.moe_router(x, Wr[:, :E], dt, 2)
+    lg, sel, wsel, _, _ = run_moe(dt, hidden, mlp, E, 2, experts_np, Wr, x, hidden // 2, mlp // 2)
+    # exact products, fp32 additions in any order
+    bound = (hidden + 1) * 2.0 ** -24 * (np.abs(oracle.decode(x, dt)[0])[:, None] * np.abs(oracle.decode(Wr[:, :E], dt))).sum(0)
+    assert (np.abs(lg - logits) <= bound).all()
+    assert sel.tolist() == ids.tolist() and np.allclose(wsel, w, rtol=1e-4)
