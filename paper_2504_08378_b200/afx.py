@@ -210,8 +210,11 @@ def _stream(stream):
         if _current_raw_stream is None:
             import torch
             torch.cuda.init()
-            device, raw = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
-            _current_raw_stream = lambda: raw(device())
+            device, raw = (getattr(torch._C, n, None) for n in ("_cuda_getDevice", "_cuda_getCurrentRawStream"))
+            if device is not None and raw is not None:
+                _current_raw_stream = lambda: raw(device())
+            else:  # not part of torch's public interface
+                _current_raw_stream = lambda: torch.cuda.current_stream().cuda_stream
         return _current_raw_stream()
     if isinstance(stream, int):
         return stream

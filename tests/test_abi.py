@@ -158,3 +158,18 @@ def test_binding_structs_have_the_headers_layout(tmp_path):
         py_names = [f[0] for f in cls._fields_]
         assert py_names == fields[cname], (cname, py_names, fields[cname])
         assert [getattr(cls, n).offset for n in py_names] == [int(o) for o in offs], cname
+
+
+@pytest.mark.parametrize("private", [True, False])
+def test_current_stream_with_and_without_torchs_private_handle(monkeypatch, private):
+    torch = pytest.importorskip("torch")
+    monkeypatch.setattr(afx, "_current_raw_stream", None)
+    monkeypatch.setattr(torch.cuda, "init", lambda: None)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: type("S", (), {"cuda_stream": 17}))
+    for name, value in (("_cuda_getDevice", lambda: 3), ("_cuda_getCurrentRawStream", lambda d: 40 + d)):
+        if private:
+            monkeypatch.setattr(torch._C, name, value, raising=False)
+        else:
+            monkeypatch.delattr(torch._C, name, raising=False)
+    assert afx._stream(None) == (43 if private else 17)
+    assert afx._stream(5) == 5
