@@ -4,15 +4,18 @@
 
 namespace afx {
 
-template <int DT, int NT, int NW, int CH, int IN, int EP, bool GRP>
+template <int DT, int NT, int NW, int CH, int IN, int EP, bool GRP, bool SPLIT>
 __global__ void __launch_bounds__(NT, 1024 / NT) slice_op_kernel(FusedArgs a) {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ RegSelScratch s;
-    slice_op_block<DT, NT, NW, CH, IN, EP, GRP>(a, dyn, &s);
+    __shared__ float recv[SPLIT ? kSlMaxSplit * kSlSplitOutputs : 1];
+    slice_op_block<DT, NT, NW, CH, IN, EP, GRP, SPLIT>(a, dyn, &s, recv);
 }
 
-template <int DT, int NT, int NW, int CH, int IN, int EP, bool GRP>
-static afx_status launch_slice(const FusedArgs& a, cudaStream_t st) {
+// split: blocks (a cluster) that share the list of a granule; a.N is then at most as wide as there is room for
+// one granule per cluster.
+template <int DT, int NT, int NW, int CH, int IN, int EP, bool GRP, bool SPLIT = false>
+static afx_status launch_slice(const FusedArgs& a, cudaStream_t st, int split = 1) {
     if (static_cast<uint64_t>(a.K) * static_cast<uint64_t>(a.ldw >> 3) > 0x100000000ull) return AFX_ERR_CAPACITY;
     FusedArgs b = a;
     b.side_cluster = a.idx_out != nullptr || a.count_out != nullptr || a.bitmap_out != nullptr ||
@@ -31,21 +34,28 @@ static afx_status launch_slice(const FusedArgs& a, cudaStream_t st) {
     b.slices = nb;
     size_t dyn = slice_dyn_smem(NT, a.K, a.idx_in != nullptr);
     if (NT == 512 && dyn < kSlAlone) dyn = kSlAlone;
-    auto kern = slice_op_kernel<DT, NT, NW, CH, IN, EP, GRP>;
+    auto kern = slice_op_kernel<DT, NT, NW, CH, IN, EP, GRP, SPLIT>;
     if (!ensure_dyn_smem(reinterpret_cast<const void*>(kern), dyn)) {
         cudaGetLastError();
         return AFX_ERR_CUDA;
     }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(nb * groups + b.side_cluster, 1, 1);
+    const int units = nb * groups + b.side_cluster;
+    // clusters that the occupancy query counts and that are then placed behind another kernel differ by a few
+    while (SPLIT && split > 1 && max_active_clusters(reinterpret_cast<const void*>(kern), split, dyn, NT) < units + 2) split >>= 1;
+    cfg.gridDim = dim3(units * split, 1, 1);
     cfg.blockDim = dim3(NT, 1, 1);
     cfg.dynamicSmemBytes = dyn;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = split;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = SPLIT ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kern, b) == cudaSuccess ? AFX_OK : AFX_ERR_CUDA;
 }
 
@@ -56,9 +66,21 @@ static afx_status launch_slice(const FusedArgs& a, cudaStream_t st) {
 // the loads in flight (4096 -> 22016: 20.0 us, with 512 threads 24.1), and from K = 4096 on that is worth
 // more than the overlap (8 layers of 8192 channels, 8000 positions: 1573 us, with 512 threads 1613).
 constexpr int kSlNarrowMaxK = 4096;
+// From here on clusters share a granule's list, where at least four blocks find an SM for each granule.  One block and
+// a cluster per granule, half of the channels kept, in a graph: 5120 -> 256 6.9 and 6.4 us, 5120 -> 1024 7.1 and 7.3,
+// 8192 -> 512 8.2 and 6.9, 8192 -> 1024 9.7 and 8.2, 16384 -> 256 12.9 and 8.2, 28672 -> 512 20.8 and 15.0; two
+// blocks per granule do not pay (8192 -> 2048 9.4 and 9.7).
+constexpr int kSlSplitMinK = 6144;
 // Selecting warps and slots: as few warps as leave a lane enough registers.
 template <int DT, int IN, int EP, bool GRP>
 static afx_status launch_slice_k(const FusedArgs& a, cudaStream_t st) {
+    if (a.K >= kSlSplitMinK) {
+        const int clusters = (a.N / 8 + kSlGranule - 1) / kSlGranule * (GRP ? a.groups : 1) + 1;  // (one for the side outputs)
+        const int fit = (sm_count() > 0 ? sm_count() : 148) / clusters;
+        const int split = fit >= 8 ? 8 : 4;
+        if (fit >= 4 && a.K <= 16384) return launch_slice<DT, 512, 16, 8, IN, EP, GRP, true>(a, st, split);
+        if (fit >= 4 && a.K <= 32768) return launch_slice<DT, 1024, 32, 8, IN, EP, GRP, true>(a, st, split);
+    }
     const bool narrow = (a.beside_attention && a.K <= kSlNarrowMaxK) || static_cast<int64_t>(a.K) * a.N <= (8 << 20);
     if (narrow && a.K <= 4096) return launch_slice<DT, 512, 8, 4, IN, EP, GRP>(a, st);
     if (narrow && a.K <= 12288) return launch_slice<DT, 512, 16, 6, IN, EP, GRP>(a, st);

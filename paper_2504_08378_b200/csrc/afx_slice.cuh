@@ -16,6 +16,8 @@
 // 17.2 and 15.3, 28672 -> 8192 70.9 and 52.0, 1024 -> 3072 7.7 and 5.7 us.
 // Sharing the selection among the eight blocks of a cluster lost again: a cluster barrier with pushed
 // operands costs 0.75 to 1 us, five of them more than the selection takes.
+// Narrow operators of many channels have fewer granules than there are SMs and long lists: there the blocks of
+// a cluster share the list of one granule (SPLIT, see launch_slice_k).
 #pragma once
 
 #include "afx_fused.cuh"
@@ -24,11 +26,14 @@
 
 namespace afx {
 
-
 constexpr int kSlGranule = 4;  // pieces (16-byte loads of a row) that one slice holds together
 // Shared memory that at least one block of 512 threads asks for, so that an SM takes one such block and
 // what it leaves free goes to a block of another kernel.
 constexpr size_t kSlAlone = 116 * 1024;
+
+// Blocks that share a granule's list at most, and outputs of a granule.
+constexpr int kSlMaxSplit = 8;
+constexpr int kSlSplitOutputs = kSlGranule * 8;
 
 // Widest slice in pieces: one output per thread in the epilogue.
 __host__ __device__ constexpr int slice_max_pieces(int threads) { return threads / 8; }
@@ -90,9 +95,11 @@ __device__ __forceinline__ void st_shared_if(uint32_t at, uint32_t v, bool on) {
 
 // The row sets' sums (thread `tid` holds row set g = tid / P, piece tid - g P, of `rows` sets) meet and leave
 // as outputs 8 piece0 .. of the operator: `parts` threads per output add every parts-th set, then in order.
-template <int DT, int NT, int EP>
-__device__ __forceinline__ void slice_finish(const f32x2 (&acc)[4], int g, int rows, int P, int piece0, unsigned char* dyn, float* y,
-                                             uint16_t* out_bits, float scale, float y_old) {
+// SPLIT: the blocks of the cluster (all have arrived once at its barrier) push their sums into block 0's `recv`,
+// which adds them in rank order.
+template <int DT, int NT, int EP, bool SPLIT>
+__device__ __forceinline__ void slice_finish(const f32x2 (&acc)[4], int g, int rows, int P, int piece0, unsigned char* dyn, float* recv,
+                                             float* y, uint16_t* out_bits, float scale, float y_old) {
     const int tid = threadIdx.x, nout = P * 8;
     const int parts = NT / nout, part = tid / nout, out = tid - part * nout;
     __syncthreads();  // the list has been read
@@ -117,10 +124,26 @@ __device__ __forceinline__ void slice_finish(const f32x2 (&acc)[4], int g, int r
         red2[tid] = sum;
     }
     __syncthreads();
-    auto total = [&](int o) {
+    auto own = [&](int o) {
         float v = red2[o];
 #pragma unroll 4
         for (int q = 1; q < parts; ++q) v += red2[q * nout + o];
+        return v;
+    };
+    const int split = SPLIT ? static_cast<int>(cg::this_cluster().num_blocks()) : 1;
+    if (SPLIT) {
+        const int rank = static_cast<int>(cg::this_cluster().block_rank());
+        cluster_wait();  // block 0 is running
+        if (tid < nout) cg::this_cluster().map_shared_rank(recv, 0)[rank * kSlSplitOutputs + tid] = own(tid);
+        __syncwarp();
+        cluster_arrive();
+        cluster_wait();
+        if (rank != 0) return;
+    }
+    auto total = [&](int o) {
+        if (!SPLIT) return own(o);
+        float v = recv[o];
+        for (int q = 1; q < split; ++q) v += recv[q * kSlSplitOutputs + o];
         return v;
     };
     if (EP == EP_SILU) {
@@ -138,13 +161,21 @@ __device__ __forceinline__ void slice_finish(const f32x2 (&acc)[4], int g, int r
 
 // GRP: the grid may hold several operators of one family (FusedArgs::groups).  The first NW of the NT / 32
 // warps select, with up to CH slots of 4 channels per lane (K <= 128 NW CH).
-template <int DT, int NT, int NW, int CH, int IN, int EP, bool GRP>
-__device__ __forceinline__ void slice_op_block(const FusedArgs& a, unsigned char* dyn, RegSelScratch* sc) {
+template <int DT, int NT, int NW, int CH, int IN, int EP, bool GRP, bool SPLIT>
+__device__ __forceinline__ void slice_op_block(const FusedArgs& a, unsigned char* dyn, RegSelScratch* sc, float* recv) {
     const int tid = threadIdx.x, warp = tid >> 5;
     const int K = a.K, m = sel_slots<NW>(K);
     const bool selects = NW == NT / 32 || warp < NW;
-    const int nb = a.slices, grp = GRP ? static_cast<int>(blockIdx.x) / nb : 0, b = static_cast<int>(blockIdx.x) - grp * nb;
-    const bool scribe = a.side_cluster != 0 && blockIdx.x == gridDim.x - 1;  // selects only, writes the side outputs
+    const int split = SPLIT ? static_cast<int>(cg::this_cluster().num_blocks()) : 1;  // blocks that share a list
+    const int rank = SPLIT ? static_cast<int>(cg::this_cluster().block_rank()) : 0;
+    const int unit = SPLIT ? static_cast<int>(blockIdx.x) / split : static_cast<int>(blockIdx.x);
+    const int units = SPLIT ? static_cast<int>(gridDim.x) / split : static_cast<int>(gridDim.x);
+    const int nb = a.slices, grp = GRP ? unit / nb : 0, b = unit - grp * nb;
+    const bool scribe = a.side_cluster != 0 && unit == units - 1;  // selects only, writes the side outputs
+    if (SPLIT) {
+        if (scribe && rank != 0) return;
+        if (!scribe) cluster_arrive();  // (the scribe's cluster never meets)
+    }
     const uint16_t* x = GRP ? a.x + grp * a.x_stride : a.x;
     uint32_t* list = reinterpret_cast<uint32_t*>(dyn);
     const bool own = a.idx_in == nullptr;
@@ -293,10 +324,11 @@ __device__ __forceinline__ void slice_op_block(const FusedArgs& a, unsigned char
     f32x2 acc[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) acc[i] = pack_f32x2(0.0f, 0.0f);
-    if (g < rows) slice_stream<DT>(Wt, a.ldw, piece0 + piece, list, cnt, g, rows, acc);
+    const int c_lo = SPLIT ? rank * cnt / split : 0, c_hi = SPLIT ? (rank + 1) * cnt / split : cnt;
+    if (g < rows) slice_stream<DT>(Wt, a.ldw, piece0 + piece, list + c_lo, c_hi - c_lo, g, rows, acc);
     AFX_MARK(5);
 
-    slice_finish<DT, NT, EP>(acc, g, rows, P, piece0, dyn, y, out_bits, scale, y_old);
+    slice_finish<DT, NT, EP, SPLIT>(acc, g, rows, P, piece0, dyn, recv, y, out_bits, scale, y_old);
     AFX_MARK(7);
 }
 

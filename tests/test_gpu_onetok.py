@@ -1,11 +1,14 @@
 """GPU parity of the one-token operator where its dispatch and its slices change: the limits of the
-selecting warps, 512 and 1024 threads, one granule, ragged last granules, more slices than SMs."""
+selecting warps, 512 and 1024 threads, one granule, ragged last granules, more slices than SMs, clusters
+that share a granule's list."""
 import numpy as np
 import pytest
 import torch
 
 import oracle
+import oracle.layer as ol
 from paper_2504_08378_b200 import afx, synth
+from test_gpu_layer import OPN, check_layer_stages, make, oracle_weights
 
 pytestmark = pytest.mark.gpu
 
@@ -14,7 +17,10 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("K,N,dt", [
     (1, 8, "bf16"), (127, 40, "f16"), (64, 80000, "bf16"),          # one channel; one granule and a bit; waves of slices
     (4096, 2048, "bf16"), (4096, 2056, "f16"), (4097, 2040, "f16"),  # 512 / 1024 threads, 8 / 16 selecting warps
-    (8200, 4104, "bf16"), (12288, 680, "f16"), (12289, 688, "bf16"),  # 16 / 32 selecting warps
+    (8200, 4104, "bf16"), (12288, 680, "f16"), (12289, 688, "bf16"),  # 6 / 8 slots per lane
+    (16384, 4608, "bf16"), (16385, 4608, "f16"), (16385, 2048, "f16"),  # 16 / 32 selecting warps
+    (6143, 64, "bf16"), (6144, 64, "bf16"), (6144, 1120, "f16"), (6144, 1160, "f16"),  # clusters that share a list
+    (16384, 520, "bf16"), (16385, 264, "bf16"), (32768, 8, "bf16"),
     (32768, 96, "f16"),
 ])
 def test_one_token_operator_at_dispatch_edges(K, N, dt, mode):
@@ -102,3 +108,56 @@ def test_calls_in_a_row_share_a_hint(K, N, dt):
     for i in range(calls):
         assert np.array_equal(idx[i, :k].cpu().numpy(), want[i % 2]), i
         assert torch.equal(y[i], y[i % 2])
+
+
+@pytest.mark.parametrize("hidden,mlp", [(12296, 2312), (16392, 264), (8192, 64)])
+def test_layer_of_very_wide_hidden_state(hidden, mlp):
+    """Gains read late (8 slots per lane), normed operators by clusters and by slices, a family of side outputs: two
+    layers, the second compared with the first one's sets."""
+    dt, pos, T = "bf16", 9, 1
+    cfg = ol.Config(dt, hidden, 1, 1, mlp, mode=oracle.TOPK, xl_depth=1, xl_mode=1)
+    k = [synth.keep_count(K, 50) for K in (hidden, 128, hidden, mlp)]
+    L = synth.layer_weights(59, 0, hidden, 1, 1, mlp, dt, gain_jitter=0.1)
+    kc, vc = synth.kv_cache(59, 0, T, 16, 1, pos)
+    L["k"], L["k_cache"], L["v_cache"] = k, kc, vc
+    m = make(cfg, [L, L], T, afx.MODE_TOPK, xl_depth=1, xl_mode=afx.XL_BOOKKEEP, max_seq=16)
+    h = synth.hidden_state(59, 5, T, hidden, scale=4.0, scales_stream=6)
+    m.h.copy_(torch.from_numpy(h).cuda())
+    sets = []
+    for layer in (0, 1):
+        h0 = m.h.cpu().numpy().copy()
+        m.layer_step(layer, pos)
+        torch.cuda.synchronize()
+        check_layer_stages(cfg, L, oracle_weights(L, k), m, layer, h0, kc, vc, pos, T)
+        stats = m.stats.cpu().numpy()[layer]
+        sets.append([m.idx(op).cpu().numpy()[: stats[op][0]].copy() for op in range(4)])
+        if layer == 1:
+            for op in range(4):
+                miss, hit = oracle.diff_active(sets[1][op], sets[0][op], m.K_op[op])
+                assert stats[op][1] == hit and stats[op][2] == len(miss), OPN[op]
+                assert np.array_equal(m.miss(op).cpu().numpy()[: len(miss)], miss)
+    m.close()
+
+
+@pytest.mark.parametrize("hidden,mlp,E,top", [(8192, 512, 3, 2), (512, 8192, 4, 3), (256, 16392, 2, 1)])
+def test_expert_families_by_clusters(hidden, mlp, E, top):
+    """Experts whose operators are narrow with long lists, against the same call's own intermediates in fp64."""
+    from test_gpu_moe import run_moe
+    dt = "bf16"
+    ex = [synth.layer_weights(61, e, hidden, 1, 1, mlp, dt) for e in range(E)]
+    Wr = synth.weight(61, 99, hidden, E, dt, sigma=0.05)
+    x = synth.laplace_bits(61, 7, (1, hidden), dt)
+    k_gu, k_down = hidden // 2, mlp // 2
+    ids, w, _ = ol.moe_router(x, Wr, dt, top)
+    lg, sel, wsel, hm, y = run_moe(dt, hidden, mlp, E, top, ex, Wr, x, k_gu, k_down)
+    assert sel.tolist() == ids.tolist()
+    ref = np.zeros((1, hidden))
+    idx = oracle.select_active(x, dt, oracle.TOPK, k=k_gu)
+    for r in range(top):
+        e = ex[int(sel[r])]
+        g, u = (oracle.sparse_gemv(e[n], dt, mlp, x, idx) for n in ("w_gate", "w_up"))
+        want = oracle.decode(oracle.silu_mul(g, u, dt), dt)
+        got = oracle.decode(hm[r][None, :], dt)
+        assert np.abs(got - want).max() <= 2.0 ** -7 * np.abs(want).max()
+        ref += float(wsel[r]) * oracle.sparse_gemv(e["w_down"], dt, hidden, hm[r], oracle.select_active(hm[r], dt, oracle.TOPK, k=k_down))
+    assert np.abs(y - ref).max() <= 2e-5 * np.sqrt((ref ** 2).mean()) * 10
