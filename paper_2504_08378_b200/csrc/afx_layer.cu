@@ -142,11 +142,22 @@ static afx_status launch_split(const FusedArgs& a, cudaStream_t st) {
     return launch_list_gemv(DT, g, st);
 }
 
+// Three or four tokens of few channels on 9 to 20 tiles of outputs: the second launch costs more than the blocks that
+// repeat the selections, unless the attention could run beside them.  With list outputs, in a graph, two kernels and
+// one: 4 tokens 256 -> 4096 14.1 and 13.1 us, 2048 -> 5120 17.0 and 15.9, 4096 -> 4096 21.4 and 20.2.  Outside:
+// 2048 -> 2048 14.9 and 15.1, 5120 -> 5120 24.1 and 24.5, 2048 -> 8192 19.1 and 19.3; 2 tokens 2048 -> 4096 13.4 and
+// 14.1; 6 tokens 2048 -> 5120 19.0 and 21.0.
+template <int IN>
+static bool one_kernel_pays(const FusedArgs& a) {
+    return IN == IN_X && !a.beside_attention && (a.T == 3 || a.T == 4) && a.K <= 4096 && a.N > 2048 && a.N <= 5120;
+}
+
 template <int DT, int IN, int EP>
 static afx_status launch_fused_dt(const FusedArgs& a, cudaStream_t st) {
     if (a.T <= 1) return launch_one_token(DT, IN, EP, ONE_TOKEN_PLAIN, a, st);
     const bool listed = a.idx_in != nullptr || (a.idx_out != nullptr && a.count_out != nullptr);
-    if (listed && (IN == IN_X || a.xnorm_out != nullptr) && a.K <= kSelectFastMaxK) return launch_split<DT, IN, EP>(a, st);
+    if (listed && (IN == IN_X || a.xnorm_out != nullptr) && a.K <= kSelectFastMaxK && !one_kernel_pays<IN>(a))
+        return launch_split<DT, IN, EP>(a, st);
     if (a.T <= 4) return launch_fused_mt<DT, 4, IN, EP>(a, st);
     return launch_fused_mt<DT, 8, IN, EP>(a, st);
 }

@@ -201,3 +201,25 @@ def test_gemv_after_a_cache_fetch_that_ran_out_of_staging_rows():
     assert rel_err(out, oracle.sparse_gemv(Wt, dt, N, x, active[:3])) <= 2e-3
     assert (buf[:guard] == -1).all() and (buf[guard + C + staging:] == -1).all()
     afx.afx_cache_destroy(handle)
+
+
+@pytest.mark.parametrize("K,N,T", [(4096, 2048, 4), (4096, 2056, 4), (4097, 2056, 4), (264, 5120, 3), (264, 5128, 3), (264, 4096, 2),
+                                   (264, 4096, 5)])
+@pytest.mark.parametrize("accumulate", [0, 1])
+def test_several_tokens_with_lists_in_one_kernel_and_in_two(K, N, T, accumulate):
+    """Either side of the sizes at which one kernel selects and multiplies, with list outputs and without."""
+    rng = np.random.default_rng(K + N + T)
+    x = torch.from_numpy(rng.laplace(size=(T, K)).astype(np.float32)).bfloat16().cuda()
+    W = (0.02 * torch.from_numpy(rng.standard_normal((K, N), dtype=np.float32))).bfloat16().cuda()
+    k = K // 3
+    want = oracle.select_active(x.view(torch.int16).cpu().numpy().view(np.uint16), "bf16", oracle.TOPK, k=k)
+    idx, count = torch.zeros(K, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    a = torch.from_numpy(want.astype(np.int64)).cuda()
+    ref, mag = x[:, a].double() @ W[a].double(), x[:, a].double().abs() @ W[a].double().abs()
+    for lists in ((idx, count), (None, None)):
+        y = torch.full((T, N), 0.5, device="cuda")
+        afx.afx_select_gemv(W.view(torch.int16), "bf16", K, N, N, x.view(torch.int16), T, afx.MODE_TOPK, k, 0.0, y, accumulate, *lists)
+        # products are exact; the tensor core may drop what lies 2^-23 below a partial sum at each of K / 16 additions
+        bound = (len(want) / 16 + 20) * 2.0 ** -23 * (mag + 0.5)
+        assert bool(((y.double() - 0.5 * accumulate - ref).abs() <= bound).all())
+    assert np.array_equal(idx.cpu().numpy()[: int(count)], want)
