@@ -35,7 +35,7 @@ CFG = dict(name="llama7b_decode_32L_bf16_top50_xl3", dtype="bf16", n_layers=32, 
            n_kv_heads=32, mlp=11008, past=2048, sparsity_percent=50, xl_depth=3, seed=3)
 ORACLE_SAMPLE_LAYERS = 16
 # DRAM bytes (dram__bytes.sum.per_second x duration) of one fused gate/up launch of this workload,
-# from the ncu capture summarised in profiles/slice_op_kernel_7b_ncu.md (None while the
+# from a capture of ncu's memory counters on the first four layers (None while the
 # kernel has changed since the counters were taken).
 NCU_TRAFFIC_BYTES_PER_LAUNCH = 93_519_000
 
@@ -1211,9 +1211,9 @@ def variant_q4_step(st, n_layers=32):
            "active_weight_bytes": int(w_bytes), "active_weight_gbs": round(w_bytes / (ms * 1e-3) / 1e9, 1),
            "weights_plus_kv_gbs": round((w_bytes + kv_bytes) / (ms * 1e-3) / 1e9, 1),
            "weight_bytes_resident": int(n_layers * sum(K * rb for (K, _), rb in zip(shapes, row_bytes))),
-           "note": "4-bit rows are 3.56x smaller than bf16 rows, but the 4-bit streaming loop is bound by instruction "
-                   "issue (5-6 instructions per weight) and the fixed phases of every operator are those of the bf16 "
-                   "step: the token takes about as long as with bf16 weights, in 0.28 of the memory"}
+           "note": "4-bit rows are 3.56x smaller than bf16 rows, but two thirds of the warp instructions of an operator "
+                   "are input stage and selection over a shared-memory histogram, repeated by every block: the token "
+                   "takes about as long as with bf16 weights, in 0.28 of the memory"}
     m.close()
     del m, layers, g
     torch.cuda.empty_cache()

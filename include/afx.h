@@ -67,8 +67,8 @@ const char* afx_status_string(afx_status s);
 /*
  * Bytes of DEVICE scratch memory the entry points below need for operators of up to K_max
  * channels, N_max outputs and T_max tokens: always 0.  Partial sums meet in shared memory and
- * in the distributed shared memory of a thread-block cluster, and the selection runs inside
- * the consuming kernel, so no call takes a workspace pointer.  (Interface bookkeeping; the
+ * in the distributed shared memory of a thread-block cluster, and a selection stays inside
+ * the consuming kernel or leaves in the caller's list, so no call takes a workspace pointer.  (Interface bookkeeping; the
  * paper has no counterpart.)
  */
 size_t afx_workspace_bytes(int K_max, int N_max, int T_max);
@@ -132,15 +132,19 @@ afx_status afx_sparse_gemv(const void* Wt, int dtype, int K, int N, int64_t ldw,
                            float* y, int accumulate, int32_t* dev_status, void* stream);
 
 /*
- * Selection and sparse GEMV in ONE kernel (the T and C operations of Sec. 4 back to back):
- * the result equals afx_select_active followed by afx_sparse_gemv on the same arguments,
- * without the list's round trip through global memory between two launches.  The paper runs T
+ * Selection and sparse GEMV in one call (the T and C operations of Sec. 4 back to back):
+ * the result equals afx_select_active followed by afx_sparse_gemv on the same arguments.  One
+ * token: ONE kernel, without the list's round trip through global memory between two launches.
+ * Several tokens (T > 1) with both list outputs given: usually two kernels, the second of which
+ * reads the list back from them -- idx_out and count_out are then working storage of the call and
+ * must not be shared with a call that may overlap it on another stream, even where the caller does
+ * not want the list (pass NULL instead).  The paper runs T
  * and C as separate pipeline stages; fusing them, and the `kth_hint` slot, are this library's
  * own design for a GPU (the hint is an accelerator only: the paper's thresholds are calibrated
  * offline, here the exact top-k search merely starts near the previous answer).
  *
  *   Wt, x, y, accumulate   as for afx_sparse_gemv;  mode, k, tau  as for afx_select_active.
- *   idx_out   DEVICE int32[K] or NULL: receives the active list.
+ *   idx_out   DEVICE int32[K] or NULL: receives the active list (T > 1: see above).
  *   count_out DEVICE int32[1] or NULL: receives its length.
  *   kth_hint  DEVICE int32[1] or NULL, read and rewritten by a top-k call with T == 1 and
  *             0 < k < K: on return 0x10000 | the k-th largest magnitude key (the 16-bit pattern
@@ -148,7 +152,7 @@ afx_status afx_sparse_gemv(const void* Wt, int dtype, int K, int N, int64_t ldw,
  *             its search for the k-th key starts (cheap when the key lies within about 19 % of
  *             it, e.g. the previous token's key for the same operator; the full search
  *             otherwise); 0 means no hint.  The selected set never depends on it.
- * K * T * 2 bytes of x are read by every thread block (they stay in L2).
+ * T == 1: K * 2 bytes of x are read by every thread block (they stay in L2).
  */
 afx_status afx_select_gemv(const void* Wt, int dtype, int K, int N, int64_t ldw, const void* x, int T,
                            int mode, int k, float tau, float* y, int accumulate, int32_t* idx_out,
@@ -174,7 +178,8 @@ afx_status afx_sparse_gemv_q4(const void* Wq, int K, int N, int64_t ldq_bytes, c
                               int32_t* dev_status, void* stream);
 
 /* ------------------------------------------------------------------------------------------
- * Decoder layers: every linear operator of a Llama-shaped layer run as ONE kernel that
+ * Decoder layers: every linear operator of a Llama-shaped layer run as ONE kernel (several tokens:
+ * a selection kernel and one that streams) that
  * normalises (where the layer does), selects the active channels of its own input and
  * evaluates the operator on them -- the paper's per-operator T (Top-K) + C (compute) pair of
  * Sec. 4 applied "to all linear transformation operators" (Sec. 2.1), with the cross-layer
@@ -270,7 +275,8 @@ afx_status afx_state_buffer(const afx_state* state, int which, int op, void** pt
 
 /*
  * One decoder layer for the T token streams at position `pos` (0 <= pos < max_seq; the
- * cache rows 0..pos-1 hold the past, row pos is written): five kernels on `stream`,
+ * cache rows 0..pos-1 hold the past, row pos is written): five kernels on `stream` (with several
+ * tokens an operator is a selection kernel and a streaming one),
  *   qkv (RMSNorm + select + GEMV) -> rotary, cache append, dense attention ->
  *   o (select + GEMV, h +=) -> gate/up (RMSNorm + select + GEMV + silu*up) ->
  *   down (select + GEMV, h +=).
@@ -279,7 +285,7 @@ afx_status afx_state_buffer(const afx_state* state, int which, int op, void** pt
 afx_status afx_layer_step(afx_model* model, int layer, afx_state* state, int pos, void* stream);
 
 /*
- * ONE of the five kernels of afx_layer_step, on whatever the state holds (afx_layer_step is
+ * ONE of the five stages of afx_layer_step, on whatever the state holds (afx_layer_step is
  * exactly the five calls in order).  For per-operator timing and profiling of the launches a
  * decode step really makes -- the same kernel instantiation, launch shape and side outputs;
  * this library's own addition, the paper has no counterpart.  One difference: inside
@@ -586,8 +592,8 @@ afx_status afx_moe_block(const afx_moe_desc* desc, const void* x, float* y, int 
  * afx_layer_step for a layer some of whose operators do not live in device memory: per
  * operator input (AFX_OP_*) either an LFU cache (afx_cache: THIS layer's operator tensor) or a
  * swapping object (afx_swap: the operator type of all layers).  Such an operator runs as the
- * paper's pipeline stages one after the other on `stream` -- T: input stage + selection (the
- * side outputs of the fused kernel: normed input, active list, cross-layer bookkeeping), L:
+ * paper's pipeline stages one after the other on `stream` -- T: input stage + selection (normed
+ * input, active list, cross-layer bookkeeping), L:
  * afx_cache_fetch / afx_swap_acquire, C: the sparse GEMV through the slot list with the
  * operator's epilogue -- while operators with neither handle run fused on the resident weights
  * of the layer descriptor.  slot[op]: DEVICE int32[K_op] scratch for the slot list.  Preloads

@@ -14,8 +14,8 @@
 //
 // 16 positions cost a warp 8 KB of K and V and about 200 instructions whatever the number of query heads,
 // where dot products on the fp32 pipe cost 45 instructions per position and query head (64 heads, kv 8, 8000
-// positions: 100 -> 15.7 us).  Bound by the latency of a warp's tile of loads: one block of 8 warps per SM
-// with a whole tile of K and V in flight each (202 registers) beats two or three blocks of 4 (23.8, 43.2 us).
+// positions: 100 -> 15.7 us, and 0.7 since the scores are summed on the fp32 pipe).  Bound by the latency of a warp's tile of loads: one block of 8 warps per SM
+// with a whole tile of K and V in flight each (206 registers) beats two or three blocks of 4 (23.8, 43.2 us).
 #pragma once
 
 #include "afx_attn.cuh"

@@ -1,11 +1,11 @@
-// One sparse operator of a decoder layer as a single kernel: input stage (optional RMSNorm),
-// active-channel selection, sparse GEMV, epilogue.  Every block repeats the cheap, exact
-// input stage and selection on its own (the activation vector is a few KB and L2 resident),
-// so nothing but the previous kernel's output stands between two operators: no separate
-// selection launch, no count/index round trips through global memory.
+// What a fused sparse operator is given (FusedArgs), and the form of it whose blocks select over a shared-memory
+// histogram: several tokens in one kernel, where the list cannot leave in the caller's memory or the second
+// launch does not pay, and one token over 4-bit rows.  (One token over 16-bit rows: afx_slice.cuh.)
+// Input stage (optional RMSNorm), active-channel selection, sparse GEMV, epilogue in one kernel; every block
+// repeats the exact input stage and selection on its own (the activation vector is a few KB and L2 resident).
 #pragma once
 
-// (the several-token instantiations leave fused_op_block before its one-token streaming loop)
+// (the several-token instantiations leave fused_op_block before its 4-bit streaming loop)
 #pragma nv_diag_suppress 128
 
 #include "afx_gemv.cuh"
@@ -21,7 +21,7 @@ constexpr int kFusedMtRows = 64;  // channels per pipeline stage of the several-
 
 struct FusedArgs {
     const uint16_t* Wt;
-    // mixture of experts: if wt_table is given, the weights are wt_table[*wt_sel] (both DEVICE;
+    // mixture of experts (one-token operator): if wt_table is given, the weights are wt_table[wt_sel[g]] (both DEVICE;
     // the choice is made on the device by the router kernel earlier in the stream)
     const uint16_t* const* wt_table;
     const int32_t* wt_sel;
@@ -38,7 +38,7 @@ struct FusedArgs {
     const int32_t* idx_in;
     const int32_t* count_in;
     EpilogueArgs ep;
-    // ---- side outputs of block (0,0); each may be NULL ----
+    // ---- side outputs, written by one block; each may be NULL ----
     int32_t* idx_out;        // the active list used (capacity K)
     int32_t* count_out;
     uint32_t* bitmap_out;    // the same set as a bitmap (own selection only)
@@ -48,13 +48,13 @@ struct FusedArgs {
     int32_t* miss_count;
     int32_t* hit_count;           // |A & P|
     // ---- top-k search hint (may be NULL): 0x10000 | k-th key of this operator's last top-k
-    // selection with T == 1; read before the selection, rewritten after it by block (0,0) ----
+    // selection with T == 1; read before the selection, rewritten after it by the block of the side outputs ----
     int32_t* kth_slot;
     // ---- the same for several tokens (T > 1; may be NULL): T consecutive slots, one per token ----
     int32_t* kth_multi;
     // ---- set by the launcher (several-token operators): column tiles per cluster, 0 or 1 = one ----
     int tiles_per_cluster;
-    // ---- set by the launcher: 1 if the grid has one more cluster than column tiles; its block 0
+    // ---- set by the launcher: 1 if the grid has one more cluster (slice operator: block) than its outputs need; its block 0
     // repeats input stage and selection only to write the side outputs, off the path of the
     // clusters that stream (its other blocks leave at once) ----
     int side_cluster;

@@ -63,8 +63,9 @@ static afx_status launch_slice(const FusedArgs& a, cudaStream_t st, int split = 
 // rows before the wait and start as soon as the operator's last block ends (4096 -> 12288, attention over
 // 2048 positions, 4096 -> 4096: 35.0 us, with 1024 threads 39.7).  Small operators too, which wait less
 // for fewer warps (1024 -> 5632: 6.2 us, with 1024 threads 8.0).  Elsewhere 1024 threads keep twice
-// the loads in flight (4096 -> 22016: 20.0 us, with 512 threads 24.1), and from K = 4096 on that is worth
-// more than the overlap (8 layers of 8192 channels, 8000 positions: 1573 us, with 512 threads 1613).
+// the loads in flight (4096 -> 22016: 20.0 us, with 512 threads 24.1), and above K = 4096 that is worth
+// more than the overlap (a layer over 2048 positions, 1024 and 512 threads beside the attention: 4608 channels
+// 77.3 and 78.3 us, 5120 97.0 and 99.8, 6144 119.2 and 123.3, 8192 with 8 kv heads 93.7 and 100.0).
 constexpr int kSlNarrowMaxK = 4096;
 // From here on clusters share a granule's list, where at least four blocks find an SM for each granule.  One block and
 // a cluster per granule, half of the channels kept, in a graph: 5120 -> 256 6.9 and 6.4 us, 5120 -> 1024 7.1 and 7.3,
