@@ -1,16 +1,12 @@
 // What a fused sparse operator is given (FusedArgs), and the form of it whose blocks select over a shared-memory
 // histogram: several tokens in one kernel, where the list cannot leave in the caller's memory or the second
-// launch does not pay, and one token over 4-bit rows.  (One token over 16-bit rows: afx_slice.cuh.)
+// launch does not pay.  (One token: afx_slice.cuh, afx_q4op.cuh.)
 // Input stage (optional RMSNorm), active-channel selection, sparse GEMV, epilogue in one kernel; every block
 // repeats the exact input stage and selection on its own (the activation vector is a few KB and L2 resident).
 #pragma once
 
-// (the several-token instantiations leave fused_op_block before its 4-bit streaming loop)
-#pragma nv_diag_suppress 128
-
 #include "afx_gemv.cuh"
 #include "afx_mma.cuh"
-#include "afx_q4.cuh"
 #include "afx_select.cuh"
 
 namespace afx {
@@ -75,6 +71,9 @@ struct FusedArgs {
 enum OneTokenForm { ONE_TOKEN_PLAIN, ONE_TOKEN_FAMILY };
 afx_status launch_one_token(int dtype, int in, int ep, OneTokenForm form, const FusedArgs& a, cudaStream_t st);
 
+// The same over 4-bit rows (afx_q4op.cu): a.Wt = the rows, a.ldw = their stride in units of 2 bytes, a.N % 32 == 0.
+afx_status launch_q4_operator(int dtype, int in, int ep, const FusedArgs& a, cudaStream_t st);
+
 // Input stage and selection of a.T tokens with the side outputs, as a kernel of its own (afx_seltok.cu).
 afx_status launch_select_tokens(int dtype, bool norm, const FusedArgs& a, cudaStream_t st);
 
@@ -94,17 +93,10 @@ __host__ __device__ inline size_t fused_dyn_smem(int in_kind, int K, int T, size
     return fused_input_smem(in_kind, K, T) + fused_flag_smem(K, T) + (work > kKeyHistBytes ? work : kKeyHistBytes);
 }
 
-// WMT > 0: several tokens, the streaming stage runs on the tensor cores (afx_mma.cuh) with WMT
-// pipeline stages: PW = 256, the work area holds an MtSmem<CAP, WMT> once the selection is over.
-// WQ4: the weights are 4-bit rows (afx_sparse_gemv_q4's layout; one token): Wt points at them,
-// ldw is the row stride in units of 2 bytes, the tile is PW = 512, 256 or 128 outputs wide and
-// the streaming loop and the reduction are the 4-bit kernel's.
-template <int DT, int TMAX, int PW, int CAP, int IN, int EP, bool WQ4 = false, int WMT = 0>
+// The streaming stage runs on the tensor cores (afx_mma.cuh) with STAGES pipeline stages: the work area holds an
+// MtSmem<CAP, STAGES> once the selection is over.
+template <int DT, int TMAX, int CAP, int IN, int EP, int STAGES>
 __device__ __forceinline__ void fused_op_block(const FusedArgs& a, unsigned char* dyn, SelectScratch* sel) {
-    static_assert(WQ4 || WMT > 0, "one token over 16-bit rows is afx_slice.cuh's");
-    constexpr int LPC = WQ4 ? PW / kQ4Opl : PW / 8;
-    static_assert(WMT > 0 || sizeof(GemvSmem<TMAX, CAP>) <= kKeyHistBytes, "work area too small");
-    static_assert(!WQ4 || (TMAX == 1 && CAP * 8 + (kQ4Warps + 1) * PW * 4 <= kKeyHistBytes), "4-bit: one token, sums behind the staged list");
     const int tid = threadIdx.x;
     const int lane = tid & 31;
     const int warp = tid >> 5;
@@ -112,7 +104,7 @@ __device__ __forceinline__ void fused_op_block(const FusedArgs& a, unsigned char
     // except for several-token operators with few tiles: there a cluster covers CS / S adjacent
     // tiles, so that more blocks share the per-token selections (a.tiles_per_cluster).
     const int CS = gridDim.x, cs = blockIdx.x;
-    const int tpc = (WMT > 0 && a.tiles_per_cluster > 1) ? a.tiles_per_cluster : 1;
+    const int tpc = a.tiles_per_cluster > 1 ? a.tiles_per_cluster : 1;
     const int S = tpc > 1 ? CS / tpc : CS, s = tpc > 1 ? cs % S : cs;
     const int T = a.T, K = a.K;
     const bool side = a.side_cluster != 0 && blockIdx.y == gridDim.y - 1;  // the cluster without a tile
@@ -126,7 +118,6 @@ __device__ __forceinline__ void fused_op_block(const FusedArgs& a, unsigned char
     uint16_t* xs = reinterpret_cast<uint16_t*>(dyn);
     unsigned char* work = dyn + fused_input_smem(IN, K, T) + fused_flag_smem(K, T);
     uint32_t* hist = reinterpret_cast<uint32_t*>(work);
-    GemvSmem<TMAX, CAP>* sm = reinterpret_cast<GemvSmem<TMAX, CAP>*>(work);
     float* red16 = reinterpret_cast<float*>(sel->hist);  // block reduction of the norm
 
     const uint32_t ld16 = static_cast<uint32_t>(a.ldw >> 3);  // row stride in 16-byte units (the launcher checked the range)
@@ -159,7 +150,7 @@ __device__ __forceinline__ void fused_op_block(const FusedArgs& a, unsigned char
     // threads of a block must search from the same one: a single thread reads it, the others
     // take it from shared memory behind the barrier of the input stage.
     if (tid < T) {
-        const int32_t* const slot = T == 1 ? a.kth_slot : a.kth_multi != nullptr ? a.kth_multi + tid : nullptr;
+        const int32_t* const slot = a.kth_multi != nullptr ? a.kth_multi + tid : nullptr;
         const uint32_t v = topk && slot != nullptr ? static_cast<uint32_t>(__ldcg(slot)) : 0u;
         sel->hint[tid] = (v & 0x10000u) ? v & 0x7FFFu : kNoKeyHint;
     }
@@ -237,7 +228,7 @@ __device__ __forceinline__ void fused_op_block(const FusedArgs& a, unsigned char
     // 16-bit input of token t, channel j, once the stage above / below has run
     auto x_at = [&](int t, int j) -> uint16_t {
         if (IN == IN_NORM) return xs[static_cast<size_t>(t) * Kp + j];
-        return T == 1 ? xs[j] : a.x[static_cast<size_t>(t) * K + j];
+        return a.x[static_cast<size_t>(t) * K + j];
     };
     AFX_MARK(2);
 
@@ -245,27 +236,14 @@ __device__ __forceinline__ void fused_op_block(const FusedArgs& a, unsigned char
     int cnt = 0;
     int pos0 = 0;                  // list position of this thread's first active channel
     unsigned long long fl = 0ull;  // this thread's active flags (own selection)
-    const int out0 = tile * PW + (lane % LPC) * (WQ4 ? kQ4Opl : 8);
-    const bool lane_ok = out0 < a.N;
-    // One token, top-k: the list length is k whatever x holds, so this block's part
-    // [c_lo, c_hi) of the list is known before the selection and the pass that decides the
-    // flags (it has the channel's bits in registers) stages the first CAP entries directly.
-    const bool early = topk && T == 1;
-    // one word per chunk, in the work area behind the staging and reduction buffers
-    constexpr size_t kXchgOffset = kKeyHistBytes - (kSelectFastMaxK / 8) * 4;
-    constexpr bool kXchgFits = sizeof(GemvSmem<TMAX, CAP>) <= kXchgOffset;
-    static_assert(TMAX > 1 || kXchgFits, "work area too small for the chunk exchange");
-    uint32_t* xchg = kXchgFits ? reinterpret_cast<uint32_t*>(work + kXchgOffset) : nullptr;
-    bool first_staged = false;
     // Several tokens: the blocks of a cluster share the work -- block s decides the sets of the
     // tokens t with t % CS == cs and writes their flags into every block's table of per-token
     // bitmaps (distributed shared memory); after one cluster barrier every thread reads the
     // union for its own chunks.  (The side cluster works alone and decides every token.)
-    const bool share = TMAX > 1 && T > 1 && own && !side && CS > 1;
+    const bool share = own && !side && CS > 1;
     uint8_t* const ftab = dyn + fused_input_smem(IN, K, T);
     const size_t fstride = fused_flag_smem(K);
     if (own) {
-        const int e_lo = s * a.k / S, e_n = min(CAP, (s + 1) * a.k / S - e_lo);
         if (share) cluster_wait();  // pairs with the cluster_arrive() at kernel start: the peers are running
         bool first = true;
         for (int t = 0; t < T; ++t) {
@@ -275,33 +253,20 @@ __device__ __forceinline__ void fused_op_block(const FusedArgs& a, unsigned char
                 if (!first) __syncthreads();  // the previous token's keys are still being read
                 block_stage_token(a.x + static_cast<size_t>(t) * K, K, xs);
             }
-            if (early) {
-                fl |= block_token_flags<DT, kGemvThreads>(
-                    xt, K, a.mode, a.k, a.tau, hist, first, sel, true, pos0, cnt, [&](int j, int pos, uint16_t bits) {
-                        const int p = pos - e_lo;
-                        if (p >= 0 && p < e_n) {  // the histogram is dead by now: its memory is the staging area
-                            sm->col[p] = static_cast<uint32_t>(j) * ld16;
-                            sm->xv[0][p] = bits_to_float<DT>(bits);
-                        }
-                    }, e_lo, e_lo + e_n, sel->hint[0], xchg);
-                first_staged = true;
-                if (scribe && tid == 0 && a.kth_slot != nullptr) *a.kth_slot = 0x10000 | sel->res[0];
-            } else {
-                uint32_t thr_t = 0;
-                const unsigned long long ft =
-                    block_token_flags<DT, kGemvThreads>(xt, K, a.mode, a.k, a.tau, hist, first, sel, T == 1, pos0, cnt,
-                                                        NoEmit(), 0, 0x7FFFFFFF, sel->hint[t], nullptr, &thr_t);
-                if (scribe && tid == 0 && topk && T > 1 && a.kth_multi != nullptr) a.kth_multi[t] = 0x10000 | thr_t;
-                if (share) {
-                    int q_lo, q_hi;
-                    thread_chunk_range(K, q_lo, q_hi);
-                    for (int q = 0; q < CS; ++q) {
-                        uint8_t* dst = cg::this_cluster().map_shared_rank(ftab + static_cast<size_t>(t) * fstride, q);
-                        for (int c = q_lo; c < q_hi; ++c) dst[c] = static_cast<uint8_t>(ft >> (8 * (c - q_lo)));
-                    }
-                } else {
-                    fl |= ft;
+            uint32_t thr_t = 0;
+            const unsigned long long ft =
+                block_token_flags<DT, kGemvThreads>(xt, K, a.mode, a.k, a.tau, hist, first, sel, false, pos0, cnt,
+                                                    NoEmit(), 0, 0x7FFFFFFF, sel->hint[t], nullptr, &thr_t);
+            if (scribe && tid == 0 && topk && a.kth_multi != nullptr) a.kth_multi[t] = 0x10000 | thr_t;
+            if (share) {
+                int q_lo, q_hi;
+                thread_chunk_range(K, q_lo, q_hi);
+                for (int q = 0; q < CS; ++q) {
+                    uint8_t* dst = cg::this_cluster().map_shared_rank(ftab + static_cast<size_t>(t) * fstride, q);
+                    for (int c = q_lo; c < q_hi; ++c) dst[c] = static_cast<uint8_t>(ft >> (8 * (c - q_lo)));
                 }
+            } else {
+                fl |= ft;
             }
             first = false;
         }
@@ -314,9 +279,8 @@ __device__ __forceinline__ void fused_op_block(const FusedArgs& a, unsigned char
                 for (int c = q_lo; c < q_hi; ++c)
                     fl |= static_cast<unsigned long long>(ftab[static_cast<size_t>(t) * fstride + c]) << (8 * (c - q_lo));
         }
-        if (T > 1) pos0 = block_prefix(__popcll(fl), sel->wtot[2], cnt);
+        pos0 = block_prefix(__popcll(fl), sel->wtot[2], cnt);
     } else {
-        if (IN == IN_X && T == 1) block_stage_token(a.x, K, xs);
         cnt = *a.count_in;
         cnt = max(0, min(cnt, K));
     }
@@ -354,94 +318,46 @@ __device__ __forceinline__ void fused_op_block(const FusedArgs& a, unsigned char
     const int c_lo = s * cnt / S;  // S <= 8, cnt <= 2^20: no overflow
     const int c_hi = (s + 1) * cnt / S;
 
-    f32x2 qacc[8];  // 4-bit weights: 16 outputs per lane
-#pragma unroll
-    for (int i = 0; i < 8; ++i) qacc[i] = pack_f32x2(0.0f, 0.0f);
-
     const int n_mine = __popcll(fl);
-    if (WMT) {
-        using MtT = MtSmem<CAP, (WMT > 0 ? WMT : 2), kFusedMtRows>;
-        MtT* mt = reinterpret_cast<MtT*>(work);
-        constexpr int kMtCap = CAP;
-        float c4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        const uint4* wtile16 = reinterpret_cast<const uint4*>(Wt + static_cast<size_t>(tile) * kMtTile);
-        const int n_chunks = max(0, min(kMtTile, a.N - tile * kMtTile)) >> 3;
-        // (the last cluster of a grid with several tiles per cluster may hold a block without a
-        // tile: it only shares the selections and meets the barriers)
-        for (int c0 = c_lo; n_chunks > 0 && c0 < c_hi; c0 += kMtCap) {
-            const int staged = min(kMtCap, c_hi - c0);
-            __syncthreads();  // the work area is free: the histogram / the previous pass has been read
-            if (own) {
-                if (pos0 < c0 + staged && pos0 + n_mine > c0) {
-                    for_each_owned_active(fl, K, pos0, [&](int j, int pos) {
-                        const int p = pos - c0;
-                        if (p >= 0 && p < staged) {
-                            mt->col[p] = static_cast<uint32_t>(j) * ld16;
+    using MtT = MtSmem<CAP, STAGES, kFusedMtRows>;
+    MtT* mt = reinterpret_cast<MtT*>(work);
+    constexpr int kMtCap = CAP;
+    float c4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    const uint4* wtile16 = reinterpret_cast<const uint4*>(Wt + static_cast<size_t>(tile) * kMtTile);
+    const int n_chunks = max(0, min(kMtTile, a.N - tile * kMtTile)) >> 3;
+    // (the last cluster of a grid with several tiles per cluster may hold a block without a
+    // tile: it only shares the selections and meets the barriers)
+    for (int c0 = c_lo; n_chunks > 0 && c0 < c_hi; c0 += kMtCap) {
+        const int staged = min(kMtCap, c_hi - c0);
+        __syncthreads();  // the work area is free: the histogram / the previous pass has been read
+        if (own) {
+            if (pos0 < c0 + staged && pos0 + n_mine > c0) {
+                for_each_owned_active(fl, K, pos0, [&](int j, int pos) {
+                    const int p = pos - c0;
+                    if (p >= 0 && p < staged) {
+                        mt->col[p] = static_cast<uint32_t>(j) * ld16;
 #pragma unroll
-                            for (int t = 0; t < TMAX; ++t)
-                                if (t < T) mt->xb[t][p] = x_at(t, j);
-                        }
-                    });
-                }
-            } else {
-                for (int i = tid; i < staged; i += kGemvThreads) {
-                    const int j = a.idx_in[c0 + i];
-                    mt->col[i] = static_cast<uint32_t>(j) * ld16;
-#pragma unroll
-                    for (int t = 0; t < TMAX; ++t)
-                        if (t < T) mt->xb[t][i] = x_at(t, j);
-                }
+                        for (int t = 0; t < TMAX; ++t)
+                            if (t < T) mt->xb[t][p] = x_at(t, j);
+                    }
+                });
             }
-            mt_pad_inputs(mt, T, staged);
-            __syncthreads();
-            mt_stream_pass<DT>(wtile16, mt, staged, n_chunks, c4);
-        }
-        EpilogueArgs ep = a.ep;
-        if (!share) cluster_wait();  // pairs with the cluster_arrive() at kernel start
-        mt_finish<DT>(c4, mt, T, tile, a.N, EP, ep, S, s, cs - s);
-        return;
-    }
-    for (int c0 = c_lo; c0 < c_hi; c0 += CAP) {
-        const int staged = min(CAP, c_hi - c0);
-        if (!(first_staged && c0 == c_lo)) {
-            __syncthreads();  // the work area is free: the histogram / the previous stage has been read
-            // ---- stage (column, x values) of list positions [c0, c0 + staged) ----
-            if (own) {
-                if (pos0 < c0 + staged && pos0 + n_mine > c0) {
-                    for_each_owned_active(fl, K, pos0, [&](int j, int pos) {
-                        const int p = pos - c0;
-                        if (p >= 0 && p < staged) {
-                            sm->col[p] = static_cast<uint32_t>(j) * ld16;
+        } else {
+            for (int i = tid; i < staged; i += kGemvThreads) {
+                const int j = a.idx_in[c0 + i];
+                mt->col[i] = static_cast<uint32_t>(j) * ld16;
 #pragma unroll
-                            for (int t = 0; t < TMAX; ++t)
-                                if (t < T) sm->xv[t][p] = bits_to_float<DT>(x_at(t, j));
-                        }
-                    });
-                }
-            } else {
-                for (int i = tid; i < staged; i += kGemvThreads) {
-                    const int j = a.idx_in[c0 + i];
-                    sm->col[i] = static_cast<uint32_t>(j) * ld16;
-#pragma unroll
-                    for (int t = 0; t < TMAX; ++t)
-                        if (t < T) sm->xv[t][i] = bits_to_float<DT>(x_at(t, j));
-                }
+                for (int t = 0; t < TMAX; ++t)
+                    if (t < T) mt->xb[t][i] = x_at(t, j);
             }
         }
+        mt_pad_inputs(mt, T, staged);
         __syncthreads();
-        AFX_MARK(4);
-        if (WQ4) {
-            if (lane_ok)
-                q4_stream<LPC>(reinterpret_cast<const unsigned char*>(Wt), a.N, out0 / kQ4Opl, sm->col, sm->xv[0], staged, qacc);
-        }
+        mt_stream_pass<DT>(wtile16, mt, staged, n_chunks, c4);
     }
-    AFX_MARK(5);
-
-    AFX_MARK(6);
-
-    cluster_wait();  // pairs with the cluster_arrive() at kernel start
-    q4_finish<DT, LPC>(qacc, reinterpret_cast<float*>(work) + 2 * CAP, tile, a.N,
-                       EP == EP_SILU ? Q4_SILU : (EP == EP_ACCUM ? Q4_ACCUM : Q4_STORE), a.ep.y, a.ep.out_bits);
+    EpilogueArgs ep = a.ep;
+    if (!share) cluster_wait();  // pairs with the cluster_arrive() at kernel start
+    mt_finish<DT>(c4, mt, T, tile, a.N, EP, ep, S, s, cs - s);
     AFX_MARK(7);
 }
 

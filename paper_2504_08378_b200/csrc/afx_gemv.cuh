@@ -13,16 +13,6 @@ constexpr int kGemvWarps = 16;
 constexpr int kGemvThreads = 32 * kGemvWarps;
 constexpr int kMaxCluster = 8;
 
-// Shared memory of one block.  CAP = channels whose (column, x) pairs are staged at once.
-// A column is staged as its offset from the start of the weights in 16-byte units
-// (row * ldw / 8: 32 bits cover operators of up to 64 GB), so that a load address is one
-// multiply-add away.
-template <int TMAX, int CAP>
-struct GemvSmem {
-    uint32_t col[CAP];
-    float xv[TMAX][CAP];
-};
-
 // Split cluster barrier.  Every block arrives once when it starts and waits just before its
 // first store into a peer's shared memory: by then every block of the cluster is running.
 __device__ __forceinline__ void cluster_arrive() {

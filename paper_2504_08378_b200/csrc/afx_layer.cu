@@ -7,7 +7,6 @@
 #include "afx_attn.cuh"
 #include "afx_fused.cuh"
 #include "afx_launch.cuh"
-#include "afx_q4.cuh"
 
 namespace afx {
 
@@ -24,45 +23,8 @@ template <int DT, int TMAX, int IN, int EP, int STAGES, int CAPM, int BPS>
 __global__ void __launch_bounds__(kGemvThreads, BPS) fused_mt_kernel(FusedArgs a) {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ SelectScratch sel;
-    fused_op_block<DT, TMAX, kMtTile, CAPM, IN, EP, false, STAGES>(a, dyn, &sel);
+    fused_op_block<DT, TMAX, CAPM, IN, EP, STAGES>(a, dyn, &sel);
 }
-
-// The one-token operator over 4-bit rows: tiles of PW = 512, 256 or 128 outputs.
-template <int DT, int PW, int IN, int EP>
-__global__ void __launch_bounds__(kGemvThreads, 2) fused_q4_kernel(FusedArgs a) {
-    constexpr int CAP = 2048;
-    extern __shared__ __align__(16) unsigned char dyn[];
-    __shared__ SelectScratch sel;
-    fused_op_block<DT, 1, PW, CAP, IN, EP, true>(a, dyn, &sel);
-}
-
-// a.Wt = the 4-bit rows, a.ldw = their stride in units of 2 bytes, a.T == 1, a.N % 32 == 0.
-template <int DT, int IN, int EP>
-static afx_status launch_fused_q4_dt(const FusedArgs& a, cudaStream_t st) {
-    if (static_cast<uint64_t>(a.K) * static_cast<uint64_t>(a.ldw >> 3) > 0x100000000ull) return AFX_ERR_CAPACITY;
-    const size_t dyn = fused_dyn_smem(IN, a.K, 1);
-    const void* kerns[3] = {reinterpret_cast<const void*>(fused_q4_kernel<DT, 512, IN, EP>),
-                            reinterpret_cast<const void*>(fused_q4_kernel<DT, 256, IN, EP>),
-                            reinterpret_cast<const void*>(fused_q4_kernel<DT, 128, IN, EP>)};
-    FusedArgs b = a;
-    b.side_cluster = (a.idx_out != nullptr || a.count_out != nullptr || a.bitmap_out != nullptr ||
-                      a.xnorm_out != nullptr || a.bitmap_pred != nullptr || a.kth_slot != nullptr)
-                         ? 1 : 0;
-    const GemvShapeChoice c = choose_gemv_shape(a.N, kerns, dyn, b.side_cluster, 512);
-    if (c.tiles + b.side_cluster > 65535) return AFX_ERR_CAPACITY;
-    const int rows = c.tiles + b.side_cluster;
-    switch (c.pw) {
-        case 512: return launch_clustered(fused_q4_kernel<DT, 512, IN, EP>, c.S, rows, dyn, b, st);
-        case 256: return launch_clustered(fused_q4_kernel<DT, 256, IN, EP>, c.S, rows, dyn, b, st);
-        default: return launch_clustered(fused_q4_kernel<DT, 128, IN, EP>, c.S, rows, dyn, b, st);
-    }
-}
-
-template <int IN, int EP>
-static afx_status launch_fused_q4(int dtype, const FusedArgs& a, cudaStream_t st) {
-    return dtype == AFX_F16 ? launch_fused_q4_dt<AFX_F16, IN, EP>(a, st) : launch_fused_q4_dt<AFX_BF16, IN, EP>(a, st);
-}
-
 
 template <int DT, int TMAX, int IN, int EP, int STAGES, int CAPM, int BPS>
 static afx_status launch_fused_mt_st(const FusedArgs& a, cudaStream_t st) {
@@ -638,6 +600,7 @@ extern "C" afx_status afx_layer_step_q4(afx_model* m, int layer, afx_state* s, i
         a.ldw = q4->ldq_bytes[op] >> 1;
         a.K = m->K_op[op];
         a.N = N_op[op];
+        a.beside_attention = op == AFX_OP_QKV || op == AFX_OP_O;
         plan_selection(m, s, layer, op, true, &a);
         switch (op) {
             case AFX_OP_QKV:
@@ -645,19 +608,19 @@ extern "C" afx_status afx_layer_step_q4(afx_model* m, int layer, afx_state* s, i
                 a.gain = L.g_attn;
                 a.xnorm_out = reinterpret_cast<uint16_t*>(s->blob + s->off_xnorm[0]);
                 a.ep = {qkv, nullptr, N_op[op]};
-                rc = launch_fused_q4<IN_NORM, EP_STORE>(d.dtype, a, st);
+                rc = launch_q4_operator(d.dtype, IN_NORM, EP_STORE, a, st);
                 break;
             case AFX_OP_GU:
                 a.h = h;
                 a.gain = L.g_mlp;
                 a.xnorm_out = reinterpret_cast<uint16_t*>(s->blob + s->off_xnorm[1]);
                 a.ep = {nullptr, hm, N_op[op]};
-                rc = launch_fused_q4<IN_NORM, EP_SILU>(d.dtype, a, st);
+                rc = launch_q4_operator(d.dtype, IN_NORM, EP_SILU, a, st);
                 break;
             default:
                 a.x = op == AFX_OP_O ? attn : hm;
                 a.ep = {h, nullptr, N_op[op]};
-                rc = launch_fused_q4<IN_X, EP_ACCUM>(d.dtype, a, st);
+                rc = launch_q4_operator(d.dtype, IN_X, EP_ACCUM, a, st);
                 break;
         }
         if (rc != AFX_OK) return rc;

@@ -204,6 +204,32 @@ def test_q4_layer_step_at_7b_size():
     m.close()
 
 
+@pytest.mark.parametrize("dt,hidden,heads,mlp", [("bf16", 512, 4, 4096),    # down: a cluster per block of 32 outputs
+                                                 ("f16", 1056, 2, 4128),    # 33 blocks: tiles of one and two in a cluster
+                                                 ("bf16", 4704, 1, 64),     # 147 blocks of outputs: one per SM
+                                                 ("bf16", 4736, 1, 2400),   # 148 blocks: two in some tiles
+                                                 ("f16", 512, 2, 16416),    # more channels than 16 warps select from, split
+                                                 ("bf16", 17408, 1, 64)])   # the same with the norm, not split
+def test_q4_layer_step_at_the_edges_of_its_tiles(dt, hidden, heads, mlp):
+    T, pos, max_seq = 1, 6, 8
+    cfg = ol.Config(dt, hidden, heads, heads, mlp, mode=oracle.TOPK)
+    k = [synth.keep_count(K, 45) for K in (hidden, heads * 128, hidden, mlp)]
+    L = synth.layer_weights(65, 0, hidden, heads, heads, mlp, dt)
+    L["k"] = k
+    kc0, vc0 = synth.kv_cache(65, 0, T, max_seq, heads, pos)
+    L["k_cache"], L["v_cache"] = kc0, vc0
+    rows = q4_layer_weights(65, 0, hidden, heads * 128, 3 * heads * 128, mlp)
+    dev = [torch.from_numpy(r).cuda() for r in rows]
+    m = make(cfg, [L], T, afx.MODE_TOPK, max_seq=max_seq)
+    h = synth.hidden_state(65, 5, T, hidden, scales_stream=6)
+    m.h.copy_(torch.from_numpy(h).cuda())
+    use = (True, True, True, True)
+    afx.afx_layer_step_q4(m.handle, 0, m.state, pos, q4_struct(dev, use))
+    torch.cuda.synchronize()
+    check_q4_stages(cfg, L, rows, use, oracle_weights(L, k), m, 0, h, kc0, vc0, pos)
+    m.close()
+
+
 def test_q4_layer_step_rejects_what_it_cannot_run():
     dt, heads, kvh, mlp, T = "bf16", 2, 1, 512, 2
     hidden = heads * 128
