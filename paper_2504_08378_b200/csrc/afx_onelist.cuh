@@ -13,11 +13,6 @@ __device__ __forceinline__ float list_x(uint32_t entry) {
     return DT == AFX_BF16 ? __uint_as_float(entry & 0xFFFF0000u) : bits_to_float<DT>(static_cast<uint16_t>(entry >> 16));
 }
 
-// Stores v to the shared-memory word at `at` where `on` holds; never a branch.
-__device__ __forceinline__ void st_shared_if(uint32_t at, uint32_t v, bool on) {
-    asm volatile("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p st.shared.u32 [%0], %1; }" ::"r"(at), "r"(v), "r"(on ? 1u : 0u) : "memory");
-}
-
 // Input stage and selection of a one-token operator: the active list, staged as entries (16-bit channel, 16-bit
 // input) at `dyn`, and its length.  `early`: the input is older than the kernel before this one, and the dependency
 // wait is left to the caller.  xs_at: where in `dyn` the inputs of a list decided earlier are staged.  The first NW of
@@ -39,7 +34,7 @@ __device__ __forceinline__ int one_token_list(const FusedArgs& a, const uint16_t
     if constexpr (kEarlyGain) {
         if (selects) sel_load_gain<CH>(a.gain, K, m, gv);
     }
-    if (own) sel_read_hint(a.kth_slot, sc);
+    if (own) sel_prepare<NW>(a.kth_slot, sc);
     if (!early) {
         asm volatile("griddepcontrol.wait;" ::: "memory");
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // only after the wait (ordering rule)
@@ -69,9 +64,7 @@ __device__ __forceinline__ int one_token_list(const FusedArgs& a, const uint16_t
             int kth, at, n;
             const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(list));
             const uint32_t fl = sel_flags<DT, NW, CH>(kw, m, K, a.mode, a.k, a.tau, sc->hint, sc, kth, at, n);
-            sel_emit<CH>(fl, m, at, [&](int i, int e, int pos, bool on) {
-                st_shared_if(base + 4 * pos, __byte_perm(kw[2 * i + (e >> 1)], static_cast<uint32_t>(sel_channel(m, i) + e), (e & 1) ? 0x3254 : 0x1054), on);
-            });
+            sel_emit<CH>(fl, m, kw, base + 4u * static_cast<uint32_t>(at));
             if (tid == 0) {
                 sc->count = n;
                 if (scribe && a.kth_slot != nullptr && a.mode == AFX_MODE_TOPK && a.k > 0 && a.k < K)

@@ -55,7 +55,7 @@ __device__ __forceinline__ void select_tokens_block(const FusedArgs& a, SelTokSm
         if (selects) sel_load_gain<CH>(a.gain, K, m, gv);
     }
     int32_t* const slot = T == 1 ? a.kth_slot : a.kth_multi != nullptr ? a.kth_multi + t : nullptr;
-    if (own) sel_read_hint(slot, &sm->sel);
+    if (own) sel_prepare<NW>(slot, &sm->sel);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // only after the wait (ordering rule)
 

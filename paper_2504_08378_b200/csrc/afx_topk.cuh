@@ -1,16 +1,17 @@
 // Active-channel selection with the keys in registers.
 //
 // The first NW warps of the block own the channels: slot s of warp w holds channels (w m + s) 128 + 4
-// lane .. + 3.  The k-th largest 15-bit magnitude key is found by a seven-way search: a step counts the
-// keys at or above six candidates (two keys per operation), adds the counts over warp and block (three
-// `redux` before and three shuffles behind one barrier of the NW warps) and keeps a seventh of the interval.
-// With a hint of the answer two steps suffice in bf16 and three in f16; without one a sample of the keys gives it.  There are no
-// atomics and no histogram, hence no shared memory to clear and no serialisation on popular keys.
+// lane .. + 3.  The k-th largest 15-bit magnitude key is found from a hint of it, the last k-th key or, without one, a
+// sample of the keys: every key of a window around the hint has a counter in shared memory, the keys above the
+// window are counted two per operation, and behind ONE barrier every warp sums the counters from the top.  Where the
+// k-th key is outside the window a seven-way search of the rest follows: a step counts the keys at or above six
+// candidates, adds the counts over warp and block (three `redux` before and three shuffles behind one barrier of the NW
+// warps) and keeps a seventh of the interval.
 //
-// What bounds it is the issue rate of integer instructions and the latency of a step's barrier and
-// reductions.  What every warp repeats behind the barrier counts NW times, so few warps with many keys
-// each beat many warps with few: K = 4096, bf16, hinted: 1.3 us for the search on 8 warps of 16 keys per
-// lane; 2.2 us where all 32 warps of an SM's two blocks searched a histogram of the same keys.
+// What bounds it is the latency of barriers and reductions and the rate of shared-memory atomics (about one in ten keys
+// is in the window).  Clocks for the k-th key, the seven-way search alone from the same hint and now: bf16 K = 4096 on 8
+// warps 2050 and 1560, K = 11008 on 16 warps 3850 and 2340; f16 K = 4096 3030 and 1640, K = 1024 2470 and 1030.  What
+// every warp repeats behind the barrier counts NW times, so few warps with many keys each beat many warps with few.
 #pragma once
 
 #include "afx_select.cuh"
@@ -20,11 +21,14 @@ namespace afx {
 constexpr uint32_t kNoHint = 0xFFFFFFFFu;
 constexpr int kRegSelMaxWarps = 32;
 
+constexpr int kSelBins = 256;
+
 struct RegSelScratch {
+    __align__(16) uint32_t win[kSelBins];  // keys around the hint, counted one by one (cleared by sel_prepare)
     __align__(16) uint32_t part[2][kRegSelMaxWarps][4];  // per-warp counts of a search step (double-buffered)
-    uint32_t scan[kRegSelMaxWarps];
+    uint32_t scan[kRegSelMaxWarps], top[kRegSelMaxWarps];
     int count;      // the list's length, for the warps that did not select
-    uint32_t hint;  // where the search starts (sel_read_hint)
+    uint32_t hint;  // where the search starts (sel_prepare)
     __align__(16) float sum[kRegSelMaxWarps];
 };
 
@@ -34,11 +38,14 @@ __device__ __forceinline__ void sel_barrier() {
     asm volatile("bar.sync 1, %0;" ::"n"(NW * 32) : "memory");
 }
 
-// The search hint in `slot` (NULL: none) for the whole block: ONE thread of the first warp reads it and leaves it in
-// sc->hint, which the others read behind a barrier of the selecting warps.  Another launch of the operator, or
-// another block of this one, may be rewriting the word: threads that read it for themselves could start with
-// different hints, take different numbers of search steps, and wait at different barriers for each other.
-__device__ __forceinline__ void sel_read_hint(const int32_t* slot, RegSelScratch* sc) {
+// Before the selection: clears the counters, and leaves the search hint in `slot` (NULL: none) for the whole block.  ONE
+// thread of the first warp reads the hint, and the others take it from sc->hint behind a barrier of the selecting warps:
+// another launch of the operator, or another block of this one, may be rewriting the word, and threads that read it for
+// themselves could start with different hints, take different numbers of search steps, and wait at different barriers.
+template <int NW>
+__device__ __forceinline__ void sel_prepare(const int32_t* slot, RegSelScratch* sc) {
+    if (threadIdx.x < NW * 32)
+        for (int i = threadIdx.x; i < kSelBins / 4; i += NW * 32) reinterpret_cast<uint4*>(sc->win)[i] = make_uint4(0u, 0u, 0u, 0u);
     if (threadIdx.x == 0) {
         const uint32_t v = slot != nullptr ? static_cast<uint32_t>(__ldcg(slot)) : 0u;
         sc->hint = (v & 0x10000u) ? v & 0x7FFFu : kNoHint;
@@ -84,6 +91,12 @@ __device__ __forceinline__ uint32_t sel_ge(uint32_t keys, uint32_t nv) {
 __device__ __forceinline__ uint32_t sel_neg(int v) { return (static_cast<uint32_t>(1 - v) & 0xFFFFu) * 0x00010001u; }
 constexpr uint32_t kMagnitudes = 0x7FFF7FFFu;
 
+// ++win[d] where d < N; never a branch (sixteen of them, as branches, cost 250 of the search's clocks).
+template <int N>
+__device__ __forceinline__ void count_below(uint32_t win, uint32_t d) {
+    asm volatile("{ .reg .pred p; .reg .b32 t; setp.lt.u32 p, %1, %2; mad.lo.u32 t, %1, 4, %0; @p red.shared.add.u32 [t], 1; }" ::"r"(win), "r"(d), "n"(N) : "memory");
+}
+
 // The k-th largest key (1 <= k <= K) of the NW warps' channels: `thr`; how many channels with exactly
 // that key belong to the top k: `need_eq`.  Same values in every thread.  `hint` only shortens the
 // search.  Zero padding behind K is never counted (candidates are >= 1).
@@ -91,12 +104,12 @@ template <int DT, int NW, int CH>
 __device__ __forceinline__ void sel_kth_key(const uint32_t (&kw)[2 * CH], int m, int K, int k, uint32_t hint, RegSelScratch* sc,
                                             int& thr, int& need_eq) {
     constexpr int C = 6;
-    // first step: candidates this far apart around the hint: +-17 keys (about +-13 % in magnitude) in
-    // bf16, +-122 (+-12 to 24 %) in f16; successive tokens' keys for one operator lie within a few percent
-    constexpr int D = DT == AFX_BF16 ? 7 : 49;
+    // A counter for every key of a window around the hint: +-32 keys (+-20 to 30 % in magnitude) in bf16, +-128 (+-13 to
+    // 25 %) in f16; successive tokens' keys for one operator lie within a few percent.
+    constexpr int kWin = DT == AFX_BF16 ? 64 : 256;
+    static_assert(kWin <= kSelBins, "counters");
     const int lane = lane_id(), warp = warp_id();
     int lo = 0, hi = 32768, above = 0;  // count(keys >= lo) >= k > count(keys >= hi) = above
-    int base = 4682, stride = 4682, stage = 2;
     if (hint == kNoHint && K >= 128 * m * 4) {
         // No hint: every warp that is full takes the like order statistic of one key per lane, and their mean is
         // the hint (500 samples at 16 warps: within 2 % of the rank).
@@ -115,11 +128,70 @@ __device__ __forceinline__ void sel_kth_key(const uint32_t (&kw)[2 * CH], int m,
         hint = __reduce_add_sync(0xFFFFFFFFu, e != kNoHint ? e : 0u) / full;
     }
     if (hint != kNoHint) {
-        base = static_cast<int>(hint) - 5 * D / 2;
-        stride = D;
-        stage = 0;
+        const uint32_t base = static_cast<uint32_t>(max(1, min(static_cast<int>(hint) - kWin / 2, 32768 - kWin)));
+        const uint32_t nv = sel_neg(static_cast<int>(base) + kWin);
+        const uint32_t win = static_cast<uint32_t>(__cvta_generic_to_shared(sc->win));
+        uint32_t n = 0;
+#pragma unroll
+        for (int w = 0; w < 2 * CH; ++w) {
+            if (w < 2 * m) {
+                const uint32_t a = kw[w] & kMagnitudes;
+                n += sel_ge(a, nv);
+                count_below<kWin>(win, (a & 0xFFFFu) - base);
+                count_below<kWin>(win, (a >> 16) - base);
+            }
+        }
+        n = __reduce_add_sync(0xFFFFFFFFu, (n & 0xFFFFu) + (n >> 16));
+        if (lane == 0) sc->top[warp] = n;
+        sel_barrier<NW>();
+        // lane l: counters kLane l .. of the window
+        constexpr int kLane = kWin / 32;
+        uint32_t c[kLane], sum = 0;
+#pragma unroll
+        for (int j = 0; j < kLane; j += 2) {
+            const uint2 v = *reinterpret_cast<const uint2*>(sc->win + kLane * lane + j);
+            c[j] = v.x;
+            c[j + 1] = v.y;
+            sum += v.x + v.y;
+        }
+        const uint32_t top = __reduce_add_sync(0xFFFFFFFFu, lane < NW ? sc->top[lane] : 0u);
+        uint32_t ge = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t v = __shfl_down_sync(0xFFFFFFFFu, ge, o);
+            if (lane + o < 32) ge += v;
+        }
+        ge += top;  // keys at or above the lane's first one
+        const uint32_t at = __ballot_sync(0xFFFFFFFFu, ge >= static_cast<uint32_t>(k));  // lanes 0 .. of the one that holds it
+        uint32_t run = ge - sum, key = 0, over = 0;
+        bool found = false;
+#pragma unroll
+        for (int j = kLane - 1; j >= 0; --j) {
+            if (!found) {
+                over = run;
+                key = j;
+                run += c[j];
+                found = run >= static_cast<uint32_t>(k);
+            }
+        }
+        if (at != 0u && top < static_cast<uint32_t>(k)) {
+            const uint32_t got = __shfl_sync(0xFFFFFFFFu, ((base + kLane * lane + key) << 16) | over, 31 - __clz(at));
+            thr = static_cast<int>(got >> 16);
+            need_eq = k - static_cast<int>(got & 0xFFFFu);
+            AFX_MARK(8);
+            return;
+        }
+        // the hint was off: the interval on that side of the window
+        if (at == 0u) {
+            hi = static_cast<int>(base);
+            above = static_cast<int>(__shfl_sync(0xFFFFFFFFu, ge, 0));
+        } else {
+            lo = static_cast<int>(base) + kWin;
+        }
     }
-    for (int it = 0;; ++it) {
+    int it = 0;
+    while (hi - lo > 1) {
+        const int stride = (hi - lo + C) / (C + 1), base = lo + stride;
         int cand[C];
         uint32_t nv[C], n[C];
 #pragma unroll
@@ -154,23 +226,13 @@ __device__ __forceinline__ void sel_kth_key(const uint32_t (&kw)[2 * CH], int m,
         const uint32_t od = __ballot_sync(0xFFFFFFFFu, static_cast<int>(tot >> 16) >= k) & 7u;
         const int c = __popc(ev | (od << 3));
         const uint32_t t = __shfl_sync(0xFFFFFFFFu, tot, c >> 1);
-        const bool none = c == 0, all = c == C;
         const int next = max(lo + 1, min(base + c * stride, hi));
-        if (!none) lo = max(lo + 1, min(base + (c - 1) * stride, hi));
-        if (!all) {
+        if (c > 0) lo = max(lo + 1, min(base + (c - 1) * stride, hi));
+        if (c < C) {
             hi = next;
             above = static_cast<int>((c & 1) ? t >> 16 : t & 0xFFFFu);
         }
-        if (hi - lo <= 1) break;
-        if (stage == 0 && (none || all)) {  // the hint was off: wider steps on that side of it
-            stage = 1;
-            stride = 8 * D;
-            base = all ? lo + stride : hi - C * stride;
-        } else {
-            stage = 2;
-            stride = (hi - lo + C) / (C + 1);
-            base = lo + stride;
-        }
+        ++it;
     }
     thr = lo;
     need_eq = k - above;
@@ -272,10 +334,19 @@ __device__ __forceinline__ uint32_t sel_flags(const uint32_t (&kw)[2 * CH], int 
     return fl;
 }
 
-// Calls emit(slot, element, position, active) for the lane's channels; the active ones' positions ascend with
-// the channel, from `at` for the warp's first.
-template <int CH, class Emit>
-__device__ __forceinline__ void sel_emit(uint32_t fl, int m, int at, Emit emit) {
+// Stores v to the shared-memory word at `at` and moves on to the next one where `fl` has `BIT`; never a branch.
+template <uint32_t BIT>
+__device__ __forceinline__ void st_shared_next(uint32_t& at, uint32_t v, uint32_t fl) {
+    asm volatile("{ .reg .pred p; .reg .b32 t; and.b32 t, %2, %3; setp.ne.u32 p, t, 0; @p st.shared.u32 [%0], %1; @p add.u32 %0, %0, 4; }"
+                 : "+r"(at)
+                 : "r"(v), "r"(fl), "n"(BIT)
+                 : "memory");
+}
+
+// Writes the lane's active channels (flags of sel_flags, words of sel_load_keys) as list entries (16-bit channel, 16-bit
+// value) to shared memory, `list` the address of the warp's first entry; entries ascend with the channel.
+template <int CH>
+__device__ __forceinline__ void sel_emit(uint32_t fl, int m, const uint32_t (&kw)[2 * CH], uint32_t list) {
     const int lane = lane_id();
     // Active channels per slot, four slots to a word (bytes 0..3 = slots 0, 2, 1, 3, then 4, 6, 5, 7), and
     // their prefix over the lanes (a slot of a warp has at most 128).
@@ -283,31 +354,39 @@ __device__ __forceinline__ void sel_emit(uint32_t fl, int m, int at, Emit emit) 
     uint32_t ev = pairs & 0x33333333u, od = (pairs >> 2) & 0x33333333u;  // slots 0, 2, 4, 6 and 1, 3, 5, 7
     ev += ev >> 16;
     od += od >> 16;
+    constexpr int NH = (CH + 3) / 4;
+    uint32_t cnt4[NH], incl[NH];
 #pragma unroll
-    for (int h = 0; h < (CH + 3) / 4; ++h) {
-        if (4 * h < m) {
-            const uint32_t e2 = ev >> (8 * h), o2 = od >> (8 * h);
-            const uint32_t cnt4 = (e2 & 15u) | ((e2 & 0xF0u) << 4) | ((o2 & 15u) << 16) | ((o2 & 0xF0u) << 20);
-            uint32_t incl = cnt4;
+    for (int h = 0; h < NH; ++h) {
+        const uint32_t e2 = ev >> (8 * h), o2 = od >> (8 * h);
+        cnt4[h] = (e2 & 15u) | ((e2 & 0xF0u) << 4) | ((o2 & 15u) << 16) | ((o2 & 0xF0u) << 20);
+        incl[h] = cnt4[h];
+    }
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t n = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-                if (lane >= o) incl += n;
-            }
-            const uint32_t whole = __shfl_sync(0xFFFFFFFFu, incl, 31), excl = incl - cnt4;
+    for (int o = 1; o < 32; o <<= 1) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int s = 4 * h + q, sh = q == 0 ? 0 : q == 1 ? 16 : q == 2 ? 8 : 24;
-                if (s < CH) {
-                    int pos = at + static_cast<int>((excl >> sh) & 0xFFu);
+        for (int h = 0; h < NH; ++h) {
+            const uint32_t n = __shfl_up_sync(0xFFFFFFFFu, incl[h], o);
+            if (lane >= o) incl[h] += n;
+        }
+    }
+    uint32_t chan = static_cast<uint32_t>(sel_channel(m, 0));
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const uint32_t in = fl & sel_bit(s, e);
-                        emit(s, e, pos, in != 0u);
-                        pos += in != 0u ? 1 : 0;
-                    }
-                    at += static_cast<int>((whole >> sh) & 0xFFu);
-                }
+    for (int h = 0; h < NH; ++h) {
+        const uint32_t whole = __shfl_sync(0xFFFFFFFFu, incl[h], 31), excl = incl[h] - cnt4[h];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            constexpr int kShift[4] = {0, 16, 8, 24};
+            const int s = 4 * h + q;
+            if (s < CH) {
+                uint32_t at = list + 4u * ((excl >> kShift[q]) & 0xFFu);
+                const uint32_t f = fl >> (2 * s);
+                st_shared_next<0x00001u>(at, __byte_perm(kw[2 * s], chan, 0x1054), f);
+                st_shared_next<0x10000u>(at, __byte_perm(kw[2 * s], chan + 1u, 0x3254), f);
+                st_shared_next<0x00002u>(at, __byte_perm(kw[2 * s + 1], chan + 2u, 0x1054), f);
+                st_shared_next<0x20000u>(at, __byte_perm(kw[2 * s + 1], chan + 3u, 0x3254), f);
+                list += 4u * ((whole >> kShift[q]) & 0xFFu);
+                chan += 128u;
             }
         }
     }

@@ -110,6 +110,28 @@ def test_calls_in_a_row_share_a_hint(K, N, dt):
         assert torch.equal(y[i], y[i % 2])
 
 
+@pytest.mark.parametrize("dt,half", [("bf16", 32), ("f16", 128)])
+@pytest.mark.parametrize("K", [160, 4096, 12296])
+@pytest.mark.parametrize("lo,hi", [(0, 40), (0x3C00, 0x3C90), (0x7F00, 0x7F81)])
+def test_hints_at_the_edges_of_the_counted_window(K, dt, half, lo, hi):
+    """Keys at the bottom, in the middle and at the top of the range (f16: NaN patterns), many of them equal; the k-th
+    key lies at the first and last key of the window around the hint, and just outside."""
+    rng = np.random.default_rng(K + lo)
+    keys = rng.integers(lo, hi, K)
+    x = (keys | (rng.integers(0, 2, K) << 15)).astype(np.uint16)
+    k = K // 2
+    want = oracle.select_active(x[None], dt, oracle.TOPK, k=k)
+    kth = int(np.sort(keys)[::-1][k - 1])
+    W = torch.zeros((K, 256), dtype=torch.int16, device="cuda")
+    xd, y = torch.from_numpy(x.view(np.int16)).cuda(), torch.zeros(256, device="cuda")
+    for off in (0, half - 1, half, half + 1, -half + 1, -half, -half - 1):
+        hint = torch.tensor([0x10000 | min(0x7FFF, max(0, kth + off))], dtype=torch.int32, device="cuda")
+        idx, count = torch.zeros(K, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+        afx.afx_select_gemv(W, dt, K, 256, 256, xd, 1, afx.MODE_TOPK, k, 0.0, y, 0, idx, count, kth_hint=hint)
+        assert int(count) == k and np.array_equal(idx[:k].cpu().numpy(), want), off
+        assert int(hint) == 0x10000 | kth
+
+
 @pytest.mark.parametrize("hidden,mlp", [(12296, 2312), (16392, 264), (8192, 64)])
 def test_layer_of_very_wide_hidden_state(hidden, mlp):
     """Gains read late (8 slots per lane), normed operators by clusters and by slices, a family of side outputs: two
