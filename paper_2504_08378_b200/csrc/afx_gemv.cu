@@ -1,7 +1,7 @@
 // afx_sparse_gemv: host-side shape selection and launch.
 #include "afx_launch.cuh"
 #include "afx_list.cuh"
-#include "afx_mma.cuh"
+#include "afx_mtlist.cuh"
 
 namespace afx {
 
@@ -12,39 +12,46 @@ __global__ void __launch_bounds__(kGemvThreads, 2) sparse_gemv_kernel(GemvListAr
     gemv_list_block<DT, 1, PW, 1024>(a, &sm, &recv);
 }
 
-// A few tokens at once: the tensor-core kernel (afx_mma.cuh).  2048 staged entries per pass
-// leave room for two blocks per SM.  Six stages of 16 channels: a step of four tokens on a 13B-shaped stack
-// takes 200 us a layer, 208 with four stages of 32 (more shared memory: fewer attention blocks beside it),
-// 212 with four of 16, 217 with eight.
-using MtListSmem = MtSmem<2048, 6, 16>;
+// A few tokens at once: the tensor-core kernel (afx_mtlist.cuh), two blocks per SM.
 template <int DT>
 __global__ void __launch_bounds__(kGemvThreads, 2) sparse_gemm_mt_kernel(GemvListArgs a) {
-    extern __shared__ __align__(16) unsigned char mt_dyn[];
-    mt_list_block<DT>(a, reinterpret_cast<MtListSmem*>(mt_dyn));
+    extern __shared__ __align__(16) unsigned char ml_dyn[];
+    mt_list_block<DT>(a, ml_dyn);
 }
 
+// Granules per tile and blocks per cluster: the fewest granules per block among the shapes whose clusters are all resident
+// at once with room for eight blocks more (the occupancy query counts what fits an empty GPU; behind another kernel
+// clusters were seen to run as a second wave without it).  Of equal shapes the one whose clusters are nearest to five
+// blocks: larger ones stage less of the list per block, smaller ones meet sooner.  Four tokens, granules x cluster, us:
+// 5120 -> 15360 1 x 1 36.3, 2 x 2 32.5, 4 x 4 31.0, 5 x 5 31.0, 8 x 8 31.7, 5 x 6 (not resident) 45.6;
+// 5120 -> 5120 1 x 3 15.4, 2 x 6 14.5, 3 x 9 14.7; 13824 -> 5120 1 x 3 32.8, 2 x 6 29.1; 5120 -> 27648 2 x 1 58.2,
+// 5 x 3 47.4, 3 x 2 47.1.
 template <int DT>
 static afx_status launch_gemm_mt(const GemvListArgs& a, cudaStream_t st) {
     const void* kern = reinterpret_cast<const void*>(sparse_gemm_mt_kernel<DT>);
-    const size_t dyn = sizeof(MtListSmem);
-    const int tiles = (a.N + kMtTile - 1) / kMtTile;
-    if (tiles > 65535) return AFX_ERR_CAPACITY;
-    // the largest cluster that keeps every tile's cluster resident at once (a margin stays free, as for the fp32
-    // kernels); up to 16 blocks where few tiles would leave SMs idle (four tokens, 13824 -> 5120, 20 tiles:
-    // 39.9 us with the selection, 43.5 with clusters of 8)
-    const int margin = (tiles + 15) / 16 < 2 ? 2 : (tiles + 15) / 16;
-    int most = 16;
-    if (most > kMaxCluster && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    int most = kMlMaxCluster;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
         cudaGetLastError();
         most = kMaxCluster;
     }
-    int S = 1;
-    for (int s = most; s > 1; --s)
-        if (max_active_clusters(kern, s, dyn) >= tiles + margin) {
-            S = s;
-            break;
+    const int n = (a.N + kMlGranule - 1) / kMlGranule, sms = sm_count() > 0 ? sm_count() : 148;
+    constexpr int kSpare = 8;
+    int best_s = 1, best_g = kMlMaxGranules;
+    bool found = false;
+    for (int s = 1; s <= most; ++s)
+        for (int g = 1; g <= kMlMaxGranules; ++g) {
+            const int tiles = (n + g - 1) / g;
+            if (tiles * s + kSpare > 2 * sms) continue;
+            const int order = g * best_s - best_g * s;  // < 0: fewer granules per block
+            if (found && (order > 0 || (order == 0 && abs(s - 5) >= abs(best_s - 5)))) continue;
+            if (max_active_clusters(kern, s, ml_dyn_smem(a.T, g, s)) * s < tiles * s + kSpare) continue;
+            found = true;
+            best_s = s;
+            best_g = g;
         }
-    return launch_clustered(sparse_gemm_mt_kernel<DT>, S, tiles, dyn, a, st);
+    const int tiles = (n + best_g - 1) / best_g;
+    if (tiles > 65535) return AFX_ERR_CAPACITY;
+    return launch_clustered(sparse_gemm_mt_kernel<DT>, best_s, tiles, ml_dyn_smem(a.T, best_g, best_s), a, st);
 }
 
 int sm_count() {

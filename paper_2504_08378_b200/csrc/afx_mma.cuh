@@ -209,69 +209,4 @@ __device__ __forceinline__ void mt_finish(const float (&c)[4], SMT* sm, int T, i
     cluster.sync();  // peers may still be reading this block's sums
 }
 
-// grid = (S, tiles of 256 outputs), cluster = (S, 1, 1), 512 threads.
-template <int DT, class SMT>
-__device__ __forceinline__ void mt_list_block(const GemvListArgs& a, SMT* sm) {
-    constexpr int kMtCap = SMT::kCap;
-    namespace cg = cooperative_groups;
-    cg::cluster_group cluster = cg::this_cluster();
-    const int S = static_cast<int>(cluster.num_blocks());
-    const int rank = static_cast<int>(cluster.block_rank());
-    const int tid = threadIdx.x;
-    const int tile = blockIdx.y, T = a.T;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // only after the wait (ordering rule of the library)
-    int cnt = *a.count;
-    if (cnt < 0 || cnt > a.K) {
-        if (tid == 0 && rank == 0 && tile == 0) report_status(a.status, AFX_ERR_CAPACITY);
-        cnt = max(0, min(cnt, a.K));
-    }
-    const int c_lo = static_cast<int>(static_cast<int64_t>(rank) * cnt / S);
-    const int c_hi = static_cast<int>(static_cast<int64_t>(rank + 1) * cnt / S);
-    const uint64_t ld16 = static_cast<uint64_t>(a.ldw >> 3);
-    const uint4* wtile16 = reinterpret_cast<const uint4*>(a.Wt + static_cast<size_t>(tile) * kMtTile);
-    const int n_chunks = min(kMtTile, a.N - tile * kMtTile) >> 3;
-
-    float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    __shared__ int first_ok;
-
-    for (int c0 = c_lo; c0 < c_hi; c0 += kMtCap) {
-        int staged = min(kMtCap, c_hi - c0);
-        __syncthreads();  // the previous pass has been multiplied
-        bool skipped = false;
-        for (int i = tid; i < staged; i += kGemvThreads) {
-            // as in the fp32 kernel: an entry outside [0, K) or with a negative cache slot takes no part
-            const int j = a.idx[c0 + i];
-            const int col = a.slot != nullptr ? a.slot[c0 + i] : j;
-            const bool in_range = static_cast<unsigned>(j) < static_cast<unsigned>(a.K);
-            const uint64_t off = static_cast<uint64_t>(col < 0 ? 0 : col) * ld16;
-            const bool ok = in_range && col >= 0 && off + static_cast<uint64_t>(a.N >> 3) <= 0xFFFFFFFFull;
-            if (!ok && tile == 0) report_status(a.status, in_range ? AFX_ERR_CAPACITY : AFX_ERR_INVALID_ARG);
-            skipped |= !ok;
-            sm->col[i] = ok ? static_cast<uint32_t>(off) : kSkippedEntry;
-            for (int t = 0; t < T; ++t) sm->xb[t][i] = ok ? a.x[static_cast<size_t>(t) * a.K + j] : uint16_t(0);
-        }
-        mt_pad_inputs(sm, T, staged);
-        if (__syncthreads_or(skipped)) {  // rare: a skipped entry reads the row of one that takes part (x = 0)
-            if (tid == 0) first_ok = staged;
-            __syncthreads();
-            for (int i = tid; i < staged; i += kGemvThreads)
-                if (sm->col[i] != kSkippedEntry) atomicMin(&first_ok, i);
-            __syncthreads();
-            const int f = first_ok;
-            if (f < staged) {
-                const uint32_t safe = sm->col[f];
-                __syncthreads();
-                for (int i = tid; i < staged; i += kGemvThreads)
-                    if (sm->col[i] == kSkippedEntry) sm->col[i] = safe;
-            } else {
-                staged = 0;
-            }
-            __syncthreads();
-        }
-        mt_stream_pass<DT>(wtile16, sm, staged, n_chunks, c);
-    }
-    mt_finish<DT>(c, sm, T, tile, a.N, a.silu ? EP_SILU : (a.accumulate ? EP_ACCUM : EP_STORE), a.ep);
-}
-
 }  // namespace afx

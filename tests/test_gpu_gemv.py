@@ -253,3 +253,30 @@ def test_several_tokens_slot_list_bad_entries_and_nan_inputs():
     padded = np.concatenate([full, np.full(K - full.size, 3, np.int32)])  # K entries: the count is clamped to K
     st, out = gemv(padded, K + 9)
     assert st == 3 and np.isfinite(out).all()
+
+
+@pytest.mark.parametrize("K,N,T,n", [(64, 8, 2, 1), (64, 56, 3, 15), (64, 64, 8, 16), (100, 72, 5, 17), (100, 520, 7, 0),
+                                     (3000, 1992, 4, 2999), (9000, 120, 6, 8999),  # few outputs: large clusters
+                                     (4600, 57344, 2, 4500),  # more than one pass of staged entries per block
+                                     (600, 15368, 8, 555)])
+@pytest.mark.parametrize("dt", ["bf16", "f16"])
+def test_few_tokens_at_the_edges_of_granules_steps_and_passes(K, N, T, n, dt):
+    """Rows outside the list are NaN: nothing but the list's rows may reach a sum."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(K + N)
+    td = torch.bfloat16 if dt == "bf16" else torch.float16
+    W = torch.randn(K, N, generator=g, device="cuda").mul_(0.02).to(td)
+    idx = torch.randperm(K, generator=g, device="cuda")[:n].sort().values
+    out = torch.ones(K, dtype=torch.bool, device="cuda")
+    out[idx] = False
+    W[out] = float("nan")
+    x = torch.randn(T, K, generator=g, device="cuda").to(td)
+    lst = torch.zeros(K, dtype=torch.int32, device="cuda")
+    lst[:n] = idx.int()
+    count = torch.tensor([n], dtype=torch.int32, device="cuda")
+    y = torch.full((T, N), 0.25, device="cuda")
+    afx.afx_sparse_gemv(W.view(torch.int16), dt, K, N, N, x.view(torch.int16), T, lst, count, None, y, 1)
+    w, xa = W[idx].double(), x[:, idx].double()
+    # any order of fp32 additions, each rounded or truncated to 24 bits
+    bound = (n + 3) * 2.0 ** -23 * (xa.abs() @ w.abs() + 0.25)
+    assert bool(((y.double() - 0.25 - xa @ w).abs() <= bound).all())
