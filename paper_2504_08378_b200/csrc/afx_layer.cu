@@ -78,9 +78,9 @@ static afx_status launch_fused_mt(const FusedArgs& a, cudaStream_t st) {
 
 // Several tokens with room for the list in device memory: the selection of every token on an SM of its own,
 // then the list kernel, two blocks per SM.  In one kernel (launch_fused_mt) every cluster selects for itself
-// over all tokens before it streams, one block per SM.  Four tokens of 5120 channels, 60 %, split and in one:
-// 5120 -> 15360 34.1 and 39.2 us, 5120 -> 5120 22.6 and 24.2, 5120 -> 27648 53.6 and 63.1, 13824 -> 5120
-// 39.9 and 56.6.
+// over all tokens before it streams, one block per SM.  Half of the channels of four tokens kept, in a graph, split and
+// in one: 256 -> 4096 11.6 and 12.4 us, 2048 -> 5120 14.7 and 16.6, 4096 -> 4096 17.4 and 19.4; the larger the
+// operator the more (a list kernel that was slower than now: 13824 -> 5120 39.9 and 56.6).
 template <int DT, int IN, int EP>
 static afx_status launch_split(const FusedArgs& a, cudaStream_t st) {
     // The list kernel's 32-bit row offsets would drop the channels behind them, and nothing may fail behind the
@@ -104,21 +104,11 @@ static afx_status launch_split(const FusedArgs& a, cudaStream_t st) {
     return launch_list_gemv(DT, g, st);
 }
 
-// Three or four tokens of few channels on 9 to 20 tiles of outputs: the second launch costs more than the blocks that
-// repeat the selections, unless the attention could run beside them.  With list outputs, in a graph, two kernels and
-// one: 4 tokens 256 -> 4096 14.1 and 13.1 us, 2048 -> 5120 17.0 and 15.9, 4096 -> 4096 21.4 and 20.2.  Outside:
-// 2048 -> 2048 14.9 and 15.1, 5120 -> 5120 24.1 and 24.5, 2048 -> 8192 19.1 and 19.3; 2 tokens 2048 -> 4096 13.4 and
-// 14.1; 6 tokens 2048 -> 5120 19.0 and 21.0.
-template <int IN>
-static bool one_kernel_pays(const FusedArgs& a) {
-    return IN == IN_X && !a.beside_attention && (a.T == 3 || a.T == 4) && a.K <= 4096 && a.N > 2048 && a.N <= 5120;
-}
-
 template <int DT, int IN, int EP>
 static afx_status launch_fused_dt(const FusedArgs& a, cudaStream_t st) {
     if (a.T <= 1) return launch_one_token(DT, IN, EP, ONE_TOKEN_PLAIN, a, st);
     const bool listed = a.idx_in != nullptr || (a.idx_out != nullptr && a.count_out != nullptr);
-    if (listed && (IN == IN_X || a.xnorm_out != nullptr) && a.K <= kSelectFastMaxK && !one_kernel_pays<IN>(a))
+    if (listed && (IN == IN_X || a.xnorm_out != nullptr) && a.K <= kSelectFastMaxK)
         return launch_split<DT, IN, EP>(a, st);
     if (a.T <= 4) return launch_fused_mt<DT, 4, IN, EP>(a, st);
     return launch_fused_mt<DT, 8, IN, EP>(a, st);
