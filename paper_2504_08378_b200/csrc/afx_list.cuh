@@ -23,7 +23,9 @@
 
 namespace afx {
 
-constexpr int kGemvUnroll = 8;
+// Rows in flight per lane.  Eight cost registers that 64 do not hold: 8192 -> 57344 with its selection and set difference,
+// half of the channels, 92.7 us, six 89.3, four 100.
+constexpr int kGemvUnroll = 6;
 
 template <int TMAX, int CAP>
 struct ListSmem {

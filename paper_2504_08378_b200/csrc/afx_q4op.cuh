@@ -4,13 +4,13 @@
 // The outputs are cut into tiles of whole blocks of 32, one tile per SM, and a block streams the whole active list for its
 // tile (few outputs of many channels: a cluster shares the list of a wider tile, see afx_q4op.cu).  A row's piece
 // of a tile is its codes, 16 bytes per block of 32 outputs, and its scales; a thread takes W words of codes (8 W
-// outputs) of every (NT / threads per piece)-th entry, six or eight entries in flight.
+// outputs) of every (NT / threads per piece)-th entry, five (W = 4) or four (W = 2) entries in flight (six and eight: 1 % more).
 //
 // What bounds it: the same chain of latencies as over 16-bit rows (afx_slice.cuh) and, while it streams, instruction
 // issue: three per weight, of which codes to fp32 take 1.4 and the products 0.5.  It replaced clusters of two blocks
 // per SM that each selected over a shared-memory histogram, two thirds of all instructions; a layer of 4096 and 11008
 // channels over 2048 positions, one token: 81 and 60 us.  Loading an entry's registers again as soon as it has been
-// multiplied, instead of six entries together: 63.
+// multiplied, instead of some entries together: 63.
 #pragma once
 
 #include "afx_onelist.cuh"
@@ -100,7 +100,7 @@ __device__ __forceinline__ void q4op_stream(const unsigned char* codes, const un
 template <int DT, int NT, int NW, int CH, int W, int IN, int EP, bool SPLIT>
 __device__ __forceinline__ void q4op_block(const FusedArgs& a, unsigned char* dyn, RegSelScratch* sc, float* recv) {
     constexpr int kPerBlock = 4 / W;  // threads per block of 32 outputs
-    constexpr int U = W == 4 ? 6 : 8;
+    constexpr int U = W == 4 ? 5 : 4;
     const int tid = threadIdx.x;
     const int split = SPLIT ? static_cast<int>(cg::this_cluster().num_blocks()) : 1;
     const int rank = SPLIT ? static_cast<int>(cg::this_cluster().block_rank()) : 0;

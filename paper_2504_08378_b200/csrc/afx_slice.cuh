@@ -5,7 +5,8 @@
 // one DRAM access), and a block streams the WHOLE active list for its slice: sums meet inside the block
 // only, every SM carries the same bytes, and the input stage and the selection run once per SM.  A
 // row's piece of a slice is P 16-byte loads; thread t takes piece t mod P of the list entries t div P,
-// t div P + rows, ..., eight of them in flight.
+// t div P + rows, ..., six of them in flight (eight spill at 64 registers: 7B-shaped decode step 2312 and 2244 us; four
+// 2299, five 2257, seven 2271).
 //
 // What bounds it: HBM while it streams (a 4096 -> 22016 operator at 50 %: 6.1 TB/s between the first load and
 // the last), and before and after that a chain of latencies in which HBM is idle: dependency wait 1.0 us,
@@ -51,7 +52,7 @@ __host__ __device__ inline size_t slice_dyn_smem(int threads, int K, bool list_g
 template <int DT>
 __device__ __forceinline__ void slice_stream(const uint16_t* Wt, int64_t ldw, int piece, const uint32_t* list, int cnt, int g,
                                              int groups, f32x2 (&acc)[4]) {
-    constexpr int U = 8;
+    constexpr int U = 6;
     const char* base = reinterpret_cast<const char*>(Wt + static_cast<size_t>(piece) * 8);
     const uint64_t row = static_cast<uint64_t>(ldw) * 2;
     auto consume = [&](const uint4& raw, uint32_t e) {
