@@ -111,3 +111,26 @@ def test_diff_active_matches_oracle():
     assert int(mc.item()) == 0 and int(hc.item()) == P.size
     afx.afx_diff_active(idxA, dev_i32([0]), bm, K, miss, mc, hc)
     assert int(mc.item()) == 0 and int(hc.item()) == 0
+
+
+@pytest.mark.parametrize("K", [33, 8200, 32768, 40000])
+@pytest.mark.parametrize("n", [1, 31, 33, 1024, 1025, 8192, 8193, 16385, 33000])
+def test_diff_active_at_the_edges_of_its_passes(K, n):
+    """Lists shorter and longer than one pass, predicted sets inside and outside shared memory; two entries out of range."""
+    rng = np.random.default_rng(K + n)
+    n = min(n, K)
+    A = np.sort(rng.permutation(K)[:n]).astype(np.int32)
+    P = rng.random(K) < 0.7
+    words = np.zeros((K + 31) // 32, np.uint32)
+    np.bitwise_or.at(words, np.flatnonzero(P) >> 5, np.uint32(1) << (np.flatnonzero(P) & 31).astype(np.uint32))
+    bad = [0, n - 1] if n > 2 else []
+    A[bad] = [-1, K][: len(bad)]
+    ok = (A >= 0) & (A < K)
+    want = A[ok][~P[A[ok]]]
+    miss = torch.full((K,), -1, dtype=torch.int32, device="cuda")
+    mc, hc, status = (torch.zeros(1, dtype=torch.int32, device="cuda") for _ in range(3))
+    afx.afx_diff_active(dev_i32(A), dev_i32([n]), torch.from_numpy(words.view(np.int32)).cuda(), K, miss, mc, hc, dev_status=status)
+    assert int(mc) == want.size and int(hc) == ok.sum() - want.size
+    assert np.array_equal(miss.cpu().numpy()[: want.size], want)
+    assert bool((miss[want.size:] == -1).all())
+    assert int(status) == (1 if bad else 0)
