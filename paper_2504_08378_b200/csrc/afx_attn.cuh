@@ -2,24 +2,23 @@
 // the decoder layer; the paper keeps attention dense and so does this kernel).
 //
 // grid = (S, kv_heads, T), cluster = (S,1,1): the S blocks of a cluster split the L = pos+1
-// cached positions of one (token, kv head) and meet their (max, sum, weighted V) partials
-// through distributed shared memory (softmax in base 2: exp(s) = 2^(s * log2 e)).  The block owning the last position first rotates and
+// cached positions of one (token, kv head) and push their (max, sum, weighted V) partials
+// into each other's shared memory (softmax in base 2: exp(s) = 2^(s * log2 e)).  The block owning the last position first rotates and
 // stores the current token's k and v into the cache.  head_dim is fixed at 128.  This kernel takes one
 // query head per kv head, the one in afx_attn_mma.cuh several.
 #pragma once
 
 #include <cooperative_groups.h>
 
-#include "afx_common.cuh"
+#include "afx_gemv.cuh"
 
 namespace afx {
-
-namespace cg = cooperative_groups;
 
 constexpr int kAttnThreads = 256;
 constexpr int kAttnWarps = kAttnThreads / 32;
 constexpr int kAttnWorkers = 2 * kAttnWarps;  // half warps: each walks its own positions
 constexpr int kHeadDim = 128;
+constexpr int kAttnBlocks = 8;  // blocks of a cluster at most
 constexpr int kAttnMaxRep = 8;  // query heads per kv head
 
 struct AttnArgs {
@@ -43,7 +42,8 @@ struct AttnSmem {
     __align__(16) float red[kAttnWorkers][kHeadDim];
     float red_m[kAttnWorkers];
     float red_l[kAttnWorkers];
-    float part_m, part_l, part_acc[kHeadDim];  // this block's partials, read by the cluster
+    // the cluster's partials, pushed by its blocks: every S-th dim of the head (S values of padding), and what goes with them
+    float recv_acc[kHeadDim + kAttnBlocks], recv_m[kAttnBlocks], recv_l[kAttnBlocks];
 };
 
 __device__ __forceinline__ void unpack8_f16(const uint4& raw, float (&w)[8]) {
@@ -84,6 +84,7 @@ __device__ __forceinline__ void attention_block(const AttnArgs& a, AttnSmem* sm)
 
     AFX_TRACE_REGION(0);
     AFX_MARK(0);
+    cluster_arrive();
     const size_t row_stride = static_cast<size_t>(a.kv_heads) * kHeadDim;
     const size_t head_off = static_cast<size_t>(hk) * kHeadDim + l16 * 8;
     uint16_t* kc = a.k_cache + static_cast<size_t>(t) * a.max_seq * a.kv_heads * kHeadDim;
@@ -196,7 +197,11 @@ __device__ __forceinline__ void attention_block(const AttnArgs& a, AttnSmem* sm)
         sm->red_l[worker] = l_run;
     }
     __syncthreads();
-    if (tid <= kHeadDim) {
+    // Block d % S of the cluster finishes dim d: its partial sums are pushed there, behind one cluster barrier.  (Partials
+    // that the owners fetched cost two barriers and a round trip: 0.45 us of a launch inside a layer step.)
+    const int per = (kHeadDim + S - 1) / S;
+    cluster_wait();  // the peers are running
+    if (tid < kHeadDim + S) {
         float M = -INFINITY;
 #pragma unroll
         for (int g = 0; g < kAttnWorkers; ++g) M = fmaxf(M, sm->red_m[g]);
@@ -208,44 +213,35 @@ __device__ __forceinline__ void attention_block(const AttnArgs& a, AttnSmem* sm)
             s = fmaf(w, tid < kHeadDim ? sm->red[g][tid] : sm->red_l[g], s);
         }
         if (tid < kHeadDim) {
-            sm->part_acc[tid] = s;
+            cluster.map_shared_rank(&sm->recv_acc[0], tid % S)[rank * per + tid / S] = s;
         } else {
-            sm->part_l = s;
-            sm->part_m = M;
+            cluster.map_shared_rank(&sm->recv_l[0], tid - kHeadDim)[rank] = s;
+            cluster.map_shared_rank(&sm->recv_m[0], tid - kHeadDim)[rank] = M;
         }
     }
     AFX_MARK(4);
-    cluster.sync();
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
     AFX_MARK(5);
-    for (int d = rank + S * tid; d < kHeadDim; d += S * kAttnThreads) {
-        // all remote reads first (they are independent), then the merge in block order
-        float mq[8], aq[8], lq[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            mq[q] = -INFINITY;
-            aq[q] = 0.0f;
-            lq[q] = 0.0f;
-            if (q < S) {
-                mq[q] = *cluster.map_shared_rank(&sm->part_m, q);
-                aq[q] = cluster.map_shared_rank(&sm->part_acc[0], q)[d];
-                lq[q] = *cluster.map_shared_rank(&sm->part_l, q);
-            }
-        }
+    const int d = rank + S * tid;
+    if (d < kHeadDim) {  // the merge in block order
         float M = -INFINITY;
 #pragma unroll
-        for (int q = 0; q < 8; ++q) M = fmaxf(M, mq[q]);
+        for (int q = 0; q < kAttnBlocks; ++q)
+            if (q < S) M = fmaxf(M, sm->recv_m[q]);
         float num = 0.0f, den = 0.0f;
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const float w = mq[q] == -INFINITY ? 0.0f : fast_exp2(mq[q] - M);
-            num = fmaf(w, aq[q], num);
-            den = fmaf(w, lq[q], den);
+        for (int q = 0; q < kAttnBlocks; ++q) {
+            if (q < S) {
+                const float w = sm->recv_m[q] == -INFINITY ? 0.0f : fast_exp2(sm->recv_m[q] - M);
+                num = fmaf(w, sm->recv_acc[q * per + tid], num);
+                den = fmaf(w, sm->recv_l[q], den);
+            }
         }
         a.out[static_cast<size_t>(t) * a.q_heads * kHeadDim + static_cast<size_t>(hk) * kHeadDim + d] =
             float_to_bits<DT>(num / den);
     }
-    AFX_MARK(6);
-    cluster.sync();
     AFX_MARK(7);
 }
 

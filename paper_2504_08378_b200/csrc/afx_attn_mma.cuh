@@ -35,9 +35,10 @@ struct AttnMmaSmem {
     __align__(16) float acc[kAttnMmaWarps + 1][kAttnMaxRep][kHeadDim];  // the warps' partial outputs; the last one: the new position
     float m[kAttnMmaWarps + 1][kAttnMaxRep];
     float l[kAttnMmaWarps + 1][kAttnMaxRep];
-    float part_m[kAttnMaxRep];  // this block's partials, read by the cluster
-    float part_l[kAttnMaxRep];
-    float part_acc[kAttnMaxRep][kHeadDim];
+    // the cluster's partials, pushed by its blocks: every S-th value of the heads, and what goes with them
+    float recv_acc[kAttnMaxRep * kHeadDim + kAttnMaxCluster];
+    float recv_m[kAttnMaxCluster][kAttnMaxRep];
+    float recv_l[kAttnMaxCluster][kAttnMaxRep];
 };
 
 // c += A . B, 16 x 8 x 16, fp16 in, fp32 out
@@ -74,6 +75,7 @@ __device__ __forceinline__ void attention_mma_block(const AttnArgs& a, AttnMmaSm
 
     AFX_TRACE_REGION(0);
     AFX_MARK(0);
+    cluster_arrive();
     const size_t row_stride = static_cast<size_t>(a.kv_heads) * kHeadDim;
     uint16_t* kc = a.k_cache + (static_cast<size_t>(t) * a.max_seq * a.kv_heads + hk) * kHeadDim;
     uint16_t* vc = a.v_cache + (static_cast<size_t>(t) * a.max_seq * a.kv_heads + hk) * kHeadDim;
@@ -289,6 +291,9 @@ __device__ __forceinline__ void attention_mma_block(const AttnArgs& a, AttnMmaSm
             }
     }
     __syncthreads();
+    // Block e % S of the cluster finishes value e of the heads: the partial sums are pushed there, behind one cluster barrier.
+    const int per = (rep * kHeadDim + S - 1) / S;
+    cluster_wait();  // the peers are running
     for (int e = tid; e < rep * kHeadDim; e += NT) {
         const int r = e / kHeadDim, d = e - r * kHeadDim;
         float M = -INFINITY;
@@ -302,45 +307,31 @@ __device__ __forceinline__ void attention_mma_block(const AttnArgs& a, AttnMmaSm
             acc = fmaf(w, sm->acc[g][r][d], acc);
             l = fmaf(w, sm->l[g][r], l);
         }
-        sm->part_acc[r][d] = acc;
-        if (d == 0) {
-            sm->part_m[r] = M;
-            sm->part_l[r] = l;
+        cluster.map_shared_rank(&sm->recv_acc[0], e % S)[rank * per + e / S] = acc;
+        if (d < S) {
+            cluster.map_shared_rank(&sm->recv_m[0][0], d)[rank * kAttnMaxRep + r] = M;
+            cluster.map_shared_rank(&sm->recv_l[0][0], d)[rank * kAttnMaxRep + r] = l;
         }
     }
     AFX_MARK(4);
-    cluster.sync();
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
     AFX_MARK(5);
-    for (int e = rank + S * tid; e < rep * kHeadDim; e += S * NT) {
-        const int r = e / kHeadDim, d = e - r * kHeadDim;
-        // all remote reads first (they are independent), then the merge in block order
-        float mq[kAttnMaxCluster], aq[kAttnMaxCluster], lq[kAttnMaxCluster];
-#pragma unroll
-        for (int q = 0; q < kAttnMaxCluster; ++q) {
-            mq[q] = -INFINITY;
-            aq[q] = 0.0f;
-            lq[q] = 0.0f;
-            if (q < S) {
-                mq[q] = cluster.map_shared_rank(&sm->part_m[0], q)[r];
-                aq[q] = cluster.map_shared_rank(&sm->part_acc[0][0], q)[r * kHeadDim + d];
-                lq[q] = cluster.map_shared_rank(&sm->part_l[0], q)[r];
-            }
-        }
+    for (int i = tid; rank + S * i < rep * kHeadDim; i += NT) {
+        const int e = rank + S * i, r = e / kHeadDim, d = e - r * kHeadDim;
+        // the merge in block order
         float M = -INFINITY;
-#pragma unroll
-        for (int q = 0; q < kAttnMaxCluster; ++q) M = fmaxf(M, mq[q]);
+        for (int q = 0; q < S; ++q) M = fmaxf(M, sm->recv_m[q][r]);
         float num = 0.0f, den = 0.0f;
-#pragma unroll
-        for (int q = 0; q < kAttnMaxCluster; ++q) {
-            const float w = mq[q] == -INFINITY ? 0.0f : fast_exp2(mq[q] - M);
-            num = fmaf(w, aq[q], num);
-            den = fmaf(w, lq[q], den);
+        for (int q = 0; q < S; ++q) {
+            const float w = sm->recv_m[q][r] == -INFINITY ? 0.0f : fast_exp2(sm->recv_m[q][r] - M);
+            num = fmaf(w, sm->recv_acc[q * per + i], num);
+            den = fmaf(w, sm->recv_l[q][r], den);
         }
         a.out[static_cast<size_t>(t) * a.q_heads * kHeadDim + static_cast<size_t>(hk * rep + r) * kHeadDim + d] =
             float_to_bits<DT>(num / den);
     }
-    AFX_MARK(6);
-    cluster.sync();
     AFX_MARK(7);
 }
 
