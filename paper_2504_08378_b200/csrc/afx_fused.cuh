@@ -64,6 +64,7 @@ struct FusedArgs {
     // ---- family: x was written before the kernel in front of this one started (that one decides wt_sel) ----
     int x_early;
     int slices;  // set by the launcher: slices per operator
+    int granule;  // set by the launcher (16-bit rows): 16-byte pieces of a row that a slice holds together
     int64_t x_stride, out_stride;
 };
 

@@ -4,18 +4,19 @@
 
 namespace afx {
 
-template <int DT, int NT, int NW, int CH, int IN, int EP, bool GRP, bool SPLIT>
+template <int DT, int NT, int NW, int CH, int IN, int EP, bool GRP, int FORM>
 __global__ void __launch_bounds__(NT, 1024 / NT) slice_op_kernel(FusedArgs a) {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ RegSelScratch s;
-    __shared__ float recv[SPLIT ? kSlMaxSplit * kSlSplitOutputs : 1];
-    slice_op_block<DT, NT, NW, CH, IN, EP, GRP, SPLIT>(a, dyn, &s, recv);
+    __shared__ float recv[FORM == SLICE_SPLIT ? kSlMaxSplit * kSlSplitOutputs : 1];
+    slice_op_block<DT, NT, NW, CH, IN, EP, GRP, FORM>(a, dyn, &s, recv);
 }
 
 // split: blocks (a cluster) that share the list of a granule; a.N is then at most as wide as there is room for
 // one granule per cluster.
-template <int DT, int NT, int NW, int CH, int IN, int EP, bool GRP, bool SPLIT = false>
+template <int DT, int NT, int NW, int CH, int IN, int EP, bool GRP, int FORM = SLICE_PLAIN>
 static afx_status launch_slice(const FusedArgs& a, cudaStream_t st, int split = 1) {
+    constexpr bool SPLIT = FORM == SLICE_SPLIT;
     if (static_cast<uint64_t>(a.K) * static_cast<uint64_t>(a.ldw >> 3) > 0x100000000ull) return AFX_ERR_CAPACITY;
     FusedArgs b = a;
     b.side_cluster = a.idx_out != nullptr || a.count_out != nullptr || a.bitmap_out != nullptr ||
@@ -24,9 +25,12 @@ static afx_status launch_slice(const FusedArgs& a, cudaStream_t st, int split = 
     // where one would exceed the widest a block can finish
     const int groups = GRP ? a.groups : 1;
     const int sms = sm_count() > 0 ? sm_count() : 148;
-    const int most = slice_max_pieces(NT) / kSlGranule;  // granules per slice
-    const int granules = (a.N / 8 + kSlGranule - 1) / kSlGranule;
     int nb = (sms - b.side_cluster - (GRP && a.x_early ? 1 : 0)) / groups;  // (that kernel's block keeps one SM busy)
+    b.granule = kSlGranule;
+    if (FORM == SLICE_FINE)
+        while (b.granule > (EP == EP_SILU ? 2 : 1) && 2 * ((a.N / 8 + b.granule - 1) / b.granule) <= nb) b.granule >>= 1;
+    const int most = slice_max_pieces(NT) / b.granule;  // granules per slice
+    const int granules = (a.N / 8 + b.granule - 1) / b.granule;
     if (nb > granules) nb = granules;
     if (nb < 1) nb = 1;
     if ((granules + nb - 1) / nb > most) nb = ((granules + most - 1) / most + nb - 1) / nb * nb;
@@ -34,7 +38,7 @@ static afx_status launch_slice(const FusedArgs& a, cudaStream_t st, int split = 
     b.slices = nb;
     size_t dyn = slice_dyn_smem(NT, a.K, a.idx_in != nullptr);
     if (NT == 512 && dyn < kSlAlone) dyn = kSlAlone;
-    auto kern = slice_op_kernel<DT, NT, NW, CH, IN, EP, GRP, SPLIT>;
+    auto kern = slice_op_kernel<DT, NT, NW, CH, IN, EP, GRP, FORM>;
     if (!ensure_dyn_smem(reinterpret_cast<const void*>(kern), dyn)) {
         cudaGetLastError();
         return AFX_ERR_CUDA;
@@ -72,6 +76,12 @@ constexpr int kSlNarrowMaxK = 4096;
 // 8192 -> 512 8.2 and 6.9, 8192 -> 1024 9.7 and 8.2, 16384 -> 256 12.9 and 8.2, 28672 -> 512 20.8 and 15.0; two
 // blocks per granule do not pay (8192 -> 2048 9.4 and 9.7).
 constexpr int kSlSplitMinK = 6144;
+// From here on slices of two pieces of a row, or one, where that puts twice as many SMs to work (a gate | up pair needs two
+// pieces); neighbouring SMs then share the sectors of L2.  Half of the channels kept, in a graph, four pieces, two and one:
+// 2048 -> 1024 5.3, 4.7, 4.8 us, 2816 -> 1024 5.6, 5.2, 5.1, 4096 -> 512 6.5, 5.9, 5.5, 5504 -> 1024 8.2, 7.1, 6.8,
+// 2048 -> 2048 5.5, 5.0, 4096 -> 2048 7.4, 7.0, 16384 -> 2048 15.9, 15.2; below, a list is short enough for few SMs:
+// 512 -> 1376 3.9, 4.0, 1024 -> 1024 4.2, 4.2, 4.3.
+constexpr int kSlFineMinK = 1536, kSlFineMaxN = 2336;  // (73 granules of four pieces and the block of the side outputs)
 // Selecting warps and slots: as few warps as leave a lane enough registers.
 template <int DT, int IN, int EP, bool GRP>
 static afx_status launch_slice_k(const FusedArgs& a, cudaStream_t st) {
@@ -79,10 +89,15 @@ static afx_status launch_slice_k(const FusedArgs& a, cudaStream_t st) {
         const int clusters = (a.N / 8 + kSlGranule - 1) / kSlGranule * (GRP ? a.groups : 1) + 1;  // (one for the side outputs)
         const int fit = (sm_count() > 0 ? sm_count() : 148) / clusters;
         const int split = fit >= 8 ? 8 : 4;
-        if (fit >= 4 && a.K <= 16384) return launch_slice<DT, 512, 16, 8, IN, EP, GRP, true>(a, st, split);
-        if (fit >= 4 && a.K <= 32768) return launch_slice<DT, 1024, 32, 8, IN, EP, GRP, true>(a, st, split);
+        if (fit >= 4 && a.K <= 16384) return launch_slice<DT, 512, 16, 8, IN, EP, GRP, SLICE_SPLIT>(a, st, split);
+        if (fit >= 4 && a.K <= 32768) return launch_slice<DT, 1024, 32, 8, IN, EP, GRP, SLICE_SPLIT>(a, st, split);
     }
     const bool narrow = (a.beside_attention && a.K <= kSlNarrowMaxK) || static_cast<int64_t>(a.K) * a.N <= (8 << 20);
+    if (!GRP && a.K >= kSlFineMinK && a.N <= kSlFineMaxN) {
+        if (narrow && a.K <= 4096) return launch_slice<DT, 512, 8, 4, IN, EP, GRP, SLICE_FINE>(a, st);
+        if (narrow && a.K <= 12288) return launch_slice<DT, 512, 16, 6, IN, EP, GRP, SLICE_FINE>(a, st);
+        if (a.K <= 16384) return launch_slice<DT, 1024, 16, 8, IN, EP, GRP, SLICE_FINE>(a, st);
+    }
     if (narrow && a.K <= 4096) return launch_slice<DT, 512, 8, 4, IN, EP, GRP>(a, st);
     if (narrow && a.K <= 12288) return launch_slice<DT, 512, 16, 6, IN, EP, GRP>(a, st);
     if (a.K <= 4096) return launch_slice<DT, 1024, 8, 4, IN, EP, GRP>(a, st);

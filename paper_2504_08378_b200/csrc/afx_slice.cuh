@@ -26,6 +26,8 @@
 namespace afx {
 
 constexpr int kSlGranule = 4;  // pieces (16-byte loads of a row) that one slice holds together
+// SLICE_SPLIT: the blocks of a cluster share a granule's list; SLICE_FINE: granules of fewer pieces (FusedArgs::granule).
+enum { SLICE_PLAIN = 0, SLICE_SPLIT = 1, SLICE_FINE = 2 };
 // Shared memory that at least one block of 512 threads asks for, so that an SM takes one such block and
 // what it leaves free goes to a block of another kernel.
 constexpr size_t kSlAlone = 116 * 1024;
@@ -86,7 +88,7 @@ __device__ __forceinline__ void slice_stream(const uint16_t* Wt, int64_t ldw, in
 // as outputs 8 piece0 .. of the operator: `parts` threads per output add every parts-th set, then in order.
 // SPLIT: the blocks of the cluster (all have arrived once at its barrier) push their sums into block 0's `recv`,
 // which adds them in rank order.
-template <int DT, int NT, int EP, bool SPLIT>
+template <int DT, int NT, int EP, bool SPLIT, bool FINE>
 __device__ __forceinline__ void slice_finish(const f32x2 (&acc)[4], int g, int rows, int P, int piece0, unsigned char* dyn, float* recv,
                                              float* y, uint16_t* out_bits, float scale, float y_old) {
     const int tid = threadIdx.x, nout = P * 8;
@@ -106,17 +108,26 @@ __device__ __forceinline__ void slice_finish(const f32x2 (&acc)[4], int g, int r
     }
     __syncthreads();
     float* red2 = red + NT * 8;
-    if (part < parts) {
+    // Slices of one or two pieces leave many parts per output: those of a warp meet first.
+    const bool narrow = FINE && (nout == 8 || nout == 16);
+    if (narrow) {
+        float sum = 0.0f;
+        for (int r = part; r < rows; r += parts) sum += red[r * nout + out];  // (nout divides the block: every thread has a part)
+        if (nout == 8) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 8);
+        sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 16);
+        if ((tid & 31) < nout) red2[(tid >> 5) * nout + out] = sum;
+    } else if (part < parts) {
         float sum = 0.0f;
 #pragma unroll 4
         for (int r = part; r < rows; r += parts) sum += red[r * nout + out];
         red2[tid] = sum;
     }
     __syncthreads();
+    const int sums = narrow ? NT / 32 : parts;
     auto own = [&](int o) {
         float v = red2[o];
 #pragma unroll 4
-        for (int q = 1; q < parts; ++q) v += red2[q * nout + o];
+        for (int q = 1; q < sums; ++q) v += red2[q * nout + o];
         return v;
     };
     const int split = SPLIT ? static_cast<int>(cg::this_cluster().num_blocks()) : 1;
@@ -149,8 +160,9 @@ __device__ __forceinline__ void slice_finish(const f32x2 (&acc)[4], int g, int r
 }
 
 // GRP: the grid may hold several operators of one family (FusedArgs::groups).
-template <int DT, int NT, int NW, int CH, int IN, int EP, bool GRP, bool SPLIT>
+template <int DT, int NT, int NW, int CH, int IN, int EP, bool GRP, int FORM>
 __device__ __forceinline__ void slice_op_block(const FusedArgs& a, unsigned char* dyn, RegSelScratch* sc, float* recv) {
+    constexpr bool SPLIT = FORM == SLICE_SPLIT, FINE = FORM == SLICE_FINE;
     const int tid = threadIdx.x;
     const int split = SPLIT ? static_cast<int>(cg::this_cluster().num_blocks()) : 1;  // blocks that share a list
     const int rank = SPLIT ? static_cast<int>(cg::this_cluster().block_rank()) : 0;
@@ -168,9 +180,10 @@ __device__ __forceinline__ void slice_op_block(const FusedArgs& a, unsigned char
     AFX_MARK(0);
 
     // ---- this block's slice: granules [g_lo, g_hi) of the operator, P pieces per row ----
-    const int pieces = a.N / 8, granules = (pieces + kSlGranule - 1) / kSlGranule;
+    const int gran = FINE ? a.granule : kSlGranule;
+    const int pieces = a.N / 8, granules = (pieces + gran - 1) / gran;
     const int g_lo = b * granules / nb, g_hi = (b + 1) * granules / nb;  // (the launcher keeps the products below 2^31)
-    const int piece0 = g_lo * kSlGranule, P = max(1, min(g_hi * kSlGranule, pieces) - piece0);  // 1 <= P <= slice_max_pieces
+    const int piece0 = g_lo * gran, P = max(1, min(g_hi * gran, pieces) - piece0);  // 1 <= P <= slice_max_pieces
     const int nout = P * 8;
     const int rows = NT / P;                  // list entries the block takes at once
     const int g = tid / P, piece = tid - g * P;
@@ -206,7 +219,7 @@ __device__ __forceinline__ void slice_op_block(const FusedArgs& a, unsigned char
     if (g < rows) slice_stream<DT>(Wt, a.ldw, piece0 + piece, list + c_lo, c_hi - c_lo, g, rows, acc);
     AFX_MARK(5);
 
-    slice_finish<DT, NT, EP, SPLIT>(acc, g, rows, P, piece0, dyn, recv, y, out_bits, scale, y_old);
+    slice_finish<DT, NT, EP, SPLIT, FINE>(acc, g, rows, P, piece0, dyn, recv, y, out_bits, scale, y_old);
     AFX_MARK(7);
 }
 

@@ -110,6 +110,29 @@ def test_calls_in_a_row_share_a_hint(K, N, dt):
         assert torch.equal(y[i], y[i % 2])
 
 
+@pytest.mark.parametrize("K", [1536, 5000])
+@pytest.mark.parametrize("N", [8, 264, 1168, 1176, 1184, 2352, 2360, 2368])
+def test_one_token_on_slices_of_fewer_pieces(K, N):
+    """Slices of one and two 16-byte pieces per row, at the outputs where the next smaller ones begin."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(K + N)
+    W = torch.randn(K, N, generator=g, device="cuda").mul_(0.02).to(torch.bfloat16)
+    x = torch.randn(K, generator=g, device="cuda").to(torch.bfloat16)
+    k = K // 2
+    want = oracle.select_active(x.view(torch.int16).cpu().numpy().view(np.uint16)[None], "bf16", oracle.TOPK, k=k)
+    a = torch.from_numpy(want.astype(np.int64)).cuda()
+    w, xa = W[a].double(), x[a].double()[:, None]
+    bound = (k + 3) * 2.0 ** -24 * ((w.abs() * xa.abs()).sum(0) + 0.5)  # any order of fp32 additions
+    for side in (False, True):
+        y = torch.full((N,), 0.5, device="cuda")
+        idx, count = torch.zeros(K, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+        afx.afx_select_gemv(W.view(torch.int16), "bf16", K, N, N, x.view(torch.int16), 1, afx.MODE_TOPK, k, 0.0, y, 1,
+                            idx if side else None, count if side else None)
+        assert bool(((y.double() - 0.5 - (w * xa).sum(0)).abs() <= bound).all())
+        if side:
+            assert int(count) == k and np.array_equal(idx[:k].cpu().numpy(), want)
+
+
 @pytest.mark.parametrize("dt,half", [("bf16", 32), ("f16", 128)])
 @pytest.mark.parametrize("K", [160, 4096, 12296])
 @pytest.mark.parametrize("lo,hi", [(0, 40), (0x3C00, 0x3C90), (0x7F00, 0x7F81)])
@@ -132,7 +155,7 @@ def test_hints_at_the_edges_of_the_counted_window(K, dt, half, lo, hi):
         assert int(hint) == 0x10000 | kth
 
 
-@pytest.mark.parametrize("hidden,mlp", [(12296, 2312), (16392, 264), (8192, 64)])
+@pytest.mark.parametrize("hidden,mlp", [(12296, 2312), (16392, 264), (8192, 64), (2048, 552), (1536, 1192)])
 def test_layer_of_very_wide_hidden_state(hidden, mlp):
     """Gains read late (8 slots per lane), normed operators by clusters and by slices, a family of side outputs: two
     layers, the second compared with the first one's sets."""
