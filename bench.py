@@ -1211,9 +1211,8 @@ def variant_q4_step(st, n_layers=32):
            "active_weight_bytes": int(w_bytes), "active_weight_gbs": round(w_bytes / (ms * 1e-3) / 1e9, 1),
            "weights_plus_kv_gbs": round((w_bytes + kv_bytes) / (ms * 1e-3) / 1e9, 1),
            "weight_bytes_resident": int(n_layers * sum(K * rb for (K, _), rb in zip(shapes, row_bytes))),
-           "note": "4-bit rows are 3.56x smaller than bf16 rows, but two thirds of the warp instructions of an operator "
-                   "are input stage and selection over a shared-memory histogram, repeated by every block: the token "
-                   "takes about as long as with bf16 weights, in 0.28 of the memory"}
+           "note": "4-bit rows are 3.56x smaller than bf16 rows; an operator is bound by the latencies of input stage, "
+                   "selection and sums and by the instructions that turn codes into fp32, not by bytes"}
     m.close()
     del m, layers, g
     torch.cuda.empty_cache()
