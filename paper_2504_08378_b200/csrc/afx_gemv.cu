@@ -1,4 +1,8 @@
 // afx_sparse_gemv: host-side shape selection and launch.
+#include <algorithm>
+#include <atomic>
+#include <cstdlib>
+
 #include "afx_launch.cuh"
 #include "afx_list.cuh"
 #include "afx_mtlist.cuh"
@@ -19,36 +23,53 @@ __global__ void __launch_bounds__(kGemvThreads, 2) sparse_gemm_mt_kernel(GemvLis
     mt_list_block<DT>(a, ml_dyn);
 }
 
+// Clusters of s blocks of the kernel above that are resident at once; its shared memory is never what bounds them.
+// (Asked once per device and size: a call looks through all sizes.)
+template <int DT>
+static int ml_resident(int s) {
+    static std::atomic<int> known[64][kMlMaxCluster + 1];  // + 1, 0: not asked yet
+    const void* kern = reinterpret_cast<const void*>(sparse_gemm_mt_kernel<DT>);
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    int n = known[dev][s].load(std::memory_order_relaxed) - 1;
+    if (n < 0) {
+        if (s > kMaxCluster && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        n = max_active_clusters(kern, s, ml_dyn_smem(AFX_MAX_T, kMlMaxGranules, s));
+        known[dev][s].store(n + 1, std::memory_order_relaxed);
+    }
+    return n;
+}
+
 // Granules per tile and blocks per cluster: the fewest granules per block among the shapes whose clusters are all resident
-// at once with room for eight blocks more (the occupancy query counts what fits an empty GPU; behind another kernel
-// clusters were seen to run as a second wave without it).  Of equal shapes the one whose clusters are nearest to five
-// blocks: larger ones stage less of the list per block, smaller ones meet sooner.  Four tokens, granules x cluster, us:
-// 5120 -> 15360 1 x 1 36.3, 2 x 2 32.5, 4 x 4 31.0, 5 x 5 31.0, 8 x 8 31.7, 5 x 6 (not resident) 45.6;
+// at once with room for two clusters and eight blocks more (the occupancy query counts what fits an empty GPU; behind
+// another kernel clusters were seen to run as a second wave without it).  Of equal shapes the one whose clusters are
+// nearest to five blocks: larger ones stage less of the list per block, smaller ones meet sooner.  Four tokens, granules x
+// cluster, us: 5120 -> 15360 1 x 1 36.3, 2 x 2 32.5, 4 x 4 31.0, 5 x 5 31.0, 8 x 8 31.7, 5 x 6 (not resident) 45.6;
 // 5120 -> 5120 1 x 3 15.4, 2 x 6 14.5, 3 x 9 14.7; 13824 -> 5120 1 x 3 32.8, 2 x 6 29.1; 5120 -> 27648 2 x 1 58.2,
-// 5 x 3 47.4, 3 x 2 47.1.
+// 5 x 3 47.4, 3 x 2 47.1.  Above eight blocks only the sizes that whole GPCs hold several of (1024 outputs of 4096
+// channels: 1 x 12 7.8, 1 x 13 9.0), and no block with less than a step or so of the list per warp (1024 -> 1024,
+// three tokens: 1 x 5 5.3, 1 x 10 6.1).
 template <int DT>
 static afx_status launch_gemm_mt(const GemvListArgs& a, cudaStream_t st) {
-    const void* kern = reinterpret_cast<const void*>(sparse_gemm_mt_kernel<DT>);
-    int most = kMlMaxCluster;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-        cudaGetLastError();
-        most = kMaxCluster;
-    }
-    const int n = (a.N + kMlGranule - 1) / kMlGranule, sms = sm_count() > 0 ? sm_count() : 148;
-    constexpr int kSpare = 8;
+    constexpr int kSpare = 8, kMinEntries = 192;
+    const int n = (a.N + kMlGranule - 1) / kMlGranule;
     int best_s = 1, best_g = kMlMaxGranules;
     bool found = false;
-    for (int s = 1; s <= most; ++s)
-        for (int g = 1; g <= kMlMaxGranules; ++g) {
-            const int tiles = (n + g - 1) / g;
-            if (tiles * s + kSpare > 2 * sms) continue;
-            const int order = g * best_s - best_g * s;  // < 0: fewer granules per block
-            if (found && (order > 0 || (order == 0 && abs(s - 5) >= abs(best_s - 5)))) continue;
-            if (max_active_clusters(kern, s, ml_dyn_smem(a.T, g, s)) * s < tiles * s + kSpare) continue;
-            found = true;
-            best_s = s;
-            best_g = g;
-        }
+    for (const int s : {1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 16}) {
+        if (s > 1 && a.K < s * kMinEntries) break;
+        const int resident = ml_resident<DT>(s), clusters = resident - std::max(2, (kSpare + s - 1) / s);
+        if (clusters < 1) continue;
+        const int g = (n + clusters - 1) / clusters;  // the narrowest tile that leaves no more clusters
+        if (g > kMlMaxGranules) continue;
+        const int order = g * best_s - best_g * s;  // < 0: fewer granules per block
+        if (found && (order > 0 || (order == 0 && std::abs(s - 5) >= std::abs(best_s - 5)))) continue;
+        found = true;
+        best_s = s;
+        best_g = g;
+    }
     const int tiles = (n + best_g - 1) / best_g;
     if (tiles > 65535) return AFX_ERR_CAPACITY;
     return launch_clustered(sparse_gemm_mt_kernel<DT>, best_s, tiles, ml_dyn_smem(a.T, best_g, best_s), a, st);
