@@ -256,8 +256,7 @@ __device__ __forceinline__ void fused_op_block(const FusedArgs& a, unsigned char
             }
             uint32_t thr_t = 0;
             const unsigned long long ft =
-                block_token_flags<DT, kGemvThreads>(xt, K, a.mode, a.k, a.tau, hist, first, sel, false, pos0, cnt,
-                                                    NoEmit(), 0, 0x7FFFFFFF, sel->hint[t], nullptr, &thr_t);
+                block_token_flags<DT, kGemvThreads>(xt, K, a.mode, a.k, a.tau, hist, first, sel, sel->hint[t], &thr_t);
             if (scribe && tid == 0 && topk && a.kth_multi != nullptr) a.kth_multi[t] = 0x10000 | thr_t;
             if (share) {
                 int q_lo, q_hi;

@@ -17,8 +17,6 @@
 // the same arguments.
 #pragma once
 
-#include <type_traits>
-
 #include "afx_common.cuh"
 
 namespace afx {
@@ -338,41 +336,13 @@ __device__ __forceinline__ bool block_kth_key_near(const uint16_t* xs, int K, in
 // Active flags of ONE token for the calling thread's chunks: byte v of the result covers the
 // 8 channels of chunk c_lo + v (bit e = channel 8 * (c_lo + v) + e).  xs as for
 // block_kth_key.  `hist` is the key histogram (top-k only); `hist_clean` says that it is
-// already zero and visible.  With `single` set (the token is the only one) the call also
-// returns the list position of the thread's first active channel in `pos0` and the length
-// of the list in `cnt`, from the same scan that orders the tie-break, and calls
-// emit(channel, list position, 16-bit pattern) for the thread's active channels (only for a
-// thread that can own a position in [emit_lo, emit_hi)).  `hint` (top-k; kNoKeyHint = none) is
+// already zero and visible.  `hint` (top-k; kNoKeyHint = none) is
 // a guess of the k-th key that shortens the search and never changes the result; `thr_out`
-// (top-k with 0 < k < K) receives the k-th key found, in every thread.  `xchg` (top-k emits; may be NULL) is ceil(K/8) words of shared
-// memory apart from the histogram's first KeyWindow bins and from whatever emit writes.
-// After a top-k selection with 0 < k < K, s->res[0] holds the k-th
-// key until the next selection.
-struct NoEmit {
-    __device__ __forceinline__ void operator()(int, int, uint16_t) const {}
-};
-
-// emit(channel, list position, 16-bit pattern) for the set bits of chunk c's flag byte (w = the
-// chunk's four words); the first set bit gets position `pos`.  Eight independent predicated
-// calls, no loop over the set bits: nothing waits for the previous channel.
-template <class Emit>
-__device__ __forceinline__ void emit_chunk(uint32_t byte, int c, const uint32_t (&w)[4], int pos, Emit& emit) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e)
-        if (byte & (1u << e))
-            emit((c << 3) + e, pos + __popc(byte & ((1u << e) - 1u)),
-                 static_cast<uint16_t>(w[e >> 1] >> (16 * (e & 1))));
-}
-
-template <int DT, int NT, class Emit = NoEmit>
+// (top-k with 0 < k < K) receives the k-th key found, in every thread.
+template <int DT, int NT>
 __device__ __forceinline__ unsigned long long block_token_flags(const uint16_t* xs, int K, int mode, int k,
                                                                 float tau, uint32_t* hist, bool hist_clean,
-                                                                SelectScratch* s, bool single, int& pos0,
-                                                                int& cnt, Emit emit = Emit(), int emit_lo = 0,
-                                                                int emit_hi = 0x7FFFFFFF,
-                                                                uint32_t hint = kNoKeyHint,
-                                                                uint32_t* xchg = nullptr,
-                                                                uint32_t* thr_out = nullptr) {
+                                                                SelectScratch* s, uint32_t hint, uint32_t* thr_out) {
     int c_lo, c_hi;
     thread_chunk_range(K, c_lo, c_hi);
     unsigned long long fl = 0ull;
@@ -392,20 +362,6 @@ __device__ __forceinline__ unsigned long long block_token_flags(const uint16_t* 
             }
             fl |= static_cast<unsigned long long>(byte) << (8 * (c - c_lo));
         }
-        if (single) {
-            pos0 = block_prefix(__popcll(fl), s->wtot[1], cnt);
-            int pos = pos0;
-            if (!std::is_same<Emit, NoEmit>::value && pos0 < emit_hi && pos0 + __popcll(fl) > emit_lo) {
-                for (int c = c_lo; c < c_hi; ++c) {
-                    const uint32_t byte = static_cast<uint32_t>(fl >> (8 * (c - c_lo))) & 0xFFu;
-                    if (byte == 0u) continue;
-                    const uint4 raw = *reinterpret_cast<const uint4*>(xs + (c << 3));
-                    const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
-                    emit_chunk(byte, c, w, pos, emit);
-                    pos += __popc(byte);
-                }
-            }
-        }
         return fl;
     }
     if (!hist_clean) {
@@ -417,7 +373,7 @@ __device__ __forceinline__ unsigned long long block_token_flags(const uint16_t* 
     int need_eq, tot_eq;
     if (!(hint != kNoKeyHint && block_kth_key_near<DT, NT>(xs, K, k, hint, hist, s, thr, need_eq, tot_eq)))
         block_kth_key<NT>(xs, K, k, hist, s, thr, need_eq, tot_eq);
-    if (thr_out != nullptr) *thr_out = thr;
+    *thr_out = thr;
     AFX_MARK(8);
     // Channels above the k-th key are in; of those equal to it, the need_eq lowest ids.  One
     // pass over the thread's chunks, two keys per operation (swar_*), leaves two flag sets in
@@ -442,18 +398,11 @@ __device__ __forceinline__ unsigned long long block_token_flags(const uint16_t* 
         fg |= static_cast<unsigned long long>(gbyte) << (8 * (c - c_lo));
         fe |= static_cast<unsigned long long>(ebyte) << (8 * (c - c_lo));
     }
-    const int g = __popcll(fg), e_cnt = __popcll(fe);
     AFX_MARK(9);
     int pre_e = 0;
-    if (single) {
+    if (need_eq != tot_eq) {
         int tot;
-        const int pre = block_prefix((g << 16) | e_cnt, s->wtot[1], tot);  // g < 2^15, e <= 2^15: no carry
-        pre_e = pre & 0xFFFF;
-        pos0 = (pre >> 16) + min(pre_e, need_eq);
-        cnt = k;
-    } else if (need_eq != tot_eq) {
-        int tot;
-        pre_e = block_prefix(e_cnt, s->wtot[1], tot);
+        pre_e = block_prefix(__popcll(fe), s->wtot[1], tot);
     }
     AFX_MARK(10);
     fl = fg;
@@ -467,44 +416,6 @@ __device__ __forceinline__ unsigned long long block_token_flags(const uint16_t* 
             const unsigned long long low = rest & (0ull - rest);
             rest ^= low;
             fl |= low;
-        }
-    }
-    if (single && !std::is_same<Emit, NoEmit>::value) {
-        const int nchunks = (K + 7) >> 3;
-        if (xchg != nullptr && nchunks > NT) {
-            // Several chunks per thread: the few owners of the positions [emit_lo, emit_hi)
-            // would emit chunk after chunk.  Every owner posts (position, flags) of its chunks
-            // instead, and the chunks that touch the range are emitted by one thread each.
-            int pos = pos0;
-            for (int c = c_lo; c < c_hi; ++c) {
-                const uint32_t byte = static_cast<uint32_t>(fl >> (8 * (c - c_lo))) & 0xFFu;
-                xchg[c] = (static_cast<uint32_t>(pos) << 8) | byte;
-                pos += __popc(byte);
-            }
-            __syncthreads();
-            for (int c = threadIdx.x; c < nchunks; c += NT) {
-                const uint32_t v = xchg[c];
-                const uint32_t byte = v & 0xFFu;
-                const int p = static_cast<int>(v >> 8);
-                if (byte != 0u && p < emit_hi && p + __popc(byte) > emit_lo) {
-                    const uint4 raw = *reinterpret_cast<const uint4*>(xs + (c << 3));
-                    const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
-                    emit_chunk(byte, c, w, p, emit);
-                }
-            }
-        } else {
-            const int n = __popcll(fl);
-            if (pos0 < emit_hi && pos0 + n > emit_lo) {
-                int pos = pos0;
-                for (int c = c_lo; c < c_hi; ++c) {
-                    const uint32_t byte = static_cast<uint32_t>(fl >> (8 * (c - c_lo))) & 0xFFu;
-                    if (byte == 0u) continue;
-                    const uint4 raw = *reinterpret_cast<const uint4*>(xs + (c << 3));
-                    const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
-                    emit_chunk(byte, c, w, pos, emit);
-                    pos += __popc(byte);
-                }
-            }
         }
     }
     return fl;
