@@ -33,7 +33,11 @@ struct EpilogueArgs {
                          // expert's routing weight), or NULL for 1
 };
 
-constexpr uint32_t kSkippedEntry = 0xFFFFFFFFu;  // staged column of a list entry that takes no part
+// A staged list entry holds its row's offset from the start of the weights in 16-byte units, in 32 bits; the place inside
+// the row is added in 64 bits, so that only the offset itself has to fit.  (An operator of K rows whose K * ldw / 8 is at
+// most 2^32, 64 GB, has no row whose offset does not.)
+constexpr uint32_t kSkippedEntry = 0xFFFFFFFFu;  // of an entry that takes no part
+__device__ __forceinline__ bool row_offset_fits(uint64_t off) { return off < kSkippedEntry; }
 
 struct GemvListArgs {
     const uint16_t* Wt;

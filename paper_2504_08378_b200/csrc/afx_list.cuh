@@ -245,7 +245,7 @@ __device__ __forceinline__ void gemv_list_block(const GemvListArgs& a, ListSmem<
             const int col = a.slot != nullptr ? a.slot[c0 + i] : j;
             const bool in_range = static_cast<unsigned>(j) < static_cast<unsigned>(a.K);
             const uint64_t off = static_cast<uint64_t>(col < 0 ? 0 : col) * ld16;
-            const bool ok = in_range && col >= 0 && off + static_cast<uint64_t>(a.N >> 3) <= 0xFFFFFFFFull;
+            const bool ok = in_range && col >= 0 && row_offset_fits(off);
             if (!ok && tile == 0) report_status(a.status, in_range ? AFX_ERR_CAPACITY : AFX_ERR_INVALID_ARG);
             skipped |= !ok;
             sm->col[i] = ok ? static_cast<uint32_t>(off) : kSkippedEntry;

@@ -61,24 +61,24 @@ __global__ void __launch_bounds__(kQ4Threads, 2) sparse_gemv_q4_kernel(Q4Args a)
         for (int i = tid; i < staged; i += kQ4Threads) {
             const int j = a.idx[c0 + i];
             const uint64_t off = static_cast<uint64_t>(j < 0 ? 0 : j) * ld16;
-            const bool ok = static_cast<unsigned>(j) < static_cast<unsigned>(a.K) && off + ld16 <= 0xFFFFFFFFull;
+            const bool ok = static_cast<unsigned>(j) < static_cast<unsigned>(a.K) && row_offset_fits(off);
             if (!ok && tile == 0) report_status(a.status, AFX_ERR_INVALID_ARG);
             skipped |= !ok;
-            s_off[i] = ok ? static_cast<uint32_t>(off) : 0xFFFFFFFFu;
+            s_off[i] = ok ? static_cast<uint32_t>(off) : kSkippedEntry;
             s_x[i] = ok ? bits_to_float<XDT>(a.x[j]) : 0.0f;
         }
         if (__syncthreads_or(skipped)) {  // rare: a skipped entry reads the row of one that takes part
             if (tid == 0) first_ok = staged;
             __syncthreads();
             for (int i = tid; i < staged; i += kQ4Threads)
-                if (s_off[i] != 0xFFFFFFFFu) atomicMin(&first_ok, i);
+                if (s_off[i] != kSkippedEntry) atomicMin(&first_ok, i);
             __syncthreads();
             const int f = first_ok;
             if (f < staged) {
                 const uint32_t safe = s_off[f];
                 __syncthreads();
                 for (int i = tid; i < staged; i += kQ4Threads)
-                    if (s_off[i] == 0xFFFFFFFFu) s_off[i] = safe;
+                    if (s_off[i] == kSkippedEntry) s_off[i] = safe;
             } else {
                 staged = 0;
             }

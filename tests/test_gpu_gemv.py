@@ -280,3 +280,46 @@ def test_few_tokens_at_the_edges_of_granules_steps_and_passes(K, N, T, n, dt):
     # any order of fp32 additions, each rounded or truncated to 24 bits
     bound = (n + 3) * 2.0 ** -23 * (xa.abs() @ w.abs() + 0.25)
     assert bool(((y.double() - 0.25 - xa @ w).abs() <= bound).all())
+
+
+def test_last_row_of_an_operator_of_64_gib():
+    """Row offsets are 32-bit counts of 16 bytes: 2^32 of them make up the largest operator, and its last row takes part
+    like any other, in the calls over a list and in the operator that selects."""
+    K, N, dt = 32768, 1 << 20, "bf16"
+    torch.cuda.empty_cache()
+    if torch.cuda.mem_get_info()[0] < 72 << 30:
+        pytest.skip("needs 72 GiB of free device memory")
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    W = torch.empty((K, N), dtype=torch.bfloat16, device="cuda")
+    rows = [3, K - 1]
+    W[rows] = torch.randn(2, N, generator=g, device="cuda").to(W.dtype)
+    x = torch.zeros((2, K), dtype=torch.bfloat16, device="cuda")
+    x[:, rows] = torch.tensor([[1.5, -2.25], [0.375, 3.0]], dtype=torch.bfloat16, device="cuda")
+    idx = torch.zeros(K, dtype=torch.int32, device="cuda")
+    idx[:2] = torch.tensor(rows, dtype=torch.int32)
+    count = torch.tensor([2], dtype=torch.int32, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    want = x[:, rows].double() @ W[rows].double()
+    bound = 4 * 2.0 ** -23 * (x[:, rows].double().abs() @ W[rows].double().abs())  # exact products, one rounded sum
+    for T in (1, 2):
+        y = torch.zeros((T, N), device="cuda")
+        afx.afx_sparse_gemv(W.view(torch.int16), dt, K, N, N, x[:T].view(torch.int16), T, idx, count, None, y, 0, dev_status=status)
+        assert int(status.item()) == 0 and bool(((y.double() - want[:T]).abs() <= bound[:T]).all())
+        out, n = torch.zeros_like(idx), torch.zeros_like(count)
+        y.zero_()
+        afx.afx_select_gemv(W.view(torch.int16), dt, K, N, N, x[:T].view(torch.int16), T, afx.MODE_TOPK, 2, 0.0, y, 0, out, n)
+        assert int(n.item()) == 2 and out[:2].tolist() == rows
+        assert bool(((y.double() - want[:T]).abs() <= bound[:T]).all())
+    # 4-bit rows a 32768th of the same memory apart
+    n4 = 64
+    q = W.view(torch.uint8)
+    q[:, : n4 // 2] = torch.arange(K, device="cuda", dtype=torch.int64).view(K, 1).remainder(251).to(torch.uint8)
+    q[:, n4 // 2: n4 // 2 + n4 // 16] = torch.tensor([1.0, 0.5], dtype=torch.float16, device="cuda").view(torch.uint8)
+    y = torch.zeros(n4, device="cuda")
+    afx.afx_sparse_gemv_q4(q, K, n4, 2 * N, x[0].view(torch.int16), dt, idx, count, y, 0, dev_status=status)
+    byte = torch.tensor([r % 251 for r in rows], dtype=torch.float64, device="cuda")
+    code = torch.stack([byte.remainder(16), (byte / 16).floor()], 1) - 8.0  # low and high nibbles of every byte of a row
+    per_block = (x[0, rows].double().view(2, 1) * code).sum(0).repeat_interleave(16)
+    assert int(status.item()) == 0
+    assert torch.equal(y.double(), torch.cat([per_block, 0.5 * per_block]))  # small integers and halves: exact
