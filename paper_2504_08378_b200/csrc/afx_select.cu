@@ -45,54 +45,81 @@ select_kernel(const uint16_t* __restrict__ x, int K, int T, int mode, int k, flo
 // What bounds it is latency: of the dependency wait, the count, the list and P, one behind the other.  All entries of a
 // pass are on their way together and stay in registers until they are written; P is in shared memory by then, where it
 // fits.  A warp that took its chunks one after the other, twice, needed two loads in a row for each (selection,
-// difference of 4096 entries and list operator 8192 -> 57344: 89.3 us, now 87.7).
+// difference of 4096 entries and list operator 8192 -> 57344: 89.3 us, now 87.7).  A short list is done in a pass with
+// room for one chunk per warp, or four: the instructions of eight cost more than the loads.  us in a graph, one
+// after the other, with eight always, and now: 51 of 512 entries 2.1, 2.7, 1.7; 2048 of 4096 2.8, 3.0, 2.1; 7372 of 8192
+// 5.6, 3.4, 3.1; 100000 of 200000 60.0, 28.7, 25.8.
 constexpr int kDiffChunks = 8;                     // chunks of 32 entries per warp and pass
 constexpr int kDiffWords = kSelectFastMaxK / 32;   // words of P in shared memory
-__global__ void __launch_bounds__(kSelectThreads, 1)
-diff_kernel(const int32_t* __restrict__ idxA, const int32_t* __restrict__ cntA,
-            const uint32_t* __restrict__ bitmapP, int K, int32_t* __restrict__ miss,
-            int32_t* __restrict__ miss_count, int32_t* __restrict__ hit_count, int32_t* __restrict__ status) {
-    __shared__ int scan[2][33];
-    __shared__ uint32_t words[kDiffWords];
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // only after the wait (ordering rule of the library)
-    const bool staged = K <= kSelectFastMaxK;
-    if (staged)
-        for (int w = threadIdx.x; w < (K + 31) / 32; w += kSelectThreads) words[w] = bitmapP[w];
-    int n = *cntA;
-    if (n < 0 || n > K) {
-        if (threadIdx.x == 0) report_status(status, AFX_ERR_CAPACITY);
-        n = max(0, min(n, K));
-    }
+
+struct DiffArgs {
+    const int32_t* idxA;
+    const uint32_t* bitmapP;
+    int32_t* miss;
+    int K, n;
+};
+// The chunks c_lo .. of the list, `per` <= CH of them per warp: writes their misses from position n_miss on; the number
+// of misses, and of entries out of range above bit 16.  Every thread calls it; a block barrier is part of it.
+template <int CH, bool STAGED>
+__device__ __forceinline__ int diff_pass(const DiffArgs& a, int c_lo, int per, const uint32_t* words, bool first, int* scan, int n_miss) {
     const int lane = lane_id();
     const uint32_t lt_mask = (1u << lane) - 1u;
+    const int p0 = ((c_lo + warp_id() * per) << 5) + lane;  // (a position beyond the run of another warp is beyond n as well)
+    int j[CH];
+#pragma unroll
+    for (int c = 0; c < CH; ++c) j[c] = c < per && p0 + 32 * c < a.n ? __ldg(a.idxA + p0 + 32 * c) : 0;
+    if (first) __syncthreads();  // P is in place
+    uint32_t m[CH];
+    int mine = 0;
+#pragma unroll
+    for (int c = 0; c < CH; ++c) {
+        const bool here = c < per && p0 + 32 * c < a.n, ok = static_cast<unsigned>(j[c]) < static_cast<unsigned>(a.K);
+        uint32_t w = 0xFFFFFFFFu;
+        if (here && ok) w = STAGED ? words[j[c] >> 5] : __ldg(a.bitmapP + (j[c] >> 5));
+        m[c] = __ballot_sync(0xFFFFFFFFu, here && ok && ((w >> (j[c] & 31)) & 1u) == 0u);
+        mine += __popc(m[c]) + (__popc(__ballot_sync(0xFFFFFFFFu, here && !ok)) << 16);
+    }
+    int total;
+    int at = n_miss + (warp_prefix(mine, scan, total) & 0xFFFF);
+#pragma unroll
+    for (int c = 0; c < CH; ++c) {
+        if ((m[c] >> lane) & 1u) a.miss[at + __popc(m[c] & lt_mask)] = j[c];
+        at += __popc(m[c]);
+    }
+    return total;
+}
+
+__global__ void __launch_bounds__(kSelectThreads, 1)
+diff_kernel(DiffArgs a, const int32_t* __restrict__ cntA, int32_t* __restrict__ miss_count, int32_t* __restrict__ hit_count,
+            int32_t* __restrict__ status) {
+    __shared__ int scan[2][33];
+    __shared__ uint32_t words[kDiffWords];
     constexpr int kWarps = kSelectThreads / 32;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // only after the wait (ordering rule of the library)
+    const bool staged = a.K <= kSelectFastMaxK;
+    int n = *cntA;
+    if (staged)
+        for (int w = threadIdx.x; w < (a.K + 31) / 32; w += kSelectThreads) words[w] = a.bitmapP[w];
+    if (n < 0 || n > a.K) {
+        if (threadIdx.x == 0) report_status(status, AFX_ERR_CAPACITY);
+        n = max(0, min(n, a.K));
+    }
+    a.n = n;
     const int nchunks = (n + 31) >> 5;
     int n_miss = 0, n_bad = 0;
     for (int pass = 0, c_lo = 0; c_lo < nchunks; ++pass, c_lo += kWarps * kDiffChunks) {
         const int per = min(kDiffChunks, (nchunks - c_lo + kWarps - 1) / kWarps);
-        const int p0 = ((c_lo + warp_id() * per) << 5) + lane;  // (a position beyond the run of another warp is beyond n as well)
-        int j[kDiffChunks];
-#pragma unroll
-        for (int c = 0; c < kDiffChunks; ++c) j[c] = c < per && p0 + 32 * c < n ? idxA[p0 + 32 * c] : 0;
-        if (pass == 0) __syncthreads();  // P is in place
-        uint32_t m[kDiffChunks];
-        int mine = 0;  // misses, and entries out of range above bit 16
-#pragma unroll
-        for (int c = 0; c < kDiffChunks; ++c) {
-            const bool here = c < per && p0 + 32 * c < n, ok = static_cast<unsigned>(j[c]) < static_cast<unsigned>(K);
-            uint32_t w = 0xFFFFFFFFu;
-            if (here && ok) w = staged ? words[j[c] >> 5] : bitmapP[j[c] >> 5];
-            m[c] = __ballot_sync(0xFFFFFFFFu, here && ok && ((w >> (j[c] & 31)) & 1u) == 0u);
-            mine += __popc(m[c]) + (__popc(__ballot_sync(0xFFFFFFFFu, here && !ok)) << 16);
-        }
+        int* const sc = scan[pass & 1];
         int total;
-        int at = n_miss + (warp_prefix(mine, scan[pass & 1], total) & 0xFFFF);
-#pragma unroll
-        for (int c = 0; c < kDiffChunks; ++c) {
-            if ((m[c] >> lane) & 1u) miss[at + __popc(m[c] & lt_mask)] = j[c];
-            at += __popc(m[c]);
-        }
+        if (!staged)
+            total = diff_pass<kDiffChunks, false>(a, c_lo, per, words, false, sc, n_miss);
+        else if (per == 1)
+            total = diff_pass<1, true>(a, c_lo, per, words, pass == 0, sc, n_miss);
+        else if (per <= 4)
+            total = diff_pass<4, true>(a, c_lo, per, words, pass == 0, sc, n_miss);
+        else
+            total = diff_pass<kDiffChunks, true>(a, c_lo, per, words, pass == 0, sc, n_miss);
         n_miss += total & 0xFFFF;
         n_bad += total >> 16;
     }
@@ -165,7 +192,7 @@ extern "C" afx_status afx_diff_active(const int32_t* idxA, const int32_t* cntA,
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, diff_kernel, idxA, cntA, bitmapP, K, miss, miss_count, hit_count, dev_status) == cudaSuccess
+    return cudaLaunchKernelEx(&cfg, diff_kernel, DiffArgs{idxA, bitmapP, miss, K, 0}, cntA, miss_count, hit_count, dev_status) == cudaSuccess
                ? AFX_OK
                : AFX_ERR_CUDA;
 }

@@ -134,3 +134,9 @@ def test_diff_active_at_the_edges_of_its_passes(K, n):
     assert np.array_equal(miss.cpu().numpy()[: want.size], want)
     assert bool((miss[want.size:] == -1).all())
     assert int(status) == (1 if bad else 0)
+
+
+@pytest.mark.parametrize("K", [32768, 40000])
+@pytest.mark.parametrize("n", [2048, 4095, 4096, 4097])
+def test_diff_active_where_a_pass_makes_more_room(K, n):
+    test_diff_active_at_the_edges_of_its_passes(K, n)
