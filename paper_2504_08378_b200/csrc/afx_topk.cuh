@@ -4,12 +4,13 @@
 // lane .. + 3.  The k-th largest 15-bit magnitude key is found from a hint of it, the last k-th key or, without one, a
 // sample of the keys: every key of a window around the hint has a counter in shared memory, the keys above the
 // window are counted two per operation, and behind ONE barrier every warp sums the counters from the top.  Where the
-// k-th key is outside the window a seven-way search of the rest follows: a step counts the keys at or above six
-// candidates, adds the counts over warp and block (three `redux` before and three shuffles behind one barrier of the NW
-// warps) and keeps a seventh of the interval.
+// k-th key is outside the window a seven-way search of the rest follows, from the window outwards: a step counts the keys
+// at or above six candidates, adds the counts over warp and block (three `redux` before and three shuffles behind one
+// barrier of the NW warps) and keeps the interval between two of them.
 //
 // What bounds it is the latency of barriers and reductions and the rate of shared-memory atomics (about one in ten keys
-// is in the window).  Clocks for the k-th key, the seven-way search alone from the same hint and now: bf16 K = 4096 on 8
+// is in the window; all of them on one counter cost no more: one token of 28672 equal magnitudes 8.8 us, of Laplace ones
+// 9.6).  Clocks for the k-th key, the seven-way search alone from the same hint and now: bf16 K = 4096 on 8
 // warps 2050 and 1560, K = 11008 on 16 warps 3850 and 2340; f16 K = 4096 3030 and 1640, K = 1024 2470 and 1030.  What
 // every warp repeats behind the barrier counts NW times, so few warps with many keys each beat many warps with few.
 #pragma once
@@ -104,12 +105,20 @@ template <int DT, int NW, int CH>
 __device__ __forceinline__ void sel_kth_key(const uint32_t (&kw)[2 * CH], int m, int K, int k, uint32_t hint, RegSelScratch* sc,
                                             int& thr, int& need_eq) {
     constexpr int C = 6;
-    // A counter for every key of a window around the hint: +-32 keys (+-20 to 30 % in magnitude) in bf16, +-128 (+-13 to
-    // 25 %) in f16; successive tokens' keys for one operator lie within a few percent.
+    // A counter for every key of a window around the hint: +-32 keys in bf16 (+-12 to 25 % in magnitude), +-128 in f16
+    // (+-6 to 12 %); successive tokens' keys for one operator lie within a few percent.
     constexpr int kWin = DT == AFX_BF16 ? 64 : 256;
     static_assert(kWin <= kSelBins, "counters");
     const int lane = lane_id(), warp = warp_id();
     int lo = 0, hi = 32768, above = 0;  // count(keys >= lo) >= k > count(keys >= hi) = above
+    // The candidates of a search step are a seventh of the interval apart.  Behind a missed window they are a power of seven
+    // apart, next to it, since that is where the k-th key usually is: two steps are left in bf16, three in f16, instead of
+    // five (a hint off by more than a factor of four pays one step more).  From below the farthest one is key 1: more than
+    // half of some inputs are zeros.  us, the whole selection, a missed window behind which the search took sevenths at
+    // once, and now: one token of 4096 4-bit values 5.1 and 4.7, half of 4096 zeros 6.1 and 4.5; f16, four tokens of 4096
+    // 7.1 and 6.6, one of 11008 values half of them zeros 11.0 and 7.4.
+    constexpr int kNear = DT == AFX_BF16 ? 49 : 343;
+    int stride = (32768 + C) / (C + 1), from = stride;
     if (hint == kNoHint && K >= 128 * m * 4) {
         // No hint: every warp that is full takes the like order statistic of one key per lane, and their mean is
         // the hint (500 samples at 16 warps: within 2 % of the rank).
@@ -185,19 +194,20 @@ __device__ __forceinline__ void sel_kth_key(const uint32_t (&kw)[2 * CH], int m,
         if (at == 0u) {
             hi = static_cast<int>(base);
             above = static_cast<int>(__shfl_sync(0xFFFFFFFFu, ge, 0));
+            from = hi - C * kNear;
         } else {
             lo = static_cast<int>(base) + kWin;
+            from = lo + kNear;
         }
+        stride = kNear;
     }
     int it = 0;
     while (hi - lo > 1) {
-        const int stride = (hi - lo + C) / (C + 1), base = lo + stride;
-        int cand[C];
+        const bool zeros = it == 0 && stride == kNear && lo == 0;
         uint32_t nv[C], n[C];
 #pragma unroll
         for (int j = 0; j < C; ++j) {
-            cand[j] = max(lo + 1, min(base + j * stride, hi));
-            nv[j] = sel_neg(cand[j]);
+            nv[j] = sel_neg(j == 0 && zeros ? 1 : max(lo + 1, min(from + j * stride, hi)));
             n[j] = 0;
         }
 #pragma unroll
@@ -226,12 +236,14 @@ __device__ __forceinline__ void sel_kth_key(const uint32_t (&kw)[2 * CH], int m,
         const uint32_t od = __ballot_sync(0xFFFFFFFFu, static_cast<int>(tot >> 16) >= k) & 7u;
         const int c = __popc(ev | (od << 3));
         const uint32_t t = __shfl_sync(0xFFFFFFFFu, tot, c >> 1);
-        const int next = max(lo + 1, min(base + c * stride, hi));
-        if (c > 0) lo = max(lo + 1, min(base + (c - 1) * stride, hi));
+        const int next = c == 0 && zeros ? 1 : max(lo + 1, min(from + c * stride, hi));
+        if (c > 0) lo = c == 1 && zeros ? 1 : max(lo + 1, min(from + (c - 1) * stride, hi));
         if (c < C) {
             hi = next;
             above = static_cast<int>((c & 1) ? t >> 16 : t & 0xFFFFu);
         }
+        stride = (hi - lo + C) / (C + 1);
+        from = lo + stride;
         ++it;
     }
     thr = lo;

@@ -155,6 +155,29 @@ def test_hints_at_the_edges_of_the_counted_window(K, dt, half, lo, hi):
         assert int(hint) == 0x10000 | kth
 
 
+@pytest.mark.parametrize("dt,half,near", [("bf16", 32, 49), ("f16", 128, 343)])
+@pytest.mark.parametrize("K,zeros", [(160, 0.0), (4096, 0.0), (12296, 0.0), (1000, 0.49), (4096, 0.6)])
+def test_hints_whose_window_misses(K, zeros, dt, half, near):
+    """The search from the window outwards: the k-th key at, before and behind the first, second and last of the next
+    candidates, beyond all of them, and among zeros."""
+    rng = np.random.default_rng(K)
+    keys = rng.integers(0x1000, 0x6000, K)
+    keys[rng.random(K) < zeros] = 0
+    x = (keys | (rng.integers(0, 2, K) << 15)).astype(np.uint16)
+    k = K // 2
+    want = oracle.select_active(x[None], dt, oracle.TOPK, k=k)
+    kth = int(np.sort(keys)[::-1][k - 1])
+    W = torch.zeros((K, 256), dtype=torch.int16, device="cuda")
+    xd, y = torch.from_numpy(x.view(np.int16)).cuda(), torch.zeros(256, device="cuda")
+    for d in [half + m * near + e for m in (0, 1, 2, 6) for e in (-1, 0, 1, 2)] + [6000, 12000, 24000]:
+        for hint in {min(0x7FFF, kth + d), max(0, kth - d)}:
+            slot = torch.tensor([0x10000 | hint], dtype=torch.int32, device="cuda")
+            idx, count = torch.zeros(K, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+            afx.afx_select_gemv(W, dt, K, 256, 256, xd, 1, afx.MODE_TOPK, k, 0.0, y, 0, idx, count, kth_hint=slot)
+            assert int(count) == k and np.array_equal(idx[:k].cpu().numpy(), want), (d, hint)
+            assert int(slot) == 0x10000 | kth
+
+
 @pytest.mark.parametrize("hidden,mlp", [(12296, 2312), (16392, 264), (8192, 64), (2048, 552), (1536, 1192)])
 def test_layer_of_very_wide_hidden_state(hidden, mlp):
     """Gains read late (8 slots per lane), normed operators by clusters and by slices, a family of side outputs: two
