@@ -1,7 +1,7 @@
 // afx_sparse_gemv: host-side shape selection and launch.
 #include <algorithm>
 #include <atomic>
-#include <cstdlib>
+#include <cmath>
 
 #include "afx_launch.cuh"
 #include "afx_list.cuh"
@@ -43,30 +43,35 @@ static int ml_resident(int s) {
     return n;
 }
 
-// Granules per tile and blocks per cluster: the fewest granules per block among the shapes whose clusters are all resident
-// at once with room for two clusters and eight blocks more (the occupancy query counts what fits an empty GPU; behind
-// another kernel clusters were seen to run as a second wave without it).  Of equal shapes the one whose clusters are
-// nearest to five blocks: larger ones stage less of the list per block, smaller ones meet sooner.  Four tokens, granules x
-// cluster, us: 5120 -> 15360 1 x 1 36.3, 2 x 2 32.5, 4 x 4 31.0, 5 x 5 31.0, 8 x 8 31.7, 5 x 6 (not resident) 45.6;
-// 5120 -> 5120 1 x 3 15.4, 2 x 6 14.5, 3 x 9 14.7; 13824 -> 5120 1 x 3 32.8, 2 x 6 29.1; 5120 -> 27648 2 x 1 58.2,
-// 5 x 3 47.4, 3 x 2 47.1.  Above eight blocks only the sizes that whole GPCs hold several of (1024 outputs of 4096
-// channels: 1 x 12 7.8, 1 x 13 9.0), and no block with less than a step or so of the list per warp (1024 -> 1024,
-// three tokens: 1 x 5 5.3, 1 x 10 6.1).
+// Granules g per tile and blocks s per cluster.  Of every cluster size that keeps all clusters resident at once, with room
+// for two clusters and eight blocks more (the occupancy query counts what fits an empty GPU; behind another kernel
+// clusters were seen to run as a second wave without it), the narrowest tile; of these the shape of least cost.  The cost
+// is that of a block, in parts that were fitted to 207 calls of 1024 to 13824 channels on 1024 to 57344 outputs with two,
+// four and eight tokens, each in 5 to 25 shapes: the entries that a warp multiplies (16 / g warps share a granule's
+// list, so that three, five, six or seven granules leave warps idle), the entries that it stages, and the rows and peers
+// that its sums meet.  It is within 1 % of the best resident shape in the mean and 18 % at worst; the fewest granules per
+// block, the nearest to five blocks of equals, were within 4 % and 38 %.  By that rule and now, us: eight tokens
+// 1024 -> 16384 14.3 and 11.6, 2048 -> 20480 25.2 and 19.9, 5120 -> 24576 43.0 and 40.9, 5120 -> 16384 31.0 and 29.3;
+// four tokens 5120 -> 14336 27.1 and 26.5, 1024 -> 10240 9.9 and 8.8; two tokens 2048 -> 10240 11.4 and 10.4.
+// Sizes above eight only where whole GPCs hold several of them, and not nine (28 of 30 clusters of nine ran as one wave or
+// two from call to call).  No block with less than a step or so of the list per warp (1024 -> 1024, three tokens: 1 x 5
+// 5.3, 1 x 10 6.1).
 template <int DT>
 static afx_status launch_gemm_mt(const GemvListArgs& a, cudaStream_t st) {
     constexpr int kSpare = 8, kMinEntries = 192;
     const int n = (a.N + kMlGranule - 1) / kMlGranule;
     int best_s = 1, best_g = kMlMaxGranules;
-    bool found = false;
+    float least = INFINITY;
     for (const int s : {1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 16}) {
         if (s > 1 && a.K < s * kMinEntries) break;
         const int resident = ml_resident<DT>(s), clusters = resident - std::max(2, (kSpare + s - 1) / s);
         if (clusters < 1) continue;
         const int g = (n + clusters - 1) / clusters;  // the narrowest tile that leaves no more clusters
         if (g > kMlMaxGranules) continue;
-        const int order = g * best_s - best_g * s;  // < 0: fewer granules per block
-        if (found && (order > 0 || (order == 0 && std::abs(s - 5) >= std::abs(best_s - 5)))) continue;
-        found = true;
+        const float T = static_cast<float>(a.T), warps = static_cast<float>(kGemvWarps / g);  // that share a granule's list
+        const float cost = static_cast<float>(a.K) / s * (100.0f / warps + T) + T * (300.0f * g + 100.0f * s);
+        if (cost >= least) continue;
+        least = cost;
         best_s = s;
         best_g = g;
     }

@@ -282,6 +282,14 @@ def test_few_tokens_at_the_edges_of_granules_steps_and_passes(K, N, T, n, dt):
     assert bool(((y.double() - 0.25 - xa @ w).abs() <= bound).all())
 
 
+@pytest.mark.parametrize("T", [2, 8])
+@pytest.mark.parametrize("K,N", [(1024, 1024), (1024, 10240), (1024, 16376), (1024, 20480), (1024, 32768), (2048, 20488),
+                                 (2048, 32768), (5120, 14344), (5120, 20480)])
+def test_few_tokens_over_shapes_of_tiles_and_clusters(K, N, T):
+    """Sizes whose tiles have one to five granules and whose clusters have one to nine blocks."""
+    test_few_tokens_at_the_edges_of_granules_steps_and_passes(K, N, T, K * 5 // 8 + 3, "bf16")
+
+
 def test_last_row_of_an_operator_of_64_gib():
     """Row offsets are 32-bit counts of 16 bytes: 2^32 of them make up the largest operator, and its last row takes part
     like any other, in the calls over a list and in the operator that selects."""
