@@ -82,6 +82,10 @@ constexpr int kSlSplitMinK = 6144;
 // 2048 -> 2048 5.5, 5.0, 4096 -> 2048 7.4, 7.0, 16384 -> 2048 15.9, 15.2; below, a list is short enough for few SMs:
 // 512 -> 1376 3.9, 4.0, 1024 -> 1024 4.2, 4.2, 4.3.
 constexpr int kSlFineMinK = 1536, kSlFineMaxN = 2336;  // (73 granules of four pieces and the block of the side outputs)
+// Top-k operators of 16-bit inputs on 1024 threads where a thread takes seven or eight rows: all of them in flight instead
+// of six and then the rest.  us, eight rows in flight always, six, and now, half of the channels kept: 2048 -> 5632 7.0,
+// 7.2, 6.7, 4096 -> 4096 8.0, 8.1, 7.7, 2048 -> 8192 7.4, 7.7, 7.2; 40 %: 4096 -> 4096 7.5, 7.6, 7.3.  More rows than
+// eight lose with two passes of eight what three of six cost (13 rows, 4096 -> 6144: 9.6 and 9.1).
 // Selecting warps and slots: as few warps as leave a lane enough registers.
 template <int DT, int IN, int EP, bool GRP>
 static afx_status launch_slice_k(const FusedArgs& a, cudaStream_t st) {
@@ -100,6 +104,14 @@ static afx_status launch_slice_k(const FusedArgs& a, cudaStream_t st) {
     }
     if (narrow && a.K <= 4096) return launch_slice<DT, 512, 8, 4, IN, EP, GRP>(a, st);
     if (narrow && a.K <= 12288) return launch_slice<DT, 512, 16, 6, IN, EP, GRP>(a, st);
+    if constexpr (!GRP && IN == IN_X && EP != EP_SILU) {
+        const int granules = (a.N / 8 + kSlGranule - 1) / kSlGranule, sms = (sm_count() > 1 ? sm_count() : 148) - 1;
+        const int rows = 1024 / (kSlGranule * ((granules + sms - 1) / sms));  // list entries the widest slice takes at once
+        if (a.idx_in == nullptr && a.mode == AFX_MODE_TOPK && a.k > 6 * rows && a.k <= kSlDeepRows * rows) {
+            if (a.K <= 4096) return launch_slice<DT, 1024, 8, 4, IN, EP, GRP, SLICE_DEEP>(a, st);
+            if (a.K <= 12288) return launch_slice<DT, 1024, 16, 6, IN, EP, GRP, SLICE_DEEP>(a, st);
+        }
+    }
     if (a.K <= 4096) return launch_slice<DT, 1024, 8, 4, IN, EP, GRP>(a, st);
     if (a.K <= 12288) return launch_slice<DT, 1024, 16, 6, IN, EP, GRP>(a, st);
     if (a.K <= 16384) return launch_slice<DT, 1024, 16, 8, IN, EP, GRP>(a, st);

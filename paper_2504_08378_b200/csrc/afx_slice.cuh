@@ -26,8 +26,10 @@
 namespace afx {
 
 constexpr int kSlGranule = 4;  // pieces (16-byte loads of a row) that one slice holds together
-// SLICE_SPLIT: the blocks of a cluster share a granule's list; SLICE_FINE: granules of fewer pieces (FusedArgs::granule).
-enum { SLICE_PLAIN = 0, SLICE_SPLIT = 1, SLICE_FINE = 2 };
+// SLICE_SPLIT: the blocks of a cluster share a granule's list; SLICE_FINE: granules of fewer pieces (FusedArgs::granule);
+// SLICE_DEEP: kSlDeepRows rows in flight.
+constexpr int kSlDeepRows = 8;
+enum { SLICE_PLAIN = 0, SLICE_SPLIT = 1, SLICE_FINE = 2, SLICE_DEEP = 3 };
 // Shared memory that at least one block of 512 threads asks for, so that an SM takes one such block and
 // what it leaves free goes to a block of another kernel.
 constexpr size_t kSlAlone = 116 * 1024;
@@ -50,11 +52,10 @@ __host__ __device__ inline size_t slice_dyn_smem(int threads, int K, bool list_g
     return slice_list_bytes(threads, K) + (list_given ? (static_cast<size_t>(K) + 7) / 8 * 16 : 0);
 }
 
-// Streams list entries [0, cnt) for one piece: acc += x * W[channel][8 outputs].
-template <int DT>
+// Streams list entries [0, cnt) for one piece, U of them in flight: acc += x * W[channel][8 outputs].
+template <int DT, int U>
 __device__ __forceinline__ void slice_stream(const uint16_t* Wt, int64_t ldw, int piece, const uint32_t* list, int cnt, int g,
                                              int groups, f32x2 (&acc)[4]) {
-    constexpr int U = 6;
     const char* base = reinterpret_cast<const char*>(Wt + static_cast<size_t>(piece) * 8);
     const uint64_t row = static_cast<uint64_t>(ldw) * 2;
     auto consume = [&](const uint4& raw, uint32_t e) {
@@ -216,7 +217,7 @@ __device__ __forceinline__ void slice_op_block(const FusedArgs& a, unsigned char
 #pragma unroll
     for (int i = 0; i < 4; ++i) acc[i] = pack_f32x2(0.0f, 0.0f);
     const int c_lo = SPLIT ? rank * cnt / split : 0, c_hi = SPLIT ? (rank + 1) * cnt / split : cnt;
-    if (g < rows) slice_stream<DT>(Wt, a.ldw, piece0 + piece, list + c_lo, c_hi - c_lo, g, rows, acc);
+    if (g < rows) slice_stream<DT, FORM == SLICE_DEEP ? kSlDeepRows : 6>(Wt, a.ldw, piece0 + piece, list + c_lo, c_hi - c_lo, g, rows, acc);
     AFX_MARK(5);
 
     slice_finish<DT, NT, EP, SPLIT, FINE>(acc, g, rows, P, piece0, dyn, recv, y, out_bits, scale, y_old);

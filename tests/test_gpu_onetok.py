@@ -133,6 +133,28 @@ def test_one_token_on_slices_of_fewer_pieces(K, N):
             assert int(count) == k and np.array_equal(idx[:k].cpu().numpy(), want)
 
 
+@pytest.mark.parametrize("dt", ["bf16", "f16"])
+@pytest.mark.parametrize("K,N,rows", [(2304, 4096, 256), (4096, 4072, 256), (2304, 5632, 128), (1200, 7272, 128), (8192, 4096, 256)])
+def test_one_token_where_all_rows_of_a_thread_are_in_flight(K, N, rows, dt):
+    """Lists of six rows per thread, just above, eight, and just above; stored and added."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(K + N)
+    td = torch.bfloat16 if dt == "bf16" else torch.float16
+    W = torch.randn(K, N, generator=g, device="cuda").mul_(0.02).to(td)
+    x = torch.randn(K, generator=g, device="cuda").to(td)
+    for k in (6 * rows, 6 * rows + 1, 7 * rows - 3, 8 * rows, 8 * rows + 1):
+        want = oracle.select_active(x.view(torch.int16).cpu().numpy().view(np.uint16)[None], dt, oracle.TOPK, k=k)
+        a = torch.from_numpy(want.astype(np.int64)).cuda()
+        w, xa = W[a].double(), x[a].double()
+        for accumulate in (0, 1):
+            y = torch.full((N,), 0.5, device="cuda")
+            idx, count = torch.zeros(K, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+            afx.afx_select_gemv(W.view(torch.int16), dt, K, N, N, x.view(torch.int16), 1, afx.MODE_TOPK, k, 0.0, y, accumulate, idx, count)
+            bound = (k + 3) * 2.0 ** -24 * (xa.abs() @ w.abs() + 0.5)  # any order of fp32 additions
+            assert bool(((y.double() - 0.5 * accumulate - xa @ w).abs() <= bound).all()), k
+            assert int(count) == k and np.array_equal(idx[:k].cpu().numpy(), want), k
+
+
 @pytest.mark.parametrize("dt,half", [("bf16", 32), ("f16", 128)])
 @pytest.mark.parametrize("K", [160, 4096, 12296])
 @pytest.mark.parametrize("lo,hi", [(0, 40), (0x3C00, 0x3C90), (0x7F00, 0x7F81)])
