@@ -249,6 +249,7 @@ afx_status afx_model_destroy(afx_model* model);
  * active sets of the four operator inputs, and per-layer counters.  The caller allocates
  * afx_state_bytes() of DEVICE memory (256-byte aligned); afx_state_create clears it on
  * `stream` and returns a HOST handle that only records where things live in the blob.
+ * AFX_ERR_UNSUPPORTED: mlp or n_heads * head_dim above 32768, or, with several tokens, hidden.
  */
 size_t afx_state_bytes(const afx_model* model, int T);
 afx_status afx_state_create(const afx_model* model, int T, void* blob, size_t bytes, void* stream,

@@ -1,8 +1,8 @@
-// What a fused sparse operator is given (FusedArgs), and the form of it whose blocks select over a shared-memory
-// histogram: several tokens in one kernel, where the list cannot leave in the caller's memory or the second
-// launch does not pay.  (One token: afx_slice.cuh, afx_q4op.cuh.)
-// Input stage (optional RMSNorm), active-channel selection, sparse GEMV, epilogue in one kernel; every block
-// repeats the exact input stage and selection on its own (the activation vector is a few KB and L2 resident).
+// What a fused sparse operator is given (FusedArgs), and the form of it for several tokens in one kernel, whose clusters
+// select over a shared-memory histogram: where the caller has no room for the list between two launches
+// (afx_seltok.cuh, afx_mtlist.cuh).  (One token: afx_slice.cuh, afx_q4op.cuh.)
+// Active-channel selection, sparse GEMV, epilogue in one kernel; every cluster repeats the exact selection on its own
+// (the activation vectors are a few KB and L2 resident).
 #pragma once
 
 #include "afx_gemv.cuh"
@@ -78,31 +78,26 @@ afx_status launch_q4_operator(int dtype, int in, int ep, const FusedArgs& a, cud
 // Input stage and selection of a.T tokens with the side outputs, as a kernel of its own (afx_seltok.cu).
 afx_status launch_select_tokens(int dtype, bool norm, const FusedArgs& a, cudaStream_t st);
 
-// Dynamic shared memory: [16-bit inputs: T tokens (IN_NORM) or one token (IN_X), each padded
-// to a multiple of 8 elements] [T bitmaps of ceil(K/32) flag words, each padded to 16 bytes: where
-// the blocks of a cluster exchange the per-token sets they decided] [work area: the key
-// histogram during the selection, then the GEMV staging and reduction buffers].
-__host__ __device__ inline size_t fused_input_smem(int in_kind, int K, int T) {
-    const size_t Kp = (static_cast<size_t>(K) + 7) / 8 * 8;
-    return (in_kind == IN_NORM ? static_cast<size_t>(T) : 1) * Kp * 2;
-}
+// Dynamic shared memory: [16-bit inputs of one token, padded to a multiple of 8 elements] [T bitmaps of ceil(K/32) flag
+// words, each padded to 16 bytes: where the blocks of a cluster exchange the per-token sets they decided] [work area:
+// the key histogram during the selection, then the staging and pipeline buffers].
+__host__ __device__ inline size_t fused_input_smem(int K) { return (static_cast<size_t>(K) + 7) / 8 * 16; }
 __host__ __device__ inline size_t fused_flag_smem(int K, int T = 1) {
     return static_cast<size_t>(T) * ((static_cast<size_t>((K + 31) / 32) * 4 + 15) / 16 * 16);
 }
 // work = bytes of the work area: the key histogram, or more where the streaming stage needs more
-__host__ __device__ inline size_t fused_dyn_smem(int in_kind, int K, int T, size_t work = kKeyHistBytes) {
-    return fused_input_smem(in_kind, K, T) + fused_flag_smem(K, T) + (work > kKeyHistBytes ? work : kKeyHistBytes);
+__host__ __device__ inline size_t fused_dyn_smem(int K, int T, size_t work) {
+    return fused_input_smem(K) + fused_flag_smem(K, T) + (work > kKeyHistBytes ? work : kKeyHistBytes);
 }
 
-// The streaming stage runs on the tensor cores (afx_mma.cuh) with STAGES pipeline stages: the work area holds an
-// MtSmem<CAP, STAGES> once the selection is over.
-template <int DT, int TMAX, int CAP, int IN, int EP, int STAGES>
+// Reads a.x, a.mode, a.k, a.tau; a.idx_out and a.count_out are the only side outputs.  The streaming stage runs on the
+// tensor cores (afx_mma.cuh) with STAGES pipeline stages: the work area holds an MtSmem<CAP, STAGES> once the
+// selection is over.
+template <int DT, int TMAX, int CAP, int EP, int STAGES>
 __device__ __forceinline__ void fused_op_block(const FusedArgs& a, unsigned char* dyn, SelectScratch* sel) {
     const int tid = threadIdx.x;
-    const int lane = tid & 31;
-    const int warp = tid >> 5;
     // CS blocks form a cluster; S of them split the active list of one column tile.  CS == S
-    // except for several-token operators with few tiles: there a cluster covers CS / S adjacent
+    // except for operators with few tiles: there a cluster covers CS / S adjacent
     // tiles, so that more blocks share the per-token selections (a.tiles_per_cluster).
     const int CS = gridDim.x, cs = blockIdx.x;
     const int tpc = a.tiles_per_cluster > 1 ? a.tiles_per_cluster : 1;
@@ -111,24 +106,16 @@ __device__ __forceinline__ void fused_op_block(const FusedArgs& a, unsigned char
     const bool side = a.side_cluster != 0 && blockIdx.y == gridDim.y - 1;  // the cluster without a tile
     const int tile = tpc > 1 ? blockIdx.y * tpc + cs / S : blockIdx.y;
     if (side && blockIdx.x != 0) return;  // (a block that has left no longer holds back the next grid)
-    // writes the side outputs: block 0 of the side cluster, else block (0,0) next to its GEMV work
-    const bool scribe = a.side_cluster != 0 ? side : (blockIdx.x == 0 && blockIdx.y == 0);
-    const int nwords = (K + 31) >> 5;
 
-    const int Kp = (K + 7) & ~7;
     uint16_t* xs = reinterpret_cast<uint16_t*>(dyn);
-    unsigned char* work = dyn + fused_input_smem(IN, K, T) + fused_flag_smem(K, T);
+    unsigned char* work = dyn + fused_input_smem(K) + fused_flag_smem(K, T);
     uint32_t* hist = reinterpret_cast<uint32_t*>(work);
-    float* red16 = reinterpret_cast<float*>(sel->hist);  // block reduction of the norm
 
     const uint32_t ld16 = static_cast<uint32_t>(a.ldw >> 3);  // row stride in 16-byte units (the launcher checked the range)
-    const bool own = (a.idx_in == nullptr);
-    const bool topk = own && a.mode == AFX_MODE_TOPK && a.k > 0 && a.k < K;
-    // kernel kinds of a decode step: 1 q|k|v, 2 gate|up, 3 down (the wider plain input), 4 o
-    AFX_TRACE_REGION(IN == IN_NORM ? (EP == EP_SILU ? 2 : 1) : (K > a.N ? 3 : 4));
+    AFX_TRACE_REGION(EP == EP_SILU ? 2 : (K > a.N ? 3 : 4));
     AFX_MARK(0);
     if (!side) cluster_arrive();  // the side cluster never meets
-    if (topk) block_clear_key_hist<kGemvThreads>(hist);  // does not depend on the previous kernel
+    if (a.mode == AFX_MODE_TOPK && a.k > 0 && a.k < K) block_clear_key_hist<kGemvThreads>(hist);  // does not depend on the previous kernel
 
     // Ordering rule of every kernel of this library: a grid lets its successor be scheduled
     // only AFTER its own dependency wait.  When a grid runs its prologue, its predecessor has
@@ -136,228 +123,89 @@ __device__ __forceinline__ void fused_op_block(const FusedArgs& a, unsigned char
     // before the wait below must have been written at least two grids earlier (weights and
     // gains: never; the predicted set: by the same operator of an earlier layer, at least five
     // grids back).  The search hint is the exception: it may be rewritten while it is read.
-    // the norm's gains are weights: they can be on their way before the wait for h
-    constexpr int NH = 4;  // float4 pieces of h (and of the gain) a thread keeps in registers
-    float4 gv[NH];
-    if (IN == IN_NORM) {
-#pragma unroll
-        for (int i = 0; i < NH; ++i) {
-            const int c = tid + i * kGemvThreads;
-            gv[i] = c < (K >> 2) ? reinterpret_cast<const float4*>(a.gain)[c] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        }
-    }
-    // The hints, one per token, are written by an earlier launch of this operator, which may still be
-    // running, and by this launch's own scribe block.  The selection does not depend on them, but all
-    // threads of a block must search from the same one: a single thread reads it, the others
-    // take it from shared memory behind the barrier of the input stage.
-    if (tid < T) {
-        const int32_t* const slot = a.kth_multi != nullptr ? a.kth_multi + tid : nullptr;
-        const uint32_t v = topk && slot != nullptr ? static_cast<uint32_t>(__ldcg(slot)) : 0u;
-        sel->hint[tid] = (v & 0x10000u) ? v & 0x7FFFu : kNoKeyHint;
-    }
-    // likewise the predicted set this selection is compared with: the same operator of the
-    // predictor layer wrote it, at least one layer (five grids) ago (byte v = the flags of the
-    // v-th chunk this thread owns, like `fl`)
-    unsigned long long pm = 0ull;
-    if (scribe && own && a.bitmap_pred != nullptr) {
-        int q_lo, q_hi;
-        thread_chunk_range(K, q_lo, q_hi);
-        const uint8_t* pred = reinterpret_cast<const uint8_t*>(a.bitmap_pred);
-        for (int c = q_lo; c < q_hi; ++c) pm |= static_cast<unsigned long long>(__ldcg(pred + c)) << (8 * (c - q_lo));
-    }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    AFX_MARK(1);
-
-    // ---- input stage --------------------------------------------------------------------
-    if (IN == IN_NORM) {
-        // x = round(h / rms(h) * gain), every block for itself (K % 8 == 0, 16-byte aligned rows)
-        const int nq = K >> 2;
-        for (int t = 0; t < T; ++t) {
-            const float4* ht = reinterpret_cast<const float4*>(a.h + static_cast<size_t>(t) * K);
-            float4 hv[NH];
-            float ss = 0.0f;
-#pragma unroll
-            for (int i = 0; i < NH; ++i) {
-                const int c = tid + i * kGemvThreads;
-                hv[i] = c < nq ? ht[c] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                ss = fmaf(hv[i].x, hv[i].x, ss);
-                ss = fmaf(hv[i].y, hv[i].y, ss);
-                ss = fmaf(hv[i].z, hv[i].z, ss);
-                ss = fmaf(hv[i].w, hv[i].w, ss);
-            }
-            for (int c = tid + NH * kGemvThreads; c < nq; c += kGemvThreads) {
-                const float4 v = ht[c];
-                ss = fmaf(v.x, v.x, ss);
-                ss = fmaf(v.y, v.y, ss);
-                ss = fmaf(v.z, v.z, ss);
-                ss = fmaf(v.w, v.w, ss);
-            }
-            ss = warp_sum(ss);
-            if (t > 0) __syncthreads();  // the previous token's sums have been read
-            if (lane == 0) red16[warp] = ss;
-            __syncthreads();
-            float tot = 0.0f;  // the 16 warp sums in warp order, read four at a time
-#pragma unroll
-            for (int w = 0; w < kGemvWarps; w += 4) {
-                const float4 v = *reinterpret_cast<const float4*>(red16 + w);
-                tot += v.x;
-                tot += v.y;
-                tot += v.z;
-                tot += v.w;
-            }
-            const float inv = 1.0f / sqrtf(tot / static_cast<float>(K) + a.eps);
-            const float4* gq = reinterpret_cast<const float4*>(a.gain);
-            auto emit = [&](int c, const float4& v, const float4& g) {
-                const uint32_t lo = static_cast<uint32_t>(float_to_bits<DT>(v.x * inv * g.x)) |
-                                    (static_cast<uint32_t>(float_to_bits<DT>(v.y * inv * g.y)) << 16);
-                const uint32_t hi = static_cast<uint32_t>(float_to_bits<DT>(v.z * inv * g.z)) |
-                                    (static_cast<uint32_t>(float_to_bits<DT>(v.w * inv * g.w)) << 16);
-                reinterpret_cast<uint2*>(xs + static_cast<size_t>(t) * Kp)[c] = make_uint2(lo, hi);
-                if (scribe && a.xnorm_out != nullptr)
-                    reinterpret_cast<uint2*>(a.xnorm_out + static_cast<size_t>(t) * K)[c] = make_uint2(lo, hi);
-            };
-#pragma unroll
-            for (int i = 0; i < NH; ++i) {
-                const int c = tid + i * kGemvThreads;
-                if (c < nq) emit(c, hv[i], gv[i]);
-            }
-            for (int c = tid + NH * kGemvThreads; c < nq; c += kGemvThreads) emit(c, ht[c], gq[c]);
-        }
-        __syncthreads();
-    }
-    // 16-bit input of token t, channel j, once the stage above / below has run
-    auto x_at = [&](int t, int j) -> uint16_t {
-        if (IN == IN_NORM) return xs[static_cast<size_t>(t) * Kp + j];
-        return a.x[static_cast<size_t>(t) * K + j];
-    };
     AFX_MARK(2);
 
     // ---- selection ----------------------------------------------------------------------
-    int cnt = 0;
-    int pos0 = 0;                  // list position of this thread's first active channel
-    unsigned long long fl = 0ull;  // this thread's active flags (own selection)
-    // Several tokens: the blocks of a cluster share the work -- block s decides the sets of the
+    unsigned long long fl = 0ull;  // this thread's active flags
+    // The blocks of a cluster share the work -- block s decides the sets of the
     // tokens t with t % CS == cs and writes their flags into every block's table of per-token
     // bitmaps (distributed shared memory); after one cluster barrier every thread reads the
     // union for its own chunks.  (The side cluster works alone and decides every token.)
-    const bool share = own && !side && CS > 1;
-    uint8_t* const ftab = dyn + fused_input_smem(IN, K, T);
+    const bool share = !side && CS > 1;
+    uint8_t* const ftab = dyn + fused_input_smem(K);
     const size_t fstride = fused_flag_smem(K);
-    if (own) {
-        if (share) cluster_wait();  // pairs with the cluster_arrive() at kernel start: the peers are running
-        bool first = true;
-        for (int t = 0; t < T; ++t) {
-            if (share && t % CS != cs) continue;
-            const uint16_t* xt = xs + (IN == IN_NORM ? static_cast<size_t>(t) * Kp : 0);
-            if (IN == IN_X) {
-                if (!first) __syncthreads();  // the previous token's keys are still being read
-                block_stage_token(a.x + static_cast<size_t>(t) * K, K, xs);
-            }
-            uint32_t thr_t = 0;
-            const unsigned long long ft =
-                block_token_flags<DT, kGemvThreads>(xt, K, a.mode, a.k, a.tau, hist, first, sel, sel->hint[t], &thr_t);
-            if (scribe && tid == 0 && topk && a.kth_multi != nullptr) a.kth_multi[t] = 0x10000 | thr_t;
-            if (share) {
-                int q_lo, q_hi;
-                thread_chunk_range(K, q_lo, q_hi);
-                for (int q = 0; q < CS; ++q) {
-                    uint8_t* dst = cg::this_cluster().map_shared_rank(ftab + static_cast<size_t>(t) * fstride, q);
-                    for (int c = q_lo; c < q_hi; ++c) dst[c] = static_cast<uint8_t>(ft >> (8 * (c - q_lo)));
-                }
-            } else {
-                fl |= ft;
-            }
-            first = false;
-        }
+    int q_lo, q_hi;
+    thread_chunk_range(K, q_lo, q_hi);
+    if (share) cluster_wait();  // pairs with the cluster_arrive() at kernel start: the peers are running
+    bool first = true;
+    for (int t = 0; t < T; ++t) {
+        if (share && t % CS != cs) continue;
+        if (!first) __syncthreads();  // the previous token's keys are still being read
+        block_stage_token(a.x + static_cast<size_t>(t) * K, K, xs);
+        const unsigned long long ft = block_token_flags<DT, kGemvThreads>(xs, K, a.mode, a.k, a.tau, hist, first, sel);
         if (share) {
-            cluster_arrive();  // the flags written above are visible to the peers after their wait
-            cluster_wait();
-            int q_lo, q_hi;
-            thread_chunk_range(K, q_lo, q_hi);
-            for (int t = 0; t < T; ++t)
-                for (int c = q_lo; c < q_hi; ++c)
-                    fl |= static_cast<unsigned long long>(ftab[static_cast<size_t>(t) * fstride + c]) << (8 * (c - q_lo));
+            for (int q = 0; q < CS; ++q) {
+                uint8_t* dst = cg::this_cluster().map_shared_rank(ftab + static_cast<size_t>(t) * fstride, q);
+                for (int c = q_lo; c < q_hi; ++c) dst[c] = static_cast<uint8_t>(ft >> (8 * (c - q_lo)));
+            }
+        } else {
+            fl |= ft;
         }
-        pos0 = block_prefix(__popcll(fl), sel->wtot[2], cnt);
-    } else {
-        cnt = *a.count_in;
-        cnt = max(0, min(cnt, K));
+        first = false;
     }
-    // ---- side outputs (one block of the grid): plain stores that drain while the block streams ----
-    if (scribe) {
-        if (own) {
-            if (a.idx_out != nullptr) for_each_owned_active(fl, K, pos0, [&](int j, int pos) { a.idx_out[pos] = j; });
-            int q_lo, q_hi;
-            thread_chunk_range(K, q_lo, q_hi);
-            if (a.bitmap_out != nullptr) {  // byte c of the bitmap = the flags of chunk c
-                uint8_t* bytes = reinterpret_cast<uint8_t*>(a.bitmap_out);
-                for (int c = q_lo; c < q_hi; ++c) bytes[c] = static_cast<uint8_t>(fl >> (8 * (c - q_lo)));
-                for (int c = ((K + 7) >> 3) + tid; c < nwords * 4; c += kGemvThreads) bytes[c] = 0;
-            }
-            if (a.bitmap_pred != nullptr) {
-                // A \ P in ascending order, |A & P|
-                const unsigned long long ms = fl & ~pm;
-                int n_miss;
-                const int m0 = block_prefix(__popcll(ms), sel->wtot[3], n_miss);
-                if (a.miss_out != nullptr)
-                    for_each_owned_active(ms, K, m0, [&](int j, int pos) { a.miss_out[pos] = j; });
-                if (tid == 0) {
-                    if (a.miss_count != nullptr) *a.miss_count = n_miss;
-                    if (a.hit_count != nullptr) *a.hit_count = cnt - n_miss;
-                }
-            }
-        } else if (a.idx_out != nullptr && a.idx_out != a.idx_in) {
-            for (int i = tid; i < cnt; i += kGemvThreads) a.idx_out[i] = a.idx_in[i];
-        }
+    if (share) {
+        cluster_arrive();  // the flags written above are visible to the peers after their wait
+        cluster_wait();
+        for (int t = 0; t < T; ++t)
+            for (int c = q_lo; c < q_hi; ++c)
+                fl |= static_cast<unsigned long long>(ftab[static_cast<size_t>(t) * fstride + c]) << (8 * (c - q_lo));
+    }
+    int cnt = 0;
+    const int pos0 = block_prefix(__popcll(fl), sel->wtot[2], cnt);  // list position of this thread's first active channel
+    // ---- side outputs ----
+    if (side) {
+        if (a.idx_out != nullptr) for_each_owned_active(fl, K, pos0, [&](int j, int pos) { a.idx_out[pos] = j; });
         if (tid == 0 && a.count_out != nullptr) *a.count_out = cnt;
-        if (side) return;
+        return;
     }
     AFX_MARK(3);
-    const uint16_t* Wt = a.Wt;
     const int c_lo = s * cnt / S;  // S <= 8, cnt <= 2^20: no overflow
     const int c_hi = (s + 1) * cnt / S;
 
     const int n_mine = __popcll(fl);
     using MtT = MtSmem<CAP, STAGES, kFusedMtRows>;
     MtT* mt = reinterpret_cast<MtT*>(work);
-    constexpr int kMtCap = CAP;
     float c4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    const uint4* wtile16 = reinterpret_cast<const uint4*>(Wt + static_cast<size_t>(tile) * kMtTile);
+    const uint4* wtile16 = reinterpret_cast<const uint4*>(a.Wt + static_cast<size_t>(tile) * kMtTile);
     const int n_chunks = max(0, min(kMtTile, a.N - tile * kMtTile)) >> 3;
     // (the last cluster of a grid with several tiles per cluster may hold a block without a
     // tile: it only shares the selections and meets the barriers)
-    for (int c0 = c_lo; n_chunks > 0 && c0 < c_hi; c0 += kMtCap) {
-        const int staged = min(kMtCap, c_hi - c0);
+    for (int c0 = c_lo; n_chunks > 0 && c0 < c_hi; c0 += CAP) {
+        const int staged = min(CAP, c_hi - c0);
         __syncthreads();  // the work area is free: the histogram / the previous pass has been read
-        if (own) {
-            if (pos0 < c0 + staged && pos0 + n_mine > c0) {
-                for_each_owned_active(fl, K, pos0, [&](int j, int pos) {
-                    const int p = pos - c0;
-                    if (p >= 0 && p < staged) {
-                        mt->col[p] = static_cast<uint32_t>(j) * ld16;
+        if (pos0 < c0 + staged && pos0 + n_mine > c0) {
+            for_each_owned_active(fl, K, pos0, [&](int j, int pos) {
+                const int p = pos - c0;
+                if (p >= 0 && p < staged) {
+                    uint16_t xv[TMAX];  // (all on their way before the first store)
 #pragma unroll
-                        for (int t = 0; t < TMAX; ++t)
-                            if (t < T) mt->xb[t][p] = x_at(t, j);
-                    }
-                });
-            }
-        } else {
-            for (int i = tid; i < staged; i += kGemvThreads) {
-                const int j = a.idx_in[c0 + i];
-                mt->col[i] = static_cast<uint32_t>(j) * ld16;
+                    for (int t = 0; t < TMAX; ++t)
+                        if (t < T) xv[t] = a.x[static_cast<size_t>(t) * K + j];
+                    mt->col[p] = static_cast<uint32_t>(j) * ld16;
 #pragma unroll
-                for (int t = 0; t < TMAX; ++t)
-                    if (t < T) mt->xb[t][i] = x_at(t, j);
-            }
+                    for (int t = 0; t < TMAX; ++t)
+                        if (t < T) mt->xb[t][p] = xv[t];
+                }
+            });
         }
         mt_pad_inputs(mt, T, staged);
         __syncthreads();
         mt_stream_pass<DT>(wtile16, mt, staged, n_chunks, c4);
     }
-    EpilogueArgs ep = a.ep;
     if (!share) cluster_wait();  // pairs with the cluster_arrive() at kernel start
-    mt_finish<DT>(c4, mt, T, tile, a.N, EP, ep, S, s, cs - s);
+    mt_finish<DT>(c4, mt, T, tile, a.N, EP, a.ep, S, s, cs - s);
     AFX_MARK(7);
 }
 

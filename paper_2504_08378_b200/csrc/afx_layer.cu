@@ -18,23 +18,20 @@ template <int TMAX>
 struct FusedMtCap {
     static constexpr int value = TMAX <= 4 ? 4096 : 1024;  // (multiples of kFusedMtRows)
 };
-// CAPM staged entries per pass, STAGES pipeline stages, BPS blocks per SM.
-template <int DT, int TMAX, int IN, int EP, int STAGES, int CAPM, int BPS>
-__global__ void __launch_bounds__(kGemvThreads, BPS) fused_mt_kernel(FusedArgs a) {
+// CAPM staged entries per pass, STAGES pipeline stages.
+template <int DT, int TMAX, int EP, int STAGES, int CAPM>
+__global__ void __launch_bounds__(kGemvThreads, 1) fused_mt_kernel(FusedArgs a) {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ SelectScratch sel;
-    fused_op_block<DT, TMAX, CAPM, IN, EP, STAGES>(a, dyn, &sel);
+    fused_op_block<DT, TMAX, CAPM, EP, STAGES>(a, dyn, &sel);
 }
 
-template <int DT, int TMAX, int IN, int EP, int STAGES, int CAPM, int BPS>
+template <int DT, int TMAX, int EP, int STAGES, int CAPM>
 static afx_status launch_fused_mt_st(const FusedArgs& a, cudaStream_t st) {
-    const void* kern = reinterpret_cast<const void*>(fused_mt_kernel<DT, TMAX, IN, EP, STAGES, CAPM, BPS>);
-    const size_t dyn = fused_dyn_smem(IN, a.K, a.T, sizeof(MtSmem<CAPM, STAGES, kFusedMtRows>));
+    const void* kern = reinterpret_cast<const void*>(fused_mt_kernel<DT, TMAX, EP, STAGES, CAPM>);
+    const size_t dyn = fused_dyn_smem(a.K, a.T, sizeof(MtSmem<CAPM, STAGES, kFusedMtRows>));
     FusedArgs b = a;
-    b.side_cluster = (a.idx_out != nullptr || a.count_out != nullptr || a.bitmap_out != nullptr ||
-                      a.xnorm_out != nullptr || a.bitmap_pred != nullptr || a.kth_slot != nullptr ||
-                      a.kth_multi != nullptr)
-                         ? 1 : 0;
+    b.side_cluster = a.idx_out != nullptr || a.count_out != nullptr;
     const int tiles = (a.N + kMtTile - 1) / kMtTile;
     if (tiles + b.side_cluster > 65535) return AFX_ERR_CAPACITY;
     const int margin = (tiles + 15) / 16 < 2 ? 2 : (tiles + 15) / 16;
@@ -45,19 +42,18 @@ static afx_status launch_fused_mt_st(const FusedArgs& a, cudaStream_t st) {
             break;
         }
     // Few tiles leave the clusters smaller than the number of tokens: let a cluster cover several
-    // adjacent tiles, so that its blocks share the per-token selections (own selection only).
+    // adjacent tiles, so that its blocks share the per-token selections.
     int tpc = 1;
-    if (a.idx_in == nullptr)
-        for (int t2 = 8; t2 > 1; t2 >>= 1) {
-            const int cs = S * t2, rows2 = (tiles + t2 - 1) / t2 + b.side_cluster;
-            if (cs <= kMaxCluster && cs <= 2 * a.T && max_active_clusters(kern, cs, dyn) >= rows2 + (margin + t2 - 1) / t2) {
-                tpc = t2;
-                break;
-            }
+    for (int t2 = 8; t2 > 1; t2 >>= 1) {
+        const int cs = S * t2, rows2 = (tiles + t2 - 1) / t2 + b.side_cluster;
+        if (cs <= kMaxCluster && cs <= 2 * a.T && max_active_clusters(kern, cs, dyn) >= rows2 + (margin + t2 - 1) / t2) {
+            tpc = t2;
+            break;
         }
+    }
     b.tiles_per_cluster = tpc;
     const int rows = (tiles + tpc - 1) / tpc + b.side_cluster;
-    return launch_clustered(fused_mt_kernel<DT, TMAX, IN, EP, STAGES, CAPM, BPS>, S * tpc, rows, dyn, b, st);
+    return launch_clustered(fused_mt_kernel<DT, TMAX, EP, STAGES, CAPM>, S * tpc, rows, dyn, b, st);
 }
 
 // One block per SM (the inputs of several tokens and the tensor-core buffers fill its shared
@@ -65,14 +61,14 @@ static afx_status launch_fused_mt_st(const FusedArgs& a, cudaStream_t st) {
 // with the buffers inside the histogram's 64 KB -- 512 staged entries per pass, 3 stages, twice
 // as many blocks to share the per-token selections -- measured slower: 295 instead of 255 us per
 // 13B layer at 4 tokens.)
-template <int DT, int TMAX, int IN, int EP>
+template <int DT, int TMAX, int EP>
 static afx_status launch_fused_mt(const FusedArgs& a, cudaStream_t st) {
     if (static_cast<uint64_t>(a.K) * static_cast<uint64_t>(a.ldw >> 3) > 0x100000000ull) return AFX_ERR_CAPACITY;
     constexpr int kCap1 = FusedMtCap<TMAX>::value;
-    if (fused_dyn_smem(IN, a.K, a.T, sizeof(MtSmem<kCap1, kFusedMtStages, kFusedMtRows>)) <= kMaxDynSmem)
-        return launch_fused_mt_st<DT, TMAX, IN, EP, kFusedMtStages, kCap1, 1>(a, st);
-    if (fused_dyn_smem(IN, a.K, a.T, sizeof(MtSmem<kCap1, kFusedMtStagesSmall, kFusedMtRows>)) <= kMaxDynSmem)
-        return launch_fused_mt_st<DT, TMAX, IN, EP, kFusedMtStagesSmall, kCap1, 1>(a, st);
+    if (fused_dyn_smem(a.K, a.T, sizeof(MtSmem<kCap1, kFusedMtStages, kFusedMtRows>)) <= kMaxDynSmem)
+        return launch_fused_mt_st<DT, TMAX, EP, kFusedMtStages, kCap1>(a, st);
+    if (fused_dyn_smem(a.K, a.T, sizeof(MtSmem<kCap1, kFusedMtStagesSmall, kFusedMtRows>)) <= kMaxDynSmem)
+        return launch_fused_mt_st<DT, TMAX, EP, kFusedMtStagesSmall, kCap1>(a, st);
     return AFX_ERR_CAPACITY;
 }
 
@@ -107,11 +103,12 @@ static afx_status launch_split(const FusedArgs& a, cudaStream_t st) {
 template <int DT, int IN, int EP>
 static afx_status launch_fused_dt(const FusedArgs& a, cudaStream_t st) {
     if (a.T <= 1) return launch_one_token(DT, IN, EP, ONE_TOKEN_PLAIN, a, st);
-    const bool listed = a.idx_in != nullptr || (a.idx_out != nullptr && a.count_out != nullptr);
-    if (listed && (IN == IN_X || a.xnorm_out != nullptr) && a.K <= kSelectFastMaxK)
+    if constexpr (IN == IN_NORM) {  // (layer operators: the state holds the list and the normed input)
         return launch_split<DT, IN, EP>(a, st);
-    if (a.T <= 4) return launch_fused_mt<DT, 4, IN, EP>(a, st);
-    return launch_fused_mt<DT, 8, IN, EP>(a, st);
+    } else {
+        if (a.idx_in != nullptr || (a.idx_out != nullptr && a.count_out != nullptr)) return launch_split<DT, IN, EP>(a, st);
+        return a.T <= 4 ? launch_fused_mt<DT, 4, EP>(a, st) : launch_fused_mt<DT, 8, EP>(a, st);
+    }
 }
 
 template <int IN, int EP>
@@ -254,12 +251,8 @@ extern "C" afx_status afx_state_create(const afx_model* model, int T, void* blob
         delete s;
         return AFX_ERR_CAPACITY;
     }
-    // the widest input stage must fit one block's shared memory
-    const size_t dyn_max = afx::fused_dyn_smem(
-        afx::IN_NORM, model->d.hidden, T,
-        T > 4 ? sizeof(afx::MtSmem<afx::FusedMtCap<8>::value, afx::kFusedMtStagesSmall, afx::kFusedMtRows>)
-              : (T > 1 ? sizeof(afx::MtSmem<afx::FusedMtCap<4>::value, afx::kFusedMtStagesSmall, afx::kFusedMtRows>) : 0));
-    if (dyn_max > afx::kMaxDynSmem || model->d.mlp > afx::kSelectFastMaxK ||
+    // what an operator of several tokens selects from (a one-token operator refuses more channels itself)
+    if ((T > 1 && model->d.hidden > afx::kSelectFastMaxK) || model->d.mlp > afx::kSelectFastMaxK ||
         model->d.n_heads * model->d.head_dim > afx::kSelectFastMaxK) {
         delete s;
         return AFX_ERR_UNSUPPORTED;

@@ -154,16 +154,12 @@ __device__ __forceinline__ void mt_pad_inputs(SMT* sm, int T, int staged) {
 // EP_SILU as in gemv_finish_tile).  Every thread of every block of the cluster calls it; no
 // cluster barrier arrival may be pending.
 // S blocks of the cluster, ranks base .. base + S - 1, worked on this tile; the caller is the
-// rank-th of them (S < 0: the whole cluster).
+// rank-th of them.
 template <int DT, class SMT>
 __device__ __forceinline__ void mt_finish(const float (&c)[4], SMT* sm, int T, int tile, int N, int ep_kind,
-                                          const EpilogueArgs& ep, int S = -1, int rank = 0, int base = 0) {
+                                          const EpilogueArgs& ep, int S, int rank, int base) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
-    if (S < 0) {
-        S = static_cast<int>(cluster.num_blocks());
-        rank = static_cast<int>(cluster.block_rank());
-    }
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     __syncthreads();  // the last stage has been multiplied by everybody
     float* part = reinterpret_cast<float*>(sm->w[0]);  // [8 tokens][kMtPartStride]

@@ -26,11 +26,10 @@ constexpr int kKeyHistWords = 16384;    // 32768 16-bit counters
 constexpr size_t kKeyHistBytes = static_cast<size_t>(kKeyHistWords) * 4;
 
 struct SelectScratch {
-    int wtot[4][32];  // per-warp totals for the ordered scans
+    int wtot[3][32];  // per-warp totals for the ordered scans
     int res[4];       // broadcast of the k-th key search
-    __align__(16) int hist[256];  // large-K path; the fused operators borrow it for the norm's reduction
+    int hist[256];    // large-K path
     int scan[33];
-    uint32_t hint[AFX_MAX_T];  // the fused operators: where each token's search starts
 };
 
 // Words [w0, w1) of a ceil(K/32)-word bitmap owned by the calling warp (contiguous, so that
@@ -217,132 +216,14 @@ __device__ __forceinline__ void block_kth_key(const uint16_t* xs, int K, int k, 
     tot_eq = s->res[2];
 }
 
-// Keys searched around a hint of the k-th key: about +-19 % in magnitude for either type.
-template <int DT>
-struct KeyWindow {
-    static constexpr int kBins = DT == AFX_BF16 ? 64 : 512;
-};
-constexpr uint32_t kNoKeyHint = 0xFFFFFFFFu;
-
-// block_kth_key with a hint (a key near the expected answer, e.g. the one found for the
-// previous token): counts the keys above a window of KeyWindow<DT>::kBins keys around the hint
-// and histograms only the keys inside it -- two masked compares per word and a few
-// uncontended atomics instead of one atomic per key, and one warp resolves the window.
-// Exact whenever it returns true; returns false (same value in every thread, outputs
-// untouched, `hist` clean again) when the k-th key lies outside the window.  `hist` as for
-// block_kth_key; words [0, kBins) are left dirty and may be rewritten only after the block's
-// next barrier (the warps read them at their own pace).
-template <int DT, int NT>
-__device__ __forceinline__ bool block_kth_key_near(const uint16_t* xs, int K, int k, uint32_t hint,
-                                                   uint32_t* hist, SelectScratch* s, uint32_t& thr,
-                                                   int& need_eq, int& tot_eq) {
-    constexpr int WB = KeyWindow<DT>::kBins;
-    constexpr int P = WB / 32;  // bins per lane of the resolving warp
-    static_assert(P == 2 || P % 4 == 0, "window bins per lane: 2 or a multiple of 4");
-    const int lane = lane_id();
-    const int lo = max(0, min(static_cast<int>(hint & 0x7FFFu) - WB / 2, 32768 - WB));
-    // swar_gt(keys, pair(v)) marks keys >= v (it tests key > v - 1); lo + WB <= 0x8000 keeps
-    // the subtraction inside its half
-    const uint32_t lo2 = swar_pair(static_cast<uint32_t>(lo)), hi2 = swar_pair(static_cast<uint32_t>(lo + WB));
-    int c_lo, c_hi;
-    thread_chunk_range(K, c_lo, c_hi);
-    int above = 0;
-    for (int c = c_lo; c < c_hi; ++c) {
-        const uint4 raw = *reinterpret_cast<const uint4*>(xs + (c << 3));
-        const uint32_t r[4] = {raw.x & 0x7FFF7FFFu, raw.y & 0x7FFF7FFFu, raw.z & 0x7FFF7FFFu, raw.w & 0x7FFF7FFFu};
-        const int nvalid = K - (c << 3);
-        uint32_t am = 0;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const uint32_t a = swar_gt(r[i], hi2);
-            uint32_t in = swar_gt(r[i], lo2) & ~a;
-            // the zero padding of a partial last chunk would fall into a window that starts at 0
-            if (nvalid < 8) in &= (2 * i < nvalid ? 0x8000u : 0u) | (2 * i + 1 < nvalid ? 0x80000000u : 0u);
-            am |= a >> i;
-            if (in & 0x8000u) atomicAdd(&hist[(r[i] & 0xFFFFu) - lo], 1u);
-            if (in & 0x80000000u) atomicAdd(&hist[(r[i] >> 16) - lo], 1u);
-        }
-        above += __popc(am);
-    }
-    AFX_MARK(11);
-    above = __reduce_add_sync(0xFFFFFFFFu, above);
-    if (lane == 0) s->wtot[0][warp_id()] = above;
-    AFX_MARK(12);
-    __syncthreads();
-    AFX_MARK(13);
-    // Every warp resolves the window for itself from the same counters: nothing to broadcast.
-    constexpr int NW = NT / 32;
-    const int ab = __reduce_add_sync(0xFFFFFFFFu, lane < NW ? s->wtot[0][lane] : 0);
-    uint32_t cnt[P];
-    if (P == 2) {
-        const uint2 v = *reinterpret_cast<const uint2*>(hist + lane * 2);
-        cnt[0] = v.x;
-        cnt[1] = v.y;
-    } else {
-#pragma unroll
-        for (int q = 0; q < P / 4; ++q) {
-            const uint4 v = *reinterpret_cast<const uint4*>(hist + lane * P + q * 4);
-            cnt[4 * q] = v.x;
-            cnt[4 * q + 1] = v.y;
-            cnt[4 * q + 2] = v.z;
-            cnt[4 * q + 3] = v.w;
-        }
-    }
-    int lane_sum = 0;
-#pragma unroll
-    for (int q = 0; q < P; ++q) lane_sum += static_cast<int>(cnt[q]);
-    int suf = lane_sum;  // inclusive suffix sums: higher lanes hold higher keys
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int n = __shfl_down_sync(0xFFFFFFFFu, suf, o);
-        if (lane + o < 32) suf += n;
-    }
-    const int inside = __shfl_sync(0xFFFFFFFFu, suf, 0);
-    if (!(ab < k && k <= ab + inside)) {  // same outcome in every warp
-        __syncthreads();                  // every warp has read the window
-        for (int i = threadIdx.x; i < WB; i += NT) hist[i] = 0u;
-        __syncthreads();
-        return false;
-    }
-    int rem = k - ab;  // rank from the top inside the window
-    const uint32_t has = __ballot_sync(0xFFFFFFFFu, suf >= rem);
-    const int l_star = 31 - __clz(static_cast<int>(has));
-    int my_thr = 0, my_need = 0, my_tot = 0;
-    if (lane == l_star) {
-        rem -= suf - lane_sum;
-        bool done = false;
-#pragma unroll
-        for (int q = P - 1; q >= 0; --q) {
-            const int cq = static_cast<int>(cnt[q]);
-            if (!done) {
-                if (rem <= cq) {
-                    done = true;
-                    my_thr = lo + lane * P + q;
-                    my_need = rem;
-                    my_tot = cq;
-                } else {
-                    rem -= cq;
-                }
-            }
-        }
-        if (warp_id() == 0) s->res[0] = my_thr;  // for the caller that records the key
-    }
-    thr = static_cast<uint32_t>(__shfl_sync(0xFFFFFFFFu, my_thr, l_star));
-    need_eq = __shfl_sync(0xFFFFFFFFu, my_need, l_star);
-    tot_eq = __shfl_sync(0xFFFFFFFFu, my_tot, l_star);
-    return true;
-}
-
 // Active flags of ONE token for the calling thread's chunks: byte v of the result covers the
 // 8 channels of chunk c_lo + v (bit e = channel 8 * (c_lo + v) + e).  xs as for
 // block_kth_key.  `hist` is the key histogram (top-k only); `hist_clean` says that it is
-// already zero and visible.  `hint` (top-k; kNoKeyHint = none) is
-// a guess of the k-th key that shortens the search and never changes the result; `thr_out`
-// (top-k with 0 < k < K) receives the k-th key found, in every thread.
+// already zero and visible.
 template <int DT, int NT>
 __device__ __forceinline__ unsigned long long block_token_flags(const uint16_t* xs, int K, int mode, int k,
                                                                 float tau, uint32_t* hist, bool hist_clean,
-                                                                SelectScratch* s, uint32_t hint, uint32_t* thr_out) {
+                                                                SelectScratch* s) {
     int c_lo, c_hi;
     thread_chunk_range(K, c_lo, c_hi);
     unsigned long long fl = 0ull;
@@ -364,16 +245,13 @@ __device__ __forceinline__ unsigned long long block_token_flags(const uint16_t* 
         }
         return fl;
     }
-    if (!hist_clean) {
-        __syncthreads();  // a hinted search of the previous token may still be read by slower warps
+    if (!hist_clean) {  // (the previous token's search ended with a barrier behind its last read)
         block_clear_key_hist<NT>(hist);
         __syncthreads();
     }
     uint32_t thr;
     int need_eq, tot_eq;
-    if (!(hint != kNoKeyHint && block_kth_key_near<DT, NT>(xs, K, k, hint, hist, s, thr, need_eq, tot_eq)))
-        block_kth_key<NT>(xs, K, k, hist, s, thr, need_eq, tot_eq);
-    *thr_out = thr;
+    block_kth_key<NT>(xs, K, k, hist, s, thr, need_eq, tot_eq);
     AFX_MARK(8);
     // Channels above the k-th key are in; of those equal to it, the need_eq lowest ids.  One
     // pass over the thread's chunks, two keys per operation (swar_*), leaves two flag sets in

@@ -146,6 +146,33 @@ def test_layer_step_every_stage_matches_oracle(dt, T, mode, heads, kvh):
     m.close()
 
 
+@pytest.mark.parametrize("T,hidden,mlp", [(4, 9752, 264), (8, 8488, 264), (2, 16392, 64), (8, 32768, 64)])
+def test_layer_step_of_several_tokens_on_a_wide_model(T, hidden, mlp):
+    """As many channels as the selection takes, whatever the number of tokens."""
+    dt, pos = "bf16", 9
+    cfg = ol.Config(dt, hidden, 1, 1, mlp, mode=oracle.TOPK)
+    k = [synth.keep_count(K, 50) for K in (hidden, 128, hidden, mlp)]
+    L = synth.layer_weights(37, 0, hidden, 1, 1, mlp, dt, gain_jitter=0.1)
+    kc, vc = synth.kv_cache(37, 0, T, 16, 1, pos)
+    L["k"], L["k_cache"], L["v_cache"] = k, kc, vc
+    m = make(cfg, [L], T, afx.MODE_TOPK, max_seq=16)
+    h0 = synth.hidden_state(37, 5, T, hidden, scale=4.0, scales_stream=6)
+    m.h.copy_(torch.from_numpy(h0).cuda())
+    m.layer_step(0, pos)
+    torch.cuda.synchronize()
+    check_layer_stages(cfg, L, oracle_weights(L, k), m, 0, h0, kc, vc, pos, T)
+    m.close()
+
+
+def test_state_of_several_tokens_beyond_the_selection_is_refused():
+    cfg = ol.Config("bf16", 32776, 1, 1, 64, mode=oracle.TOPK)
+    w = torch.zeros(16, dtype=torch.int16, device="cuda")
+    L = dict(w_qkv=w, w_o=w, w_gu=w, w_down=w, g_attn=torch.ones(8, device="cuda"), g_mlp=torch.ones(8, device="cuda"), k=[1] * 4)
+    with pytest.raises(afx.AfxError) as e:
+        make(cfg, [L], 2, afx.MODE_TOPK, max_seq=16)
+    assert e.value.status == 4
+
+
 @pytest.mark.parametrize("xl_mode", [afx.XL_BOOKKEEP, afx.XL_REUSE])
 def test_cross_layer_prediction_matches_oracle_free_running(xl_mode):
     """Four layers, depth 3: free-running GPU vs free-running oracle.  Index sets are compared
