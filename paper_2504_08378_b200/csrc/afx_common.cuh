@@ -38,24 +38,6 @@ __device__ __forceinline__ float bits_to_float(uint16_t bits) {
     }
 }
 
-// Eight packed 16-bit weights (one 128-bit load) to fp32.
-template <int DT>
-__device__ __forceinline__ void unpack8(const uint4& raw, float (&w)[8]) {
-    const uint32_t r[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        if (DT == AFX_F16) {
-            __half2 h = *reinterpret_cast<const __half2*>(&r[i]);
-            float2 f = __half22float2(h);
-            w[2 * i] = f.x;
-            w[2 * i + 1] = f.y;
-        } else {
-            w[2 * i] = __uint_as_float(r[i] << 16);
-            w[2 * i + 1] = __uint_as_float(r[i] & 0xFFFF0000u);
-        }
-    }
-}
-
 // ---- packed fp32 pairs (two-wide fused multiply-add of sm_100) ------------------------
 
 typedef unsigned long long f32x2;  // two fp32 values in one 64-bit register pair (low, high)
@@ -125,9 +107,6 @@ __device__ __forceinline__ uint4 ld_stream_16B(const void* p) {
 }
 
 // ---- warp / block primitives ---------------------------------------------------------
-
-__host__ __device__ __forceinline__ int64_t min64(int64_t a, int64_t b) { return a < b ? a : b; }
-__host__ __device__ __forceinline__ int64_t max64(int64_t a, int64_t b) { return a > b ? a : b; }
 
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 __device__ __forceinline__ int warp_id() { return threadIdx.x >> 5; }

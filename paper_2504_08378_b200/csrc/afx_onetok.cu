@@ -97,10 +97,12 @@ static afx_status launch_slice_k(const FusedArgs& a, cudaStream_t st) {
         if (fit >= 4 && a.K <= 32768) return launch_slice<DT, 1024, 32, 8, IN, EP, GRP, SLICE_SPLIT>(a, st, split);
     }
     const bool narrow = (a.beside_attention && a.K <= kSlNarrowMaxK) || static_cast<int64_t>(a.K) * a.N <= (8 << 20);
-    if (!GRP && a.K >= kSlFineMinK && a.N <= kSlFineMaxN) {
-        if (narrow && a.K <= 4096) return launch_slice<DT, 512, 8, 4, IN, EP, GRP, SLICE_FINE>(a, st);
-        if (narrow && a.K <= 12288) return launch_slice<DT, 512, 16, 6, IN, EP, GRP, SLICE_FINE>(a, st);
-        if (a.K <= 16384) return launch_slice<DT, 1024, 16, 8, IN, EP, GRP, SLICE_FINE>(a, st);
+    if constexpr (!GRP) {
+        if (a.K >= kSlFineMinK && a.N <= kSlFineMaxN) {
+            if (narrow && a.K <= 4096) return launch_slice<DT, 512, 8, 4, IN, EP, GRP, SLICE_FINE>(a, st);
+            if (narrow && a.K <= 12288) return launch_slice<DT, 512, 16, 6, IN, EP, GRP, SLICE_FINE>(a, st);
+            if (a.K <= 16384) return launch_slice<DT, 1024, 16, 8, IN, EP, GRP, SLICE_FINE>(a, st);
+        }
     }
     if (narrow && a.K <= 4096) return launch_slice<DT, 512, 8, 4, IN, EP, GRP>(a, st);
     if (narrow && a.K <= 12288) return launch_slice<DT, 512, 16, 6, IN, EP, GRP>(a, st);

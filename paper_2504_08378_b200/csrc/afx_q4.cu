@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(kQ4Threads, 2) sparse_gemv_q4_kernel(Q4Args a)
         }
         if (lane_ok) q4_stream<LPC>(a.Wq, a.N, half, s_off, s_x, staged, acc);
     }
-    q4_finish<XDT, LPC>(acc, s_red, tile, a.N, a.ep, a.y, a.out_bits);
+    q4_finish<LPC>(acc, s_red, tile, a.N, a.accumulate, a.y);
 }
 
 static size_t q4_dyn_smem(int lpc) {
@@ -127,10 +127,6 @@ static afx_status launch_q4(const Q4Args& a, cudaStream_t st) {
     }
 }
 
-afx_status launch_q4_list(int x_dtype, const Q4Args& a, cudaStream_t st) {
-    return x_dtype == AFX_F16 ? launch_q4<AFX_F16>(a, st) : launch_q4<AFX_BF16>(a, st);
-}
-
 }  // namespace afx
 
 extern "C" size_t afx_q4_row_bytes(int N) {
@@ -159,8 +155,8 @@ extern "C" afx_status afx_sparse_gemv_q4(const void* Wq, int K, int N, int64_t l
     a.idx = idx;
     a.count = count;
     a.y = y;
-    a.ep = accumulate ? Q4_ACCUM : Q4_STORE;
+    a.accumulate = accumulate ? 1 : 0;
     a.status = dev_status;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    return launch_q4_list(x_dtype, a, st);
+    return x_dtype == AFX_F16 ? launch_q4<AFX_F16>(a, st) : launch_q4<AFX_BF16>(a, st);
 }

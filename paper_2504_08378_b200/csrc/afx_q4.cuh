@@ -1,5 +1,5 @@
-// Arguments and launcher of the 4-bit sparse GEMV kernel (afx_q4.cu), shared with the layer
-// step over 4-bit weights (afx_layer.cu).
+// 4-bit blocks to fp32, shared with the layer operators over 4-bit rows (afx_q4op.cuh); streaming loop and reduction of
+// the sparse GEMV over a list (afx_q4.cu).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -18,8 +18,6 @@ constexpr int kQ4Unroll = 8;   // 8-byte loads in flight per lane
 constexpr int kQ4Cap = 1024;   // staged list entries per pass of the list kernel
 constexpr int kQ4Opl = 16;     // outputs per lane and channel: half a block of 32
 
-enum { Q4_STORE = 0, Q4_ACCUM = 1, Q4_SILU = 2 };
-
 struct Q4Args {
     const unsigned char* Wq;
     int64_t ldq;  // row stride in bytes (multiple of 16)
@@ -27,20 +25,10 @@ struct Q4Args {
     const uint16_t* x;
     const int32_t* idx;
     const int32_t* count;
-    // how a finished sum leaves: Q4_STORE y[i] = sum, Q4_ACCUM y[i] += sum; Q4_SILU: every block
-    // of 32 outputs is 16 "gate" outputs (the low 4 bits of its 16 bytes) and 16 "up" outputs
-    // (the high 4 bits), out_bits[16 b + m] = round(silu(gate_m) * up_m) in x's 16-bit type
-    int ep;
+    int accumulate;  // 0: y = sum, 1: y += sum
     float* y;
-    uint16_t* out_bits;
     int32_t* status;
 };
-
-// x_dtype AFX_F16 / AFX_BF16; arguments already validated.
-afx_status launch_q4_list(int x_dtype, const Q4Args& a, cudaStream_t st);
-
-
-// ---- device side: streaming loop and reduction shared by the list kernel and the fused operator ----
 
 __device__ __forceinline__ uint2 ld_stream_8B(const void* p) {
     uint2 v;
@@ -115,12 +103,11 @@ __device__ __forceinline__ void q4_stream(const unsigned char* Wq, int N, int ha
 }
 
 // Meeting of the sums of one tile -- lane groups of a warp, warps of the block, blocks of the
-// cluster, in that fixed order -- and the epilogue `ep` (Q4_*).  s_red: (kQ4Warps + 1) * LPC * 16
+// cluster, in that fixed order.  s_red: (kQ4Warps + 1) * LPC * 16
 // floats of shared memory, free on entry (a block barrier comes first).  Every thread of every
 // block of the cluster calls it; no cluster barrier arrival may be pending.
-template <int XDT, int LPC>
-__device__ __forceinline__ void q4_finish(const f32x2 (&acc)[8], float* s_red, int tile, int N, int ep, float* y,
-                                          uint16_t* out_bits) {
+template <int LPC>
+__device__ __forceinline__ void q4_finish(const f32x2 (&acc)[8], float* s_red, int tile, int N, int accumulate, float* y) {
     namespace cg = cooperative_groups;
     constexpr int PW = LPC * kQ4Opl;
     cg::cluster_group cluster = cg::this_cluster();
@@ -155,30 +142,12 @@ __device__ __forceinline__ void q4_finish(const f32x2 (&acc)[8], float* s_red, i
         part[o] = s;
     }
     cluster.sync();
-    if (ep == Q4_SILU) {
-        // pair r of the tile: gate = output 32 * (r / 16) + r % 16, up = 16 further on
-        constexpr int HP = PW / 2;
-        for (int r = rank + S * tid; r < HP; r += S * kQ4Threads) {
-            const int og = (r >> 4) * 32 + (r & 15);
-            const int m = tile * HP + r;
-            if (2 * m < N) {
-                float g = 0.0f, u = 0.0f;
-                for (int q = 0; q < S; ++q) {
-                    const float* pq = cluster.map_shared_rank(part, q);
-                    g += pq[og];
-                    u += pq[og + 16];
-                }
-                out_bits[m] = float_to_bits<XDT>(g / (1.0f + expf(-g)) * u);
-            }
-        }
-    } else {
-        for (int o = rank + S * tid; o < PW; o += S * kQ4Threads) {
-            const int out = tile * PW + o;
-            if (out < N) {
-                float s = 0.0f;
-                for (int q = 0; q < S; ++q) s += cluster.map_shared_rank(part, q)[o];
-                y[out] = ep == Q4_ACCUM ? y[out] + s : s;
-            }
+    for (int o = rank + S * tid; o < PW; o += S * kQ4Threads) {
+        const int out = tile * PW + o;
+        if (out < N) {
+            float s = 0.0f;
+            for (int q = 0; q < S; ++q) s += cluster.map_shared_rank(part, q)[o];
+            y[out] = accumulate ? y[out] + s : s;
         }
     }
     cluster.sync();  // peers may still be reading this block's sums

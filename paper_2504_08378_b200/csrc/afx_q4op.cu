@@ -31,7 +31,8 @@ static afx_status launch_q4op(const FusedArgs& a, cudaStream_t st) {
     const int split = SPLIT ? kQoSplit : 1;
     int room = sms - b.side_cluster;
     if (SPLIT) {
-        // clusters that the occupancy query counts and that are then placed behind another kernel differ by a few
+        // All clusters that the occupancy query counts (32 on 148 SMs): one, two or three spare ones make the tiles wider
+        // and a layer slower, 8192 channels 122.7 and 125.5 us, 4096 58.3 and 59.2, 2048 37.3 and 38.4.
         const int fit = max_active_clusters(reinterpret_cast<const void*>(kern), split, dyn, NT) - b.side_cluster;
         room = fit < 1 ? 1 : fit;
     }
@@ -70,12 +71,16 @@ constexpr int kQoBesideMaxK = 4096;
 template <int DT, int IN, int EP>
 static afx_status launch_q4op_dt(const FusedArgs& a, cudaStream_t st) {
     if (static_cast<uint64_t>(a.K) * static_cast<uint64_t>(a.ldw >> 3) > 0x100000000ull) return AFX_ERR_CAPACITY;
-    if (IN == IN_X && a.K >= kQoSplitMinK && a.K >= 2 * static_cast<int64_t>(a.N)) {
-        if (a.K <= 16384) return launch_q4op<DT, 512, 16, 8, 4, IN, EP, true>(a, st);
-        if (a.K <= 32768) return launch_q4op<DT, 1024, 32, 8, 2, IN, EP, true>(a, st);
-        return AFX_ERR_CAPACITY;
+    if constexpr (IN == IN_X) {
+        if (a.K >= kQoSplitMinK && a.K >= 2 * static_cast<int64_t>(a.N)) {
+            if (a.K <= 16384) return launch_q4op<DT, 512, 16, 8, 4, IN, EP, true>(a, st);
+            if (a.K <= 32768) return launch_q4op<DT, 1024, 32, 8, 2, IN, EP, true>(a, st);
+            return AFX_ERR_CAPACITY;
+        }
     }
-    if (a.beside_attention && a.K <= kQoBesideMaxK) return launch_q4op<DT, 512, 8, 4, 2, IN, EP, false>(a, st);
+    if constexpr (EP != EP_SILU) {
+        if (a.beside_attention && a.K <= kQoBesideMaxK) return launch_q4op<DT, 512, 8, 4, 2, IN, EP, false>(a, st);
+    }
     if (a.K <= 4096) return launch_q4op<DT, 512, 8, 4, 4, IN, EP, false>(a, st);
     if (a.K <= 16384) return launch_q4op<DT, 512, 16, 8, 4, IN, EP, false>(a, st);
     if (a.K <= 32768) return launch_q4op<DT, 1024, 32, 8, 2, IN, EP, false>(a, st);
