@@ -113,9 +113,8 @@ afx_status afx_diff_active(const int32_t* idxA, const int32_t* cntA, const uint3
  * with col(c) = idx[c], or slot[c] when `slot` is given (the columns then live in a cache
  * whose slot list afx_cache_fetch produced).  Products are exact in fp32; sums are fp32 in
  * a fixed order (same inputs on the same device give the same bits).  One token is multiplied
- * on the fp32 pipe; with 2..8 tokens the active rows are gathered into shared memory and
- * multiplied on the tensor cores (16-bit inputs, fp32 accumulation): the order of the sums, and
- * with it the last bits of y, differ between the two, the rules above hold for both.
+ * on the fp32 pipe, 2..8 tokens on the tensor cores (16-bit inputs, fp32 accumulation): the order of
+ * the sums, and with it the last bits of y, differ between the two, the rules above hold for both.
  *
  *   Wt        DEVICE, channel-contiguous weights (see the conventions above).
  *   x         DEVICE, [T][K] 16-bit floats; every token uses the whole list.
@@ -149,9 +148,9 @@ afx_status afx_sparse_gemv(const void* Wt, int dtype, int K, int N, int64_t ldw,
  *   kth_hint  DEVICE int32[1] or NULL, read and rewritten by a top-k call with T == 1 and
  *             0 < k < K: on return 0x10000 | the k-th largest magnitude key (the 16-bit pattern
  *             with the sign cleared).  A value with bit 16 set that a call finds there is where
- *             its search for the k-th key starts (cheap when the key lies within about 19 % of
- *             it, e.g. the previous token's key for the same operator; the full search
- *             otherwise); 0 means no hint.  The selected set never depends on it.
+ *             its search for the k-th key starts (cheap when the key lies within about 12 % of
+ *             it, 6 % in f16, e.g. the previous token's key for the same operator; a search from
+ *             there outwards otherwise); 0 means no hint.  The selected set never depends on it.
  * T == 1: K * 2 bytes of x are read by every thread block (they stay in L2).
  */
 afx_status afx_select_gemv(const void* Wt, int dtype, int K, int N, int64_t ldw, const void* x, int T,

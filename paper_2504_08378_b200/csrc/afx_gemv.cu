@@ -54,8 +54,8 @@ static int ml_resident(int s) {
 // 1024 -> 16384 14.3 and 11.6, 2048 -> 20480 25.2 and 19.9, 5120 -> 24576 43.0 and 40.9, 5120 -> 16384 31.0 and 29.3;
 // four tokens 5120 -> 14336 27.1 and 26.5, 1024 -> 10240 9.9 and 8.8; two tokens 2048 -> 10240 11.4 and 10.4.
 // Sizes above eight only where whole GPCs hold several of them, and not nine (28 of 30 clusters of nine ran as one wave or
-// two from call to call).  No block with less than a step or so of the list per warp (1024 -> 1024, three tokens: 1 x 5
-// 5.3, 1 x 10 6.1).
+// two from call to call).  No block with less than a step or so of the list per warp (1024 -> 1024, three tokens: 1 x 10
+// 6.1; the rule's 1 x 5 5.0, 2048 -> 1024 with four tokens 5.6).
 template <int DT>
 static afx_status launch_gemm_mt(const GemvListArgs& a, cudaStream_t st) {
     constexpr int kSpare = 8, kMinEntries = 192;

@@ -17,8 +17,10 @@
 // steps per warp, together or one ahead of the other, cost registers that 64 do not hold (5120 -> 27648, four tokens: 57
 // to 68 us; with one block per SM and 128 registers 55 to 70; one step 47).  It replaced stages of 16 channels
 // in shared memory (cp.async, ldmatrix.trans, a block barrier per stage): four tokens 5120 -> 27648 53.6 and 47.1 us,
-// 5120 -> 5120 16.9 and 14.5, 13824 -> 5120 33.1 and 29.1, 5120 -> 15360 30.3 and 31.0; eight tokens 5120 -> 27648 61.8
-// and 53.7; two tokens 8192 -> 57344 132.7 and 122.8; three tokens 5003 -> 7208 17.4 and 15.7.
+// 5120 -> 5120 16.9 and 14.5, 13824 -> 5120 33.1 and 29.1, 5120 -> 15360 (4096 entries) 27.5 and 27.8; eight tokens
+// 5120 -> 27648 61.8 and 53.7; two tokens 8192 -> 57344 132.7 and 122.8; three tokens 5003 -> 7208 17.4 and 15.7.  It
+// loses where few channels meet many outputs, whose blocks have little to stream beside the sums of many granules: eight
+// tokens 2048 -> 20480 17.4 and 19.9, 1024 -> 20480 12.1 and 14.3.
 #pragma once
 
 #include "afx_gemv.cuh"

@@ -7,7 +7,8 @@
 // outputs) of every (NT / threads per piece)-th entry, five (W = 4) or four (W = 2) entries in flight (six and eight: 1 % more).
 //
 // What bounds it: the same chain of latencies as over 16-bit rows (afx_slice.cuh) and, while it streams, instruction
-// issue: three per weight, of which codes to fp32 take 1.4 and the products 0.5.  It replaced clusters of two blocks
+// issue: three per weight, of which codes to fp32 take 1.4 and the products 0.5.  (Over a whole launch, chain included,
+// a gate | up operator of 4096 and 11008 channels issues in 40 % of its cycles, 4.5 instructions per weight.)  It replaced clusters of two blocks
 // per SM that each selected over a shared-memory histogram, two thirds of all instructions; a layer of 4096 and 11008
 // channels over 2048 positions, one token: 81 and 60 us.  Loading an entry's registers again as soon as it has been
 // multiplied, instead of some entries together: 63.

@@ -9,8 +9,8 @@
 // 2299, five 2257, seven 2271).
 //
 // What bounds it: HBM while it streams (a 4096 -> 22016 operator at 50 %: 6.1 TB/s between the first load and
-// the last), and before and after that a chain of latencies in which HBM is idle: dependency wait 1.0 us,
-// input and norm 1.5, search 1.3, list 1.0, sums 0.8 at K = 4096.  Clusters of 3 to 8 blocks of 512 threads,
+// the last), and before and after that a chain of latencies in which HBM is idle: dependency wait 0.2 us,
+// input and norm 1.1, search 0.9, list 0.6, first load 1, sums 0.6 to 1.2 at K = 4096.  Clusters of 3 to 8 blocks of 512 threads,
 // two per SM, that shared a tile ran the input stage and the selection twice per SM, bound by instruction
 // issue, left 6 to 14 SMs without a block and needed a cluster barrier for the sums.  Alone in a
 // graph, before and after: 4096 -> 22016 21.8 and 20.0 us, 4096 -> 4096 9.6 and 8.5, 11008 -> 4096
