@@ -331,3 +331,5 @@ def test_last_row_of_an_operator_of_64_gib():
     per_block = (x[0, rows].double().view(2, 1) * code).sum(0).repeat_interleave(16)
     assert int(status.item()) == 0
     assert torch.equal(y.double(), torch.cat([per_block, 0.5 * per_block]))  # small integers and halves: exact
+    del W, q
+    torch.cuda.empty_cache()
